@@ -218,8 +218,9 @@ int idtx_ctx_set_graphs(idtx_ctx *ctx, int enable);
  *     full scan for a (query, estimate) whose neighbourhood the lists do not
  *     cover.  Needs dz >= 1 (dz = 0 calls use the tile kernel).
  *   IDTX_KERNEL_AUTO (default): on the first call of a shape (kernel
- *     variant, floor(log2 N)) both kernels run, timed, and the faster serves
- *     that shape from then on in this context.
+ *     variant, floor(log2 N)) both kernels run, timed; from then on in this
+ *     context the one serves a call of that shape that is the faster by these
+ *     times, scaled to the call's N and number of estimates.
  * Returns IDTX_EINVAL for a NULL ctx or an unknown value. */
 #define IDTX_KERNEL_AUTO 0
 #define IDTX_KERNEL_TILE 1

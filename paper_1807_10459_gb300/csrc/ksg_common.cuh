@@ -91,6 +91,7 @@ struct KsgLaunch {
     const int2 *list_b;
     const int4 *lmeta;
     double *ring;  // kListRingBytes of scratch for the list kernel's term ring
+    void *lscratch;  // list_scratch_bytes of scratch for build_lists
     int cap_a, cap_b;
 };
 
@@ -133,9 +134,13 @@ struct KsgVariant {
 };
 
 // Per-query sorted neighbour lists of a group prepared into sh (lists.cu):
-// z columns [0, dzb), y columns [dzb, dsb) of rows of dsp floats.
-cudaError_t build_lists(const float *sh, int dsp, int dzb, int dsb, int64_t n, int cap_a,
-                        int cap_b, int2 *list_a, int2 *list_b, int4 *meta, cudaStream_t st);
+// rows of dzb z columns, then dyb y columns.  scratch: list_scratch_bytes(n,
+// cap_a, cap_b), which also covers smaller capacities.  *launches (nullable)
+// receives the kernels launched.  n <= 0 only sets kernel attributes.
+size_t list_scratch_bytes(int64_t n, int cap_a, int cap_b);
+cudaError_t build_lists(const float *sh, int dzb, int dyb, int64_t n, int cap_a, int cap_b,
+                        int2 *list_a, int2 *list_b, int4 *meta, void *scratch, cudaStream_t st,
+                        int *launches);
 
 // Radix sort of (key, index) pairs on the low end_bit key bits (sort.cu).
 // With tmp == nullptr only sets tmp_bytes.

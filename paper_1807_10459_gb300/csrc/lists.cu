@@ -2,20 +2,29 @@
 // subspaces, the preparation step of ksg_list_kernel (ksg_list.cuh).
 //
 // For every query i (sorted sample position) and every other sample j that
-// may belong to a list (whole tiles that cannot are skipped: see the
-// kernel), the max-norm distances d_Z(i,j) over the z columns and d_YZ(i,j)
-// over the z and y columns of sh are formed exactly as in the estimator's
-// definition (fp32 |a-b| and maxima).  List A holds every j != i with
-// d_YZ < r_A(i), list B every j != i with d_Z < r_B(i), each ascending by
-// distance (equal distances in any order); r_A, r_B are the largest
-// histogram-bin edges for which the lists fit their capacities (+inf when
-// every sample fits).
+// may belong to a list, the max-norm distances d_Z(i,j) over the z columns
+// and d_YZ(i,j) over the z and y columns of sh are formed exactly as in the
+// estimator's definition (fp32 |a-b| and maxima).  List A holds every j != i
+// with d_YZ < r_A(i), list B every j != i with d_Z < r_B(i), each ascending
+// by distance (equal distances in any order; entries at r itself may follow).
+// r_A, r_B are any radii for which the lists fit their capacities.
+//
+// Two kernels per chunk of queries, with the unsorted entries in scratch
+// between them:
+//   k_collect     a warp per QW consecutive queries: a radius for each list
+//                 from a sample of the distances, then one pass over the
+//                 tiles whose box is within a radius, appending the entries.
+//   k_sort_lists  a block per (query, list): counting sort on the distance.
+// Measured on GB300 against one block per query with two histogram passes over
+// all rows and block radix sorts, both kernels together: N = 9995, three z and
+// one y column, lists of 2048 and 4096: 1.68 -> 0.98 ms; N = 4997, six z,
+// 1024 and 2048: 0.51 -> 0.33 ms; N = 99850, ten z, 512 and 1024: 44.3 ->
+// 9.1 ms (that kernel read every visited row once per query, and visited 60 to
+// 95 % of the tiles for its histogram).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cstdint>
-
-#include <cub/block/block_radix_sort.cuh>
 
 #include "ksg_common.cuh"
 
@@ -23,457 +32,677 @@ namespace idtx {
 
 namespace {
 
-constexpr int kLThreads = 256;
-constexpr int kBins = 4096;          // bins on bits 30..19 of a non-negative float
-constexpr int kBinShift = 19;
-constexpr int kBinsPerThread = kBins / kLThreads;
+constexpr unsigned kFull = 0xffffffffu;
+constexpr int kBinShift = 19;       // histogram bins: 16 per octave of distance
+constexpr int kHistBins = 256;      // 16 octaves
+constexpr int kHistPerLane = kHistBins / 32;
+constexpr int kCollectWarps = 8;
+constexpr int kCollectThreads = kCollectWarps * 32;
 
-// Digit width of the block radix sorts: 7 passes over a 32-bit key instead
-// of CUB's default 8 (measured on GB300: 1.82 against 1.97 ms for 9995
-// queries, lists of 2048 and 4096; 6 bits spills).
-constexpr int kSortRadixBits = 5;
+// Sampling.  A list's radius is the distance within which 1.15 capacities of
+// samples are expected, from a sample holding `hits` of its shorter list's
+// entries (a spread of 1 / sqrt(hits)): 64 for lists of 1024 entries or more,
+// 28 below, where the sample is a larger share of the work.  A scratch buffer
+// takes two capacities, 1.5 from 2048 entries on (their spread is smaller),
+// so most lists end full and buffers rarely overflow.
+constexpr float kTargetFill = 1.15f;
 
-// Largest tile-visit bitmap (32-bit words): calls with more tiles visit all.
-constexpr int kMaxVisitWords = 1024;
-// Tile pruning runs for calls of at least kPruneMinTiles tiles whose lists
-// hold at most an eighth of the samples: otherwise its per-query set-up (two
-// histogram clears, bounds of every tile, two ranking scans) costs more than
-// it saves (measured on GB300: N = 1000 lost 7 %; the greedy step's build,
-// N = 9995 with lists of 2048 and 4096, 0.15 ms; N = 99850 with lists of
-// 512 and 1024 was built 1.8x faster).
-constexpr int kPruneMinTiles = 64;
-constexpr int kPruneMaxListShare = 8;  // lists of at most n / 8 entries
+struct CollectArgs {
+    const float *sh;
+    int64_t n;
+    int64_t q0;          // first query of the chunk
+    int n_q;             // queries of the chunk
+    int cap_a, cap_b;    // list capacities
+    int buf_a, buf_b;    // scratch entries per query
+    int n_sample;        // sampled rows (0: no sampling), at `stride`
+    int stride;
+    int2 *raw_a, *raw_b; // scratch [n_q][buf]
+    int4 *raw_meta;      // per query of the chunk: counts, radii (bits)
+};
 
-constexpr int kMaxRow4 = 5;  // float4 columns of a row of sh: dsp <= 20 (dz' <= 16, dy <= 4)
-constexpr int kUnrollJ = 4;  // samples a thread has in flight per step of a distance pass
-
-// Fold float4 column c of a row into the running maxima of d_Z (the first
-// dzb columns) and d_YZ (the first dsb): the estimator's fp32 |a-b| and maxima.
-__device__ __forceinline__ void fold4(const float4 q, const float4 r, int c, int dzb, int dsb,
-                                      float &mz, float &my)
+// The radius of a list from a histogram of sampled distances (bin 0 at float
+// bits base << 19): the distance below which `want` of them lie, linear
+// within its bin; +inf when the histogram's last octave does not reach it.
+// Warp-uniform; the lanes hold consecutive bins.
+__device__ float hist_radius(const int *hist, int base, float want)
 {
-    const float a[4] = {fabsf(q.x - r.x), fabsf(q.y - r.y), fabsf(q.z - r.z), fabsf(q.w - r.w)};
+    const int lane = threadIdx.x & 31;
+    int c[kHistPerLane], sum = 0;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const int d = 4 * c + e;
-        if (d < dzb) mz = fmaxf(mz, a[e]);
-        if (d < dsb) my = fmaxf(my, a[e]);
+    for (int b = 0; b < kHistPerLane; ++b) {
+        c[b] = hist[lane * kHistPerLane + b];
+        sum += c[b];
     }
-}
-
-// First bin b with (count of bins <= b) > cap, or kBins if the total fits.
-// All threads of the block call it; the result is returned to every thread.
-__device__ int cut_bin(const int *hist, int cap, int *s_part, int *s_cut)
-{
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int local = 0;
-    for (int b = 0; b < kBinsPerThread; ++b) local += hist[tid * kBinsPerThread + b];
-    // inclusive scan over threads
-    int inc = local;
+    int inc = sum;
     for (int off = 1; off < 32; off <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, inc, off);
+        const int v = __shfl_up_sync(kFull, inc, off);
         if (lane >= off) inc += v;
     }
-    if (lane == 31) s_part[warp] = inc;
-    if (tid == 0) *s_cut = kBins;
-    __syncthreads();
-    int before = 0;
-    for (int w = 0; w < warp; ++w) before += s_part[w];
-    int cum = before + inc - local;  // count in bins before this thread's range
-    if (cum <= cap && cum + local > cap) {
-        for (int b = 0; b < kBinsPerThread; ++b) {
-            cum += hist[tid * kBinsPerThread + b];
+    const uint32_t over = __ballot_sync(kFull, (float)inc > want);
+    float r = INFINITY;
+    if (over) {
+        const int l = __ffs(over) - 1;
+        float mine = 0.0f;
+        if (lane == l) {
+            int cum = inc - sum;
+#pragma unroll
+            for (int b = 0; b < kHistPerLane; ++b) {
+                if ((float)cum <= want && (float)(cum + c[b]) > want) {
+                    const int at = base + l * kHistPerLane + b;
+                    const float lo = __uint_as_float((unsigned)max(at, 0) << kBinShift);
+                    const float hi = __uint_as_float((unsigned)max(at + 1, 0) << kBinShift);
+                    mine = l * kHistPerLane + b == kHistBins - 1
+                               ? INFINITY
+                               : lo + (hi - lo) * ((want - (float)cum) / (float)c[b]);
+                }
+                cum += c[b];
+            }
+        }
+        r = __shfl_sync(kFull, mine, l);
+    }
+    return r;
+}
+
+// A full scratch buffer: lower the radius to a bin edge below which at most
+// cap entries lie and keep those (in order).  Called by a whole warp.  Every
+// sample closer than the new radius that has been met stays listed.
+struct Shrunk {
+    int kept;
+    float radius;
+};
+__device__ __noinline__ Shrunk shrink_list(int2 *buf, int cnt, int cap, int *hist)
+{
+    const int lane = threadIdx.x & 31;
+    for (int b = lane; b < kHistBins; b += 32) hist[b] = 0;
+    unsigned top = 0;
+    for (int p = lane; p < cnt; p += 32) top = max(top, (unsigned)buf[p].y);
+    top = __reduce_max_sync(kFull, top);
+    const int base = (int)(top >> kBinShift) - (kHistBins - 1);
+    __syncwarp();
+    for (int p = lane; p < cnt; p += 32)
+        atomicAdd(&hist[max((int)((unsigned)buf[p].y >> kBinShift) - base, 0)], 1);
+    __syncwarp();
+    int sum = 0;
+    for (int b = 0; b < kHistPerLane; ++b) sum += hist[lane * kHistPerLane + b];
+    int inc = sum;
+    for (int off = 1; off < 32; off <<= 1) {
+        const int v = __shfl_up_sync(kFull, inc, off);
+        if (lane >= off) inc += v;
+    }
+    // the first bin at which the running count exceeds cap (cnt > cap here)
+    const int l = __ffs(__ballot_sync(kFull, inc > cap)) - 1;
+    int cut = 0;
+    if (lane == l) {
+        int cum = inc - sum;
+        for (int b = 0; b < kHistPerLane; ++b) {
+            cum += hist[lane * kHistPerLane + b];
             if (cum > cap) {
-                *s_cut = tid * kBinsPerThread + b;
+                cut = lane * kHistPerLane + b;
                 break;
             }
         }
     }
-    __syncthreads();
-    const int r = *s_cut;
-    __syncthreads();
-    return r;
-}
-
-// Sort the n collected (distance bits, sample) pairs of one list ascending by
-// distance and write them, then +inf sentinels up to a multiple of 32 (at
-// most cap), to out.  Ties may land in any order: nothing downstream depends
-// on the order of equal distances.  Every key is below `bound` (the bits of
-// the list's cut, a non-negative float), so only its low 32 - clz(bound)
-// bits can differ and the sort passes over those alone; the padding keys
-// (all ones) stay above every real key in those bits.  The pairs are first
-// taken into registers, so the sort's scratch may overlay the collection
-// buffers (tmp); all threads of the block call it.
-template <int ITEMS>
-__device__ void sort_and_store(const uint32_t *keys, const int32_t *vals, int n, int cap,
-                               uint32_t bound, void *tmp, int2 *out)
-{
-    using Sort = cub::BlockRadixSort<uint32_t, kLThreads, ITEMS, int32_t, kSortRadixBits>;
-    uint32_t k[ITEMS];
-    int32_t v[ITEMS];
-    const int t0 = threadIdx.x * ITEMS;
-#pragma unroll
-    for (int i = 0; i < ITEMS; ++i) {
-        const int at = t0 + i;
-        k[i] = at < n ? keys[at] : 0xFFFFFFFFu;
-        v[i] = at < n ? vals[at] : 0;
+    cut = __shfl_sync(kFull, cut, l);
+    // bin 0 also holds what is more than 16 octaves below the largest
+    const float radius = cut == 0 ? 0.0f : __uint_as_float((unsigned)max(base + cut, 0) << kBinShift);
+    int kept = 0;
+    for (int p0 = 0; p0 < cnt; p0 += 32) {
+        const int p = p0 + lane;
+        const int2 e = p < cnt ? buf[p] : make_int2(0, __float_as_int(INFINITY));
+        const bool keep = __int_as_float(e.y) < radius;
+        const uint32_t m = __ballot_sync(kFull, keep);  // also orders the reads before the writes
+        if (keep) buf[kept + __popc(m & ((1u << lane) - 1u))] = e;
+        kept += __popc(m);
+        __syncwarp();
     }
-    __syncthreads();  // the collection buffers may now be overwritten
-    const int end_bit = max(1, 32 - __clz(bound));
-    Sort(*reinterpret_cast<typename Sort::TempStorage *>(tmp)).Sort(k, v, 0, end_bit);
-    const int end = min(cap, (n + 31) & ~31);
-#pragma unroll
-    for (int i = 0; i < ITEMS; ++i) {
-        const int at = t0 + i;
-        if (at < end)
-            out[at] = at < n ? make_int2(v[i], (int)k[i]) : make_int2(0, __float_as_int(INFINITY));
-    }
-    __syncthreads();
+    return Shrunk{kept, radius};
 }
 
-template <int ITEMS>
-constexpr size_t sort_tmp_bytes()
-{
-    return sizeof(typename cub::BlockRadixSort<uint32_t, kLThreads, ITEMS, int32_t, kSortRadixBits>::TempStorage);
-}
-
-// One block per query.  Dynamic shared memory: the two histograms, later
-// overlaid by the collected keys and samples of both lists, later by the
-// sort's scratch (build_smem bytes), then at visit_off the tile-visit bitmap
-// and its per-word prefix counts.
-// IA, IB: sort items per thread (kLThreads * IA >= cap_a, kLThreads * IB >=
-// cap_b).
+// One warp per two consecutive queries.
 //
-// Tile pruning.  Rows kTJ and kTJ+1 of every tile of sh hold its samples'
-// per-dimension minimum and maximum.  For the query, a tile's box gap G (the
-// largest over dimensions of the distance from the query to the box, 0
-// inside) bounds its samples' distances from below and its far corner F
-// (the largest over dimensions of the query's distance to the farther face)
-// from above, in the subspaces Z and (Y,Z), both in the definition's fp32
-// arithmetic (rounding is monotone, so the bounds hold for the computed
-// distances).  Summing tile sizes by F gives a radius R within which more
-// than cap samples lie: the list's cut is at most R, so the histogram pass
-// needs only the tiles with G < R (it is exact below R).  The collecting
-// pass needs only the tiles with G below the cut.
-template <int IA, int IB>
-__global__ void __launch_bounds__(kLThreads, 3)
-    k_build_lists(const float *sh, int dsp, int dzb, int dsb, int64_t n, int cap_a, int cap_b,
-                  int2 *list_a, int2 *list_b, int4 *meta, int visit_off)
+// Radii.  The distances to n_sample rows spread evenly over the samples (in
+// Morton order, so over space) go into a histogram per list; the radius is
+// the distance at the wanted rank of the sample (hist_radius).  It only
+// decides how long the lists get: they hold every sample below it.
+//
+// Tiles.  Rows kTJ and kTJ+1 of every tile of sh hold its samples'
+// per-dimension minimum and maximum.  A tile's box gap (the largest over
+// dimensions of the distance from the query to the box, 0 inside) bounds its
+// samples' distances from below in the definition's fp32 arithmetic (rounding
+// is monotone, so the bound holds for the computed distances): tiles whose
+// gap reaches both radii of both queries are skipped, 32 tiles being tested
+// at a time, one per lane.
+//
+// A visited tile's rows are loaded once for the two queries, whose
+// coordinates stay in registers, and the entries below a radius are appended
+// to the query's buffers (the counts are the warp's own: no atomics).  With
+// more than six dimensions the first four are tested first: a group of 32
+// rows none of which is within a radius there goes no further.
+// Bound by issue (the differences and maxima) at few dimensions and by L1 at
+// many; two queries per warp at 80 registers ran N = 99850, ten z in 7.1 ms,
+// four queries at 167 registers (half the warps) in 15.4.
+template <int DZ, int DY>
+__global__ void __launch_bounds__(kCollectThreads, DZ + DY <= 12 ? 3 : 2)
+    k_collect(const CollectArgs a)
 {
-    extern __shared__ __align__(16) unsigned char l_smem[];
-    __shared__ int s_part[kLThreads / 32];
-    __shared__ int s_cut;
-    __shared__ int s_cnt[2];
-    __shared__ int s_nvis;
-    int *hist_a = reinterpret_cast<int *>(l_smem);
-    int *hist_b = hist_a + kBins;
-    const int64_t i = blockIdx.x;
-    const int tid = threadIdx.x;
-    const int nc = dsp / 4;  // float4 columns per row
-    auto row4 = [&](int64_t j) {
-        return reinterpret_cast<const float4 *>(sh + ((j / kTJ) * kTileRows + (j % kTJ)) * dsp);
+    constexpr int DS = DZ + DY, NC = (DS + 3) / 4, DSP = NC * 4;
+    constexpr int QW = 2, kSegs = kTJ / 32;
+    constexpr int U = NC == 1 ? 4 : 2;  // rows a lane has in flight
+    constexpr bool EARLY = DZ > 6;
+    static_assert(kTJ % QW == 0 && kSegs % U == 0, "query groups and row steps tile a tile");
+    __shared__ int s_hist[kCollectWarps][QW][2][kHistBins];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g0 = (blockIdx.x * kCollectWarps + warp) * QW;  // first query, within the chunk
+    if (g0 >= a.n_q) return;
+    const int n = (int)a.n;  // at most IDTX_MAX_N; row offsets in float4 fit an int
+    const float4 *sh = reinterpret_cast<const float4 *>(a.sh);
+    auto row_of = [&](int j) { return sh + ((j / kTJ) * kTileRows + (j % kTJ)) * NC; };
+    auto load = [&](const float4 *p, float(&r)[DSP]) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            const float4 v = __ldg(p + c);
+            r[4 * c] = v.x, r[4 * c + 1] = v.y, r[4 * c + 2] = v.z, r[4 * c + 3] = v.w;
+        }
     };
-    float4 q4[kMaxRow4];
-    {
-        const float4 *qr = row4(i);
+    auto dist = [](const float(&q)[DSP], const float(&r)[DSP], float &dz, float &dyz) {
+        dz = fabsf(q[0] - r[0]);
 #pragma unroll
-        for (int c = 0; c < kMaxRow4; ++c) q4[c] = c < nc ? qr[c] : make_float4(0, 0, 0, 0);
+        for (int d = 1; d < DZ; ++d) dz = fmaxf(dz, fabsf(q[d] - r[d]));
+        dyz = dz;
+#pragma unroll
+        for (int d = DZ; d < DS; ++d) dyz = fmaxf(dyz, fabsf(q[d] - r[d]));
+    };
+    // The second query past the chunk's end (odd counts) repeats the first
+    // and lists nothing.
+    const bool two = g0 + 1 < a.n_q;
+    const int q0 = (int)a.q0 + g0;
+    float q[QW][DSP], ra[QW], rb[QW];
+    int ca[QW], cb[QW];
+#pragma unroll
+    for (int u = 0; u < QW; ++u) {
+        load(row_of(q0 + (two ? u : 0)), q[u]);
+        ra[u] = rb[u] = INFINITY;
+        ca[u] = cb[u] = 0;
     }
-    const int warp = tid >> 5;
-    const int n_tiles = (int)((n + kTJ - 1) / kTJ);
-    const int vwords = (n_tiles + 31) / 32;
-    const bool prune = vwords <= kMaxVisitWords && n_tiles >= kPruneMinTiles &&
-                       (int64_t)max(cap_a, cap_b) * kPruneMaxListShare <= n;
-    uint32_t *visit = reinterpret_cast<uint32_t *>(l_smem + visit_off);
-    // Box gap and far-corner bounds of tile t in Z and (Y,Z).
-    auto tile_bounds = [&](int t, float &gz, float &gyz, float &fz, float &fyz) {
-        const float4 *lo = reinterpret_cast<const float4 *>(sh + ((int64_t)t * kTileRows + kTJ) * dsp);
-        const float4 *hi = lo + nc;
-        gz = gyz = fz = fyz = 0.0f;
+    int *hist = s_hist[warp][0][0];
+    if (a.n_sample > 0) {
+        for (int b = lane; b < QW * 2 * kHistBins; b += 32) hist[b] = 0;
+        __syncwarp();
+        int base[QW][2];
+        for (int s0 = 0; s0 < a.n_sample; s0 += 32) {
+            const bool in = s0 + lane < a.n_sample;
+            float r[DSP];
+            load(row_of(in ? (s0 + lane) * a.stride : 0), r);
 #pragma unroll
-        for (int c = 0; c < kMaxRow4; ++c) {
-            if (c < nc) {
-                const float4 a4 = lo[c], b4 = hi[c], q = q4[c];
-                const float qa[4] = {q.x, q.y, q.z, q.w}, la[4] = {a4.x, a4.y, a4.z, a4.w},
-                            ha[4] = {b4.x, b4.y, b4.z, b4.w};
+            for (int u = 0; u < QW; ++u) {
+                float dz, dyz;
+                dist(q[u], r, dz, dyz);
+                const unsigned k[2] = {__float_as_uint(dyz) >> kBinShift, __float_as_uint(dz) >> kBinShift};
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int d = 4 * c + e;
-                    const float g = fmaxf(fmaxf(la[e] - qa[e], qa[e] - ha[e]), 0.0f);
-                    const float f = fmaxf(fabsf(qa[e] - la[e]), fabsf(qa[e] - ha[e]));
-                    if (d < dzb) {
-                        gz = fmaxf(gz, g);
-                        fz = fmaxf(fz, f);
-                    }
-                    if (d < dsb) {
-                        gyz = fmaxf(gyz, g);
-                        fyz = fmaxf(fyz, f);
-                    }
+                for (int l = 0; l < 2; ++l) {
+                    // the bins end an octave above the first rows' largest
+                    if (s0 == 0) base[u][l] = (int)__reduce_max_sync(kFull, k[l]) + 17 - kHistBins;
+                    if (in)
+                        atomicAdd(&hist[(u * 2 + l) * kHistBins +
+                                        min(max((int)k[l] - base[u][l], 0), kHistBins - 1)], 1);
                 }
             }
         }
-    };
-    // Bit t of the visit bitmap: tile t has G < lim in either subspace.
-    auto mark_tiles = [&](float lim_a, float lim_b) {
-        for (int w = warp; w < vwords; w += kLThreads / 32) {
-            const int t = w * 32 + (tid & 31);
-            bool vis = false;
-            if (t < n_tiles) {
-                float gz, gyz, fz, fyz;
-                tile_bounds(t, gz, gyz, fz, fyz);
-                vis = gyz < lim_a || gz < lim_b;
-            }
-            const uint32_t bits = __ballot_sync(0xffffffffu, vis);
-            if ((tid & 31) == 0) visit[w] = bits;
-        }
-    };
-    // The visited tiles are taken by the warps in turn (the visited tile of
-    // rank k by warp k mod 8); vpre[w] counts the visited tiles in the
-    // bitmap's words before w.
-    int *vpre = reinterpret_cast<int *>(visit + vwords);
-    auto rank_tiles = [&]() {  // all threads; the bitmap written and synced before
-        if (warp == 0) {
-            const int lane = tid & 31;
-            const int per = (vwords + 31) / 32;
-            const int w0 = lane * per, w1 = min(w0 + per, vwords);
-            int sum = 0;
-            for (int w = w0; w < w1; ++w) sum += __popc(visit[w]);
-            int inc = sum;
-            for (int off = 1; off < 32; off <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, inc, off);
-                if (lane >= off) inc += v;
-            }
-            int run = inc - sum;
-            for (int w = w0; w < w1; ++w) {
-                vpre[w] = run;
-                run += __popc(visit[w]);
-            }
-            if (lane == 31) s_nvis = inc;
-        }
-        __syncthreads();
-    };
-    // The tile of rank k (all tiles in order when not pruning); wp: the
-    // bitmap word to search from (a warp's ranks only grow).
-    auto tile_of = [&](int k, int &wp) -> int {
-        if (!prune) return k;
-        while (wp + 1 < vwords && vpre[wp + 1] <= k) ++wp;
-        return wp * 32 + (int)__fns(visit[wp], 0, k - vpre[wp] + 1);
-    };
-    constexpr int kSegs = kTJ / 32;  // 32-sample segments per tile
-    // Distances of samples j[u] = tile t's segment s0 + u, this lane's
-    // sample (kUnrollJ segments, their rows loaded back to back); the query
-    // itself and samples past the tile or n get +inf (and read the query's
-    // own row, an L1 hit).
-    auto dists_tile = [&](int t, int s0, int64_t (&j)[kUnrollJ], float (&dz)[kUnrollJ],
-                          float (&dyz)[kUnrollJ]) {
-        const float4 *r[kUnrollJ];
-        bool ok[kUnrollJ];
+        __syncwarp();
+        const float part = kTargetFill * (float)a.n_sample / (float)n;
 #pragma unroll
-        for (int u = 0; u < kUnrollJ; ++u) {
-            j[u] = (int64_t)t * kTJ + (s0 + u) * 32 + (tid & 31);
-            ok[u] = s0 + u < kSegs && j[u] < n && j[u] != i;
-            r[u] = row4(ok[u] ? j[u] : i);
-            dz[u] = dyz[u] = 0.0f;
+        for (int u = 0; u < QW; ++u) {
+            if (a.cap_a < n - 1)
+                ra[u] = hist_radius(hist + u * 2 * kHistBins, base[u][0], part * (float)a.cap_a);
+            if (a.cap_b < n - 1)
+                rb[u] = hist_radius(hist + (u * 2 + 1) * kHistBins, base[u][1], part * (float)a.cap_b);
         }
-#pragma unroll
-        for (int c = 0; c < kMaxRow4; ++c) {
-            if (c < nc) {
-                float4 v[kUnrollJ];
-#pragma unroll
-                for (int u = 0; u < kUnrollJ; ++u) v[u] = r[u][c];
-#pragma unroll
-                for (int u = 0; u < kUnrollJ; ++u) fold4(q4[c], v[u], c, dzb, dsb, dz[u], dyz[u]);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kUnrollJ; ++u)
-            if (!ok[u]) dz[u] = dyz[u] = INFINITY;
-    };
-    constexpr int kWarps = kLThreads / 32;
-
-    // The radii R: tile sizes summed into the histograms by far corner.
-    // Bins hold bits 30..19 of a non-negative float, so the upper edge of
-    // bin b is the float with bits (b + 1) << 19; from bin 4079 on that is
-    // +inf or past it.
-    auto upper_edge = [](int b) {
-        return b + 1 >= (0x7F800000 >> kBinShift) ? INFINITY : __uint_as_float((unsigned)(b + 1) << kBinShift);
-    };
-    if (prune) {
-        for (int b = tid; b < 2 * kBins; b += kLThreads) hist_a[b] = 0;
-        __syncthreads();
-        for (int t = tid; t < n_tiles; t += kLThreads) {
-            float gz, gyz, fz, fyz;
-            tile_bounds(t, gz, gyz, fz, fyz);
-            const int64_t left = n - (int64_t)t * kTJ;
-            const int size = left < kTJ ? (int)left : kTJ;
-            atomicAdd(&hist_a[__float_as_uint(fyz) >> kBinShift], size);
-            atomicAdd(&hist_b[__float_as_uint(fz) >> kBinShift], size);
-        }
-        __syncthreads();
-        // more than cap + 1 samples (the query among them) within the bin's upper edge
-        const int fa = cut_bin(hist_a, cap_a + 1, s_part, &s_cut);
-        const int fb = cut_bin(hist_b, cap_b + 1, s_part, &s_cut);
-        mark_tiles(fa >= kBins ? INFINITY : upper_edge(fa), fb >= kBins ? INFINITY : upper_edge(fb));
+        __syncwarp();
     }
-    for (int b = tid; b < 2 * kBins; b += kLThreads) hist_a[b] = 0;
-    __syncthreads();
-    if (prune) rank_tiles();
-    {
-        const int n_iter = prune ? s_nvis : n_tiles;
-        int wp = 0;
-        for (int k = warp; k < n_iter; k += kWarps) {
-            const int t = tile_of(k, wp);
-            for (int s0 = 0; s0 < kSegs; s0 += kUnrollJ) {
-                int64_t j[kUnrollJ];
-                float dz[kUnrollJ], dyz[kUnrollJ];
-                dists_tile(t, s0, j, dz, dyz);
-#pragma unroll
-                for (int u = 0; u < kUnrollJ; ++u) {
-                    if (dz[u] == INFINITY) continue;  // the query itself or past n
-                    atomicAdd(&hist_a[__float_as_uint(dyz[u]) >> kBinShift], 1);
-                    atomicAdd(&hist_b[__float_as_uint(dz[u]) >> kBinShift], 1);
-                }
-            }
-        }
-    }
-    __syncthreads();
-    const int cut_a = cut_bin(hist_a, cap_a, s_part, &s_cut);
-    const int cut_b = cut_bin(hist_b, cap_b, s_part, &s_cut);
-    const float r_a = cut_a >= kBins ? INFINITY : __uint_as_float((unsigned)cut_a << kBinShift);
-    const float r_b = cut_b >= kBins ? INFINITY : __uint_as_float((unsigned)cut_b << kBinShift);
-    if (prune) {
-        mark_tiles(r_a, r_b);  // the histogram pass is done with the bitmap (cut_bin syncs)
-        __syncthreads();
-        rank_tiles();
-    }
-
-    // Collect the samples below the cuts (in order of arrival; a warp claims
-    // the slots of all its qualifying lanes with one atomic per list).
-    uint32_t *key_a = reinterpret_cast<uint32_t *>(l_smem);
-    int32_t *val_a = reinterpret_cast<int32_t *>(key_a + kLThreads * IA);
-    uint32_t *key_b = reinterpret_cast<uint32_t *>(val_a + kLThreads * IA);
-    int32_t *val_b = reinterpret_cast<int32_t *>(key_b + kLThreads * IB);
-    if (tid < 2) s_cnt[tid] = 0;
-    __syncthreads();  // histograms are dead from here on
-    const int lane = tid & 31;
+    if (!two) ra[1] = rb[1] = -1.0f;
+    int2 *const oa = a.raw_a + (int64_t)g0 * a.buf_a, *const ob = a.raw_b + (int64_t)g0 * a.buf_b;
+    const int n_tiles = (n + kTJ - 1) / kTJ;
+    const int home = q0 / kTJ;  // the tile of both queries
     const uint32_t below = (1u << lane) - 1u;
-    {
-        const int n_iter = prune ? s_nvis : n_tiles;
-        int wp = 0;
-        for (int k = warp; k < n_iter; k += kWarps) {  // whole warps iterate
-            const int t = tile_of(k, wp);
-            for (int s0 = 0; s0 < kSegs; s0 += kUnrollJ) {
-                int64_t j[kUnrollJ];
-                float dz[kUnrollJ], dyz[kUnrollJ];
-                dists_tile(t, s0, j, dz, dyz);
+    for (int tb = 0; tb < n_tiles; tb += 32) {
+        bool vis = false;
+        if (tb + lane < n_tiles) {
+            const float4 *bx = sh + ((tb + lane) * kTileRows + kTJ) * NC;
+            float lo[DSP], hi[DSP];
+            load(bx, lo);
+            load(bx + NC, hi);
 #pragma unroll
-                for (int u = 0; u < kUnrollJ; ++u) {
-                    const bool in_a = dyz[u] < r_a, in_b = dz[u] < r_b;
-                    const uint32_t ma = __ballot_sync(0xffffffffu, in_a);
-                    const uint32_t mb = __ballot_sync(0xffffffffu, in_b);
-                    int base_a = 0, base_b = 0;
-                    if (lane == 0) {
-                        if (ma) base_a = atomicAdd(&s_cnt[0], __popc(ma));
-                        if (mb) base_b = atomicAdd(&s_cnt[1], __popc(mb));
-                    }
-                    base_a = __shfl_sync(0xffffffffu, base_a, 0);
-                    base_b = __shfl_sync(0xffffffffu, base_b, 0);
-                    if (in_a) {
-                        const int at = base_a + __popc(ma & below);
-                        if (at < cap_a) {
-                            key_a[at] = __float_as_uint(dyz[u]);
-                            val_a[at] = (int32_t)j[u];
+            for (int u = 0; u < QW; ++u) {
+                float gz = 0.0f;
+#pragma unroll
+                for (int d = 0; d < DZ; ++d) gz = fmaxf(gz, fmaxf(lo[d] - q[u][d], q[u][d] - hi[d]));
+                float gyz = gz;
+#pragma unroll
+                for (int d = DZ; d < DS; ++d) gyz = fmaxf(gyz, fmaxf(lo[d] - q[u][d], q[u][d] - hi[d]));
+                vis |= gyz < ra[u] || gz < rb[u];
+            }
+        }
+        uint32_t todo = __ballot_sync(kFull, vis);
+        while (todo) {
+            const int t = tb + __ffs(todo) - 1;
+            todo &= todo - 1;
+            const float4 *rows = sh + (t * kTileRows + lane) * NC;
+            const int self = t == home ? q0 % kTJ : -2;  // the first query's row of this tile
+#pragma unroll 1
+            for (int s0 = 0; s0 < kSegs; s0 += U) {
+                float r[U][DSP];
+#pragma unroll
+                for (int v = 0; v < U; ++v) load(rows + (s0 + v) * 32 * NC, r[v]);
+#pragma unroll
+                for (int v = 0; v < U; ++v) {
+                    const int at = (s0 + v) * 32 + lane;
+#pragma unroll
+                    for (int u = 0; u < QW; ++u) {
+                        if (EARLY) {
+                            float d4 = fabsf(q[u][0] - r[v][0]);
+#pragma unroll
+                            for (int d = 1; d < 4; ++d) d4 = fmaxf(d4, fabsf(q[u][d] - r[v][d]));
+                            if (!__any_sync(kFull, d4 < fmaxf(ra[u], rb[u]))) continue;
                         }
-                    }
-                    if (in_b) {
-                        const int at = base_b + __popc(mb & below);
-                        if (at < cap_b) {
-                            key_b[at] = __float_as_uint(dz[u]);
-                            val_b[at] = (int32_t)j[u];
+                        float dz, dyz;
+                        dist(q[u], r[v], dz, dyz);
+                        const bool other = at != self + u;
+                        bool pa = dyz < ra[u] && other, pb = dz < rb[u] && other;
+                        uint32_t ma = __ballot_sync(kFull, pa), mb = __ballot_sync(kFull, pb);
+                        if (ma) {
+                            int2 *out = oa + u * a.buf_a;
+                            if (ca[u] + __popc(ma) > a.buf_a) {
+                                __syncwarp();
+                                const Shrunk w = shrink_list(out, ca[u], a.cap_a, hist);
+                                ca[u] = w.kept;
+                                ra[u] = w.radius;
+                                pa = pa && dyz < ra[u];
+                                ma = __ballot_sync(kFull, pa);
+                            }
+                            if (pa) out[ca[u] + __popc(ma & below)] = make_int2(t * kTJ + at, __float_as_int(dyz));
+                            ca[u] += __popc(ma);
+                        }
+                        if (mb) {
+                            int2 *out = ob + u * a.buf_b;
+                            if (cb[u] + __popc(mb) > a.buf_b) {
+                                __syncwarp();
+                                const Shrunk w = shrink_list(out, cb[u], a.cap_b, hist);
+                                cb[u] = w.kept;
+                                rb[u] = w.radius;
+                                pb = pb && dz < rb[u];
+                                mb = __ballot_sync(kFull, pb);
+                            }
+                            if (pb) out[cb[u] + __popc(mb & below)] = make_int2(t * kTJ + at, __float_as_int(dz));
+                            cb[u] += __popc(mb);
                         }
                     }
                 }
             }
         }
     }
+    if (lane == 0) {
+        a.raw_meta[g0] = make_int4(ca[0], cb[0], __float_as_int(ra[0]), __float_as_int(rb[0]));
+        if (two) a.raw_meta[g0 + 1] = make_int4(ca[1], cb[1], __float_as_int(ra[1]), __float_as_int(rb[1]));
+    }
+}
+
+constexpr int kBigBin = 16;  // bins above this are sorted by the whole block
+
+struct SortArgs {
+    const int2 *raw;       // [query of the chunk][buf]
+    const int4 *raw_meta;
+    int buf, cap;
+    int is_b;              // list B's (else list A's) fields of the metas
+    int pow;               // squarings of the scaled distance before binning
+    int64_t q0;
+    int2 *list;
+    int4 *meta;
+};
+
+struct SortPair {
+    SortArgs l[2];
+};
+
+// Dynamic shared memory: the entries, then the bins' offsets.
+__host__ __device__ constexpr size_t sort_smem(int buf, int bins)
+{
+    return (size_t)buf * sizeof(int2) + (size_t)(bins + 1) * sizeof(int);
+}
+
+// One block per (query, list): the collected entries in ascending order of
+// distance, the first `cap` of them written out.  A counting sort over bins
+// that are even in a power of the distance (a neighbourhood of dimension D
+// holds about r^D samples, so the power evens out the bins), then exchanges
+// of neighbours within the bins (one or two entries on average).  Bins of
+// more than kBigBin entries (data with many equal distances) are sorted in
+// place by the whole block first.  Bound by shared memory (LSU 88 % busy at
+// lists of 4096): N = 9995, lists of 2048 and 4096, 0.27 + 0.45 ms.
+// T threads, E entries per thread, BINS bins.
+template <int T, int E, int BINS>
+__global__ void __launch_bounds__(T, E > 8 ? 1536 / T : 2048 / T)
+    k_sort_lists(const SortPair pair)
+{
+    constexpr int kSortThreads = T, kSortWarps = T / 32;
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    __shared__ int s_part[kSortWarps];
+    __shared__ unsigned s_top;
+    __shared__ int s_big;
+    const SortArgs &a = pair.l[blockIdx.y];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int qr = blockIdx.x;
+    const int64_t i = a.q0 + qr;
+    const int cap = a.cap;
+    const int2 *raw = a.raw + (int64_t)qr * a.buf;
+    int2 *out = a.list + i * cap;
+    const int4 rm = a.raw_meta[qr];
+    const int n = a.is_b ? rm.y : rm.x;
+    const float radius = __int_as_float(a.is_b ? rm.w : rm.z);
+    constexpr int nb = BINS;
+    const int sq = a.pow;
+    int2 *ent = reinterpret_cast<int2 *>(s_raw);
+    int *base = reinterpret_cast<int *>(s_raw + (size_t)a.buf * sizeof(int2));
+    for (int b = tid; b <= nb; b += kSortThreads) base[b] = 0;
+    if (tid == 0) {
+        s_big = 0;
+        s_top = 0;
+    }
     __syncthreads();
-    const int na = min(s_cnt[0], cap_a), nb = min(s_cnt[1], cap_b);
-    // List B first: its pairs go to registers, then its scratch overlays
-    // list B's buffers (list A's stay intact below them).
-    sort_and_store<IB>(key_b, val_b, nb, cap_b, __float_as_uint(r_b), key_b, list_b + i * cap_b);
-    sort_and_store<IA>(key_a, val_a, na, cap_a, __float_as_uint(r_a), key_a, list_a + i * cap_a);
-    if (tid == 0) meta[i] = make_int4(na, nb, __float_as_int(r_a), __float_as_int(r_b));
+    float top = radius;
+    if (!(radius < INFINITY)) {  // no radius: the bins span up to the largest distance
+        unsigned m = 0;
+        for (int p = tid; p < n; p += kSortThreads) m = max(m, (unsigned)raw[p].y);
+        m = __reduce_max_sync(kFull, m);
+        if (lane == 0) atomicMax(&s_top, m);
+        __syncthreads();
+        top = __uint_as_float(s_top);
+    }
+    const float inv = top > 0.0f ? 1.0f / top : 0.0f, fnb = (float)nb;
+    // The loads of kBatch entries are in flight together (E a multiple of it).
+    constexpr int kBatch = E < 8 ? E : 8;
+    unsigned at[E];  // bin << 16 | place within the bin (buffers hold under 65536 entries)
+#pragma unroll
+    for (int e0 = 0; e0 < E; e0 += kBatch) {
+        if (e0 * kSortThreads >= n) break;
+        int key[kBatch];
+#pragma unroll
+        for (int e = 0; e < kBatch; ++e) {
+            const int p = (e0 + e) * kSortThreads + tid;
+            key[e] = p < n ? raw[p].y : 0;
+        }
+#pragma unroll
+        for (int e = 0; e < kBatch; ++e) {
+            float t = __int_as_float(key[e]) * inv;  // non-decreasing in the distance
+            if (sq >= 1) t *= t;
+            if (sq >= 2) t *= t;
+            const int b = min(max((int)(t * fnb), 0), nb - 1);
+            if ((e0 + e) * kSortThreads + tid < n)
+                at[e0 + e] = (unsigned)b << 16 | (unsigned)atomicAdd(&base[b], 1);
+        }
+    }
+    __syncthreads();
+    {  // exclusive scan of the bins' counts: a warp takes nb / kSortWarps
+       // consecutive bins, 32 at a time (a thread per run of bins would meet
+       // bank conflicts as wide as the run)
+        constexpr int kSteps = nb / kSortThreads;
+        int *mine = base + warp * kSteps * 32 + lane;
+        int ex[kSteps], run = 0;
+        bool big = false;
+#pragma unroll
+        for (int b = 0; b < kSteps; ++b) {
+            const int c = mine[b * 32];
+            big |= c > kBigBin;
+            int inc = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(kFull, inc, o);
+                if (lane >= o) inc += v;
+            }
+            ex[b] = run + inc - c;
+            run += __shfl_sync(kFull, inc, 31);
+        }
+        if (lane == 0) s_part[warp] = run;
+        if (big) s_big = 1;
+        __syncthreads();
+        int before = 0;
+        for (int w = 0; w < warp; ++w) before += s_part[w];
+#pragma unroll
+        for (int b = 0; b < kSteps; ++b) {
+            mine[b * 32] = before + ex[b];
+        }
+        if (tid == 0) base[nb] = n;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e0 = 0; e0 < E; e0 += kBatch) {
+        if (e0 * kSortThreads >= n) break;
+        int2 v[kBatch];
+#pragma unroll
+        for (int e = 0; e < kBatch; ++e) {
+            const int p = (e0 + e) * kSortThreads + tid;
+            v[e] = p < n ? raw[p] : make_int2(0, 0);
+        }
+#pragma unroll
+        for (int e = 0; e < kBatch; ++e)
+            if ((e0 + e) * kSortThreads + tid < n)
+                ent[base[at[e0 + e] >> 16] + (int)(at[e0 + e] & 0xffffu)] = v[e];
+    }
+    __syncthreads();
+    if (s_big) {
+        // Bitonic sort (ascending-only form, so that any length works: an
+        // index past the end counts as +inf and never moves) of each big bin.
+        for (int b = 0; b < nb; ++b) {
+            const int s0 = base[b], m = base[b + 1] - s0;
+            if (m <= kBigBin) continue;
+            int2 *v = ent + s0;
+            int half = 1;
+            while (2 * half < m) half <<= 1;
+            auto exchange = [&](int x, int y) {
+                if (y < m) {
+                    const int2 p = v[x], r = v[y];
+                    if (p.y > r.y) {
+                        v[x] = r;
+                        v[y] = p;
+                    }
+                }
+            };
+            for (int k = 2; k <= 2 * half; k <<= 1) {
+                for (int t = tid; t < half; t += kSortThreads) {
+                    const int blk = t / (k / 2), w = t % (k / 2);
+                    exchange(blk * k + w, blk * k + k - 1 - w);
+                }
+                __syncthreads();
+                for (int j = k / 4; j > 0; j >>= 1) {
+                    for (int t = tid; t < half; t += kSortThreads) {
+                        const int x = (t / j) * 2 * j + t % j;
+                        exchange(x, x + j);
+                    }
+                    __syncthreads();
+                }
+            }
+        }
+    }
+    // Entries now lie at most kBigBin places from their own: exchanges of
+    // neighbours, even and odd pairs in turn, until a round moves nothing
+    // (about as many passes as the fullest small bin has entries).  Only the
+    // places up to the first dropped entry's bin matter.
+    const int m = min(n, cap + 1 + kBigBin);
+    bool moved = true;
+    while (moved) {
+        bool mv = false;
+        for (int x = 2 * tid; x + 1 < m; x += 2 * kSortThreads) {
+            const int4 v = *reinterpret_cast<const int4 *>(&ent[x]);
+            if (v.y > v.w) {  // bit patterns of non-negative floats order like integers
+                *reinterpret_cast<int4 *>(&ent[x]) = make_int4(v.z, v.w, v.x, v.y);
+                mv = true;
+            }
+        }
+        __syncthreads();
+        for (int x = 2 * tid + 1; x + 1 < m; x += 2 * kSortThreads) {
+            const int2 v = ent[x], w = ent[x + 1];
+            if (v.y > w.y) {
+                ent[x] = w;
+                ent[x + 1] = v;
+                mv = true;
+            }
+        }
+        moved = __syncthreads_or(mv) != 0;
+    }
+    const int len = min(n, cap), end = min(cap, (n + 31) & ~31);
+    for (int p = tid; p < end; p += kSortThreads)
+        out[p] = p < len ? ent[p] : make_int2(0, __float_as_int(INFINITY));
+    if (tid == 0) {
+        // a cut list's radius is its first dropped distance
+        const int r = n > cap ? ent[cap].y : __float_as_int(radius);
+        if (a.is_b) {
+            a.meta[i].y = len;
+            a.meta[i].w = r;
+        } else {
+            a.meta[i].x = len;
+            a.meta[i].z = r;
+        }
+    }
 }
 
-// Items per thread covering a capacity (a power of two, at least 1).
-int items_for(int cap)
+template <int DZ, int DY>
+cudaError_t launch_collect(const CollectArgs &a, cudaStream_t st)
 {
-    int it = 1;
-    while (it * kLThreads < cap) it <<= 1;
-    return it;
+    const int per = kCollectWarps * 2;  // queries per block
+    k_collect<DZ, DY><<<(unsigned)((a.n_q + per - 1) / per), kCollectThreads, 0, st>>>(a);
+    return cudaGetLastError();
 }
 
-// Shared memory of k_build_lists<ia, ib>: the histograms, or the collected
-// pairs of both lists, or list A's pairs plus list B's sort scratch,
-// whichever is largest.
-size_t build_smem(int ia, int ib, size_t tmp_b, size_t tmp_a)
+template <int DY>
+cudaError_t collect_dz(int dzb, const CollectArgs &a, cudaStream_t st)
 {
-    const size_t hist = 2 * (size_t)kBins * sizeof(int);
-    const size_t pairs_a = (size_t)kLThreads * ia * 8, pairs_b = (size_t)kLThreads * ib * 8;
-    size_t m = hist;
-    m = std::max(m, pairs_a + pairs_b);
-    m = std::max(m, pairs_a + tmp_b);
-    m = std::max(m, tmp_a);
-    return (m + 15) & ~size_t(15);
+    switch (dzb) {
+    case 1: return launch_collect<1, DY>(a, st);
+    case 2: return launch_collect<2, DY>(a, st);
+    case 3: return launch_collect<3, DY>(a, st);
+    case 4: return launch_collect<4, DY>(a, st);
+    case 5: return launch_collect<5, DY>(a, st);
+    case 6: return launch_collect<6, DY>(a, st);
+    case 8: return launch_collect<8, DY>(a, st);
+    case 10: return launch_collect<10, DY>(a, st);
+    case 12: return launch_collect<12, DY>(a, st);
+    case 16: return launch_collect<16, DY>(a, st);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
-template <int IA, int IB>
-cudaError_t launch_build(const float *sh, int dsp, int dzb, int dsb, int64_t n, int cap_a,
-                         int cap_b, int2 *list_a, int2 *list_b, int4 *meta, cudaStream_t st)
+template <int T, int E, int BINS>
+cudaError_t launch_sort(const SortPair &p, int n_q, int lists, int buf, cudaStream_t st)
 {
     static DeviceOnce attr;  // the attribute is per function and device
-    const size_t main = build_smem(IA, IB, sort_tmp_bytes<IB>(), sort_tmp_bytes<IA>());
     cudaError_t e = once_per_device(attr, [&](int) {
-        return cudaFuncSetAttribute(k_build_lists<IA, IB>,
+        return cudaFuncSetAttribute(k_sort_lists<T, E, BINS>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)(main + 2 * kMaxVisitWords * sizeof(uint32_t)));
+                                    (int)sort_smem(E * T, BINS));
     });
-    if (e != cudaSuccess) return e;
-    if (n <= 0) return cudaSuccess;
-    const int64_t vwords = ((n + kTJ - 1) / kTJ + 31) / 32;
-    const size_t smem =
-        main + (vwords <= kMaxVisitWords ? 2 * (size_t)vwords * sizeof(uint32_t) : 0);
-    k_build_lists<IA, IB><<<(unsigned)n, kLThreads, smem, st>>>(
-        sh, dsp, dzb, dsb, n, cap_a, cap_b, list_a, list_b, meta, (int)main);
+    if (e != cudaSuccess || n_q <= 0) return e;
+    k_sort_lists<T, E, BINS>
+        <<<dim3((unsigned)n_q, (unsigned)lists), T, sort_smem(buf, BINS), st>>>(p);
     return cudaGetLastError();
+}
+
+// Lists of `buf` scratch entries (n_q = 0: set-up only).  Threads per block
+// by the buffer, so that a thread has at most 12 entries and the SM's threads
+// are full or nearly so.
+cudaError_t sort_lists(const SortPair &p, int n_q, int lists, int buf, cudaStream_t st)
+{
+    if (buf <= 512) return launch_sort<128, 4, 512>(p, n_q, lists, buf, st);
+    if (buf <= 1024) return launch_sort<128, 8, 1024>(p, n_q, lists, buf, st);
+    if (buf <= 2048) return launch_sort<256, 8, 2048>(p, n_q, lists, buf, st);
+    if (buf <= 4096) return launch_sort<512, 8, 4096>(p, n_q, lists, buf, st);
+    return launch_sort<512, 12, 4096>(p, n_q, lists, buf, st);
+}
+
+// Scratch entries per query of a list (see the sampling above), or every sample.
+int buf_of(int cap, int64_t n)
+{
+    const int64_t all = (n + 31) / 32 * 32;
+    return (int)std::max<int64_t>(64, std::min<int64_t>(cap >= 2048 ? cap + cap / 2 : 2 * cap, all));
+}
+static_assert(kMaxListB + kMaxListB / 2 <= 512 * 12, "the largest buffer");
+
+size_t query_scratch(int64_t n, int cap_a, int cap_b)
+{
+    return ((size_t)buf_of(cap_a, n) + buf_of(cap_b, n)) * sizeof(int2) + sizeof(int4);
+}
+
+// Scratch of one chunk of queries: enough of them to fill the GPU several
+// times over, without another list-sized buffer for large n.
+constexpr size_t kScratchBudget = size_t(5) << 28;
+constexpr int64_t kMinChunk = 4096;
+
+int64_t chunk_of(int64_t n, int cap_a, int cap_b)
+{
+    const int64_t fit = (int64_t)(kScratchBudget / query_scratch(n, cap_a, cap_b));
+    return std::min(n, std::max(kMinChunk, fit / kTJ * kTJ));  // whole tiles: warps share their home tile
 }
 
 }  // namespace
 
-cudaError_t build_lists(const float *sh, int dsp, int dzb, int dsb, int64_t n, int cap_a,
-                        int cap_b, int2 *list_a, int2 *list_b, int4 *meta, cudaStream_t st)
+// Enough for these capacities and for any smaller ones.
+size_t list_scratch_bytes(int64_t n, int cap_a, int cap_b)
 {
-    // One instantiation per size class s: list A up to 128 s entries, list B
-    // up to 256 s (s = 2, 4, 8, 16).
-    int s = std::max(items_for(cap_b), 2 * items_for(cap_a));
-    s = std::max(s, 2);
+    const size_t per = query_scratch(n, cap_a, cap_b);
+    return std::min((size_t)n * per, std::max(kScratchBudget, (size_t)kMinChunk * per)) + 512;
+}
+
+cudaError_t build_lists(const float *sh, int dzb, int dyb, int64_t n, int cap_a, int cap_b,
+                        int2 *list_a, int2 *list_b, int4 *meta, void *scratch, cudaStream_t st,
+                        int *launches)
+{
+    if (launches) *launches = 0;
     if (n <= 0) {  // set-up only: every instantiation's attribute (outside captures)
-        cudaError_t e = launch_build<1, 2>(sh, dsp, dzb, dsb, 0, 0, 0, nullptr, nullptr, nullptr, st);
-        if (e == cudaSuccess) e = launch_build<2, 4>(sh, dsp, dzb, dsb, 0, 0, 0, nullptr, nullptr, nullptr, st);
-        if (e == cudaSuccess) e = launch_build<4, 8>(sh, dsp, dzb, dsb, 0, 0, 0, nullptr, nullptr, nullptr, st);
-        if (e == cudaSuccess) e = launch_build<8, 16>(sh, dsp, dzb, dsb, 0, 0, 0, nullptr, nullptr, nullptr, st);
+        cudaError_t e = cudaSuccess;
+        for (int buf = 512; buf <= 8192 && e == cudaSuccess; buf *= 2)
+            e = sort_lists(SortPair{}, 0, 0, buf, st);
         return e;
     }
-    switch (s) {
-    case 2:
-        return launch_build<1, 2>(sh, dsp, dzb, dsb, n, cap_a, cap_b, list_a, list_b, meta, st);
-    case 4:
-        return launch_build<2, 4>(sh, dsp, dzb, dsb, n, cap_a, cap_b, list_a, list_b, meta, st);
-    case 8:
-        return launch_build<4, 8>(sh, dsp, dzb, dsb, n, cap_a, cap_b, list_a, list_b, meta, st);
-    default:
-        return launch_build<8, 16>(sh, dsp, dzb, dsb, n, cap_a, cap_b, list_a, list_b, meta, st);
+    const int64_t chunk = chunk_of(n, cap_a, cap_b);
+    CollectArgs c{};
+    c.sh = sh;
+    c.n = n;
+    c.cap_a = cap_a;
+    c.cap_b = cap_b;
+    c.buf_a = buf_of(cap_a, n);
+    c.buf_b = buf_of(cap_b, n);
+    c.raw_a = (int2 *)scratch;
+    c.raw_b = c.raw_a + chunk * c.buf_a;
+    c.raw_meta = (int4 *)(((uintptr_t)(c.raw_b + chunk * c.buf_b) + 15) & ~(uintptr_t)15);
+    // No sample when it would be half of the samples or every list holds all.
+    const int cut = cap_a < n - 1 ? cap_a : cap_b;
+    if (cut < n - 1) {
+        const int64_t m = (cut >= 1024 ? 64 : 28) * n / cut;
+        if (2 * m <= n) {
+            c.stride = (int)(n / m);
+            c.n_sample = (int)((n + c.stride - 1) / c.stride);
+        }
     }
+    // squarings: the power of the distance that evens out the bins
+    auto squarings = [](int d) { return d >= 4 ? 2 : (d >= 2 ? 1 : 0); };
+    SortPair s{};
+    s.l[0] = SortArgs{c.raw_a, c.raw_meta, c.buf_a, cap_a, 0, squarings(dzb + dyb), 0, list_a, meta};
+    s.l[1] = SortArgs{c.raw_b, c.raw_meta, c.buf_b, cap_b, 1, squarings(dzb), 0, list_b, meta};
+    for (int64_t q0 = 0; q0 < n; q0 += chunk) {
+        const int n_q = (int)std::min(chunk, n - q0);
+        c.q0 = s.l[0].q0 = s.l[1].q0 = q0;
+        c.n_q = n_q;
+        cudaError_t e = dyb == 1   ? collect_dz<1>(dzb, c, st)
+                        : dyb == 2 ? collect_dz<2>(dzb, c, st)
+                        : dyb == 4 && dzb == 16 ? launch_collect<16, 4>(c, st)
+                                                : cudaErrorInvalidValue;
+        if (e != cudaSuccess) return e;
+        // Short lists in one launch; long ones apart, with the blocks of each size.
+        const int buf = std::max(c.buf_a, c.buf_b);
+        const bool together = buf <= 1024 || c.buf_a == c.buf_b;
+        e = sort_lists(s, n_q, together ? 2 : 1, together ? buf : c.buf_a, st);
+        if (e == cudaSuccess && !together) e = sort_lists(SortPair{{s.l[1], s.l[1]}}, n_q, 1, c.buf_b, st);
+        if (e != cudaSuccess) return e;
+        if (launches) *launches += together ? 2 : 3;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace idtx

@@ -702,14 +702,21 @@ struct idtx_ctx {
     std::vector<uint64_t> graph_key;
     cudaStream_t cap_stream = nullptr;
     cudaStream_t side_stream = nullptr;  // second stream of a call (prep_group)
-    // kernel choice: IDTX_KERNEL_AUTO picks per (variant, log2 N) by timing
-    // both kernels on the first call of that shape; list capacities (0: default)
+    // kernel choice: IDTX_KERNEL_AUTO times the kernels on the first call of a
+    // shape (variant, log2 N) and picks by these times, scaled to the call at
+    // hand; list capacities (0: default)
     int kernel_pref = IDTX_KERNEL_AUTO;
-    struct Choice {
-        bool list;         // list kernel (else tile kernel)
-        int cap_a, cap_b;  // its list capacities
+    struct Timed {
+        bool list;                // list kernel (else tile kernel)
+        int cap_a, cap_b;         // its list capacities
+        float build_ms, est_ms;   // building the lists, the estimator
     };
-    std::map<std::pair<const KsgVariant *, int>, Choice> tuned;
+    struct Trial {
+        int64_t n;
+        int groups;               // job groups of the timed call
+        std::vector<Timed> way;
+    };
+    std::map<std::pair<const KsgVariant *, int>, Trial> tuned;
     int cap_a = 0, cap_b = 0;
     long long wait_ns = 0;  // bound of device waits (0: settings->timeout_ms)
 };
@@ -861,6 +868,36 @@ std::pair<const KsgVariant *, int> tune_key(const Group &g)
     return {g.v, lg};
 }
 
+// The way of running g that the trial's times, scaled to g, put first.
+// Building lists and the tile kernel grow as n^2, the walks as n; the
+// estimators with the job groups, while the lists are built once for all of
+// them: a call of few groups may want the tile kernel or shorter lists where
+// one of many groups does not.
+const idtx_ctx::Timed &best_way(const idtx_ctx::Trial &t, const Group &g)
+{
+    const float rn = (float)g.n / (float)t.n, rg = (float)g.n_groups / (float)t.groups;
+    size_t best = 0;
+    float best_ms = 0.0f;
+    for (size_t i = 0; i < t.way.size(); ++i) {
+        const idtx_ctx::Timed &w = t.way[i];
+        const float ms = w.build_ms * rn * rn + w.est_ms * rg * (w.list ? rn : rn * rn);
+        if (i == 0 || ms < best_ms) {
+            best = i;
+            best_ms = ms;
+        }
+    }
+    return t.way[best];
+}
+
+void take_way(Group &g, const idtx_ctx::Timed &w)
+{
+    g.use_list = w.list;
+    if (w.list) {
+        g.cap_a = std::min(g.cap_a, w.cap_a);
+        g.cap_b = std::min(g.cap_b, w.cap_b);
+    }
+}
+
 int plan(idtx_ctx *c, Group &g)
 {
     g.v = pick_variant(c, g.dx, g.dy, g.dz, g.k);
@@ -886,11 +923,7 @@ int plan(idtx_ctx *c, Group &g)
                 if (it == c->tuned.end()) {
                     g.tune = true;
                 } else {
-                    g.use_list = it->second.list;
-                    if (g.use_list) {
-                        g.cap_a = it->second.cap_a;
-                        g.cap_b = it->second.cap_b;
-                    }
+                    take_way(g, best_way(it->second, g));
                 }
             }
         }
@@ -935,7 +968,7 @@ struct CallBuffers {
 };
 
 // B_LIST layout for n queries: list_a [n][cap_a] | list_b [n][cap_b] | meta [n]
-// | the list kernel's term ring.
+// | the list kernel's term ring, all counted here | build_lists' scratch.
 size_t list_bytes(int64_t n, int cap_a, int cap_b)
 {
     return align_up((size_t)n * cap_a * sizeof(int2), 256) +
@@ -960,7 +993,8 @@ CallBuffers bytes_of(const Group &g)
     b.xi = align_up((size_t)g.n_groups * g.n_pad * g.v->gb * g.v->dx * sizeof(float), 256);
     b.perm = align_up(g.slot_stream.size() * (size_t)(g.n + g.n_reps) * sizeof(int32_t), 256);
     b.partial = align_up(g.jobs.size() * (size_t)g.n_qt * sizeof(double), 256);
-    if (g.use_list || g.tune) b.lists = list_bytes(g.n, g.cap_a, g.cap_b);
+    if (g.use_list || g.tune)
+        b.lists = list_bytes(g.n, g.cap_a, g.cap_b) + list_scratch_bytes(g.n, g.cap_a, g.cap_b);
     return b;
 }
 
@@ -1091,6 +1125,7 @@ void fill_launch(const idtx_ctx *c, const Group &g, const Slices &sl, float *eps
     a.list_b = nullptr;
     a.lmeta = nullptr;
     a.ring = nullptr;
+    a.lscratch = nullptr;
     a.cap_a = g.cap_a;
     a.cap_b = g.cap_b;
     if ((g.use_list || g.tune) && sl.lists) {
@@ -1101,6 +1136,7 @@ void fill_launch(const idtx_ctx *c, const Group &g, const Slices &sl, float *eps
         a.list_b = (const int2 *)(sl.lists + oa);
         a.lmeta = (const int4 *)(sl.lists + oa + ob);
         a.ring = (double *)(sl.lists + oa + ob + om);
+        a.lscratch = sl.lists + list_bytes(g.n, g.cap_a, g.cap_b);
     }
 }
 
@@ -1200,14 +1236,15 @@ int prep_group(idtx_ctx *c, const Group &g, cudaStream_t st, const Slices &sl, f
     IDTX_CUDA(cudaGetLastError());
     if (a.list_a) {
         IDTX_CUDA(cudaEventRecord(join, xs));
-        IDTX_CUDA(build_lists(sh, v.dsp, v.dz, v.dz + v.dy, g.n, g.cap_a, g.cap_b,
+        int built = 0;
+        IDTX_CUDA(build_lists(sh, v.dz, v.dy, g.n, g.cap_a, g.cap_b,
                               const_cast<int2 *>(a.list_a), const_cast<int2 *>(a.list_b),
-                              const_cast<int4 *>(a.lmeta), st));
+                              const_cast<int4 *>(a.lmeta), a.lscratch, st, &built));
         IDTX_CUDA(cudaStreamWaitEvent(st, join, 0));
         // a later record of these events does not disturb the waits above
         c->event_pool.push_back(fork);
         c->event_pool.push_back(join);
-        launches += 1;
+        launches += built;
     }
     launches += 5;  // pack, boxes, gather, fused, finalize
     return IDTX_OK;
@@ -1238,69 +1275,61 @@ void note_group(idtx_ctx *c, const Group &g, int launches, bool list)
 }
 
 // Time the candidate ways of running a prepared group -- the tile kernel, and
-// the list kernel (list building included) with the group's list capacities
-// and with two smaller ones -- and remember the fastest for this (variant,
-// log2 N).  Every candidate writes the same partial sums.  On return the
-// lists in the buffer, and a's capacities, are those of the choice.
+// the list kernel with the group's list capacities and with two smaller ones
+// -- and remember the times for this (variant, log2 N).  Every candidate
+// writes the same partial sums.  On return the lists in the buffer, and a's
+// capacities, are those of the choice.
 int tune_group(idtx_ctx *c, const Group &g, KsgLaunch &a, cudaStream_t st, bool &use_list)
 {
-    struct Cand {
-        bool list;
-        int ca, cb;
-        float ms;
-    };
-    std::vector<Cand> cands{{false, 0, 0, 0.0f}, {true, g.cap_a, g.cap_b, 0.0f}};
+    idtx_ctx::Trial trial{g.n, g.n_groups, {{false, 0, 0, 0.0f, 0.0f}, {true, g.cap_a, g.cap_b, 0.0f, 0.0f}}};
+    std::vector<idtx_ctx::Timed> &way = trial.way;
     if (c->cap_a == 0 && c->cap_b == 0)  // capacities not fixed by the caller
         for (int sh = 1; sh <= 2; ++sh) {
             const int ca = (g.cap_a >> sh) / 32 * 32, cb = (g.cap_b >> sh) / 32 * 32;
-            if (ca >= 256 && cb >= 256) cands.push_back({true, ca, cb, 0.0f});
+            if (ca >= 256 && cb >= 256) way.push_back({true, ca, cb, 0.0f, 0.0f});
         }
     const KsgVariant &v = *g.v;
     KsgLaunch t = a;
     t.work = nullptr;
-    std::vector<cudaEvent_t> ev(cands.size() + 1);
+    auto build = [&](int ca, int cb) -> int {
+        int built = 0;
+        IDTX_CUDA(build_lists(a.sh, v.dz, v.dy, g.n, ca, cb, const_cast<int2 *>(a.list_a),
+                              const_cast<int2 *>(a.list_b), const_cast<int4 *>(a.lmeta),
+                              a.lscratch, st, &built));
+        c->stats.kernel_launches += built;
+        return IDTX_OK;
+    };
+    std::vector<cudaEvent_t> ev(2 * way.size() + 1);  // before way 0; after each build and estimator
     for (auto &e : ev) IDTX_TRY(take_event(c, &e));
     IDTX_CUDA(cudaEventRecord(ev[0], st));
-    int built_a = g.cap_a, built_b = g.cap_b;  // the lists prep_group built
-    for (size_t i = 0; i < cands.size(); ++i) {
-        const Cand &cd = cands[i];
-        if (!cd.list) {
-            IDTX_CUDA(v.fn(t, g.n_groups, st));
-        } else {
-            // the first list candidate re-times the build prep_group did
-            IDTX_CUDA(build_lists(t.sh, v.dsp, v.dz, v.dz + v.dy, g.n, cd.ca, cd.cb,
-                                  const_cast<int2 *>(t.list_a), const_cast<int2 *>(t.list_b),
-                                  const_cast<int4 *>(t.lmeta), st));
-            built_a = cd.ca;
-            built_b = cd.cb;
-            t.cap_a = cd.ca;
-            t.cap_b = cd.cb;
-            IDTX_CUDA(v.fn_list(t, g.n_groups, st));
-        }
-        IDTX_CUDA(cudaEventRecord(ev[i + 1], st));
+    for (size_t i = 0; i < way.size(); ++i) {
+        // the first list candidate re-times the build prep_group did
+        if (way[i].list) IDTX_TRY(build(way[i].cap_a, way[i].cap_b));
+        IDTX_CUDA(cudaEventRecord(ev[2 * i + 1], st));
+        t.cap_a = way[i].cap_a;
+        t.cap_b = way[i].cap_b;
+        IDTX_CUDA(way[i].list ? v.fn_list(t, g.n_groups, st) : v.fn(t, g.n_groups, st));
+        IDTX_CUDA(cudaEventRecord(ev[2 * i + 2], st));
     }
     IDTX_CUDA(cudaEventSynchronize(ev.back()));
-    size_t best = 0;
-    for (size_t i = 0; i < cands.size(); ++i) {
-        IDTX_CUDA(cudaEventElapsedTime(&cands[i].ms, ev[i], ev[i + 1]));
-        if (cands[i].ms < cands[best].ms) best = i;
+    for (size_t i = 0; i < way.size(); ++i) {
+        IDTX_CUDA(cudaEventElapsedTime(&way[i].build_ms, ev[2 * i], ev[2 * i + 1]));
+        IDTX_CUDA(cudaEventElapsedTime(&way[i].est_ms, ev[2 * i + 1], ev[2 * i + 2]));
     }
+    way[0].build_ms = 0.0f;
     for (auto &e : ev) c->event_pool.push_back(e);
-    const Cand &b = cands[best];
+    const idtx_ctx::Timed b = best_way(trial, g);
     use_list = b.list;
-    c->tuned[tune_key(g)] = idtx_ctx::Choice{b.list, b.ca, b.cb};
-    if (b.list && (built_a != b.ca || built_b != b.cb)) {
-        IDTX_CUDA(build_lists(a.sh, v.dsp, v.dz, v.dz + v.dy, g.n, b.ca, b.cb,
-                              const_cast<int2 *>(a.list_a), const_cast<int2 *>(a.list_b),
-                              const_cast<int4 *>(a.lmeta), st));
-        c->stats.kernel_launches += 1;
-    }
     if (b.list) {
-        a.cap_a = b.ca;
-        a.cap_b = b.cb;
+        // the lists in the buffer are the last candidate's
+        if (b.cap_a != way.back().cap_a || b.cap_b != way.back().cap_b)
+            IDTX_TRY(build(b.cap_a, b.cap_b));
+        a.cap_a = b.cap_a;
+        a.cap_b = b.cap_b;
     }
     c->stats.tune_trials += 1;
-    c->stats.kernel_launches += (int64_t)(2 * cands.size() - 1);
+    c->stats.kernel_launches += (int64_t)way.size();  // the estimator launches
+    c->tuned[tune_key(g)] = std::move(trial);
     return IDTX_OK;
 }
 
@@ -1553,12 +1582,7 @@ int resolve_tuning(idtx_ctx *c, std::vector<Group> &gs, cudaStream_t st, long lo
             IDTX_TRY(tune_group(c, g, a, st, unused));
             c->stats.kernel_launches += launches - 2;
         }
-        const idtx_ctx::Choice ch = c->tuned[tune_key(g)];
-        g.use_list = ch.list;
-        if (ch.list) {
-            g.cap_a = ch.cap_a;
-            g.cap_b = ch.cap_b;
-        }
+        take_way(g, best_way(c->tuned[tune_key(g)], g));
         g.tune = false;
     }
     return IDTX_OK;
@@ -2076,8 +2100,8 @@ int idtx_cmi_batch(idtx_ctx *c, const idtx_problem *probs, int n_probs, int k, d
             else
                 c->event_pool.push_back(ev);
         }
-        if (rc == IDTX_OK && build_lists(nullptr, 4, 1, 1, 0, 0, 0, nullptr, nullptr, nullptr, st) !=
-                                 cudaSuccess)
+        if (rc == IDTX_OK && build_lists(nullptr, 1, 1, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, st,
+                                         nullptr) != cudaSuccess)
             rc = fail(IDTX_ECUDA, "list kernel attribute setup failed");
         for (const KsgVariant *v : bp.vars)
             if (rc == IDTX_OK && v->fn_table(KsgTable{nullptr, nullptr, nullptr, 0, 0}, st) !=

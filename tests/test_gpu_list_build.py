@@ -1,0 +1,67 @@
+"""List building where it can go wrong: more queries than one chunk of scratch,
+an odd query count, scratch buffers that overflow (a radius sampled too wide)
+and runs of equal distances longer than a sorting bin.  The estimates, eps and
+counts over the lists are compared with the tile kernel's, which uses no lists
+(bit for bit, as both sum in the same order), or with the oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1807_10459_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def idtx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1807_10459_gb300 as m
+    from paper_1807_10459_gb300 import build
+    build.build()
+    return m
+
+
+def _both(idtx, x, y, z, caps, S=2, k=4):
+    out = []
+    for kernel in (idtx.KERNEL_LIST, idtx.KERNEL_TILE):
+        ctx = idtx.Context(0)
+        ctx.set_kernel(kernel)
+        ctx.set_list_caps(*caps)
+        dev = [torch.from_numpy(np.ascontiguousarray(c)).cuda() for c in (x, y, z)]
+        r = idtx.cmi_ksg(*dev, k=k, n_surr=S, seed=11, want_eps=True, want_counts=True, ctx=ctx)
+        out.append([t.cpu().numpy() for t in r])
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+    return out[0]
+
+
+@pytest.mark.parametrize("n,dims,caps", [
+    (18501, (1, 1, 2), (0, 0)),      # two chunks of scratch, the second one short
+    (4097, (1, 1, 7), (96, 160)),    # a tile of one sample; first dimensions tested first
+    (2047, (2, 2, 3), (512, 1024)),
+    (700, (1, 1, 1), (32, 64)),
+])
+def test_lists_give_the_tile_kernels_results(idtx, n, dims, caps):
+    g = synth.gaussian_problem(n, *dims, seed=n)
+    _both(idtx, g.x, g.y, g.z, caps)
+
+
+def test_lists_of_uneven_density_and_equal_distances(idtx):
+    """Half of the samples in tight clusters the sampled rows hardly meet, a
+    fifth on a coarse grid (equal distances by the hundred), the rest wide."""
+    rng = np.random.default_rng(8)
+    n = 1500
+    s = rng.standard_normal((4, n)) * 5
+    c = rng.random(n) < 0.5
+    s[:, c] = rng.integers(0, 3, (4, c.sum())) + 1e-4 * rng.standard_normal((4, c.sum()))
+    g = rng.random(n) < 0.2
+    s[:, g] = rng.integers(-2, 3, (4, g.sum()))
+    s = s.astype(np.float32)
+    x, y, z = s[:1], s[1:2], s[2:]
+    for caps in ((32, 32), (96, 160), (512, 1024)):
+        _, eps, cnt = _both(idtx, x, y, z, caps)
+        e, a, b, d = oracle.ksg_counts(x, y, z, 4)
+        assert np.array_equal(eps[0], e)
+        assert np.array_equal(cnt[0], np.stack([a, b, d]))
