@@ -92,8 +92,19 @@ struct KsgLaunch {
     const int4 *lmeta;
     double *ring;  // kListRingBytes of scratch for the list kernel's term ring
     void *lscratch;  // list_scratch_bytes of scratch for build_lists
+    // list kernel, n_pad <= 65536 (else null): the counts n_yz, n_z, n_xz of
+    // every (group, query, job), [n_groups][n_pad][32], for sum_terms
+    uint16_t *cyz, *cz, *cxz;
+    // with them: (group, query, jobs) left to ksg_scan_kernel, and counters, 0
+    // between launches: the next chunk, the CTAs done, the entries of scans
+    int4 *scans;
+    int *next;
     int cap_a, cap_b;
 };
+
+// The digamma terms of the list kernel's counts, summed into partial: query
+// tiles of qc queries, nws interleaved sums each (sums.cu).
+cudaError_t sum_terms(const KsgLaunch &a, int qc, int nws, int n_groups, cudaStream_t st);
 
 typedef cudaError_t (*KsgLaunchFn)(const KsgLaunch &, int n_groups, cudaStream_t);
 

@@ -19,8 +19,8 @@
 //     one, so the walk stops there.  If the list runs out while the k-th
 //     value is still above r_A, an unlisted sample might enter: that job is
 //     recomputed by a full scan.
-//   pass B: n_yz = #{list A entries with d_YZ < eps} (binary search over the
-//     prefix pass A walked); n_z and n_xz counted over the list B entries with
+//   pass B: n_yz = #{list A entries with d_YZ < eps} (bisection of the prefix
+//     pass A walked); n_z and n_xz counted over the list B entries with
 //     d_Z < eps, using max(d_X, d_Z) < eps <=> d_X < eps and d_Z < eps.  Both
 //     are exact when eps <= r_A and eps <= r_B (every sample closer than eps
 //     is listed); otherwise the job's counts come from a full scan.
@@ -30,43 +30,49 @@
 // bit-identical estimates and either may serve a call.
 //
 // Design (GB300).  The kernel is persistent: one CTA of 32 warps per SM, one
-// job per lane.  A CTA takes chunks of up to 8 consecutive query tiles of one
-// job group (chunks ordered query block by query block, so the CTAs in flight
-// share the lists of one block of queries), and its warps take the chunk's
-// queries one at a time from a shared counter.  So at any moment the
-// SM's warps serve ~32 consecutive queries of one group: samples are in Morton
-// order of (Z, Y), the neighbourhoods of consecutive queries overlap, and the
-// X rows the walks gather (one 128-byte row of xi per list entry: the 32 jobs'
-// X at that sample) are reused from L1 instead of L2.  Shared memory holds
-// only the per-query digamma terms of the last few query tiles (a ring of
-// tile slots, so the terms can be summed in the fixed order once a tile's 64
-// queries are done), the warps' staged list entries and work counters; the
-// rest of the SM's 256 KB serves as L1.
-//   * Walks read their list 32 entries at a time with one coalesced load (the
-//     next chunk prefetched), stage them in the warp's shared buffer and
-//     consume them in sub-chunks whose X rows are loaded back to back.  The
-//     shared walks are warp-uniform (they stop when every lane's job is done);
-//     the one or two jobs that would lengthen a walk most finish lane-split
-//     (the 32 lanes splitting the entries), two or four blocks of entries per
-//     step so that the loads of a step are in flight together.
-//   * The only waits are on the tile ring: a warp that takes a query of tile
-//     t waits until tile t - RING has been summed (that tile's queries were
-//     all taken earlier, so the wait always ends); the wait is bounded by
-//     %globaltimer, and on expiry the CTA records kErrTimeout and stops.
+// job per lane.  A CTA takes chunks of consecutive queries of one job group
+// (chunks ordered query block by query block, so the CTAs in flight share the
+// lists of one block of queries), and its warps take the chunk's queries one
+// at a time.  So at any moment the SM's warps serve ~32 consecutive queries of
+// one group: samples are in Morton order of (Z, Y), the neighbourhoods of
+// consecutive queries overlap, and the X rows the walks gather (one 128-byte
+// row of xi per list entry: the 32 jobs' X at that sample) are reused from L1
+// instead of L2.
+//   * Walks stage their list 32 entries at a time into the warp's buffer and
+//     fetch the X rows of the next IDTX_LIST_SA entries while they use those
+//     of the last.  The shared walks are warp-uniform (they stop when every
+//     lane's job is done); the one or two jobs that would lengthen the
+//     neighbour walk most finish lane-split (the 32 lanes splitting the
+//     entries), the last of the count walk with the lanes shared out among
+//     them.
+//   * Split form (n_pad <= 65536): the counts go out as 16-bit numbers and
+//     sum_terms (sums.cu) forms and sums the terms.  No order of the queries
+//     matters then, so the CTAs take chunks as they come free; (query, group)s
+//     that need full scans are queued for ksg_scan_kernel.
+//   * Otherwise the terms go through a ring of tile slots in global memory, so
+//     that they can be summed in the fixed order once a tile's queries are
+//     done, the CTAs' chunks are fixed, and full scans run in place.  A warp
+//     that takes a query of tile t waits until tile t - RING has been summed
+//     (that tile's queries were all taken earlier, so the wait always ends).
+//     Every wait is bounded by %globaltimer; on expiry the CTA records
+//     kErrTimeout and stops.
+// Measured on GB300, greedy step of N = 9995 with 9447 estimates (one network;
+// lists of 2048 and 4096): 19.1 -> 13.2 ms with sum_terms; of N = 4997, six
+// conditions, 28341 estimates: 10.8 -> 9.7 ms; N = 1000, 101 estimates: 163 ->
+// 70 us.  Bound by issue (58 % of the slots) and the latency behind it: fewer,
+// fatter warps (24 of 80 registers) were 8 % slower.
 #pragma once
+
+#include <type_traits>
 
 #include "ksg_kernel.cuh"
 #include "ksg_plain.cuh"
 
-// List entries per sub-chunk of the neighbour-pass and count-pass walks
-// (even divisors of 32; compile-time knobs, the defaults are the tuned values:
-// on GB300, list kernel of the greedy step, interleaved runs, SA/SB = 16/16
-// 15.55-15.73 ms, 8/16 15.53-15.55, 16/8 15.55, 8/8 16.05).
+// List entries whose X rows a walk has in flight (a multiple of 4, at most 16;
+// compile-time knobs, the defaults are the tuned values: 4 / 8 / 16 give the
+// greedy step 13.8 / 13.2 / 13.4 ms).
 #ifndef IDTX_LIST_SA
 #define IDTX_LIST_SA 8
-#endif
-#ifndef IDTX_LIST_SB
-#define IDTX_LIST_SB 16
 #endif
 // Jobs of a warp whose neighbour walk goes on past the others' and is
 // finished with the lanes splitting its entries.
@@ -74,41 +80,45 @@
 #define IDTX_LIST_TAIL_A 2
 #endif
 // The shared count walk hands over to the repacked phases once at most this
-// many jobs (a power of two <= 16) still need entries.
+// many jobs (a power of two <= 16) still need entries (4 / 8 / 16: within 1 %).
 #ifndef IDTX_LIST_REPACK
 #define IDTX_LIST_REPACK 8
 #endif
-// Entries a lane takes per step of a repacked count phase (their X loads are
-// in flight together; a step's entries past the lane's share are predicated
-// off).  Measured on GB300, list kernel of the greedy step: 1 / 2 / 4 / 8
-// entries 15.80 / 15.75 / 16.05 / 17.72 ms.
+// Entries a lane takes per step of a repacked count phase (their loads are in
+// flight together; entries past the lane's job are predicated off): 2 / 4
+// entries give the greedy step 13.5 / 13.2 ms.
 #ifndef IDTX_LIST_PHASE_STEP
-#define IDTX_LIST_PHASE_STEP 2
+#define IDTX_LIST_PHASE_STEP 4
 #endif
 // Job groups per super-block of the chunk order (see the kernel).
 #ifndef IDTX_LIST_GSB
 #define IDTX_LIST_GSB 16
 #endif
-// Most consecutive query tiles a CTA takes at a time (fewer when the call
-// has too few tiles to give every SM two chunks; the ring's depth,
-// kListRing, is in ksg_common.cuh).
+// The form with the ring: most consecutive query tiles a CTA takes at a time
+// (fewer when the call has too few tiles to give every SM two chunks; the
+// ring's depth, kListRing, is in ksg_common.cuh).  The split form: queries
+// (256 to 1024 are alike).
 #ifndef IDTX_LIST_CHUNK
 #define IDTX_LIST_CHUNK 8
+#endif
+#ifndef IDTX_LIST_CHUNKQ
+#define IDTX_LIST_CHUNKQ 256
 #endif
 
 namespace idtx {
 
-// Number of entries of the ascending list l[0..hi) whose distance is below v.
+// Number of entries of the ascending list l[0..hi) (hi the lane's own) whose
+// distance is below v, for every lane of a warp.  Warp-uniform probes of
+// every lane at once first bound the answers by a power of two (most are far
+// below hi); then each lane bisects without branches.
 __device__ __forceinline__ int list_lower(const int2 *l, int hi, float v)
 {
+    constexpr unsigned kFull = 0xffffffffu;
+    int bits = 4;  // the answers are below 2^bits
+    while (__any_sync(kFull, (1 << bits) <= hi && __int_as_float(__ldg(&l[(1 << bits) - 1].y)) < v)) ++bits;
     int lo = 0;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (__int_as_float(__ldg(&l[mid].y)) < v)
-            lo = mid + 1;
-        else
-            hi = mid;
-    }
+    for (int b = (1 << bits) >> 1; b; b >>= 1)
+        if (lo + b <= hi && __int_as_float(__ldg(&l[lo + b - 1].y)) < v) lo += b;
     return lo;
 }
 
@@ -138,14 +148,48 @@ struct ListShape {
     static constexpr int RING = kListRing;
     static_assert(QC <= 64, "the term ring holds tiles of up to 64 queries");
     struct Smem {
-        int2 ent[NW][32];  // per warp: staged list entries
+        int2 ent[NW][64];  // per warp: two chunks of staged list entries
         unsigned long long work[NW][kNumWork];
         int owner[RING];  // the CTA-local tile number a slot currently serves
         int done[RING];   // queries of that tile finished
         int next;         // next CTA-local query position
+        // split form: the CTA's chunks in their order (number, chunk; a ring),
+        // the next query (number << 16 | query within the chunk), and the
+        // chunk to follow (-1: being fetched)
+        int2 chunk[8];
+        unsigned cur;
+        int ahead;
     };
     static constexpr size_t SMEM = sizeof(Smem);
 };
+
+// Merge four distances into the ascending h[0..4): sort them, take the four
+// smallest of both (the element-wise minimum of one and the other reversed),
+// and order that bitonic sequence.  22 minima and maxima without a branch,
+// against 28 for four insertions; in a warp of 32 jobs nearly every group of
+// four holds a distance for some job's h, so skipping it rarely pays.
+__device__ __forceinline__ void cmp_swap(float &a, float &b)
+{
+    const float lo = fminf(a, b);
+    b = fmaxf(a, b);
+    a = lo;
+}
+__device__ __forceinline__ void merge4(float (&h)[4], float s0, float s1, float s2, float s3)
+{
+    cmp_swap(s0, s1);
+    cmp_swap(s2, s3);
+    cmp_swap(s0, s2);
+    cmp_swap(s1, s3);
+    cmp_swap(s1, s2);
+    h[0] = fminf(h[0], s3);
+    h[1] = fminf(h[1], s2);
+    h[2] = fminf(h[2], s1);
+    h[3] = fminf(h[3], s0);
+    cmp_swap(h[0], h[2]);
+    cmp_swap(h[1], h[3]);
+    cmp_swap(h[0], h[1]);
+    cmp_swap(h[2], h[3]);
+}
 
 // Wait until *owner == want (tile slot free), bounded by timeout_ns.
 __device__ __forceinline__ bool wait_slot(const int *owner, int want, long long timeout_ns)
@@ -160,9 +204,9 @@ __device__ __forceinline__ bool wait_slot(const int *owner, int want, long long 
     return true;
 }
 
-template <int DX, int DY, int DZ, int K1, bool EXACT, int QCTA, int NWARPS>
+template <int DX, int DY, int DZ, int K1, bool EXACT, int QCTA, int NWARPS, bool SPLIT>
 __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>::THREADS, 1)
-    ksg_list_kernel(const KsgLaunch a, const int n_groups, const int n_chunks, const int chunk_lg)
+    ksg_list_kernel(const KsgLaunch a, const int n_groups, const int n_chunks, const int chunk_q)
 {
     using S = KsgShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>;
     using LS = ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>;
@@ -172,8 +216,7 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
     constexpr int KH = K1 - 1;  // smallest distances kept (EXACT: exactly k)
     constexpr int kShStage = kTileRows * DSP;
     constexpr unsigned kFull = 0xffffffffu;
-    constexpr int SA = IDTX_LIST_SA, SB = IDTX_LIST_SB;  // entries per sub-chunk of the walks
-    constexpr int TAIL_A = IDTX_LIST_TAIL_A;  // and after the shared neighbour walk
+    constexpr int TAIL_A = IDTX_LIST_TAIL_A;  // jobs left after the shared neighbour walk
     const float kInf = CUDART_INF_F;
 
     extern __shared__ __align__(16) unsigned char l_smem[];
@@ -185,8 +228,14 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
         sm.owner[tid] = tid;
         sm.done[tid] = 0;
     }
-    if (tid == 0) sm.next = 0;
-    for (int i = tid; i < NW * kNumWork; i += LS::THREADS) (&sm.work[0][0])[i] = 0;
+    if (tid == 0) {
+        sm.next = 0;
+        if (SPLIT) {
+            sm.cur = 0;
+            sm.chunk[0] = make_int2(0, atomicAdd(a.next, 1));
+            sm.ahead = atomicAdd(a.next, 1);
+        }
+    }
     __syncthreads();
 
     int2 *ent = sm.ent[warp];
@@ -195,74 +244,140 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
     auto kth = [&](const float(&h)[KH]) { return EXACT ? h[KH - 1] : select_kth<KH>(h, kk - 1); };
     auto sh_row = [&](int64_t j) { return a.sh + (j / kTJ) * kShStage + (j % kTJ) * DSP; };
     const long long t_begin = clock64();
+    unsigned long long my_work = 0;   // work counter `lane` of this warp (5: cycles)
+    int grp = 0, qt = 0, num_of = -1, q_of = 0;  // the last query's group, tile or chunk
 
     while (true) {
-        // ---------------- take the CTA's next query: tile lt of its stream is
-        // tile lt mod 2^chunk_lg of chunk blockIdx.x + (lt >> chunk_lg) *
-        // gridDim.x.  Chunks run in super-blocks of GSB groups, query block
+        // ---------------- take the CTA's next query.  Chunks of consecutive
+        // queries of one group run in super-blocks of GSB groups, query block
         // by query block within a super-block, so the CTAs in flight share a
         // few groups' X rows and a range of queries' lists in L2, while each
-        // CTA's warps serve consecutive queries of one group.  Tiles past a
-        // group's last one (its last block may be short) are claimed as
-        // empty.
-        int p = 0;
-        if (lane == 0) p = atomicAdd(&sm.next, 1);
-        p = __shfl_sync(kFull, p, 0);
-        const int lt = p / QC, m = p - lt * QC;
-        const int chunk = static_cast<int>(blockIdx.x) + (lt >> chunk_lg) * static_cast<int>(gridDim.x);
-        if (chunk >= n_chunks) break;
-        const int slot = lt % RING;
-        int ok = 1;
-        if (lane == 0) ok = wait_slot(&sm.owner[slot], lt, a.timeout_ns) ? 1 : 0;
-        ok = __shfl_sync(kFull, ok, 0);
-        if (!ok) {
-            if (lane == 0) atomicOr(a.err, kErrTimeout);
-            break;
+        // CTA's warps serve consecutive queries of one group.
+        int slot = 0, lt = 0, m = 0;
+        int qi;  // the query (sorted position)
+        if constexpr (SPLIT) {
+            // Chunks of `chunk_q` queries, taken by the CTAs as they come free
+            // (the queries' work differs).  The warp that takes the first
+            // query past a chunk brings in the one fetched ahead; others that
+            // come before it has try again.
+            unsigned v = 0;
+            if (lane == 0) v = atomicAdd(&sm.cur, 1u);
+            v = __shfl_sync(kFull, v, 0);
+            const int num = static_cast<int>(v >> 16), at = static_cast<int>(v & 0xffffu);
+            if (at >= chunk_q) {
+                int ok = 1;
+                if (lane == 0) {
+                    const long long t0 = global_ns();
+                    if (at == chunk_q) {
+                        volatile int *ahead = &sm.ahead;
+                        while (ok && *ahead < 0) {
+                            __nanosleep(32);
+                            ok = global_ns() - t0 <= a.timeout_ns;
+                        }
+                        if (ok) {
+                            const int next = *ahead;
+                            *ahead = -1;
+                            sm.chunk[(num + 1) & 7] = make_int2((num + 1) & 0xffff, next);
+                            __threadfence_block();
+                            atomicExch(&sm.cur, static_cast<unsigned>(num + 1) << 16);
+                            *ahead = next < n_chunks ? atomicAdd(a.next, 1) : next;
+                        }
+                    } else {
+                        const volatile unsigned *cur = &sm.cur;
+                        while (ok && (*cur >> 16) == (v >> 16)) {
+                            __nanosleep(32);
+                            ok = global_ns() - t0 <= a.timeout_ns;
+                        }
+                    }
+                }
+                if (!__shfl_sync(kFull, ok, 0)) {
+                    if (lane == 0) atomicOr(a.err, kErrTimeout);
+                    break;
+                }
+                continue;
+            }
+            if (num != num_of) {
+                num_of = num;
+                __threadfence_block();
+                const int2 mine = sm.chunk[num & 7];
+                if (mine.x != num) {  // overtaken by seven chunks: cannot be, and is not passed over
+                    if (lane == 0) atomicOr(a.err, kErrInternal);
+                    break;
+                }
+                const int chunk = mine.y;
+                if (chunk >= n_chunks) break;
+                const int n_qb = (static_cast<int>(a.n) + chunk_q - 1) / chunk_q;
+                const int per_sb = IDTX_LIST_GSB * n_qb;
+                const int sb = chunk / per_sb;
+                const int g0 = sb * IDTX_LIST_GSB;
+                const int gs = n_groups - g0 < IDTX_LIST_GSB ? n_groups - g0 : IDTX_LIST_GSB;
+                const int rc = chunk - sb * per_sb;
+                const int qblock = rc / gs;
+                grp = g0 + (rc - qblock * gs);
+                q_of = qblock * chunk_q;
+            }
+            qi = q_of + at;
+        } else {
+            // The ring sums the tiles in their order, so the CTA's stream is
+            // fixed: tile lt of it is tile lt mod 2^chunk_lg of chunk
+            // blockIdx.x + (lt >> chunk_lg) * gridDim.x; tiles past a group's
+            // last one (its last block may be short) are claimed as empty.
+            int p = 0;
+            if (lane == 0) p = atomicAdd(&sm.next, 1);
+            p = __shfl_sync(kFull, p, 0);
+            lt = p / QC;
+            m = p - lt * QC;
+            const int chunk_lg = chunk_q;
+            const int chunk =
+                static_cast<int>(blockIdx.x) + (lt >> chunk_lg) * static_cast<int>(gridDim.x);
+            if (chunk >= n_chunks) break;
+            slot = lt % RING;
+            int ok = 1;
+            if (lane == 0) ok = wait_slot(&sm.owner[slot], lt, a.timeout_ns) ? 1 : 0;
+            ok = __shfl_sync(kFull, ok, 0);
+            if (!ok) {
+                if (lane == 0) atomicOr(a.err, kErrTimeout);
+                break;
+            }
+            __threadfence_block();
+            // (32-bit: n_chunks, the chunk count, fits an int; see the launcher)
+            const int n_qb = (a.n_qt + (1 << chunk_lg) - 1) >> chunk_lg;
+            const int per_sb = IDTX_LIST_GSB * n_qb;
+            const int sb = chunk / per_sb;
+            const int g0 = sb * IDTX_LIST_GSB;
+            const int gs = n_groups - g0 < IDTX_LIST_GSB ? n_groups - g0 : IDTX_LIST_GSB;
+            const int rc = chunk - sb * per_sb;
+            const int qblock = rc / gs;
+            grp = g0 + (rc - qblock * gs);
+            qt = (qblock << chunk_lg) + (lt & ((1 << chunk_lg) - 1));
+            qi = qt * QC + m;  // >= n_pad past the last tile
         }
-        __threadfence_block();
-        // (32-bit: n_chunks, the chunk count, fits an int; see the launcher)
-        const int n_qb = (a.n_qt + (1 << chunk_lg) - 1) >> chunk_lg;
-        const int per_sb = IDTX_LIST_GSB * n_qb;
-        const int sb = chunk / per_sb;
-        const int g0 = sb * IDTX_LIST_GSB;
-        const int gs = n_groups - g0 < IDTX_LIST_GSB ? n_groups - g0 : IDTX_LIST_GSB;
-        const int rc = chunk - sb * per_sb;
-        const int qblock = rc / gs;
-        const int grp = g0 + (rc - qblock * gs);
-        const int qt = (qblock << chunk_lg) + (lt & ((1 << chunk_lg) - 1));
-        const int64_t qi = static_cast<int64_t>(qt) * QC + m;  // >= n_pad past the last tile
         const int job = grp * GB + lane;
         const bool job_ok = job < a.n_jobs;
         double term = 0.0;
 
         if (qi < a.n) {
             const float *xg = a.xi + static_cast<int64_t>(grp) * a.n_pad * XW + lane * DX;
-            auto x_dist = [&](const float(&xq)[DX], int64_t j) {
-                const float *xr = xg + j * XW;
+            // per-query work counters (warp-uniform)
+            unsigned ta = 0, tb = 0, nfa = 0, nfb = 0;
+            float xq[DX];
+#pragma unroll
+            for (int d = 0; d < DX; ++d) xq[d] = xg[static_cast<int64_t>(qi) * XW + d];
+            const int len_a = __ldg(&a.lmeta[qi].x);
+            const int2 *la = a.list_a + static_cast<int64_t>(qi) * a.cap_a;
+
+            auto x_dist = [&](int j) {
+                const float *xr = xg + static_cast<int64_t>(j) * XW;
                 float dx = fabsf(xq[0] - xr[0]);
 #pragma unroll
                 for (int d = 1; d < DX; ++d) dx = fmaxf(dx, fabsf(xq[d] - xr[d]));
                 return dx;
             };
-            // per-query work counters (warp-uniform)
-            unsigned ta = 0, tb = 0, nfa = 0, nfb = 0;
-            float xq[DX];
-#pragma unroll
-            for (int d = 0; d < DX; ++d) xq[d] = xg[qi * XW + d];
-            const int4 meta = __ldg(&a.lmeta[qi]);
-            const int len_a = meta.x, len_b = meta.y;
-            const float r_a = __int_as_float(meta.z), r_b = __int_as_float(meta.w);
-            const int2 *la = a.list_a + qi * a.cap_a;
-            const int2 *lb = a.list_b + qi * a.cap_b;
-
-            float qc[DS];  // the query's shared coordinates (full-scan fallbacks only)
-            bool have_q = false;
-            auto load_q = [&]() {
-                if (have_q) return;
+            // the query's shared coordinates (full-scan fallbacks only)
+            auto load_q = [&](float(&qc)[DS]) {
                 const float *qr = sh_row(qi);
 #pragma unroll
                 for (int d = 0; d < DS; ++d) qc[d] = qr[d];
-                have_q = true;
             };
 
             // ---------------- pass A: the k smallest joint distances
@@ -272,56 +387,88 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
             float th = job_ok ? kInf : -1.0f;  // padding jobs never insert
             int walked_a = 0;
             uint32_t amask = 0;  // jobs the shared walk left to finish lane-split
-            {
-                int2 nxt = len_a > 0 ? __ldg(la + lane) : sentinel;
-                for (int e = 0; e < len_a; e += 32) {
-                    const int2 cur = nxt;
-                    if (e + 32 < len_a) nxt = __ldg(la + e + 32 + lane);
+            // A walk's next rows, fetched while the current ones are used: the
+            // entries of list l from e on (staged 32 at a time into the half
+            // of the warp's buffer that was used up; past the list's end
+            // sentinels), their distances and X values.
+            constexpr int SW = IDTX_LIST_SA;
+            float row_d[SW], row_x[SW][DX];
+            int2 nxt;
+            auto fetch = [&](int e) {
+#pragma unroll
+                for (int t = 0; t < SW; t += 2) {
+                    const int4 v = *reinterpret_cast<const int4 *>(&ent[(e & 63) + t]);
+                    row_d[t] = __int_as_float(v.y);
+                    row_d[t + 1] = __int_as_float(v.w);
+                    // (32 x 32 -> 64 bits: one multiply-add per row)
+                    const float *x0 = xg + static_cast<uint64_t>(static_cast<uint32_t>(v.x)) * XW;
+                    const float *x1 = xg + static_cast<uint64_t>(static_cast<uint32_t>(v.z)) * XW;
+#pragma unroll
+                    for (int d = 0; d < DX; ++d) {
+                        row_x[t][d] = x0[d];
+                        row_x[t + 1][d] = x1[d];
+                    }
+                }
+            };
+            auto begin = [&](const int2 *l, int len) {
+                const int2 first = len > 0 ? __ldg(l + lane) : sentinel;
+                nxt = len > 32 ? __ldg(l + 32 + lane) : sentinel;
+                __syncwarp();
+                ent[lane] = first;
+                __syncwarp();
+                fetch(0);
+            };
+            auto advance = [&](const int2 *l, int len, int e) {  // after the rows of e
+                if ((e & 31) == 32 - 2 * SW || (SW > 8 && (e & 31) == 0)) {
+                    const int at = (e & ~31) + 32;  // the chunk after e's
                     __syncwarp();
-                    ent[lane] = cur;
+                    ent[(at & 32) + lane] = nxt;
                     __syncwarp();
-                    int u = 0;
-                    for (; u < 32; u += SA) {
-                        // Ascending list: once the sub-chunk's first entry is
-                        // out of a job's reach, so is everything after it.
-                        // When at most TAIL_A jobs are still in reach the
-                        // shared walk stops and those finish lane-split below.
-                        const uint32_t act =
-                            __ballot_sync(kFull, __int_as_float(ent[u].y) < th);
-                        if (__popc(act) <= TAIL_A) {
-                            amask = act;
-                            break;
-                        }
-                        int jj[SA];
-                        float dyz[SA], dd[SA];
+                    nxt = at + 32 < len ? __ldg(l + at + 32 + lane) : sentinel;
+                }
+                fetch(e + SW);
+            };
+            begin(la, len_a);
+            for (int e = 0;; e += SW) {
+                // Ascending list: once the first of the next entries is out
+                // of a job's reach, so is everything after it.  When at most
+                // TAIL_A jobs are still in reach the shared walk stops and
+                // those finish lane-split below.
+                const uint32_t act = __ballot_sync(kFull, row_d[0] < th);
+                if (__popc(act) <= TAIL_A) {
+                    amask = act;
+                    walked_a = e;
+                    break;
+                }
+                float dd[SW];
 #pragma unroll
-                        for (int t = 0; t < SA; t += 2) {
-                            const int4 q = *reinterpret_cast<const int4 *>(&ent[u + t]);
-                            jj[t] = q.x;
-                            dyz[t] = __int_as_float(q.y);
-                            jj[t + 1] = q.z;
-                            dyz[t + 1] = __int_as_float(q.w);
-                        }
+                for (int t = 0; t < SW; ++t) {
+                    float dx = fabsf(xq[0] - row_x[t][0]);
 #pragma unroll
-                        for (int t = 0; t < SA; ++t) dd[t] = x_dist(xq, jj[t]);
+                    for (int d = 1; d < DX; ++d) dx = fmaxf(dx, fabsf(xq[d] - row_x[t][d]));
+                    dd[t] = fmaxf(dx, row_d[t]);
+                }
+                advance(la, len_a, e);
+                if constexpr (EXACT && KH == 4) {
 #pragma unroll
-                        for (int t = 0; t < SA; ++t) {
-                            const float d = fmaxf(dd[t], dyz[t]);
-                            if (d < th) {
-                                sorted_insert<KH>(h, d);
-                                th = kth(h);
-                            }
+                    for (int t = 0; t < SW; t += 4) merge4(h, dd[t], dd[t + 1], dd[t + 2], dd[t + 3]);
+                    if (job_ok) th = h[3];
+                } else {
+#pragma unroll
+                    for (int t = 0; t < SW; ++t) {
+                        if (dd[t] < th) {
+                            sorted_insert<KH>(h, dd[t]);
+                            th = kth(h);
                         }
                     }
-                    walked_a = e + u;
-                    if (u < 32) break;
                 }
             }
             if (walked_a > len_a) walked_a = len_a;
             // Lane-split finish of the remaining jobs, one at a time: steps of
             // two blocks of 32 entries, one entry per lane and block; the
             // distances below the job's k-th value are inserted smallest first
-            // (warp minimum) until the step's last entry is out of reach.
+            // (warp minimum) into its k smallest, which every lane holds,
+            // until the step's last entry is out of reach.
             // my_walked: the prefix of list A this lane's job walked.
             int my_walked = walked_a;
             while (amask) {
@@ -331,7 +478,10 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
 #pragma unroll
                 for (int d = 0; d < DX; ++d) xf[d] = __shfl_sync(kFull, xq[d], f);
                 const float *xgf = xg - lane * DX + f * DX;
-                float thf = __shfl_sync(kFull, th, f);
+                float hf[KH];
+#pragma unroll
+                for (int t = 0; t < KH; ++t) hf[t] = __shfl_sync(kFull, h[t], f);
+                float thf = kth(hf);
                 int pos = walked_a;
                 while (pos < len_a) {
                     const int p0 = pos + lane, p1 = pos + 32 + lane;
@@ -339,23 +489,15 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
                     const int2 e1 = p1 < len_a ? __ldg(la + p1) : sentinel;
                     const float y0 = __int_as_float(e0.y), y1 = __int_as_float(e1.y);
                     if (!(__shfl_sync(kFull, y0, 0) < thf)) break;
-                    float c0 = kInf, c1 = kInf;
-                    if (y0 < thf) {
-                        const float *xr = xgf + static_cast<int64_t>(e0.x) * XW;
+                    auto reach = [&](const int2 e, float y) {  // joint distance, +inf out of reach
+                        if (!(y < thf)) return kInf;
+                        const float *xr = xgf + static_cast<uint64_t>(static_cast<uint32_t>(e.x)) * XW;
                         float dx = fabsf(xf[0] - xr[0]);
 #pragma unroll
                         for (int d = 1; d < DX; ++d) dx = fmaxf(dx, fabsf(xf[d] - xr[d]));
-                        c0 = fmaxf(dx, y0);
-                    }
-                    if (y1 < thf) {
-                        const float *xr = xgf + static_cast<int64_t>(e1.x) * XW;
-                        float dx = fabsf(xf[0] - xr[0]);
-#pragma unroll
-                        for (int d = 1; d < DX; ++d) dx = fmaxf(dx, fabsf(xf[d] - xr[d]));
-                        c1 = fmaxf(dx, y1);
-                    }
-                    if (!(c0 < thf)) c0 = kInf;
-                    if (!(c1 < thf)) c1 = kInf;
+                        return fmaxf(dx, y);
+                    };
+                    float c0 = reach(e0, y0), c1 = reach(e1, y1);
                     while (true) {
                         const float mn = warp_min_nn(fminf(c0, c1));
                         if (!(mn < thf)) break;
@@ -366,29 +508,35 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
                             const uint32_t w1 = __ballot_sync(kFull, c1 == mn);
                             if (lane == __ffs(w1) - 1) c1 = kInf;
                         }
-                        if (lane == f) {
-                            sorted_insert<KH>(h, mn);
-                            th = kth(h);
-                        }
-                        thf = __shfl_sync(kFull, th, f);
+                        sorted_insert<KH>(hf, mn);
+                        thf = kth(hf);
                     }
                     ta += (len_a - pos < 64) ? static_cast<unsigned>(len_a - pos) : 64u;
                     pos += 64;
                     // ascending: if the step's last entry is out of reach, so is the rest
                     if (!(__shfl_sync(kFull, y1, 31) < thf)) break;
                 }
-                if (lane == f) my_walked = pos < len_a ? pos : len_a;
+                if (lane == f) {
+#pragma unroll
+                    for (int t = 0; t < KH; ++t) h[t] = hf[t];
+                    th = thf;
+                    my_walked = pos < len_a ? pos : len_a;
+                }
             }
             // The list ran out before the job's k-th distance dropped to r_A:
-            // recompute those jobs over every sample.  For each such job the
-            // 32 lanes split the samples, keep their own k smallest, and the
-            // warp merges them (repeatedly taking the smallest head).
+            // the job is recomputed over every sample, in the split form by
+            // ksg_scan_kernel, else here: the 32 lanes split the samples of
+            // one such job at a time, keep their own k smallest, and the warp
+            // merges them (repeatedly taking the smallest head).
+            const float r_a = __int_as_float(__ldg(&a.lmeta[qi].z));
             const bool fa = job_ok && th > r_a;
             float eps_fix = 0.0f;
             uint32_t fmask = __ballot_sync(kFull, fa);
-            if (fmask) load_q();
             nfa = __popc(fmask);
+            if (SPLIT) fmask = 0;
             while (fmask) {
+                float qc[DS];
+                load_q(qc);
                 const int f = __ffs(fmask) - 1;
                 fmask &= fmask - 1;
                 float xf[DX];
@@ -426,145 +574,125 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
                 }
                 if (lane == f) eps_fix = kv;
             }
-            const float eps = job_ok ? (fa ? eps_fix : kth(h)) : -1.0f;
+            const float eps = job_ok ? (!SPLIT && fa ? eps_fix : kth(h)) : -1.0f;
 
             // ---------------- pass B: strict-radius counts
-            const bool fb = job_ok && (eps > r_a || eps > r_b);
+            const int len_b = __ldg(&a.lmeta[qi].y);
+            const float r_b = __int_as_float(__ldg(&a.lmeta[qi].w));
+            const int2 *lb = a.list_b + static_cast<int64_t>(qi) * a.cap_b;
+            const bool fb = job_ok && (eps > r_a || eps > r_b || (SPLIT && fa));
             int nz = 0, nyz = 0, nxz = 0;
             // Every list A entry below eps lies in the walked prefix (the walk
             // went on until each job's k-th value was at most the next entry).
-            if (job_ok && !fb) nyz = list_lower(la, my_walked, eps);
-            // The count walk over list B, for every job the entries below its
-            // eps (n_z) and those also within eps in X (n_xz).  While more
-            // than 16 jobs still need entries the warp walks the list shared,
-            // one job per lane (a sub-chunk is skipped by a job whose eps is
-            // at most its first entry).  Then the jobs still walking are
-            // repacked: with c of them left, each takes 32/M lanes (M the
-            // power of two >= c), which split the entries of each staged
-            // chunk between them, and at every chunk boundary the warp
-            // repacks again once at most M/2 jobs need more -- so no more
-            // than half the lanes ever walk for jobs that are done.
+            nyz = list_lower(la, job_ok && !fb ? my_walked : 0, eps);
+            // The count walk over list B: for every job the entries below its
+            // eps (n_z) and those also within eps in X (n_xz).  Shared rows,
+            // one job per lane, while more than IDTX_LIST_REPACK jobs need
+            // entries (`reach`: a job's eps is above the next entry).
             const float ev = (job_ok && !fb) ? eps : 0.0f;
-            int walked_b = 0;
-            int cf = 0, co = 0;  // staged chunk [cf, cf+32), next entry cf+co
-            int2 nxt = len_b > 0 ? __ldg(lb + lane) : sentinel;
-            uint32_t rem = 0;  // lanes whose job still needs entries after the shared phase
-            for (; cf < len_b; cf += 32) {
-                const int2 cur = nxt;
-                if (cf + 32 < len_b) nxt = __ldg(lb + cf + 32 + lane);
-                __syncwarp();
-                ent[lane] = cur;
-                __syncwarp();
-                int u = 0;
-                for (; u < 32; u += SB) {
-                    const uint32_t act = __ballot_sync(kFull, ev > __int_as_float(ent[u].y));
-                    if (__popc(act) <= IDTX_LIST_REPACK) {
-                        rem = act;
-                        break;
-                    }
-                    int jj[SB];
-                    float dz[SB], dx[SB];
+            int pos = 0;
+            uint32_t rem;
+            begin(lb, len_b);
+            while (true) {
+                rem = __ballot_sync(kFull, ev > row_d[0]);
+                if (__popc(rem) <= IDTX_LIST_REPACK) break;
+                float dx[SW], dz[SW];
 #pragma unroll
-                    for (int t = 0; t < SB; t += 2) {
-                        const int4 q = *reinterpret_cast<const int4 *>(&ent[u + t]);
-                        jj[t] = q.x;
-                        dz[t] = __int_as_float(q.y);
-                        jj[t + 1] = q.z;
-                        dz[t + 1] = __int_as_float(q.w);
-                    }
+                for (int t = 0; t < SW; ++t) {
+                    dx[t] = fabsf(xq[0] - row_x[t][0]);
 #pragma unroll
-                    for (int t = 0; t < SB; ++t) dx[t] = x_dist(xq, jj[t]);
-#pragma unroll
-                    for (int t = 0; t < SB; ++t) {
-                        const bool pz = dz[t] < eps;
-                        nz += pz ? 1 : 0;
-                        nxz += (pz && dx[t] < eps) ? 1 : 0;
-                    }
+                    for (int d = 1; d < DX; ++d) dx[t] = fmaxf(dx[t], fabsf(xq[d] - row_x[t][d]));
+                    dz[t] = row_d[t];
                 }
-                if (u < 32) {
-                    co = u;
-                    break;
+                advance(lb, len_b, pos);
+                pos += SW;
+#pragma unroll
+                for (int t = 0; t < SW; ++t) {
+                    const bool pz = dz[t] < ev;
+                    nz += pz ? 1 : 0;
+                    nxz += (pz && dx[t] < ev) ? 1 : 0;
                 }
             }
-            walked_b = cf + co < len_b ? cf + co : len_b;
-            // Repacked phases: M job slots (M a power of two <= 16), slot s on
-            // lanes s, s+M, ..., which take the staged chunk's entries r,
-            // r + 32/M, ... (r = lane / M), IDTX_LIST_PHASE_STEP per step.
+            const int walked_b = pos < len_b ? pos : len_b;
+            // The jobs that need more share the lanes: with c of them left,
+            // M slots (the power of two >= c) of 32 / M lanes that split the
+            // entries between them; once at most M / 2 need more, the lanes
+            // are shared out again.
             while (rem) {
                 const int c = __popc(rem);
                 const int lg = c > 8 ? 4 : (c > 4 ? 3 : (c > 2 ? 2 : (c > 1 ? 1 : 0)));
                 const int M = 1 << lg, per = 32 >> lg;
                 const int s = lane & (M - 1), r = lane >> lg;
-                const bool slot_ok = s < c;
-                uint32_t mm = rem;  // the job of slot s: the (s+1)-th lane of rem
-                for (int t = 0; t < s && t < c; ++t) mm &= mm - 1;
-                const int home = slot_ok ? __ffs(mm) - 1 : lane;
+                const int rank = __popc(rem & ((1u << lane) - 1u));
+                int *tab = &ent[0].x;  // the staged entries are done with
+                __syncwarp();
+                if ((rem >> lane) & 1u) tab[rank] = lane;
+                __syncwarp();
+                const int home = s < c ? tab[s] : lane;
                 const float e_home = __shfl_sync(kFull, ev, home);
-                const float es = slot_ok ? e_home : 0.0f;
+                const float es = s < c ? e_home : 0.0f;
                 float xs[DX];
 #pragma unroll
                 for (int d = 0; d < DX; ++d) xs[d] = __shfl_sync(kFull, xq[d], home);
                 const float *xgs = xg + (home - lane) * DX;
+                const int from = pos;
                 int cz = 0, cx = 0;
-                uint32_t still = 0;
-                while (true) {
-                    for (int u0 = 0; u0 < M; u0 += IDTX_LIST_PHASE_STEP) {
-                        constexpr int PS = IDTX_LIST_PHASE_STEP;
-                        bool in[PS];
-                        float xv[PS][DX];
+                uint32_t still;
+                do {
+                    constexpr int PS = IDTX_LIST_PHASE_STEP;
+                    int js[PS];
+                    float xv[PS][DX];
 #pragma unroll
-                        for (int t = 0; t < PS; ++t) {
-                            const int idx = r + per * (u0 + t);
-                            const int2 e = ent[idx & 31];
-                            in[t] = u0 + t < M && idx >= co && __int_as_float(e.y) < es;
-                            const float *xr = xgs + static_cast<int64_t>(e.x) * XW;
-#pragma unroll
-                            for (int d = 0; d < DX; ++d) xv[t][d] = in[t] ? xr[d] : xs[d];
-                        }
-#pragma unroll
-                        for (int t = 0; t < PS; ++t) {
-                            float dxv = fabsf(xs[0] - xv[t][0]);
-#pragma unroll
-                            for (int d = 1; d < DX; ++d) dxv = fmaxf(dxv, fabsf(xs[d] - xv[t][d]));
-                            cz += in[t] ? 1 : 0;
-                            cx += (in[t] && dxv < es) ? 1 : 0;
-                        }
+                    for (int t = 0; t < PS; ++t) {
+                        const int e = pos + r + per * t;
+                        const int2 v = e < len_b ? __ldg(lb + e) : sentinel;
+                        js[t] = __int_as_float(v.y) < es ? v.x : -1;
                     }
-                    tb += static_cast<unsigned>(c * (32 - co));
-                    cf += 32;
-                    co = 0;
-                    still = 0;
-                    if (cf >= len_b) break;  // the list is done: so is every job
-                    // jobs that need entries of the next chunk (slot lanes 0..M-1)
-                    const float dn = __int_as_float(__shfl_sync(kFull, nxt.y, 0));
-                    still = __ballot_sync(kFull, r == 0 && es > dn);
-                    const int2 cur = nxt;
-                    if (cf + 32 < len_b) nxt = __ldg(lb + cf + 32 + lane);
-                    __syncwarp();
-                    ent[lane] = cur;
-                    __syncwarp();
-                    if (__popc(still) <= (M >> 1)) break;
-                }
-                // each slot's total over its lanes, then to the job's lane
+#pragma unroll
+                    for (int t = 0; t < PS; ++t) {
+                        const float *xr = xgs + static_cast<uint64_t>(static_cast<uint32_t>(js[t])) * XW;
+#pragma unroll
+                        for (int d = 0; d < DX; ++d) xv[t][d] = js[t] >= 0 ? xr[d] : CUDART_INF_F;
+                    }
+                    pos += per * PS;
+                    const float dn = pos < len_b ? __int_as_float(__ldg(&lb[pos].y)) : kInf;
+#pragma unroll
+                    for (int t = 0; t < PS; ++t) {
+                        float dxv = fabsf(xs[0] - xv[t][0]);
+#pragma unroll
+                        for (int d = 1; d < DX; ++d) dxv = fmaxf(dxv, fabsf(xs[d] - xv[t][d]));
+                        cz += js[t] >= 0 ? 1 : 0;
+                        cx += dxv < es ? 1 : 0;
+                    }
+                    still = __ballot_sync(kFull, ((rem >> lane) & 1u) && ev > dn);
+                } while (__popc(still) > (M >> 1));
+                tb += static_cast<unsigned>(c * (pos - from));
+                // each slot's totals over its lanes, then to the job's lane
                 for (int off = M; off < 32; off <<= 1) {
                     cz += __shfl_xor_sync(kFull, cz, off);
                     cx += __shfl_xor_sync(kFull, cx, off);
                 }
-                const int rank = __popc(rem & ((1u << lane) - 1u));
                 const int vz = __shfl_sync(kFull, cz, rank & 31);
                 const int vx = __shfl_sync(kFull, cx, rank & 31);
                 if ((rem >> lane) & 1u) {
                     nz += vz;
                     nxz += vx;
                 }
-                rem = __reduce_or_sync(kFull, (r == 0 && ((still >> lane) & 1u)) ? (1u << home) : 0u);
+                rem = still;
             }
-            // Jobs whose eps reaches past a list: counts by a full scan, the
-            // 32 lanes splitting the samples of one such job at a time.
+            // Jobs whose eps reaches past a list: counts by a full scan, in
+            // the split form by ksg_scan_kernel, else here, the 32 lanes
+            // splitting the samples of one such job at a time.
             uint32_t bmask = __ballot_sync(kFull, fb);
-            if (bmask) load_q();
             nfb = __popc(bmask);
+            if (SPLIT && bmask) {
+                if (lane == 0)
+                    a.scans[atomicAdd(a.next + 2, 1)] = make_int4(grp, qi, static_cast<int>(bmask), 0);
+                bmask = 0;
+            }
             while (bmask) {
+                float qc[DS];
+                load_q(qc);
                 const int f = __ffs(bmask) - 1;
                 bmask &= bmask - 1;
                 float xf[DX];
@@ -600,30 +728,46 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
                     nxz = cxz;
                 }
             }
-            if (job_ok) {
+            if constexpr (SPLIT) {
+                const int64_t at = (static_cast<int64_t>(grp) * a.n_pad + qi) * GB + lane;
+                a.cyz[at] = static_cast<uint16_t>(nyz);
+                a.cz[at] = static_cast<uint16_t>(nz);
+                a.cxz[at] = static_cast<uint16_t>(nxz);
+            } else if (job_ok) {
                 term = a.psi[nz + 1] - a.psi[nxz + 1] - a.psi[nyz + 1];
-                const int64_t orig = a.order ? static_cast<int64_t>(a.order[qi]) : qi;
-                if (a.eps_out) a.eps_out[static_cast<int64_t>(job) * a.n + orig] = eps;
-                if (a.cnt_out) {
+            }
+            if (job_ok) {
+                const int64_t orig = a.order ? static_cast<int64_t>(a.order[qi]) : static_cast<int64_t>(qi);
+                if (a.eps_out && !(SPLIT && fb)) a.eps_out[static_cast<int64_t>(job) * a.n + orig] = eps;
+                if (!SPLIT && a.cnt_out) {
                     int32_t *co = a.cnt_out + static_cast<int64_t>(job) * 3 * a.n;
                     co[orig] = nxz;
                     co[a.n + orig] = nyz;
                     co[2 * a.n + orig] = nz;
                 }
             }
-            const int snz = __reduce_add_sync(kFull, job_ok ? nz : 0);
-            const int snyz = __reduce_add_sync(kFull, job_ok ? nyz : 0);
-            if (lane == 0) {
-                unsigned long long *w = sm.work[warp];
-                w[8] += static_cast<unsigned>(snz);
-                w[9] += static_cast<unsigned>(snyz);
-                w[0] += static_cast<unsigned>(walked_a);
-                w[1] += static_cast<unsigned>(walked_b);
-                w[2] += static_cast<unsigned long long>(nfa) * static_cast<unsigned long long>(a.n - 1);
-                w[3] += static_cast<unsigned long long>(nfb) * static_cast<unsigned long long>(a.n - 1);
-                w[4] += nfa + nfb;
-                w[6] += tb;
-                w[7] += ta;
+            if (a.work) {
+                // lane k keeps counter k: no read-modify-write per query
+                unsigned snz = 0, snyz = 0;  // (the split form's are summed by sum_terms)
+                if (!SPLIT) {
+                    snz = __reduce_add_sync(kFull, static_cast<unsigned>(job_ok ? nz : 0));
+                    snyz = __reduce_add_sync(kFull, static_cast<unsigned>(job_ok ? nyz : 0));
+                }
+                unsigned v = static_cast<unsigned>(walked_a);
+                v = lane == 1 ? static_cast<unsigned>(walked_b) : v;
+                v = lane == 6 ? tb : v;
+                v = lane == 7 ? ta : v;
+                if (!SPLIT) {
+                    v = lane == 8 ? snz : v;
+                    v = lane == 9 ? snyz : v;
+                    my_work += lane < 2 || lane >= 6 ? v : 0u;
+                } else {
+                    my_work += lane < 2 || lane == 6 || lane == 7 ? v : 0u;
+                }
+                if (nfa | nfb) {
+                    const unsigned long long n1 = static_cast<unsigned long long>(a.n - 1);
+                    my_work += lane == 2 ? nfa * n1 : (lane == 3 ? nfb * n1 : (lane == 4 ? nfa + nfb : 0ull));
+                }
             }
         }
 
@@ -631,6 +775,7 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
         // finishes the tile's last query sums it in ksg_fused_kernel's order
         // (NWS sums over the queries m = w, w + NWS, ..., then their sum in
         // order of w), writes the partial and frees the slot.
+        if constexpr (SPLIT) continue;
         double *ring = a.ring + (static_cast<int64_t>(blockIdx.x) * RING + slot) * QC * 32;
         __stcg(ring + m * 32 + lane, term);
         __threadfence_block();
@@ -661,8 +806,16 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
         }
     }
 
-    if (lane == 0) sm.work[warp][5] += static_cast<unsigned long long>(clock64() - t_begin);
+    if (lane == 5) my_work = static_cast<unsigned long long>(clock64() - t_begin);
+    if (lane < kNumWork) sm.work[warp][lane] = my_work;
     __syncthreads();
+    if (SPLIT && tid == 0) {  // the last CTA to come here resets the counters for the next launch
+        __threadfence();
+        if (atomicAdd(a.next + 1, 1) == static_cast<int>(gridDim.x) - 1) {
+            a.next[0] = 0;
+            a.next[1] = 0;
+        }
+    }
     if (a.work && tid < kNumWork) {
         unsigned long long s = 0;
         for (int w = 0; w < NW; ++w) s += sm.work[w][tid];
@@ -670,11 +823,178 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
     }
 }
 
-template <int DX, int DY, int DZ, int K1, bool EXACT, int QC, int NWARPS>
-cudaError_t launch_ksg_list(const KsgLaunch &a, int n_groups, cudaStream_t stream)
+// Full scans, for the (query, group)s that the split form's lists did not
+// serve (a query far from the others has long neighbourhoods for all of its
+// jobs): eps and the counts of the marked jobs over every sample.  A CTA takes
+// one (query, group) at a time, its warps every kScanWarps-th 32 samples; in a warp
+// a lane per sample finds the samples within reach, 32 at a time, and a lane
+// per job uses them, their X rows loaded sixteen at a time.  The warps share
+// each job's smallest k-th distance so far (any warp's is at least the job's
+// own) and their heaps and counts meet in shared memory.
+// A single warp of the list kernel took up to 1 ms for one such query at N =
+// 9995 with 32 jobs, and the whole GPU often waited for it; here it takes 70
+// us, bound by the latency of its loads.
+constexpr int kScanWarps = 32;
+
+template <int DX, int DY, int DZ, int K1, bool EXACT, int QCTA, int NWARPS>
+__global__ void __launch_bounds__(kScanWarps * 32, 1)
+    ksg_scan_kernel(const KsgLaunch a)
+{
+    using S = KsgShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>;
+    constexpr int DS = S::DS, DSP = S::DSP, XW = S::XW, GB = S::GB;
+    constexpr int KH = K1 - 1, U = DX > 1 ? 8 : 16;
+    constexpr unsigned kFull = 0xffffffffu;
+    extern __shared__ __align__(16) unsigned char l_smem[];
+    float(*s_heap)[KH][32] = reinterpret_cast<float(*)[KH][32]>(l_smem);  // [kScanWarps]
+    __shared__ unsigned s_th[32];  // bits of each job's bound, then of its eps
+    __shared__ int s_cnt[3][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n = static_cast<int>(a.n), n_tiles = (n + kTJ - 1) / kTJ;
+    const int n_items = a.next[2], kk = a.k;
+    auto kth = [&](const float(&h)[KH]) { return EXACT ? h[KH - 1] : select_kth<KH>(h, kk - 1); };
+    for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
+        const int4 item = a.scans[it];
+        const int grp = item.x, qi = item.y;
+        const bool mine = (static_cast<unsigned>(item.z) >> lane) & 1u;  // this lane's job is wanted
+        const float *xg = a.xi + static_cast<int64_t>(grp) * a.n_pad * XW + lane * DX;
+        float xq[DX], q[DS];
+#pragma unroll
+        for (int d = 0; d < DX; ++d) xq[d] = xg[static_cast<int64_t>(qi) * XW + d];
+        const float *qr = a.sh + (static_cast<int64_t>(qi / kTJ) * kTileRows + qi % kTJ) * DSP;
+#pragma unroll
+        for (int d = 0; d < DS; ++d) q[d] = qr[d];
+        // use(d_X, d_Z, d_YZ of U samples) for every sample j != qi of the
+        // warp's tiles with d_YZ (ZONLY: d_Z) below limit() as it was before
+        // its 32 samples
+        auto scan = [&](auto zonly, auto limit, auto use) {
+            constexpr bool ZONLY = decltype(zonly)::value;
+            float lim = limit();
+            for (int g = warp; g < n_tiles * (kTJ / 32); g += kScanWarps) {  // 32 samples at a time
+                const int t = g / (kTJ / 32), b = g % (kTJ / 32) * 32;
+                const float *tile = a.sh + static_cast<int64_t>(t) * kTileRows * DSP;
+                if (!(point_gap<ZONLY ? DZ : DS, DSP>(tile, q) < lim)) continue;
+                const float *row = tile + (b + lane) * DSP;
+                float dz = fabsf(q[0] - row[0]);
+#pragma unroll
+                for (int d = 1; d < DZ; ++d) dz = fmaxf(dz, fabsf(q[d] - row[d]));
+                float dyz = dz;
+#pragma unroll
+                for (int d = DZ; d < DS; ++d) dyz = fmaxf(dyz, fabsf(q[d] - row[d]));
+                const int j0 = t * kTJ + b;
+                const bool other = j0 + lane < n && j0 + lane != qi;
+                uint32_t in = __ballot_sync(kFull, other && (ZONLY ? dz : dyz) < lim);
+                while (in) {
+                    float dx[U], z[U], yz[U];  // +inf where no sample is left
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int s = __ffs(in) - 1;
+                        const bool some = in != 0;
+                        in &= in - 1;
+                        const float *xr = xg + static_cast<int64_t>(some ? j0 + s : qi) * XW;
+                        dx[u] = fabsf(xq[0] - xr[0]);
+#pragma unroll
+                        for (int d = 1; d < DX; ++d) dx[u] = fmaxf(dx[u], fabsf(xq[d] - xr[d]));
+                        z[u] = __shfl_sync(kFull, dz, s & 31);
+                        yz[u] = __shfl_sync(kFull, dyz, s & 31);
+                        if (!some) z[u] = yz[u] = CUDART_INF_F;
+                    }
+                    use(dx, z, yz);
+                }
+                lim = limit();
+            }
+        };
+        if (warp == 0) {
+            s_th[lane] = __float_as_uint(mine ? CUDART_INF_F : 0.0f);
+            s_cnt[0][lane] = s_cnt[1][lane] = s_cnt[2][lane] = 0;
+        }
+        __syncthreads();
+        volatile unsigned *th_all = s_th;
+        float h[KH];
+#pragma unroll
+        for (int t = 0; t < KH; ++t) h[t] = CUDART_INF_F;
+        float th = mine ? CUDART_INF_F : 0.0f;  // other jobs do not raise the limit
+        // A distance equal to the shared bound may be the k-th itself, so the
+        // limit is the next float above it.
+        scan(std::false_type{},
+             [&] {
+                 if (mine && th < __uint_as_float(th_all[lane])) atomicMin(&s_th[lane], __float_as_uint(th));
+                 const unsigned m = __reduce_max_sync(kFull, min(th_all[lane], __float_as_uint(th)));
+                 return m < 0x7f800000u ? __uint_as_float(m + 1) : CUDART_INF_F;
+             },
+             [&](const float(&dx)[U], const float(&)[U], const float(&yz)[U]) {
+                 if constexpr (EXACT && KH == 4) {
+#pragma unroll
+                     for (int u = 0; u < U; u += 4)
+                         merge4(h, fmaxf(dx[u], yz[u]), fmaxf(dx[u + 1], yz[u + 1]),
+                                fmaxf(dx[u + 2], yz[u + 2]), fmaxf(dx[u + 3], yz[u + 3]));
+                 } else {
+#pragma unroll
+                     for (int u = 0; u < U; ++u) {
+                         const float d = fmaxf(dx[u], yz[u]);
+                         if (d < kth(h)) sorted_insert<KH>(h, d);
+                     }
+                 }
+                 if (mine) th = kth(h);
+             });
+#pragma unroll
+        for (int t = 0; t < KH; ++t) s_heap[warp][t][lane] = h[t];
+        __syncthreads();
+        if (warp == 0) {  // the k smallest of all warps
+            for (int w = 1; w < kScanWarps; ++w)
+                for (int t = 0; t < KH; ++t) {
+                    const float d = s_heap[w][t][lane];
+                    if (!__any_sync(kFull, mine && d < kth(h))) break;
+                    if (d < kth(h)) sorted_insert<KH>(h, d);
+                }
+            s_th[lane] = __float_as_uint(mine ? kth(h) : 0.0f);
+        }
+        __syncthreads();
+        const float eps = __uint_as_float(s_th[lane]);
+        const float lim = warp_max_nn(eps);
+        int cz = 0, cyz = 0, cxz = 0;
+        scan(std::true_type{}, [&] { return lim; },
+             [&](const float(&dx)[U], const float(&z)[U], const float(&yz)[U]) {
+#pragma unroll
+                 for (int u = 0; u < U; ++u) {
+                     cz += z[u] < eps ? 1 : 0;
+                     cyz += yz[u] < eps ? 1 : 0;
+                     cxz += (z[u] < eps && dx[u] < eps) ? 1 : 0;
+                 }
+             });
+        if (cz) {
+            atomicAdd(&s_cnt[0][lane], cz);
+            if (cyz) atomicAdd(&s_cnt[1][lane], cyz);
+            if (cxz) atomicAdd(&s_cnt[2][lane], cxz);
+        }
+        __syncthreads();
+        if (warp == 0 && mine) {
+            const int64_t at = (static_cast<int64_t>(grp) * a.n_pad + qi) * GB + lane;
+            a.cz[at] = static_cast<uint16_t>(s_cnt[0][lane]);
+            a.cyz[at] = static_cast<uint16_t>(s_cnt[1][lane]);
+            a.cxz[at] = static_cast<uint16_t>(s_cnt[2][lane]);
+            if (a.eps_out) {
+                const int64_t orig = a.order ? static_cast<int64_t>(a.order[qi]) : static_cast<int64_t>(qi);
+                a.eps_out[static_cast<int64_t>(grp * GB + lane) * a.n + orig] = eps;
+            }
+        }
+        __syncthreads();  // shared state is set up afresh by the next item
+    }
+    // the last CTA to come here empties the queue for the next launch
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(a.next + 1, 1) == static_cast<int>(gridDim.x) - 1) {
+            a.next[1] = 0;
+            a.next[2] = 0;
+        }
+    }
+}
+
+template <int DX, int DY, int DZ, int K1, bool EXACT, int QC, int NWARPS, bool SPLIT>
+cudaError_t launch_list_form(const KsgLaunch &a, int n_groups, cudaStream_t stream)
 {
     using LS = ListShape<DX, DY, DZ, K1, EXACT, QC, NWARPS>;
-    auto kern = ksg_list_kernel<DX, DY, DZ, K1, EXACT, QC, NWARPS>;
+    auto kern = ksg_list_kernel<DX, DY, DZ, K1, EXACT, QC, NWARPS, SPLIT>;
     // Per device: the dynamic shared memory, a carveout that leaves the rest
     // of the SM's memory to L1, and the SM count (one CTA per SM).
     static DeviceOnce setup;
@@ -692,6 +1012,10 @@ cudaError_t launch_ksg_list(const KsgLaunch &a, int n_groups, cudaStream_t strea
             }
         }
         if (r == cudaSuccess) r = cudaDeviceGetAttribute(&n_sms[d], cudaDevAttrMultiProcessorCount, d);
+        if (SPLIT && r == cudaSuccess)
+            r = cudaFuncSetAttribute(ksg_scan_kernel<DX, DY, DZ, K1, EXACT, QC, NWARPS>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     static_cast<int>(kScanWarps * (K1 - 1) * 32 * sizeof(float)));
         return r;
     });
     if (e != cudaSuccess) return e;
@@ -700,17 +1024,47 @@ cudaError_t launch_ksg_list(const KsgLaunch &a, int n_groups, cudaStream_t strea
     int dev = 0;
     e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    int chunk_lg = 0;  // the largest chunk (up to IDTX_LIST_CHUNK) giving every SM two chunks
-    while ((2 << chunk_lg) <= IDTX_LIST_CHUNK && (tiles >> (chunk_lg + 1)) >= 2 * n_sms[dev])
-        ++chunk_lg;
-    // every group's query tiles in blocks of 2^chunk_lg (the last block may be short)
-    const int64_t chunks = static_cast<int64_t>(n_groups) * ((a.n_qt + (1 << chunk_lg) - 1) >> chunk_lg);
+    int chunk = 0;
+    int64_t chunks = 0;
+    if (SPLIT) {
+        // chunks of consecutive queries: eight per SM where that leaves 16 queries
+        const int64_t per = a.n * n_groups / (8 * n_sms[dev]);
+        chunk = per > IDTX_LIST_CHUNKQ ? IDTX_LIST_CHUNKQ : (per < 16 ? 16 : static_cast<int>(per));
+        chunks = static_cast<int64_t>(n_groups) * ((a.n + chunk - 1) / chunk);
+    } else {
+        // blocks of 2^chunk query tiles (a group's last one may be short): the
+        // largest (up to IDTX_LIST_CHUNK) giving every SM two
+        while ((2 << chunk) <= IDTX_LIST_CHUNK && (tiles >> (chunk + 1)) >= 2 * n_sms[dev]) ++chunk;
+        chunks = static_cast<int64_t>(n_groups) * ((a.n_qt + (1 << chunk) - 1) >> chunk);
+    }
     if (chunks > 0x3fffffff) return cudaErrorInvalidValue;  // the kernel's chunk arithmetic is 32-bit
     int64_t grid = chunks < n_sms[dev] ? chunks : n_sms[dev];
-    if (grid > kListRingCtas) grid = kListRingCtas;
+    if (!SPLIT && grid > kListRingCtas) grid = kListRingCtas;
     kern<<<static_cast<unsigned>(grid), LS::THREADS, LS::SMEM, stream>>>(
-        a, n_groups, static_cast<int>(chunks), chunk_lg);
+        a, n_groups, static_cast<int>(chunks), chunk);
+    if (SPLIT) {
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        ksg_scan_kernel<DX, DY, DZ, K1, EXACT, QC, NWARPS>
+            <<<static_cast<unsigned>(n_sms[dev]), kScanWarps * 32, kScanWarps * (K1 - 1) * 32 * sizeof(float),
+               stream>>>(a);
+    }
     return cudaGetLastError();
+}
+
+// The split form (counts out, terms summed by sum_terms) where the counts fit
+// in 16 bits and the launch so has their buffer, else the one with the ring.
+template <int DX, int DY, int DZ, int K1, bool EXACT, int QC, int NWARPS>
+cudaError_t launch_ksg_list(const KsgLaunch &a, int n_groups, cudaStream_t stream)
+{
+    cudaError_t e = cudaSuccess;
+    const bool setup = static_cast<int64_t>(a.n_qt) * n_groups <= 0;  // of both forms
+    if (setup || !a.cz)
+        e = launch_list_form<DX, DY, DZ, K1, EXACT, QC, NWARPS, false>(a, n_groups, stream);
+    if (e == cudaSuccess && (setup || a.cz))
+        e = launch_list_form<DX, DY, DZ, K1, EXACT, QC, NWARPS, true>(a, n_groups, stream);
+    if (e == cudaSuccess && !setup && a.cz) e = sum_terms(a, QC, NWARPS, n_groups, stream);
+    return e;
 }
 
 // One compiled specialisation: the tile kernel (ksg_kernel.cuh), its

@@ -968,12 +968,22 @@ struct CallBuffers {
 };
 
 // B_LIST layout for n queries: list_a [n][cap_a] | list_b [n][cap_b] | meta [n]
-// | the list kernel's term ring, all counted here | build_lists' scratch.
+// | the list kernel's term ring, all counted here | its counts
+// | build_lists' scratch.
 size_t list_bytes(int64_t n, int cap_a, int cap_b)
 {
     return align_up((size_t)n * cap_a * sizeof(int2), 256) +
            align_up((size_t)n * cap_b * sizeof(int2), 256) +
            align_up((size_t)n * sizeof(int4), 256) + kListRingBytes;
+}
+
+// The list kernel's counts, part of B_LIST: three 16-bit ones per (group,
+// query, job) where they fit in 16 bits (else the kernel sums by its ring),
+// and its queue of (group, query)s to scan.
+size_t count_rows(const Group &g) { return g.n_pad <= 65536 ? (size_t)g.n_groups * g.n_pad * 32 : 0; }
+size_t count_bytes(const Group &g)
+{
+    return align_up(count_rows(g) * 3 * sizeof(uint16_t) + count_rows(g) / 32 * sizeof(int4), 256);
 }
 
 // B_ORDER layout for n samples: order | idx | keys_in | keys_out | column ranges.
@@ -994,7 +1004,8 @@ CallBuffers bytes_of(const Group &g)
     b.perm = align_up(g.slot_stream.size() * (size_t)(g.n + g.n_reps) * sizeof(int32_t), 256);
     b.partial = align_up(g.jobs.size() * (size_t)g.n_qt * sizeof(double), 256);
     if (g.use_list || g.tune)
-        b.lists = list_bytes(g.n, g.cap_a, g.cap_b) + list_scratch_bytes(g.n, g.cap_a, g.cap_b);
+        b.lists = list_bytes(g.n, g.cap_a, g.cap_b) + count_bytes(g) +
+                  list_scratch_bytes(g.n, g.cap_a, g.cap_b);
     return b;
 }
 
@@ -1115,6 +1126,7 @@ void fill_launch(const idtx_ctx *c, const Group &g, const Slices &sl, float *eps
     a.order = g.sort ? (const int32_t *)sl.order : nullptr;
     a.work = (unsigned long long *)c->buf[B_WORK] + (size_t)g.work_slot * kNumWork;
     a.err = c->d_err;
+    a.next = c->d_err + 32;
     a.n = g.n;
     a.n_pad = g.n_pad;
     a.n_jobs = (int)g.jobs.size();
@@ -1126,6 +1138,8 @@ void fill_launch(const idtx_ctx *c, const Group &g, const Slices &sl, float *eps
     a.lmeta = nullptr;
     a.ring = nullptr;
     a.lscratch = nullptr;
+    a.cyz = a.cz = a.cxz = nullptr;
+    a.scans = nullptr;
     a.cap_a = g.cap_a;
     a.cap_b = g.cap_b;
     if ((g.use_list || g.tune) && sl.lists) {
@@ -1136,7 +1150,14 @@ void fill_launch(const idtx_ctx *c, const Group &g, const Slices &sl, float *eps
         a.list_b = (const int2 *)(sl.lists + oa);
         a.lmeta = (const int4 *)(sl.lists + oa + ob);
         a.ring = (double *)(sl.lists + oa + ob + om);
-        a.lscratch = sl.lists + list_bytes(g.n, g.cap_a, g.cap_b);
+        unsigned char *sp = sl.lists + list_bytes(g.n, g.cap_a, g.cap_b);
+        a.lscratch = sp + count_bytes(g);
+        if (const size_t rows = count_rows(g)) {
+            a.cyz = (uint16_t *)sp;
+            a.cz = a.cyz + rows;
+            a.cxz = a.cz + rows;
+            a.scans = (int4 *)(a.cxz + rows);  // rows is a multiple of 4096: 16-byte aligned
+        }
     }
 }
 
@@ -1738,7 +1759,9 @@ int idtx_ctx_create(idtx_ctx **out, int device)
     n += ksg_variants_d22(tmp + n);
     n += ksg_variants_generic(tmp + n);
     c->variants.assign(tmp, tmp + n);
-    cudaError_t e = cudaMalloc(&c->d_err, sizeof(int));
+    // the error word, then the list kernel's two counters (zero between launches)
+    cudaError_t e = cudaMalloc(&c->d_err, 64 * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, 64 * sizeof(int));
     if (e == cudaSuccess) e = cudaMallocHost(&c->h_err, sizeof(int));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) {

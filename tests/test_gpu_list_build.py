@@ -65,3 +65,19 @@ def test_lists_of_uneven_density_and_equal_distances(idtx):
         e, a, b, d = oracle.ksg_counts(x, y, z, 4)
         assert np.array_equal(eps[0], e)
         assert np.array_equal(cnt[0], np.stack([a, b, d]))
+
+
+@pytest.mark.parametrize("n", [65536, 65537])
+def test_both_forms_of_the_list_kernel_at_their_boundary(idtx, n):
+    """Up to 65536 samples the counts leave the list kernel as 16-bit numbers
+    and the terms are summed apart; above, the kernel sums them itself."""
+    g = synth.gaussian_problem(n, 1, 1, 2, seed=9)
+    _both(idtx, g.x, g.y, g.z, (256, 512), S=1)
+
+
+@pytest.mark.parametrize("n,S,caps", [(129, 0, (32, 32)), (1000, 33, (32, 64)), (3000, 95, (96, 96))])
+def test_queued_full_scans(idtx, n, S, caps):
+    """Lists so short that most (query, group)s, some, or the far ones only go
+    to the scan kernel, with one job in the last group and with full groups."""
+    g = synth.gaussian_problem(n, 1, 1, 3, seed=n)
+    _both(idtx, g.x, g.y, g.z, caps, S=S)
