@@ -216,7 +216,11 @@ int idtx_ctx_set_graphs(idtx_ctx *ctx, int enable);
  *     by their (Y,Z) and their Z distance, keeping the nearest up to a
  *     capacity; each estimate then walks only the prefix it needs, with a
  *     full scan for a (query, estimate) whose neighbourhood the lists do not
- *     cover.  Needs dz >= 1 (dz = 0 calls use the tile kernel).
+ *     cover.  With n in (256, 65536] and one z column the samples' order by
+ *     it takes the place of the lists by Z distance; without z, counts in
+ *     sorted columns take that of both counts' walks (dx = 1; these launches
+ *     are not counted as list_launches).  Other dz = 0 calls use the tile
+ *     kernel.
  *   IDTX_KERNEL_AUTO (default): on the first call of a shape (kernel
  *     variant, floor(log2 N)) both kernels run, timed; from then on in this
  *     context the one serves a call of that shape that is the faster by these

@@ -99,6 +99,14 @@ struct KsgLaunch {
     // between launches: the next chunk, the CTAs done, the entries of scans
     int4 *scans;
     int *next;
+    // list kernel, calls of at most one z column (else 0): iv_a: no z and one
+    // y column, samples ordered by y: pass A walks that order instead of list
+    // A.  b_form 1: one z column, samples ordered by it: the count pass walks
+    // that order instead of list B; 2: no z, one x column: the counts come
+    // from xsort [sources][n], the source columns sorted, jobs[job].x its source
+    int iv_a, b_form;
+    const float *xsort;
+    const int2 *jobs;
     int cap_a, cap_b;
 };
 
@@ -158,6 +166,10 @@ cudaError_t build_lists(const float *sh, int dzb, int dyb, int64_t n, int cap_a,
 cudaError_t sort_pairs_u32(void *tmp, size_t &tmp_bytes, const uint32_t *keys_in,
                            uint32_t *keys_out, const int32_t *vals_in, int32_t *vals_out, int n,
                            int end_bit, cudaStream_t stream);
+
+// Ascending sort of n floats.  With tmp == nullptr only sets tmp_bytes.
+cudaError_t sort_floats(void *tmp, size_t &tmp_bytes, const float *in, float *out, int n,
+                        cudaStream_t stream);
 
 // Learned-screen network kernels (screen.cu).  A work area holds the batch
 // activations (B rows), the gradient and the bf16 copy of the parameters.

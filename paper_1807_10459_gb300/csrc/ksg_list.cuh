@@ -56,6 +56,15 @@
 //     (that tile's queries were all taken earlier, so the wait always ends).
 //     Every wait is bounded by %globaltimer; on expiry the CTA records
 //     kErrTimeout and stops.
+//   * Calls of at most one z column (split form) walk an order instead of a
+//     list where the subspace has one dimension: with one z column the samples
+//     are ordered by it, and the samples after and before the query, whose d_Z
+//     ascends, are list B (up to thousands of entries there, beyond any list's
+//     capacity); with none and one y column the order is by y and stands for
+//     list A.  Without z, n_z is all and n_xz with one x column is a range of
+//     the sorted column.  N = 3001, no z, 201 estimates: 2.0 ms by the tile
+//     kernel, 0.35; N = 20000: 30.1 and 1.7; one z, N = 3001: 0.95 (lists) and
+//     0.57; N = 50000, 101 estimates: 33.1 (tile) and 22.6.
 // Measured on GB300, greedy step of N = 9995 with 9447 estimates (one network;
 // lists of 2048 and 4096): 19.1 -> 13.2 ms with sum_terms; of N = 4997, six
 // conditions, 28341 estimates: 10.8 -> 9.7 ms; N = 1000, 101 estimates: 163 ->
@@ -107,19 +116,41 @@
 
 namespace idtx {
 
-// Number of entries of the ascending list l[0..hi) (hi the lane's own) whose
-// distance is below v, for every lane of a warp.  Warp-uniform probes of
-// every lane at once first bound the answers by a power of two (most are far
-// below hi); then each lane bisects without branches.
-__device__ __forceinline__ int list_lower(const int2 *l, int hi, float v)
+// Number of the ascending distances dist(0..hi-1) (hi the lane's own) that
+// are below v, for every lane of a warp.  Warp-uniform probes of every lane
+// at once first bound the answers by a power of two (most are far below hi);
+// then each lane bisects without branches.
+template <typename Dist>
+__device__ __forceinline__ int count_below(int hi, float v, Dist dist)
 {
     constexpr unsigned kFull = 0xffffffffu;
     int bits = 4;  // the answers are below 2^bits
-    while (__any_sync(kFull, (1 << bits) <= hi && __int_as_float(__ldg(&l[(1 << bits) - 1].y)) < v)) ++bits;
+    while (__any_sync(kFull, (1 << bits) <= hi && dist((1 << bits) - 1) < v)) ++bits;
     int lo = 0;
     for (int b = (1 << bits) >> 1; b; b >>= 1)
-        if (lo + b <= hi && __int_as_float(__ldg(&l[lo + b - 1].y)) < v) lo += b;
+        if (lo + b <= hi && dist(lo + b - 1) < v) lo += b;
     return lo;
+}
+
+// Number of samples other than the query's own within eps of x in the
+// ascending column xs[0..n), which holds x itself: fl(|x - v|) is monotone on
+// either side of x, so they are a contiguous range.
+__device__ __forceinline__ int count_sorted(const float *xs, int n, float x, float eps)
+{
+    int top = 1;
+    while (2 * top <= n) top <<= 1;
+    int lo = 0, hi = 0;  // entries before the range, entries up to its end
+    for (int b = top; b; b >>= 1) {
+        if (lo + b <= n) {
+            const float v = __ldg(xs + lo + b - 1);
+            if (v < x && fabsf(x - v) >= eps) lo += b;
+        }
+        if (hi + b <= n) {
+            const float v = __ldg(xs + hi + b - 1);
+            if (!(v > x && fabsf(x - v) >= eps)) hi += b;
+        }
+    }
+    return eps > 0.0f ? hi - lo - 1 : 0;
 }
 
 // Warp minimum / maximum of non-negative floats (distances, +inf allowed):
@@ -216,6 +247,7 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
     constexpr int KH = K1 - 1;  // smallest distances kept (EXACT: exactly k)
     constexpr int kShStage = kTileRows * DSP;
     constexpr unsigned kFull = 0xffffffffu;
+    constexpr bool LOW = SPLIT && (DZ == 1 || !EXACT);  // may serve calls of at most one z column
     constexpr int TAIL_A = IDTX_LIST_TAIL_A;  // jobs left after the shared neighbour walk
     const float kInf = CUDART_INF_F;
 
@@ -363,8 +395,34 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
             float xq[DX];
 #pragma unroll
             for (int d = 0; d < DX; ++d) xq[d] = xg[static_cast<int64_t>(qi) * XW + d];
-            const int len_a = __ldg(&a.lmeta[qi].x);
-            const int2 *la = a.list_a + static_cast<int64_t>(qi) * a.cap_a;
+            // Where a walk's entries come from: a list, or (dir 1 / -1) the
+            // samples after / before the query in an order sorted by column
+            // `col` of sh, which ascend in their distance in that column.
+            struct Src {
+                const int2 *l;
+                int len, dir, col;
+            };
+            auto entry = [&](const Src &src, int e) -> int2 {
+                if (e >= src.len) return sentinel;
+                if (!LOW || src.dir == 0) return __ldg(src.l + e);
+                const int j = qi + src.dir * (1 + e);
+                return make_int2(j, __float_as_int(fabsf(sh_row(qi)[src.col] - sh_row(j)[src.col])));
+            };
+            auto entry_d = [&](const Src &src, int e) {  // its distance, e < src.len
+                if (!LOW || src.dir == 0) return __int_as_float(__ldg(&src.l[e].y));
+                return fabsf(sh_row(qi)[src.col] - sh_row(qi + src.dir * (1 + e))[src.col]);
+            };
+            // the samples on one side of the query in the order by column col
+            auto side = [&](int dir, int col) {
+                return Src{nullptr, dir > 0 ? static_cast<int>(a.n) - 1 - qi : qi, dir, col};
+            };
+            const bool iv_a = LOW && a.iv_a;  // pass A over the order by the y column
+            Src la;
+            if (iv_a) {
+                la = side(1, DZ);
+            } else {
+                la = Src{a.list_a + static_cast<int64_t>(qi) * a.cap_a, __ldg(&a.lmeta[qi].x), 0, 0};
+            }
 
             auto x_dist = [&](int j) {
                 const float *xr = xg + static_cast<int64_t>(j) * XW;
@@ -410,125 +468,135 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
                     }
                 }
             };
-            auto begin = [&](const int2 *l, int len) {
-                const int2 first = len > 0 ? __ldg(l + lane) : sentinel;
-                nxt = len > 32 ? __ldg(l + 32 + lane) : sentinel;
+            auto begin = [&](const Src &src) {
+                const int2 first = entry(src, lane);
+                nxt = entry(src, 32 + lane);
                 __syncwarp();
                 ent[lane] = first;
                 __syncwarp();
                 fetch(0);
             };
-            auto advance = [&](const int2 *l, int len, int e) {  // after the rows of e
+            auto advance = [&](const Src &src, int e) {  // after the rows of e
                 if ((e & 31) == 32 - 2 * SW || (SW > 8 && (e & 31) == 0)) {
                     const int at = (e & ~31) + 32;  // the chunk after e's
                     __syncwarp();
                     ent[(at & 32) + lane] = nxt;
                     __syncwarp();
-                    nxt = at + 32 < len ? __ldg(l + at + 32 + lane) : sentinel;
+                    nxt = entry(src, at + 32 + lane);
                 }
                 fetch(e + SW);
             };
-            begin(la, len_a);
-            for (int e = 0;; e += SW) {
-                // Ascending list: once the first of the next entries is out
-                // of a job's reach, so is everything after it.  When at most
-                // TAIL_A jobs are still in reach the shared walk stops and
-                // those finish lane-split below.
-                const uint32_t act = __ballot_sync(kFull, row_d[0] < th);
-                if (__popc(act) <= TAIL_A) {
-                    amask = act;
-                    walked_a = e;
-                    break;
+            int my_walked = 0, up_walked = 0;
+            const int parts_a = iv_a ? 2 : 1;
+            int walk_total = 0;
+#pragma unroll 1
+            for (int part = 0; part < parts_a; ++part) {
+                if (part) {  // then the samples before the query
+                    up_walked = my_walked;
+                    la = side(-1, DZ);
                 }
-                float dd[SW];
-#pragma unroll
-                for (int t = 0; t < SW; ++t) {
-                    float dx = fabsf(xq[0] - row_x[t][0]);
-#pragma unroll
-                    for (int d = 1; d < DX; ++d) dx = fmaxf(dx, fabsf(xq[d] - row_x[t][d]));
-                    dd[t] = fmaxf(dx, row_d[t]);
-                }
-                advance(la, len_a, e);
-                if constexpr (EXACT && KH == 4) {
-#pragma unroll
-                    for (int t = 0; t < SW; t += 4) merge4(h, dd[t], dd[t + 1], dd[t + 2], dd[t + 3]);
-                    if (job_ok) th = h[3];
-                } else {
+                begin(la);
+                for (int e = 0;; e += SW) {
+                    // Ascending list: once the first of the next entries is out
+                    // of a job's reach, so is everything after it.  When at most
+                    // TAIL_A jobs are still in reach the shared walk stops and
+                    // those finish lane-split below.
+                    const uint32_t act = __ballot_sync(kFull, row_d[0] < th);
+                    if (__popc(act) <= TAIL_A) {
+                        amask = act;
+                        walked_a = e;
+                        break;
+                    }
+                    float dd[SW];
 #pragma unroll
                     for (int t = 0; t < SW; ++t) {
-                        if (dd[t] < th) {
-                            sorted_insert<KH>(h, dd[t]);
-                            th = kth(h);
+                        float dx = fabsf(xq[0] - row_x[t][0]);
+#pragma unroll
+                        for (int d = 1; d < DX; ++d) dx = fmaxf(dx, fabsf(xq[d] - row_x[t][d]));
+                        dd[t] = fmaxf(dx, row_d[t]);
+                    }
+                    advance(la, e);
+                    if constexpr (EXACT && KH == 4) {
+#pragma unroll
+                        for (int t = 0; t < SW; t += 4) merge4(h, dd[t], dd[t + 1], dd[t + 2], dd[t + 3]);
+                        if (job_ok) th = h[3];
+                    } else {
+#pragma unroll
+                        for (int t = 0; t < SW; ++t) {
+                            if (dd[t] < th) {
+                                sorted_insert<KH>(h, dd[t]);
+                                th = kth(h);
+                            }
                         }
                     }
                 }
-            }
-            if (walked_a > len_a) walked_a = len_a;
-            // Lane-split finish of the remaining jobs, one at a time: steps of
-            // two blocks of 32 entries, one entry per lane and block; the
-            // distances below the job's k-th value are inserted smallest first
-            // (warp minimum) into its k smallest, which every lane holds,
-            // until the step's last entry is out of reach.
-            // my_walked: the prefix of list A this lane's job walked.
-            int my_walked = walked_a;
-            while (amask) {
-                const int f = __ffs(amask) - 1;
-                amask &= amask - 1;
-                float xf[DX];
+                if (walked_a > la.len) walked_a = la.len;
+                // Lane-split finish of the remaining jobs, one at a time: steps of
+                // two blocks of 32 entries, one entry per lane and block; the
+                // distances below the job's k-th value are inserted smallest first
+                // (warp minimum) into its k smallest, which every lane holds,
+                // until the step's last entry is out of reach.
+                // my_walked: the prefix of list A this lane's job walked.
+                my_walked = walked_a;
+                while (amask) {
+                    const int f = __ffs(amask) - 1;
+                    amask &= amask - 1;
+                    float xf[DX];
 #pragma unroll
-                for (int d = 0; d < DX; ++d) xf[d] = __shfl_sync(kFull, xq[d], f);
-                const float *xgf = xg - lane * DX + f * DX;
-                float hf[KH];
+                    for (int d = 0; d < DX; ++d) xf[d] = __shfl_sync(kFull, xq[d], f);
+                    const float *xgf = xg - lane * DX + f * DX;
+                    float hf[KH];
 #pragma unroll
-                for (int t = 0; t < KH; ++t) hf[t] = __shfl_sync(kFull, h[t], f);
-                float thf = kth(hf);
-                int pos = walked_a;
-                while (pos < len_a) {
-                    const int p0 = pos + lane, p1 = pos + 32 + lane;
-                    const int2 e0 = p0 < len_a ? __ldg(la + p0) : sentinel;
-                    const int2 e1 = p1 < len_a ? __ldg(la + p1) : sentinel;
-                    const float y0 = __int_as_float(e0.y), y1 = __int_as_float(e1.y);
-                    if (!(__shfl_sync(kFull, y0, 0) < thf)) break;
-                    auto reach = [&](const int2 e, float y) {  // joint distance, +inf out of reach
-                        if (!(y < thf)) return kInf;
-                        const float *xr = xgf + static_cast<uint64_t>(static_cast<uint32_t>(e.x)) * XW;
-                        float dx = fabsf(xf[0] - xr[0]);
+                    for (int t = 0; t < KH; ++t) hf[t] = __shfl_sync(kFull, h[t], f);
+                    float thf = kth(hf);
+                    int pos = walked_a;
+                    while (pos < la.len) {
+                        const int2 e0 = entry(la, pos + lane), e1 = entry(la, pos + 32 + lane);
+                        const float y0 = __int_as_float(e0.y), y1 = __int_as_float(e1.y);
+                        if (!(__shfl_sync(kFull, y0, 0) < thf)) break;
+                        auto reach = [&](const int2 e, float y) {  // joint distance, +inf out of reach
+                            if (!(y < thf)) return kInf;
+                            const float *xr = xgf + static_cast<uint64_t>(static_cast<uint32_t>(e.x)) * XW;
+                            float dx = fabsf(xf[0] - xr[0]);
 #pragma unroll
-                        for (int d = 1; d < DX; ++d) dx = fmaxf(dx, fabsf(xf[d] - xr[d]));
-                        return fmaxf(dx, y);
-                    };
-                    float c0 = reach(e0, y0), c1 = reach(e1, y1);
-                    while (true) {
-                        const float mn = warp_min_nn(fminf(c0, c1));
-                        if (!(mn < thf)) break;
-                        const uint32_t w0 = __ballot_sync(kFull, c0 == mn);
-                        if (w0) {
-                            if (lane == __ffs(w0) - 1) c0 = kInf;
-                        } else {
-                            const uint32_t w1 = __ballot_sync(kFull, c1 == mn);
-                            if (lane == __ffs(w1) - 1) c1 = kInf;
+                            for (int d = 1; d < DX; ++d) dx = fmaxf(dx, fabsf(xf[d] - xr[d]));
+                            return fmaxf(dx, y);
+                        };
+                        float c0 = reach(e0, y0), c1 = reach(e1, y1);
+                        while (true) {
+                            const float mn = warp_min_nn(fminf(c0, c1));
+                            if (!(mn < thf)) break;
+                            const uint32_t w0 = __ballot_sync(kFull, c0 == mn);
+                            if (w0) {
+                                if (lane == __ffs(w0) - 1) c0 = kInf;
+                            } else {
+                                const uint32_t w1 = __ballot_sync(kFull, c1 == mn);
+                                if (lane == __ffs(w1) - 1) c1 = kInf;
+                            }
+                            sorted_insert<KH>(hf, mn);
+                            thf = kth(hf);
                         }
-                        sorted_insert<KH>(hf, mn);
-                        thf = kth(hf);
+                        ta += (la.len - pos < 64) ? static_cast<unsigned>(la.len - pos) : 64u;
+                        pos += 64;
+                        // ascending: if the step's last entry is out of reach, so is the rest
+                        if (!(__shfl_sync(kFull, y1, 31) < thf)) break;
                     }
-                    ta += (len_a - pos < 64) ? static_cast<unsigned>(len_a - pos) : 64u;
-                    pos += 64;
-                    // ascending: if the step's last entry is out of reach, so is the rest
-                    if (!(__shfl_sync(kFull, y1, 31) < thf)) break;
-                }
-                if (lane == f) {
+                    if (lane == f) {
 #pragma unroll
-                    for (int t = 0; t < KH; ++t) h[t] = hf[t];
-                    th = thf;
-                    my_walked = pos < len_a ? pos : len_a;
+                        for (int t = 0; t < KH; ++t) h[t] = hf[t];
+                        th = thf;
+                        my_walked = pos < la.len ? pos : la.len;
+                    }
                 }
+                walk_total += walked_a;
             }
+            walked_a = walk_total;
             // The list ran out before the job's k-th distance dropped to r_A:
             // the job is recomputed over every sample, in the split form by
             // ksg_scan_kernel, else here: the 32 lanes split the samples of
             // one such job at a time, keep their own k smallest, and the warp
             // merges them (repeatedly taking the smallest head).
-            const float r_a = __int_as_float(__ldg(&a.lmeta[qi].z));
+            const float r_a = iv_a ? kInf : __int_as_float(__ldg(&a.lmeta[qi].z));
             const bool fa = job_ok && th > r_a;
             float eps_fix = 0.0f;
             uint32_t fmask = __ballot_sync(kFull, fa);
@@ -577,108 +645,128 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
             const float eps = job_ok ? (!SPLIT && fa ? eps_fix : kth(h)) : -1.0f;
 
             // ---------------- pass B: strict-radius counts
-            const int len_b = __ldg(&a.lmeta[qi].y);
-            const float r_b = __int_as_float(__ldg(&a.lmeta[qi].w));
-            const int2 *lb = a.list_b + static_cast<int64_t>(qi) * a.cap_b;
+            const int b_form = LOW ? a.b_form : 0;
+            const float r_b = b_form ? kInf : __int_as_float(__ldg(&a.lmeta[qi].w));
             const bool fb = job_ok && (eps > r_a || eps > r_b || (SPLIT && fa));
             int nz = 0, nyz = 0, nxz = 0;
             // Every list A entry below eps lies in the walked prefix (the walk
             // went on until each job's k-th value was at most the next entry).
-            nyz = list_lower(la, job_ok && !fb ? my_walked : 0, eps);
+            nyz = count_below(job_ok && !fb ? my_walked : 0, eps, [&](int e) { return entry_d(la, e); });
+            if (iv_a) {
+                const Src up = side(1, DZ);
+                nyz += count_below(job_ok && !fb ? up_walked : 0, eps, [&](int e) { return entry_d(up, e); });
+            }
             // The count walk over list B: for every job the entries below its
             // eps (n_z) and those also within eps in X (n_xz).  Shared rows,
             // one job per lane, while more than IDTX_LIST_REPACK jobs need
             // entries (`reach`: a job's eps is above the next entry).
             const float ev = (job_ok && !fb) ? eps : 0.0f;
-            int pos = 0;
-            uint32_t rem;
-            begin(lb, len_b);
-            while (true) {
-                rem = __ballot_sync(kFull, ev > row_d[0]);
-                if (__popc(rem) <= IDTX_LIST_REPACK) break;
-                float dx[SW], dz[SW];
-#pragma unroll
-                for (int t = 0; t < SW; ++t) {
-                    dx[t] = fabsf(xq[0] - row_x[t][0]);
-#pragma unroll
-                    for (int d = 1; d < DX; ++d) dx[t] = fmaxf(dx[t], fabsf(xq[d] - row_x[t][d]));
-                    dz[t] = row_d[t];
-                }
-                advance(lb, len_b, pos);
-                pos += SW;
-#pragma unroll
-                for (int t = 0; t < SW; ++t) {
-                    const bool pz = dz[t] < ev;
-                    nz += pz ? 1 : 0;
-                    nxz += (pz && dx[t] < ev) ? 1 : 0;
-                }
+            int walked_b = 0;
+            if (LOW && b_form == 2) {
+                // no Z: every sample counts in n_z, and n_xz is a range of the
+                // job's sorted X column (a permutation does not change it)
+                nz = ev > 0.0f ? static_cast<int>(a.n) - 1 : 0;
+                nxz = count_sorted(a.xsort + static_cast<int64_t>(a.jobs[job_ok ? job : 0].x) * a.n,
+                                   static_cast<int>(a.n), xq[0], ev);
             }
-            const int walked_b = pos < len_b ? pos : len_b;
-            // The jobs that need more share the lanes: with c of them left,
-            // M slots (the power of two >= c) of 32 / M lanes that split the
-            // entries between them; once at most M / 2 need more, the lanes
-            // are shared out again.
-            while (rem) {
-                const int c = __popc(rem);
-                const int lg = c > 8 ? 4 : (c > 4 ? 3 : (c > 2 ? 2 : (c > 1 ? 1 : 0)));
-                const int M = 1 << lg, per = 32 >> lg;
-                const int s = lane & (M - 1), r = lane >> lg;
-                const int rank = __popc(rem & ((1u << lane) - 1u));
-                int *tab = &ent[0].x;  // the staged entries are done with
-                __syncwarp();
-                if ((rem >> lane) & 1u) tab[rank] = lane;
-                __syncwarp();
-                const int home = s < c ? tab[s] : lane;
-                const float e_home = __shfl_sync(kFull, ev, home);
-                const float es = s < c ? e_home : 0.0f;
-                float xs[DX];
+            // b_form 1: one z column, and the order is by it: the samples on
+            // either side of the query take the place of the list
+            const int parts_b = !LOW || b_form == 0 ? 1 : (b_form == 1 ? 2 : 0);
+#pragma unroll 1
+            for (int part = 0; part < parts_b; ++part) {
+                const Src lb = LOW && b_form == 1
+                                   ? side(part ? -1 : 1, 0)
+                                   : Src{a.list_b + static_cast<int64_t>(qi) * a.cap_b, __ldg(&a.lmeta[qi].y), 0, 0};
+                int pos = 0;
+                uint32_t rem;
+                begin(lb);
+                while (true) {
+                    rem = __ballot_sync(kFull, ev > row_d[0]);
+                    if (__popc(rem) <= IDTX_LIST_REPACK) break;
+                    float dx[SW], dz[SW];
 #pragma unroll
-                for (int d = 0; d < DX; ++d) xs[d] = __shfl_sync(kFull, xq[d], home);
-                const float *xgs = xg + (home - lane) * DX;
-                const int from = pos;
-                int cz = 0, cx = 0;
-                uint32_t still;
-                do {
-                    constexpr int PS = IDTX_LIST_PHASE_STEP;
-                    int js[PS];
-                    float xv[PS][DX];
+                    for (int t = 0; t < SW; ++t) {
+                        dx[t] = fabsf(xq[0] - row_x[t][0]);
 #pragma unroll
-                    for (int t = 0; t < PS; ++t) {
-                        const int e = pos + r + per * t;
-                        const int2 v = e < len_b ? __ldg(lb + e) : sentinel;
-                        js[t] = __int_as_float(v.y) < es ? v.x : -1;
+                        for (int d = 1; d < DX; ++d) dx[t] = fmaxf(dx[t], fabsf(xq[d] - row_x[t][d]));
+                        dz[t] = row_d[t];
                     }
+                    advance(lb, pos);
+                    pos += SW;
 #pragma unroll
-                    for (int t = 0; t < PS; ++t) {
-                        const float *xr = xgs + static_cast<uint64_t>(static_cast<uint32_t>(js[t])) * XW;
-#pragma unroll
-                        for (int d = 0; d < DX; ++d) xv[t][d] = js[t] >= 0 ? xr[d] : CUDART_INF_F;
+                    for (int t = 0; t < SW; ++t) {
+                        const bool pz = dz[t] < ev;
+                        nz += pz ? 1 : 0;
+                        nxz += (pz && dx[t] < ev) ? 1 : 0;
                     }
-                    pos += per * PS;
-                    const float dn = pos < len_b ? __int_as_float(__ldg(&lb[pos].y)) : kInf;
-#pragma unroll
-                    for (int t = 0; t < PS; ++t) {
-                        float dxv = fabsf(xs[0] - xv[t][0]);
-#pragma unroll
-                        for (int d = 1; d < DX; ++d) dxv = fmaxf(dxv, fabsf(xs[d] - xv[t][d]));
-                        cz += js[t] >= 0 ? 1 : 0;
-                        cx += dxv < es ? 1 : 0;
-                    }
-                    still = __ballot_sync(kFull, ((rem >> lane) & 1u) && ev > dn);
-                } while (__popc(still) > (M >> 1));
-                tb += static_cast<unsigned>(c * (pos - from));
-                // each slot's totals over its lanes, then to the job's lane
-                for (int off = M; off < 32; off <<= 1) {
-                    cz += __shfl_xor_sync(kFull, cz, off);
-                    cx += __shfl_xor_sync(kFull, cx, off);
                 }
-                const int vz = __shfl_sync(kFull, cz, rank & 31);
-                const int vx = __shfl_sync(kFull, cx, rank & 31);
-                if ((rem >> lane) & 1u) {
-                    nz += vz;
-                    nxz += vx;
+                walked_b += pos < lb.len ? pos : lb.len;
+                // The jobs that need more share the lanes: with c of them left,
+                // M slots (the power of two >= c) of 32 / M lanes that split the
+                // entries between them; once at most M / 2 need more, the lanes
+                // are shared out again.
+                while (rem) {
+                    const int c = __popc(rem);
+                    const int lg = c > 8 ? 4 : (c > 4 ? 3 : (c > 2 ? 2 : (c > 1 ? 1 : 0)));
+                    const int M = 1 << lg, per = 32 >> lg;
+                    const int s = lane & (M - 1), r = lane >> lg;
+                    const int rank = __popc(rem & ((1u << lane) - 1u));
+                    int *tab = &ent[0].x;  // the staged entries are done with
+                    __syncwarp();
+                    if ((rem >> lane) & 1u) tab[rank] = lane;
+                    __syncwarp();
+                    const int home = s < c ? tab[s] : lane;
+                    const float e_home = __shfl_sync(kFull, ev, home);
+                    const float es = s < c ? e_home : 0.0f;
+                    float xs[DX];
+#pragma unroll
+                    for (int d = 0; d < DX; ++d) xs[d] = __shfl_sync(kFull, xq[d], home);
+                    const float *xgs = xg + (home - lane) * DX;
+                    const int from = pos;
+                    int cz = 0, cx = 0;
+                    uint32_t still;
+                    do {
+                        constexpr int PS = IDTX_LIST_PHASE_STEP;
+                        int js[PS];
+                        float xv[PS][DX];
+#pragma unroll
+                        for (int t = 0; t < PS; ++t) {
+                            const int e = pos + r + per * t;
+                            const int2 v = entry(lb, e);
+                            js[t] = __int_as_float(v.y) < es ? v.x : -1;
+                        }
+#pragma unroll
+                        for (int t = 0; t < PS; ++t) {
+                            const float *xr = xgs + static_cast<uint64_t>(static_cast<uint32_t>(js[t])) * XW;
+#pragma unroll
+                            for (int d = 0; d < DX; ++d) xv[t][d] = js[t] >= 0 ? xr[d] : CUDART_INF_F;
+                        }
+                        pos += per * PS;
+                        const float dn = pos < lb.len ? entry_d(lb, pos) : kInf;
+#pragma unroll
+                        for (int t = 0; t < PS; ++t) {
+                            float dxv = fabsf(xs[0] - xv[t][0]);
+#pragma unroll
+                            for (int d = 1; d < DX; ++d) dxv = fmaxf(dxv, fabsf(xs[d] - xv[t][d]));
+                            cz += js[t] >= 0 ? 1 : 0;
+                            cx += dxv < es ? 1 : 0;
+                        }
+                        still = __ballot_sync(kFull, ((rem >> lane) & 1u) && ev > dn);
+                    } while (__popc(still) > (M >> 1));
+                    tb += static_cast<unsigned>(c * (pos - from));
+                    // each slot's totals over its lanes, then to the job's lane
+                    for (int off = M; off < 32; off <<= 1) {
+                        cz += __shfl_xor_sync(kFull, cz, off);
+                        cx += __shfl_xor_sync(kFull, cx, off);
+                    }
+                    const int vz = __shfl_sync(kFull, cz, rank & 31);
+                    const int vx = __shfl_sync(kFull, cx, rank & 31);
+                    if ((rem >> lane) & 1u) {
+                        nz += vz;
+                        nxz += vx;
+                    }
+                    rem = still;
                 }
-                rem = still;
             }
             // Jobs whose eps reaches past a list: counts by a full scan, in
             // the split form by ksg_scan_kernel, else here, the 32 lanes
@@ -826,7 +914,7 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
 // Full scans, for the (query, group)s that the split form's lists did not
 // serve (a query far from the others has long neighbourhoods for all of its
 // jobs): eps and the counts of the marked jobs over every sample.  A CTA takes
-// one (query, group) at a time, its warps every kScanWarps-th 32 samples; in a warp
+// one (query, group) at a time, each of its warps 32 samples of every eighth tile; in a warp
 // a lane per sample finds the samples within reach, 32 at a time, and a lane
 // per job uses them, their X rows loaded sixteen at a time.  The warps share
 // each job's smallest k-th distance so far (any warp's is at least the job's
@@ -835,6 +923,7 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
 // 9995 with 32 jobs, and the whole GPU often waited for it; here it takes 70
 // us, bound by the latency of its loads.
 constexpr int kScanWarps = 32;
+static_assert(kScanWarps % (kTJ / 32) == 0, "whole tiles per step");
 
 template <int DX, int DY, int DZ, int K1, bool EXACT, int QCTA, int NWARPS>
 __global__ void __launch_bounds__(kScanWarps * 32, 1)
@@ -868,39 +957,53 @@ __global__ void __launch_bounds__(kScanWarps * 32, 1)
         // its 32 samples
         auto scan = [&](auto zonly, auto limit, auto use) {
             constexpr bool ZONLY = decltype(zonly)::value;
+            constexpr int SEGS = kTJ / 32, STEP = kScanWarps / SEGS;  // a warp: one segment of every STEP-th tile
+            const int b = warp % SEGS * 32;
             float lim = limit();
-            for (int g = warp; g < n_tiles * (kTJ / 32); g += kScanWarps) {  // 32 samples at a time
-                const int t = g / (kTJ / 32), b = g % (kTJ / 32) * 32;
-                const float *tile = a.sh + static_cast<int64_t>(t) * kTileRows * DSP;
-                if (!(point_gap<ZONLY ? DZ : DS, DSP>(tile, q) < lim)) continue;
-                const float *row = tile + (b + lane) * DSP;
-                float dz = fabsf(q[0] - row[0]);
+            for (int i0 = 0; i0 * STEP < n_tiles; i0 += 32) {
+                // from the query's own tile outwards, so that the bounds are
+                // soon tight; 32 tiles' boxes are tested at a time
+                const int u = (i0 + lane) * STEP + warp / SEGS;
+                const int my_tile = u < n_tiles ? spiral_tile(qi / kTJ, n_tiles, u) : 0;
+                const float my_gap =
+                    u < n_tiles ? point_gap<ZONLY ? DZ : DS, DSP>(
+                                      a.sh + static_cast<int64_t>(my_tile) * kTileRows * DSP, q)
+                                : CUDART_INF_F;
+                uint32_t todo = __ballot_sync(kFull, my_gap < lim);
+                while (todo) {
+                    const int w = __ffs(todo) - 1;
+                    todo &= todo - 1;
+                    const int t = __shfl_sync(kFull, my_tile, w);
+                    if (!(__shfl_sync(kFull, my_gap, w) < lim)) continue;
+                    const float *row = a.sh + (static_cast<int64_t>(t) * kTileRows + b + lane) * DSP;
+                    float dz = fabsf(q[0] - row[0]);
 #pragma unroll
-                for (int d = 1; d < DZ; ++d) dz = fmaxf(dz, fabsf(q[d] - row[d]));
-                float dyz = dz;
+                    for (int d = 1; d < DZ; ++d) dz = fmaxf(dz, fabsf(q[d] - row[d]));
+                    float dyz = dz;
 #pragma unroll
-                for (int d = DZ; d < DS; ++d) dyz = fmaxf(dyz, fabsf(q[d] - row[d]));
-                const int j0 = t * kTJ + b;
-                const bool other = j0 + lane < n && j0 + lane != qi;
-                uint32_t in = __ballot_sync(kFull, other && (ZONLY ? dz : dyz) < lim);
-                while (in) {
-                    float dx[U], z[U], yz[U];  // +inf where no sample is left
+                    for (int d = DZ; d < DS; ++d) dyz = fmaxf(dyz, fabsf(q[d] - row[d]));
+                    const int j0 = t * kTJ + b;
+                    const bool other = j0 + lane < n && j0 + lane != qi;
+                    uint32_t in = __ballot_sync(kFull, other && (ZONLY ? dz : dyz) < lim);
+                    while (in) {
+                        float dx[U], z[U], yz[U];  // +inf where no sample is left
 #pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int s = __ffs(in) - 1;
-                        const bool some = in != 0;
-                        in &= in - 1;
-                        const float *xr = xg + static_cast<int64_t>(some ? j0 + s : qi) * XW;
-                        dx[u] = fabsf(xq[0] - xr[0]);
+                        for (int v = 0; v < U; ++v) {
+                            const int s = __ffs(in) - 1;
+                            const bool some = in != 0;
+                            in &= in - 1;
+                            const float *xr = xg + static_cast<int64_t>(some ? j0 + s : qi) * XW;
+                            dx[v] = fabsf(xq[0] - xr[0]);
 #pragma unroll
-                        for (int d = 1; d < DX; ++d) dx[u] = fmaxf(dx[u], fabsf(xq[d] - xr[d]));
-                        z[u] = __shfl_sync(kFull, dz, s & 31);
-                        yz[u] = __shfl_sync(kFull, dyz, s & 31);
-                        if (!some) z[u] = yz[u] = CUDART_INF_F;
+                            for (int d = 1; d < DX; ++d) dx[v] = fmaxf(dx[v], fabsf(xq[d] - xr[d]));
+                            z[v] = __shfl_sync(kFull, dz, s & 31);
+                            yz[v] = __shfl_sync(kFull, dyz, s & 31);
+                            if (!some) z[v] = yz[v] = CUDART_INF_F;
+                        }
+                        use(dx, z, yz);
                     }
-                    use(dx, z, yz);
+                    lim = limit();
                 }
-                lim = limit();
             }
         };
         if (warp == 0) {

@@ -7,7 +7,8 @@
 // estimator's definition (fp32 |a-b| and maxima).  List A holds every j != i
 // with d_YZ < r_A(i), list B every j != i with d_Z < r_B(i), each ascending
 // by distance (equal distances in any order; entries at r itself may follow).
-// r_A, r_B are any radii for which the lists fit their capacities.
+// r_A, r_B are any radii for which the lists fit their capacities.  With
+// cap_b = 0 there is only list A.
 //
 // Two kernels per chunk of queries, with the unsorted entries in scratch
 // between them:
@@ -259,6 +260,7 @@ __global__ void __launch_bounds__(kCollectThreads, DZ + DY <= 12 ? 3 : 2)
         }
         __syncwarp();
     }
+    if (a.cap_b == 0) rb[0] = rb[1] = -1.0f;  // list A only
     if (!two) ra[1] = rb[1] = -1.0f;
     int2 *const oa = a.raw_a + (int64_t)g0 * a.buf_a, *const ob = a.raw_b + (int64_t)g0 * a.buf_b;
     const int n_tiles = (n + kTJ - 1) / kTJ;
@@ -672,7 +674,7 @@ cudaError_t build_lists(const float *sh, int dzb, int dyb, int64_t n, int cap_a,
     c.raw_b = c.raw_a + chunk * c.buf_a;
     c.raw_meta = (int4 *)(((uintptr_t)(c.raw_b + chunk * c.buf_b) + 15) & ~(uintptr_t)15);
     // No sample when it would be half of the samples or every list holds all.
-    const int cut = cap_a < n - 1 ? cap_a : cap_b;
+    const int cut = cap_a < n - 1 || cap_b == 0 ? cap_a : cap_b;
     if (cut < n - 1) {
         const int64_t m = (cut >= 1024 ? 64 : 28) * n / cut;
         if (2 * m <= n) {
@@ -696,11 +698,12 @@ cudaError_t build_lists(const float *sh, int dzb, int dyb, int64_t n, int cap_a,
         if (e != cudaSuccess) return e;
         // Short lists in one launch; long ones apart, with the blocks of each size.
         const int buf = std::max(c.buf_a, c.buf_b);
-        const bool together = buf <= 1024 || c.buf_a == c.buf_b;
+        const bool together = cap_b > 0 && (buf <= 1024 || c.buf_a == c.buf_b);
         e = sort_lists(s, n_q, together ? 2 : 1, together ? buf : c.buf_a, st);
-        if (e == cudaSuccess && !together) e = sort_lists(SortPair{{s.l[1], s.l[1]}}, n_q, 1, c.buf_b, st);
+        if (e == cudaSuccess && !together && cap_b > 0)
+            e = sort_lists(SortPair{{s.l[1], s.l[1]}}, n_q, 1, c.buf_b, st);
         if (e != cudaSuccess) return e;
-        if (launches) *launches += together ? 2 : 3;
+        if (launches) *launches += together || cap_b == 0 ? 2 : 3;
     }
     return cudaSuccess;
 }

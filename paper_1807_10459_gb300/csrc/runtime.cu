@@ -216,6 +216,17 @@ __global__ void k_morton_keys(const Col *zc, int dz, const Col *yc, int nk, int 
     }
 }
 
+// Keys that order like the values of a column; idx[j] = j.
+__global__ void k_value_keys(const Col *col, int64_t n, uint32_t *keys, int32_t *idx)
+{
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
+         j += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t b = __float_as_uint(col->base[col->off + j]);
+        keys[j] = b & 0x80000000u ? ~b : b | 0x80000000u;
+        idx[j] = (int32_t)j;
+    }
+}
+
 // Replication-level surrogates: slot s's permutation of the samples moves
 // whole replications of len samples, pi_s(r*len + t) = blk[s][r]*len + t,
 // blk[s] the permutation of the n_reps replications.  With `order`, the row
@@ -834,13 +845,17 @@ struct Group {
     int n_qt = 0, n_groups = 0;
     size_t off_x = 0, off_y = 0, off_z = 0, off_jobs = 0, off_streams = 0, off_seeds = 0;
     size_t off_cmi = 0;  // index of the group's first job in the call's cmi buffer
-    bool sort = false;   // order the samples along a Morton curve first
+    bool sort = false;   // order the samples first: along a Morton curve, or
+    int col_order = 0;   // 1: by the one z column, 2: no z: by the one y column
     bool plain = false;  // one launch per estimate (IDTX_MODE_PLAIN)
     int work_slot = 0;   // index of the group's work counters in the call
     int64_t n_reps = 0;     // > 0: surrogates permute n_reps whole replications
     bool use_list = false;  // run the list kernel (ksg_list.cuh)
     bool tune = false;      // time both kernels first (shape not tuned yet)
     int cap_a = 0, cap_b = 0;  // list capacities
+    // list kernel, at most one z column (KsgLaunch): walks over a sorted order
+    // and counts in sorted columns in the place of lists
+    int iv_a = 0, b_form = 0;
 };
 
 // Memory the lists of one group may take; larger N gets shorter lists.
@@ -865,7 +880,7 @@ std::pair<const KsgVariant *, int> tune_key(const Group &g)
 {
     int lg = 0;
     while ((int64_t(1) << (lg + 1)) <= g.n) ++lg;
-    return {g.v, lg};
+    return {g.v, lg + 64 * (2 * g.b_form + g.iv_a)};  // the forms without lists apart
 }
 
 // The way of running g that the trial's times, scaled to g, put first.
@@ -892,6 +907,7 @@ const idtx_ctx::Timed &best_way(const idtx_ctx::Trial &t, const Group &g)
 void take_way(Group &g, const idtx_ctx::Timed &w)
 {
     g.use_list = w.list;
+    if (!w.list) g.iv_a = g.b_form = 0;
     if (w.list) {
         g.cap_a = std::min(g.cap_a, w.cap_a);
         g.cap_b = std::min(g.cap_b, w.cap_b);
@@ -908,13 +924,29 @@ int plan(idtx_ctx *c, Group &g)
     g.n_groups = (int)((g.jobs.size() + g.v->gb - 1) / g.v->gb);
     if (g.n_groups > 65535) return fail(IDTX_EINVAL, "too many estimates in one group");
     g.sort = !g.plain && g.n > 2 * kTJ;
+    // The order fixes that of the sums, so it is the same for both kernels.
+    g.col_order = 0;
+    if (g.sort && g.n_pad <= 65536)
+        g.col_order = g.dz == 1 ? 1 : (g.dz == 0 && g.dy == 1 ? 2 : 0);
     if (g.plain) g.n_qt = (int)(g.n_pad / kPlainQueriesPerPartial);
-    // The list kernel needs a Z subspace (with dz = 0 list B would hold every
-    // sample) and lists that fit the memory budget.
+    // The list kernel needs lists that fit the memory budget.  List B would
+    // be long with few z columns: with one, the samples are ordered by it and
+    // the count pass walks that order; with none, it counts in sorted columns
+    // (one x column; more go to the tile kernel), and one y column does not
+    // need list A either.  Both want an ordered call and 16-bit counts.
     g.use_list = g.tune = false;
-    g.cap_a = g.cap_b = 0;
-    if (!g.plain && g.dz >= 1 && c->kernel_pref != IDTX_KERNEL_TILE) {
-        list_caps(c, g.n, g.cap_a, g.cap_b);
+    g.cap_a = g.cap_b = g.iv_a = g.b_form = 0;
+    if (!g.plain && c->kernel_pref != IDTX_KERNEL_TILE) {
+        if (g.dz <= 1 && g.sort && g.n_pad <= 65536) {
+            if (g.dz == 1) g.b_form = 1;
+            if (g.dz == 0 && g.dx == 1) {
+                g.b_form = 2;
+                g.iv_a = g.dy == 1;
+            }
+        }
+        if (g.dz >= 1 || g.b_form) list_caps(c, g.n, g.cap_a, g.cap_b);
+        if (g.b_form) g.cap_b = 0;
+        if (g.iv_a) g.cap_a = 32;  // unused
         if (g.cap_a > 0) {
             if (c->kernel_pref == IDTX_KERNEL_LIST) {
                 g.use_list = true;
@@ -927,6 +959,7 @@ int plan(idtx_ctx *c, Group &g)
                 }
             }
         }
+        if (!g.use_list && !g.tune) g.iv_a = g.b_form = 0;
     }
     return IDTX_OK;
 }
@@ -969,7 +1002,7 @@ struct CallBuffers {
 
 // B_LIST layout for n queries: list_a [n][cap_a] | list_b [n][cap_b] | meta [n]
 // | the list kernel's term ring, all counted here | its counts
-// | build_lists' scratch.
+// | the sorted columns of a call without z | build_lists' scratch.
 size_t list_bytes(int64_t n, int cap_a, int cap_b)
 {
     return align_up((size_t)n * cap_a * sizeof(int2), 256) +
@@ -986,6 +1019,12 @@ size_t count_bytes(const Group &g)
     return align_up(count_rows(g) * 3 * sizeof(uint16_t) + count_rows(g) / 32 * sizeof(int4), 256);
 }
 
+// The sorted source columns of a call without z, part of B_LIST.
+size_t xsort_bytes(const Group &g)
+{
+    return g.b_form == 2 ? align_up(g.xcols.size() * (size_t)g.n * sizeof(float), 256) : 0;
+}
+
 // B_ORDER layout for n samples: order | idx | keys_in | keys_out | column ranges.
 size_t order_bytes(int64_t n) { return 4 * align_up((size_t)n * 4, 256) + 256; }
 
@@ -998,13 +1037,18 @@ CallBuffers bytes_of(const Group &g)
         b.order = align_up(order_bytes(g.n), 256);
         size_t tmp = 0;
         sort_pairs_u32(nullptr, tmp, nullptr, nullptr, nullptr, nullptr, (int)g.n, 32, nullptr);
+        if (g.b_form == 2) {
+            size_t keys = 0;
+            sort_floats(nullptr, keys, nullptr, nullptr, (int)g.n, nullptr);
+            tmp = std::max(tmp, keys);
+        }
         b.sort_tmp = align_up(tmp, 256);
     }
     b.xi = align_up((size_t)g.n_groups * g.n_pad * g.v->gb * g.v->dx * sizeof(float), 256);
     b.perm = align_up(g.slot_stream.size() * (size_t)(g.n + g.n_reps) * sizeof(int32_t), 256);
     b.partial = align_up(g.jobs.size() * (size_t)g.n_qt * sizeof(double), 256);
     if (g.use_list || g.tune)
-        b.lists = list_bytes(g.n, g.cap_a, g.cap_b) + count_bytes(g) +
+        b.lists = list_bytes(g.n, g.cap_a, g.cap_b) + count_bytes(g) + xsort_bytes(g) +
                   list_scratch_bytes(g.n, g.cap_a, g.cap_b);
     return b;
 }
@@ -1140,6 +1184,9 @@ void fill_launch(const idtx_ctx *c, const Group &g, const Slices &sl, float *eps
     a.lscratch = nullptr;
     a.cyz = a.cz = a.cxz = nullptr;
     a.scans = nullptr;
+    a.iv_a = a.b_form = 0;
+    a.xsort = nullptr;
+    a.jobs = nullptr;
     a.cap_a = g.cap_a;
     a.cap_b = g.cap_b;
     if ((g.use_list || g.tune) && sl.lists) {
@@ -1151,7 +1198,11 @@ void fill_launch(const idtx_ctx *c, const Group &g, const Slices &sl, float *eps
         a.lmeta = (const int4 *)(sl.lists + oa + ob);
         a.ring = (double *)(sl.lists + oa + ob + om);
         unsigned char *sp = sl.lists + list_bytes(g.n, g.cap_a, g.cap_b);
-        a.lscratch = sp + count_bytes(g);
+        a.lscratch = sp + count_bytes(g) + xsort_bytes(g);
+        if (g.b_form == 2) a.xsort = (const float *)(sp + count_bytes(g));
+        a.iv_a = g.iv_a;
+        a.b_form = g.b_form;
+        a.jobs = (const int2 *)((const unsigned char *)c->buf[B_DESC] + g.off_jobs);
         if (const size_t rows = count_rows(g)) {
             a.cyz = (uint16_t *)sp;
             a.cz = a.cyz + rows;
@@ -1197,16 +1248,24 @@ int prep_group(idtx_ctx *c, const Group &g, cudaStream_t st, const Slices &sl, f
         float *mm = (float *)(ob + 4 * col);
         int nk, bits;
         morton_shape(g.dz + g.dy, nk, bits);
-        k_minmax_cols<<<nk, 256, 0, st>>>(zc, g.dz, yc, g.dy, g.n, mm);
-        IDTX_CUDA(cudaGetLastError());
-        k_morton_keys<<<grid_for(g.n, 256), 256, 0, st>>>(zc, g.dz, yc, nk, bits, g.n, mm, kin,
-                                                          idx);
-        IDTX_CUDA(cudaGetLastError());
+        if (g.col_order) {
+            k_value_keys<<<grid_for(g.n, 256), 256, 0, st>>>(g.col_order == 2 ? yc : zc, g.n, kin, idx);
+            IDTX_CUDA(cudaGetLastError());
+            nk = 1;
+            bits = 32;
+            launches += 2;
+        } else {
+            k_minmax_cols<<<nk, 256, 0, st>>>(zc, g.dz, yc, g.dy, g.n, mm);
+            IDTX_CUDA(cudaGetLastError());
+            k_morton_keys<<<grid_for(g.n, 256), 256, 0, st>>>(zc, g.dz, yc, nk, bits, g.n, mm, kin,
+                                                              idx);
+            IDTX_CUDA(cudaGetLastError());
+            launches += 3;
+        }
         size_t tmp_bytes = sl.sort_cap;
         IDTX_CUDA(sort_pairs_u32(sl.sort_tmp, tmp_bytes, kin, kout, idx, ord, (int)g.n,
                                  nk * bits, st));
         order = ord;
-        launches += 3;
     }
     k_pack_shared<<<grid_for(g.n_pad * v.dsp, 256), 256, 0, st>>>(
         zc, g.dz, dzb, yc, g.dy, dyb, v.dsp, g.n, g.n_pad, order, sh, c->d_err);
@@ -1227,6 +1286,14 @@ int prep_group(idtx_ctx *c, const Group &g, cudaStream_t st, const Slices &sl, f
         IDTX_CUDA(cudaEventRecord(fork, st));
         IDTX_CUDA(cudaStreamWaitEvent(c->side_stream, fork, 0));
         xs = c->side_stream;
+    }
+    if (g.b_form == 2) {
+        size_t tmp_bytes = sl.sort_cap;
+        for (size_t s = 0; s < g.xcols.size(); ++s) {
+            IDTX_CUDA(sort_floats(sl.sort_tmp, tmp_bytes, g.xcols[s].base + g.xcols[s].off,
+                                  const_cast<float *>(a.xsort) + s * g.n, (int)g.n, xs));
+            launches += 1;
+        }
     }
     // Permutation rows composed with the sample order where the shuffle can
     // write them so (the gather then reads them in sequence).
@@ -1258,9 +1325,10 @@ int prep_group(idtx_ctx *c, const Group &g, cudaStream_t st, const Slices &sl, f
     if (a.list_a) {
         IDTX_CUDA(cudaEventRecord(join, xs));
         int built = 0;
-        IDTX_CUDA(build_lists(sh, v.dz, v.dy, g.n, g.cap_a, g.cap_b,
-                              const_cast<int2 *>(a.list_a), const_cast<int2 *>(a.list_b),
-                              const_cast<int4 *>(a.lmeta), a.lscratch, st, &built));
+        if (!g.iv_a)
+            IDTX_CUDA(build_lists(sh, v.dz, v.dy, g.n, g.cap_a, g.cap_b,
+                                  const_cast<int2 *>(a.list_a), const_cast<int2 *>(a.list_b),
+                                  const_cast<int4 *>(a.lmeta), a.lscratch, st, &built));
         IDTX_CUDA(cudaStreamWaitEvent(st, join, 0));
         // a later record of these events does not disturb the waits above
         c->event_pool.push_back(fork);
@@ -1292,7 +1360,7 @@ void note_group(idtx_ctx *c, const Group &g, int launches, bool list)
     c->call_shapes[g.work_slot] = ws;
     c->stats.fused_launches += 1;
     c->stats.kernel_launches += launches;
-    if (list) c->stats.list_launches += 1;
+    if (list && g.dz > 0) c->stats.list_launches += 1;  // (without z there is no list B)
 }
 
 // Time the candidate ways of running a prepared group -- the tile kernel, and
@@ -1304,16 +1372,17 @@ int tune_group(idtx_ctx *c, const Group &g, KsgLaunch &a, cudaStream_t st, bool 
 {
     idtx_ctx::Trial trial{g.n, g.n_groups, {{false, 0, 0, 0.0f, 0.0f}, {true, g.cap_a, g.cap_b, 0.0f, 0.0f}}};
     std::vector<idtx_ctx::Timed> &way = trial.way;
-    if (c->cap_a == 0 && c->cap_b == 0)  // capacities not fixed by the caller
+    if (c->cap_a == 0 && c->cap_b == 0 && !g.iv_a)  // capacities not fixed by the caller
         for (int sh = 1; sh <= 2; ++sh) {
             const int ca = (g.cap_a >> sh) / 32 * 32, cb = (g.cap_b >> sh) / 32 * 32;
-            if (ca >= 256 && cb >= 256) way.push_back({true, ca, cb, 0.0f, 0.0f});
+            if (ca >= 256 && (cb >= 256 || g.b_form)) way.push_back({true, ca, cb, 0.0f, 0.0f});
         }
     const KsgVariant &v = *g.v;
     KsgLaunch t = a;
     t.work = nullptr;
     auto build = [&](int ca, int cb) -> int {
         int built = 0;
+        if (g.iv_a) return IDTX_OK;
         IDTX_CUDA(build_lists(a.sh, v.dz, v.dy, g.n, ca, cb, const_cast<int2 *>(a.list_a),
                               const_cast<int2 *>(a.list_b), const_cast<int4 *>(a.lmeta),
                               a.lscratch, st, &built));

@@ -1,7 +1,7 @@
 // sort.cu -- the library's one use of a vendor primitive: CUB's device radix
-// sort of (32-bit key, int32 index) pairs, used to order samples along a
-// space-filling curve before the estimator runs.  Kept in its own
-// translation unit so the template instantiation compiles in parallel.
+// sort, of (32-bit key, int32 index) pairs to order the samples before the
+// estimator runs, and of a column's values for counts in it.  Kept in its own
+// translation unit so the template instantiations compile in parallel.
 #include <cub/device/device_radix_sort.cuh>
 
 #include "ksg_common.cuh"
@@ -14,6 +14,12 @@ cudaError_t sort_pairs_u32(void *tmp, size_t &tmp_bytes, const uint32_t *keys_in
 {
     return cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, keys_in, keys_out, vals_in, vals_out, n,
                                            0, end_bit, stream);
+}
+
+cudaError_t sort_floats(void *tmp, size_t &tmp_bytes, const float *in, float *out, int n,
+                        cudaStream_t stream)
+{
+    return cub::DeviceRadixSort::SortKeys(tmp, tmp_bytes, in, out, n, 0, 32, stream);
 }
 
 }  // namespace idtx

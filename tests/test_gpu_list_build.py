@@ -29,7 +29,8 @@ def _both(idtx, x, y, z, caps, S=2, k=4):
         ctx = idtx.Context(0)
         ctx.set_kernel(kernel)
         ctx.set_list_caps(*caps)
-        dev = [torch.from_numpy(np.ascontiguousarray(c)).cuda() for c in (x, y, z)]
+        dev = [None if c is None else torch.from_numpy(np.ascontiguousarray(c)).cuda()
+               for c in (x, y, z)]
         r = idtx.cmi_ksg(*dev, k=k, n_surr=S, seed=11, want_eps=True, want_counts=True, ctx=ctx)
         out.append([t.cpu().numpy() for t in r])
     for a, b in zip(*out):
@@ -81,3 +82,22 @@ def test_queued_full_scans(idtx, n, S, caps):
     to the scan kernel, with one job in the last group and with full groups."""
     g = synth.gaussian_problem(n, 1, 1, 3, seed=n)
     _both(idtx, g.x, g.y, g.z, caps, S=S)
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 0), (1, 2, 0), (2, 1, 0), (1, 1, 1), (2, 2, 1), (3, 1, 1)])
+@pytest.mark.parametrize("n,k", [(257, 4), (1100, 4), (3001, 4), (700, 7)])
+def test_at_most_one_z_column(idtx, dims, n, k):
+    """Walks over the order by the z or y column and counts in sorted columns
+    instead of lists: against the tile kernel and the oracle, on continuous
+    data and on data full of equal values."""
+    g = synth.gaussian_problem(n, *dims, seed=n + k)
+    rng = np.random.default_rng(n)
+    for grid in (False, True):
+        x, y, z = (rng.integers(-3, 4, c.shape).astype(np.float32) if grid else c
+                   for c in (g.x, g.y, g.z))
+        cmi, eps, cnt = _both(idtx, x, y, z if dims[2] else None, (0, 0), S=34, k=k)
+        e, a, b, c = oracle.ksg_counts(x, y, z if dims[2] else None, k)
+        assert np.array_equal(eps[0], e)
+        assert np.array_equal(cnt[0], np.stack([a, b, c]))
+        ref = oracle.cmi_surrogates(x, y, z if dims[2] else None, k, 1, 11)
+        assert np.max(np.abs(cmi[:2] - ref)) < 1e-10
