@@ -18,14 +18,15 @@
 //   k_sort_lists  a block per (query, list): counting sort on the distance.
 // Measured on GB300 against one block per query with two histogram passes over
 // all rows and block radix sorts, both kernels together: N = 9995, three z and
-// one y column, lists of 2048 and 4096: 1.68 -> 0.98 ms; N = 4997, six z,
-// 1024 and 2048: 0.51 -> 0.33 ms; N = 99850, ten z, 512 and 1024: 44.3 ->
-// 9.1 ms (that kernel read every visited row once per query, and visited 60 to
+// one y column, lists of 2048 and 4096: 1.68 -> 0.84 ms; N = 4997, six z,
+// 1024 and 2048: 0.51 -> 0.30 ms; N = 99850, ten z, 512 and 1024: 44.3 ->
+// 8.8 ms (that kernel read every visited row once per query, and visited 60 to
 // 95 % of the tiles for its histogram).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "ksg_common.cuh"
 
@@ -365,30 +366,38 @@ struct SortPair {
     SortArgs l[2];
 };
 
-// Dynamic shared memory: the entries, then the bins' offsets.
+// Dynamic shared memory: the bins' offsets, then the entries' keys and samples
+// (before them, a copy of the offsets).
 __host__ __device__ constexpr size_t sort_smem(int buf, int bins)
 {
-    return (size_t)buf * sizeof(int2) + (size_t)(bins + 1) * sizeof(int);
+    const size_t offs = ((size_t)bins + 4) * sizeof(int), ent = (size_t)buf * sizeof(int2);
+    return offs + (ent > offs ? ent : offs);
 }
 
 // One block per (query, list): the collected entries in ascending order of
 // distance, the first `cap` of them written out.  A counting sort over bins
 // that are even in a power of the distance (a neighbourhood of dimension D
-// holds about r^D samples, so the power evens out the bins), then exchanges
-// of neighbours within the bins (one or two entries on average).  Bins of
-// more than kBigBin entries (data with many equal distances) are sorted in
-// place by the whole block first.  Bound by shared memory (LSU 88 % busy at
-// lists of 4096): N = 9995, lists of 2048 and 4096, 0.27 + 0.45 ms.
-// T threads, E entries per thread, BINS bins.
+// holds about r^D samples, so the power evens out the bins).  Where that
+// leaves a bin of more than kBigBin entries (a list without a radius, whose
+// farthest entries stretch the bins), the bins are refined once; bins that
+// are big all the same (many equal distances) are sorted in place by the
+// whole block.  The other bins hold one or two entries on average and at most
+// W + 1; their entries find their places by comparing with the W entries
+// before and after them (reads in sequence, no barrier; exchanges of
+// neighbours until nothing moves took a third more time: N = 9995, lists of
+// 2048 and 4096, 0.74 against 0.57 ms; N = 1000, lists of 512 and 999 without
+// a radius, 35 against 27 us, and 68 before bins were refined).
+// Bound by instruction issue and shared memory.  T threads, E entries per
+// thread, BINS bins.
 template <int T, int E, int BINS>
 __global__ void __launch_bounds__(T, E > 8 ? 1536 / T : 2048 / T)
     k_sort_lists(const SortPair pair)
 {
-    constexpr int kSortThreads = T, kSortWarps = T / 32;
+    constexpr int kWarps = T / 32, nb = BINS;
     extern __shared__ __align__(16) unsigned char s_raw[];
-    __shared__ int s_part[kSortWarps];
+    __shared__ int s_part[kWarps];
     __shared__ unsigned s_top;
-    __shared__ int s_big;
+    __shared__ int s_most;  // entries of the fullest bin
     const SortArgs &a = pair.l[blockIdx.y];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int qr = blockIdx.x;
@@ -399,122 +408,159 @@ __global__ void __launch_bounds__(T, E > 8 ? 1536 / T : 2048 / T)
     const int4 rm = a.raw_meta[qr];
     const int n = a.is_b ? rm.y : rm.x;
     const float radius = __int_as_float(a.is_b ? rm.w : rm.z);
-    constexpr int nb = BINS;
     const int sq = a.pow;
-    int2 *ent = reinterpret_cast<int2 *>(s_raw);
-    int *base = reinterpret_cast<int *>(s_raw + (size_t)a.buf * sizeof(int2));
-    for (int b = tid; b <= nb; b += kSortThreads) base[b] = 0;
+    int *base = reinterpret_cast<int *>(s_raw);
+    int *keys = base + nb + 4, *vals = keys + a.buf;
+    for (int b = tid; b < nb / 4; b += T) reinterpret_cast<int4 *>(base)[b] = make_int4(0, 0, 0, 0);
     if (tid == 0) {
-        s_big = 0;
+        s_most = 0;
         s_top = 0;
     }
     __syncthreads();
     float top = radius;
     if (!(radius < INFINITY)) {  // no radius: the bins span up to the largest distance
         unsigned m = 0;
-        for (int p = tid; p < n; p += kSortThreads) m = max(m, (unsigned)raw[p].y);
+        for (int p = tid; p < n; p += T) m = max(m, (unsigned)raw[p].y);
         m = __reduce_max_sync(kFull, m);
         if (lane == 0) atomicMax(&s_top, m);
         __syncthreads();
         top = __uint_as_float(s_top);
     }
     const float inv = top > 0.0f ? 1.0f / top : 0.0f, fnb = (float)nb;
+    // The entries' bins, counted.  Refined: a second round by the places that
+    // a first round's counts give them, each bin's entries spread evenly over
+    // its places; its bins are even whatever the distances' distribution.
+    // Both are non-decreasing in the distance.
+    const int *first = keys;
+    const float per_place = fnb / (float)max(n, 1);
+    auto bin_of = [&](int key, auto again) {
+        float t = __int_as_float(key) * inv;
+        if (sq >= 1) t *= t;
+        if (sq >= 2) t *= t;
+        t *= fnb;
+        int b = min(max((int)t, 0), nb - 1);
+        if constexpr (decltype(again)::value) {
+            const int s0 = first[b], s1 = first[b + 1];
+            const float at = fminf((float)s0 + fmaxf(t - (float)b, 0.0f) * (float)(s1 - s0), (float)s1);
+            b = min(max((int)(at * per_place), 0), nb - 1);
+        }
+        return b;
+    };
     // The loads of kBatch entries are in flight together (E a multiple of it).
-    constexpr int kBatch = E < 8 ? E : 8;
+    constexpr int kBatch = E < 8 ? E : (E % 8 == 0 ? 8 : 4);
+    static_assert(E % kBatch == 0, "whole batches");
     unsigned at[E];  // bin << 16 | place within the bin (buffers hold under 65536 entries)
+    auto count = [&](auto again) {
 #pragma unroll
-    for (int e0 = 0; e0 < E; e0 += kBatch) {
-        if (e0 * kSortThreads >= n) break;
-        int key[kBatch];
+        for (int e0 = 0; e0 < E; e0 += kBatch) {
+            if (e0 * T >= n) break;
+            int key[kBatch];
 #pragma unroll
-        for (int e = 0; e < kBatch; ++e) {
-            const int p = (e0 + e) * kSortThreads + tid;
-            key[e] = p < n ? raw[p].y : 0;
+            for (int e = 0; e < kBatch; ++e) {
+                const int p = (e0 + e) * T + tid;
+                key[e] = p < n ? raw[p].y : 0;
+            }
+#pragma unroll
+            for (int e = 0; e < kBatch; ++e) {
+                const int b = bin_of(key[e], again);
+                if ((e0 + e) * T + tid < n)
+                    at[e0 + e] = (unsigned)b << 16 | (unsigned)atomicAdd(&base[b], 1);
+            }
         }
-#pragma unroll
-        for (int e = 0; e < kBatch; ++e) {
-            float t = __int_as_float(key[e]) * inv;  // non-decreasing in the distance
-            if (sq >= 1) t *= t;
-            if (sq >= 2) t *= t;
-            const int b = min(max((int)(t * fnb), 0), nb - 1);
-            if ((e0 + e) * kSortThreads + tid < n)
-                at[e0 + e] = (unsigned)b << 16 | (unsigned)atomicAdd(&base[b], 1);
-        }
-    }
-    __syncthreads();
-    {  // exclusive scan of the bins' counts: a warp takes nb / kSortWarps
-       // consecutive bins, 32 at a time (a thread per run of bins would meet
-       // bank conflicts as wide as the run)
-        constexpr int kSteps = nb / kSortThreads;
-        int *mine = base + warp * kSteps * 32 + lane;
-        int ex[kSteps], run = 0;
-        bool big = false;
+        __syncthreads();
+        // exclusive scan of the bins' counts: a warp takes nb / kWarps
+        // consecutive bins, 128 at a time, four a lane
+        constexpr int kSteps = nb / (4 * T);
+        static_assert(kSteps >= 1, "four bins a thread");
+        int4 *mine = reinterpret_cast<int4 *>(base) + warp * kSteps * 32 + lane;
+        int4 ex[kSteps];
+        int run = 0, most = 0;
 #pragma unroll
         for (int b = 0; b < kSteps; ++b) {
-            const int c = mine[b * 32];
-            big |= c > kBigBin;
-            int inc = c;
+            const int4 c = mine[b * 32];
+            most = max(most, max(max(c.x, c.y), max(c.z, c.w)));
+            const int sum = c.x + c.y + c.z + c.w;
+            int inc = sum;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const int v = __shfl_up_sync(kFull, inc, o);
                 if (lane >= o) inc += v;
             }
-            ex[b] = run + inc - c;
+            const int x = run + inc - sum;
+            ex[b] = make_int4(x, x + c.x, x + c.x + c.y, x + c.x + c.y + c.z);
             run += __shfl_sync(kFull, inc, 31);
         }
-        if (lane == 0) s_part[warp] = run;
-        if (big) s_big = 1;
+        most = __reduce_max_sync(kFull, most);
+        if (lane == 0) {
+            s_part[warp] = run;
+            atomicMax(&s_most, most);
+        }
         __syncthreads();
         int before = 0;
         for (int w = 0; w < warp; ++w) before += s_part[w];
 #pragma unroll
-        for (int b = 0; b < kSteps; ++b) {
-            mine[b * 32] = before + ex[b];
-        }
+        for (int b = 0; b < kSteps; ++b)
+            mine[b * 32] = make_int4(before + ex[b].x, before + ex[b].y, before + ex[b].z, before + ex[b].w);
         if (tid == 0) base[nb] = n;
+        __syncthreads();
+    };
+    count(std::false_type{});
+    if (s_most > kBigBin) {
+        for (int b = tid; b <= nb; b += T) {  // the entries are not placed yet
+            keys[b] = base[b];
+            base[b] = 0;
+        }
+        __syncthreads();
+        if (tid == 0) s_most = 0;
+        __syncthreads();
+        count(std::true_type{});
     }
-    __syncthreads();
 #pragma unroll
     for (int e0 = 0; e0 < E; e0 += kBatch) {
-        if (e0 * kSortThreads >= n) break;
+        if (e0 * T >= n) break;
         int2 v[kBatch];
 #pragma unroll
         for (int e = 0; e < kBatch; ++e) {
-            const int p = (e0 + e) * kSortThreads + tid;
+            const int p = (e0 + e) * T + tid;
             v[e] = p < n ? raw[p] : make_int2(0, 0);
         }
 #pragma unroll
         for (int e = 0; e < kBatch; ++e)
-            if ((e0 + e) * kSortThreads + tid < n)
-                ent[base[at[e0 + e] >> 16] + (int)(at[e0 + e] & 0xffffu)] = v[e];
+            if ((e0 + e) * T + tid < n) {
+                const int p = base[at[e0 + e] >> 16] + (int)(at[e0 + e] & 0xffffu);
+                keys[p] = v[e].y;
+                vals[p] = v[e].x;
+            }
     }
     __syncthreads();
-    if (s_big) {
+    if (s_most > kBigBin) {
         // Bitonic sort (ascending-only form, so that any length works: an
         // index past the end counts as +inf and never moves) of each big bin.
         for (int b = 0; b < nb; ++b) {
             const int s0 = base[b], m = base[b + 1] - s0;
             if (m <= kBigBin) continue;
-            int2 *v = ent + s0;
             int half = 1;
             while (2 * half < m) half <<= 1;
             auto exchange = [&](int x, int y) {
                 if (y < m) {
-                    const int2 p = v[x], r = v[y];
-                    if (p.y > r.y) {
-                        v[x] = r;
-                        v[y] = p;
+                    const int p = keys[s0 + x], r = keys[s0 + y];
+                    if (p > r) {
+                        keys[s0 + x] = r;
+                        keys[s0 + y] = p;
+                        const int v = vals[s0 + x];
+                        vals[s0 + x] = vals[s0 + y];
+                        vals[s0 + y] = v;
                     }
                 }
             };
             for (int k = 2; k <= 2 * half; k <<= 1) {
-                for (int t = tid; t < half; t += kSortThreads) {
+                for (int t = tid; t < half; t += T) {
                     const int blk = t / (k / 2), w = t % (k / 2);
                     exchange(blk * k + w, blk * k + k - 1 - w);
                 }
                 __syncthreads();
                 for (int j = k / 4; j > 0; j >>= 1) {
-                    for (int t = tid; t < half; t += kSortThreads) {
+                    for (int t = tid; t < half; t += T) {
                         const int x = (t / j) * 2 * j + t % j;
                         exchange(x, x + j);
                     }
@@ -523,44 +569,35 @@ __global__ void __launch_bounds__(T, E > 8 ? 1536 / T : 2048 / T)
             }
         }
     }
-    // Entries now lie at most kBigBin places from their own: exchanges of
-    // neighbours, even and odd pairs in turn, until a round moves nothing
-    // (about as many passes as the fullest small bin has entries).  Only the
-    // places up to the first dropped entry's bin matter.
-    const int m = min(n, cap + 1 + kBigBin);
-    bool moved = true;
-    while (moved) {
-        bool mv = false;
-        for (int x = 2 * tid; x + 1 < m; x += 2 * kSortThreads) {
-            const int4 v = *reinterpret_cast<const int4 *>(&ent[x]);
-            if (v.y > v.w) {  // bit patterns of non-negative floats order like integers
-                *reinterpret_cast<int4 *>(&ent[x]) = make_int4(v.z, v.w, v.x, v.y);
-                mv = true;
-            }
+    // An entry's place: its own, less the larger ones before it, plus the
+    // smaller ones after it (bit patterns of non-negative floats order like
+    // integers; equal ones keep their order).  Entries of other bins, and of
+    // sorted ones, are on their right side already.
+    const int len = min(n, cap), w = min(s_most, kBigBin) - 1;
+    for (int p = tid; p < n; p += T) {
+        const int key = keys[p];
+        int pos = p;
+        for (int d = 1; d <= w; ++d) {
+            pos -= p >= d && keys[p - d] > key ? 1 : 0;
+            pos += p + d < n && keys[p + d] < key ? 1 : 0;
         }
-        __syncthreads();
-        for (int x = 2 * tid + 1; x + 1 < m; x += 2 * kSortThreads) {
-            const int2 v = ent[x], w = ent[x + 1];
-            if (v.y > w.y) {
-                ent[x] = w;
-                ent[x + 1] = v;
-                mv = true;
-            }
+        if (pos < cap) out[pos] = make_int2(vals[p], key);
+        if (pos == cap) {  // a cut list's radius is its first dropped distance
+            if (a.is_b)
+                a.meta[i].w = key;
+            else
+                a.meta[i].z = key;
         }
-        moved = __syncthreads_or(mv) != 0;
     }
-    const int len = min(n, cap), end = min(cap, (n + 31) & ~31);
-    for (int p = tid; p < end; p += kSortThreads)
-        out[p] = p < len ? ent[p] : make_int2(0, __float_as_int(INFINITY));
+    const int end = min(cap, (n + 31) & ~31);
+    for (int p = n + tid; p < end; p += T) out[p] = make_int2(0, __float_as_int(INFINITY));
     if (tid == 0) {
-        // a cut list's radius is its first dropped distance
-        const int r = n > cap ? ent[cap].y : __float_as_int(radius);
         if (a.is_b) {
             a.meta[i].y = len;
-            a.meta[i].w = r;
+            if (n <= cap) a.meta[i].w = __float_as_int(radius);
         } else {
             a.meta[i].x = len;
-            a.meta[i].z = r;
+            if (n <= cap) a.meta[i].z = __float_as_int(radius);
         }
     }
 }

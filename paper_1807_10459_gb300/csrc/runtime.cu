@@ -95,67 +95,55 @@ __global__ void k_psi_table(double *psi, int64_t n_max)
     }
 }
 
-// Sample rows of sh (tiled layout, see ksg_common.cuh): sorted position j
-// holds original sample order[j]; d < dzb -> z (0 beyond dz), then dyb y
-// columns (0 beyond dy), then 0 up to dsp.  Positions j >= n are +inf in
-// the dzb + dyb used columns.
-__global__ void k_pack_shared(const Col *zc, int dz, int dzb, const Col *yc, int dy, int dyb,
-                              int dsp, int64_t n, int64_t n_pad, const int32_t *order, float *sh,
-                              int *err)
+// The tiles of sh (layout in ksg_common.cuh), one block per tile: sorted
+// position j holds original sample order[j]; d < dzb -> z (0 beyond dz), then
+// dyb y columns (0 beyond dy), then 0 up to dsp.  Positions j >= n are +inf in
+// the dzb + dyb used columns.  Rows kTJ and kTJ+1: per-dimension minimum and
+// maximum over the tile's real samples.
+constexpr int kMaxDsp = 20;  // dz' <= 16 and dy <= 4 columns
+__global__ void __launch_bounds__(kTJ)
+    k_pack_tiles(const Col *zc, int dz, int dzb, const Col *yc, int dy, int dyb, int dsp, int64_t n,
+                 const int32_t *order, float *sh, int *err)
 {
-    const int64_t total = n_pad * dsp;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = idx / dsp;
-        const int d = (int)(idx - j * dsp);
-        float v = 0.0f;
-        if (j >= n) {
-            v = d < dzb + dyb ? INFINITY : 0.0f;
-        } else {
-            const int64_t t = order ? (int64_t)order[j] : j;
-            if (d < dzb) {
-                if (d < dz) v = zc[d].base[zc[d].off + t];
-            } else if (d < dzb + dyb) {
-                const int e = d - dzb;
-                if (e < dy) v = yc[e].base[yc[e].off + t];
-            }
-            if (!isfinite(v)) atomicOr(err, kErrNonFinite);
-        }
-        const int64_t tile = j / kTJ, row = j - tile * kTJ;
-        sh[(tile * kTileRows + row) * dsp + d] = v;
-    }
-}
-
-// Rows kTJ and kTJ+1 of every sh tile: per-dimension minimum and maximum over
-// the tile's real samples (one block of kTJ threads per tile).
-__global__ void __launch_bounds__(kTJ) k_tile_boxes(float *sh, int dsp, int64_t n)
-{
-    __shared__ float s_mn[kTJ / 32], s_mx[kTJ / 32];
+    __shared__ float s_mn[kMaxDsp][kTJ / 32], s_mx[kMaxDsp][kTJ / 32];
     const int64_t tile = blockIdx.x;
     const int r = threadIdx.x;
-    const bool real = tile * kTJ + r < n;
+    const int64_t j = tile * kTJ + r;
+    const bool real = j < n;
+    const int64_t t = real ? (order ? (int64_t)order[j] : j) : 0;
     float *base = sh + tile * kTileRows * dsp;
+#pragma unroll 4
     for (int d = 0; d < dsp; ++d) {
-        const float v = base[r * dsp + d];
+        const int e = d - dzb;
+        float v = 0.0f;
+        if (!real) {
+            v = d < dzb + dyb ? INFINITY : 0.0f;
+        } else if (d < dz) {
+            v = zc[d].base[zc[d].off + t];
+        } else if (e >= 0 && e < dy) {
+            v = yc[e].base[yc[e].off + t];
+        }
+        if (real && !isfinite(v)) atomicOr(err, kErrNonFinite);
+        base[r * dsp + d] = v;
         float mn = real ? v : INFINITY, mx = real ? v : -INFINITY;
         for (int off = 16; off >= 1; off >>= 1) {
             mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, off));
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
         }
         if ((r & 31) == 0) {
-            s_mn[r >> 5] = mn;
-            s_mx[r >> 5] = mx;
+            s_mn[d][r >> 5] = mn;
+            s_mx[d][r >> 5] = mx;
         }
-        __syncthreads();
-        if (r == 0) {
-            for (int w = 1; w < kTJ / 32; ++w) {
-                mn = fminf(mn, s_mn[w]);
-                mx = fmaxf(mx, s_mx[w]);
-            }
-            base[kTJ * dsp + d] = mn;
-            base[(kTJ + 1) * dsp + d] = mx;
+    }
+    __syncthreads();
+    if (r < dsp) {
+        float mn = s_mn[r][0], mx = s_mx[r][0];
+        for (int w = 1; w < kTJ / 32; ++w) {
+            mn = fminf(mn, s_mn[r][w]);
+            mx = fmaxf(mx, s_mx[r][w]);
         }
-        __syncthreads();
+        base[kTJ * dsp + r] = mn;
+        base[(kTJ + 1) * dsp + r] = mx;
     }
 }
 
@@ -338,15 +326,60 @@ static int64_t gather_blocks(int64_t n_groups, int64_t n_pad, int gb, int dxb)
     return b > 0x7fffffff ? 0 : b;
 }
 
-// cmi[job] = psi(k) + (sum over query tiles, in order) / n.
+// cmi[job] = psi(k) + (sum over query tiles) / n, a warp per job: lane l adds
+// the tiles l, l + 32, ... in order, then the lanes' sums are added pairwise.
+// (A thread per job read its row alone: 47 us for 101 jobs of 782 tiles, 124
+// for 201 of 1561.)
+constexpr int kFinalWarps = 4;
 __global__ void k_finalize(const double *partial, int n_jobs, int n_qt, const double *psi, int k,
                            int64_t n, double *cmi)
 {
-    const int job = blockIdx.x * blockDim.x + threadIdx.x;
+    const int job = blockIdx.x * kFinalWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (job >= n_jobs) return;
     double s = 0.0;
-    for (int t = 0; t < n_qt; ++t) s += partial[(int64_t)job * n_qt + t];
-    cmi[job] = psi[k] + s / (double)n;
+    for (int t = lane; t < n_qt; t += 32) s += partial[(int64_t)job * n_qt + t];
+    for (int off = 16; off >= 1; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+    if (lane == 0) cmi[job] = psi[k] + s / (double)n;
+}
+
+// Threads of the gate kernels (one block), and the threads that share a
+// surrogate's candidates in k_gate.
+constexpr int kGateThreads = 1024, kGateSlices = 8;
+
+// The row with the largest first value of est [n][row] (ties: the lowest; -1
+// if n == 0 or none exceeds -inf) and that value, by a block of kGateThreads;
+// s_part: kGateThreads doubles of shared memory.
+__device__ int largest(const double *est, int n, int row, double *s_part, double *value)
+{
+    __shared__ int s_at[kGateThreads];
+    const int tid = threadIdx.x;
+    double t = -INFINITY;
+    int at = -1;
+    for (int c = tid; c < n; c += kGateThreads) {
+        const double v = est[(int64_t)c * row];
+        if (v > t) {
+            t = v;
+            at = c;
+        }
+    }
+    s_part[tid] = t;
+    s_at[tid] = at;
+    __syncthreads();
+    for (int half = kGateThreads / 2; half >= 1; half >>= 1) {
+        if (tid < half) {
+            const double v = s_part[tid + half];
+            const int b = s_at[tid + half];
+            if (b >= 0 && (v > s_part[tid] || (v == s_part[tid] && (s_at[tid] < 0 || b < s_at[tid])))) {
+                s_part[tid] = v;
+                s_at[tid] = b;
+            }
+        }
+        __syncthreads();
+    }
+    *value = s_part[0];
+    const int best = s_at[0];
+    __syncthreads();
+    return best;
 }
 
 // Max-statistic gate.  est_a [n_cand][1 + sa]: every candidate's estimate and
@@ -358,34 +391,32 @@ __global__ void k_finalize(const double *partial, int n_jobs, int n_qt, const do
 __global__ void k_gate(const double *est_a, int n_cand, int sa, const double *est_b, int n_keep,
                        int n_surr, const int32_t *ids, double alpha, idtx_step *out)
 {
-    __shared__ double s_tobs;
-    __shared__ int s_best;
+    __shared__ double s_part[kGateThreads];
     __shared__ int s_cnt[32];
     const int tid = threadIdx.x;
     const int row_a = 1 + sa, row_b = n_surr - sa;
-    if (tid == 0) {
-        double t = -INFINITY;
-        int b = -1;
-        for (int c = 0; c < n_cand; ++c) {
-            const double v = est_a[(int64_t)c * row_a];
-            if (v > t) {
-                t = v;
-                b = c;
-            }
-        }
-        s_tobs = t;
-        s_best = b;
-    }
-    __syncthreads();
+    double s_tobs;
+    const int s_best = largest(est_a, n_cand, row_a, s_part, &s_tobs);
+    // kGateSlices threads share a surrogate's candidates
+    const int slice = tid / (kGateThreads / kGateSlices), lane_s = tid % (kGateThreads / kGateSlices);
     int cnt = 0;
-    for (int s = tid; s < n_surr; s += blockDim.x) {
+    for (int s0 = 0; s0 < n_surr; s0 += kGateThreads / kGateSlices) {
+        const int s = s0 + lane_s;
         double ts = -INFINITY;
-        if (s < sa) {
-            for (int c = 0; c < n_cand; ++c) ts = fmax(ts, est_a[(int64_t)c * row_a + 1 + s]);
-        } else {
-            for (int c = 0; c < n_keep; ++c) ts = fmax(ts, est_b[(int64_t)c * row_b + s - sa]);
+        if (s < sa && s < n_surr) {
+#pragma unroll 8
+            for (int c = slice; c < n_cand; c += kGateSlices) ts = fmax(ts, est_a[(int64_t)c * row_a + 1 + s]);
+        } else if (s < n_surr) {
+#pragma unroll 8
+            for (int c = slice; c < n_keep; c += kGateSlices) ts = fmax(ts, est_b[(int64_t)c * row_b + s - sa]);
         }
-        cnt += ts >= s_tobs ? 1 : 0;
+        __syncthreads();
+        s_part[tid] = ts;
+        __syncthreads();
+        if (slice == 0 && s < n_surr) {
+            for (int v = 1; v < kGateSlices; ++v) ts = fmax(ts, s_part[v * (kGateThreads / kGateSlices) + lane_s]);
+            cnt += ts >= s_tobs ? 1 : 0;
+        }
     }
     for (int off = 16; off >= 1; off >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, off);
     if ((tid & 31) == 0) s_cnt[tid >> 5] = cnt;
@@ -544,22 +575,14 @@ __global__ void k_seqmax_stat(const double *est, int m, int n_surr, double alpha
 __global__ void k_gate_begin(const double *est_a, int n_cand, int sa, const int32_t *ids,
                              idtx_step *out, int *count)
 {
-    __shared__ double s_tobs;
+    __shared__ double s_part[kGateThreads];
     __shared__ int s_cnt;
+    double s_tobs;
+    const int b = largest(est_a, n_cand, 1 + sa, s_part, &s_tobs);
     if (threadIdx.x == 0) {
-        double t = -INFINITY;
-        int b = -1;
-        for (int c = 0; c < n_cand; ++c) {
-            const double v = est_a[(int64_t)c * (1 + sa)];
-            if (v > t) {
-                t = v;
-                b = c;
-            }
-        }
-        s_tobs = t;
         s_cnt = 0;
         out->cand = b >= 0 ? ids[b] : -1;
-        out->stat = t;
+        out->stat = s_tobs;
         out->n_cand = n_cand;
         out->reserved = 0;
     }
@@ -632,16 +655,32 @@ __global__ void k_screen_features(const double *est, int n_cand, int s0, float l
 __global__ void k_screen_keep(const double *est, int n_cand, int s0, const float *pred,
                               float delta, int32_t *keep, int32_t *n_keep)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double t = -INFINITY;
-    for (int c = 0; c < n_cand; ++c) t = fmax(t, est[(int64_t)c * (1 + s0)]);
+    __shared__ double s_part[kGateThreads];
+    __shared__ int s_warp[kGateThreads / 32];
+    const int tid = threadIdx.x;
+    double t;
+    largest(est, n_cand, 1 + s0, s_part, &t);
     int n = 0;
-    for (int c = 0; c < n_cand; ++c) {
-        double m = -INFINITY;
-        for (int s = 0; s < s0; ++s) m = fmax(m, est[(int64_t)c * (1 + s0) + 1 + s]);
-        if (m + fmax((double)pred[c], 0.0) + (double)delta >= t) keep[n++] = c;
+    for (int c0 = 0; c0 < n_cand; c0 += kGateThreads) {
+        const int c = c0 + tid;
+        bool kept = false;
+        if (c < n_cand) {
+            double m = -INFINITY;
+            for (int s = 0; s < s0; ++s) m = fmax(m, est[(int64_t)c * (1 + s0) + 1 + s]);
+            kept = m + fmax((double)pred[c], 0.0) + (double)delta >= t;
+        }
+        const uint32_t bits = __ballot_sync(0xffffffffu, kept);
+        __syncthreads();
+        if ((tid & 31) == 0) s_warp[tid >> 5] = __popc(bits);
+        __syncthreads();
+        int before = n;
+        for (int w = 0; w < kGateThreads / 32; ++w) {
+            if (w < (tid >> 5)) before += s_warp[w];
+            n += s_warp[w];
+        }
+        if (kept) keep[before + __popc(bits & ((1u << (tid & 31)) - 1u))] = c;
     }
-    *n_keep = n;
+    if (tid == 0) *n_keep = n;
 }
 
 static int grid_for(int64_t total, int block)
@@ -692,7 +731,8 @@ struct idtx_ctx {
     double *psi = nullptr;
     int64_t psi_n = 0;
     int *d_err = nullptr;
-    int *h_err = nullptr;  // pinned
+    unsigned char *h_status = nullptr;  // pinned copy of the status area
+    unsigned long long *work = nullptr;  // this call's work counters on the device
     std::vector<KsgVariant> variants;
     // measurement counters
     bool profiling = false;
@@ -731,6 +771,18 @@ struct idtx_ctx {
     int cap_a = 0, cap_b = 0;
     long long wait_ns = 0;  // bound of device waits (0: settings->timeout_ms)
 };
+
+// The status area: the error word and, 32 ints on, the list kernel's counters
+// (zero between launches), then the work counters of up to kStatusSlots fused
+// launches.
+constexpr size_t kStatusHead = 256;
+constexpr int kStatusSlots = 64;
+constexpr size_t kStatusBytes = kStatusHead + kStatusSlots * kNumWork * sizeof(unsigned long long);
+
+unsigned long long *status_work(const idtx_ctx *c)
+{
+    return (unsigned long long *)((unsigned char *)c->d_err + kStatusHead);
+}
 
 void drop_graph(idtx_ctx *c)
 {
@@ -1168,7 +1220,7 @@ void fill_launch(const idtx_ctx *c, const Group &g, const Slices &sl, float *eps
     a.eps_out = eps_out;
     a.cnt_out = cnt_out;
     a.order = g.sort ? (const int32_t *)sl.order : nullptr;
-    a.work = (unsigned long long *)c->buf[B_WORK] + (size_t)g.work_slot * kNumWork;
+    a.work = c->work + (size_t)g.work_slot * kNumWork;
     a.err = c->d_err;
     a.next = c->d_err + 32;
     a.n = g.n;
@@ -1267,10 +1319,8 @@ int prep_group(idtx_ctx *c, const Group &g, cudaStream_t st, const Slices &sl, f
                                  nk * bits, st));
         order = ord;
     }
-    k_pack_shared<<<grid_for(g.n_pad * v.dsp, 256), 256, 0, st>>>(
-        zc, g.dz, dzb, yc, g.dy, dyb, v.dsp, g.n, g.n_pad, order, sh, c->d_err);
-    IDTX_CUDA(cudaGetLastError());
-    k_tile_boxes<<<(unsigned)(g.n_pad / kTJ), kTJ, 0, st>>>(sh, v.dsp, g.n);
+    k_pack_tiles<<<(unsigned)(g.n_pad / kTJ), kTJ, 0, st>>>(zc, g.dz, dzb, yc, g.dy, dyb, v.dsp, g.n,
+                                                            order, sh, c->d_err);
     IDTX_CUDA(cudaGetLastError());
     fill_launch(c, g, sl, eps_out, cnt_out, timeout_ns, a);
     if ((g.use_list || g.tune) && !a.list_a)
@@ -1278,9 +1328,10 @@ int prep_group(idtx_ctx *c, const Group &g, cudaStream_t st, const Slices &sl, f
     // The permutations and the X gather do not depend on the lists: with
     // lists to build they run on the context's second stream, forked from st
     // after the sample order is known and joined back before the estimator.
+    // (Without permutations there is only the gather, shorter than the fork.)
     cudaStream_t xs = st;
     cudaEvent_t fork = nullptr, join = nullptr;
-    if (a.list_a) {
+    if (a.list_a && !g.iv_a && n_slots > 0) {
         IDTX_TRY(take_event(c, &fork));
         IDTX_TRY(take_event(c, &join));
         IDTX_CUDA(cudaEventRecord(fork, st));
@@ -1322,20 +1373,21 @@ int prep_group(idtx_ctx *c, const Group &g, cudaStream_t st, const Slices &sl, f
     k_gather_x<<<(unsigned)gblocks, kGatherThreads, gather_smem(gx, v.dx), xs>>>(
         xc, g.dx, v.dx, jobs, n_jobs, perm, g.n, g.n_pad, gx, order, composed, xi, c->d_err);
     IDTX_CUDA(cudaGetLastError());
-    if (a.list_a) {
-        IDTX_CUDA(cudaEventRecord(join, xs));
+    if (fork) IDTX_CUDA(cudaEventRecord(join, xs));
+    if (a.list_a && !g.iv_a) {
         int built = 0;
-        if (!g.iv_a)
-            IDTX_CUDA(build_lists(sh, v.dz, v.dy, g.n, g.cap_a, g.cap_b,
-                                  const_cast<int2 *>(a.list_a), const_cast<int2 *>(a.list_b),
-                                  const_cast<int4 *>(a.lmeta), a.lscratch, st, &built));
+        IDTX_CUDA(build_lists(sh, v.dz, v.dy, g.n, g.cap_a, g.cap_b,
+                              const_cast<int2 *>(a.list_a), const_cast<int2 *>(a.list_b),
+                              const_cast<int4 *>(a.lmeta), a.lscratch, st, &built));
+        launches += built;
+    }
+    if (fork) {
         IDTX_CUDA(cudaStreamWaitEvent(st, join, 0));
         // a later record of these events does not disturb the waits above
         c->event_pool.push_back(fork);
         c->event_pool.push_back(join);
-        launches += built;
     }
-    launches += 5;  // pack, boxes, gather, fused, finalize
+    launches += 4;  // pack, gather, fused, finalize
     return IDTX_OK;
 }
 
@@ -1466,7 +1518,8 @@ int enqueue_group(idtx_ctx *c, const Group &g, cudaStream_t st, double *cmi, flo
         c->pending.emplace_back(ev0, ev1);
     }
     note_group(c, g, launches, use_list && !g.plain);
-    k_finalize<<<(n_jobs + 127) / 128, 128, 0, st>>>(partial, n_jobs, g.n_qt, c->psi, g.k, g.n,
+    k_finalize<<<(n_jobs + kFinalWarps - 1) / kFinalWarps, kFinalWarps * 32, 0, st>>>(
+        partial, n_jobs, g.n_qt, c->psi, g.k, g.n,
                                                       cmi);
     IDTX_CUDA(cudaGetLastError());
     return IDTX_OK;
@@ -1614,7 +1667,6 @@ int batch_enqueue(idtx_ctx *c, const std::vector<Group> &gs, const BatchPlan &bp
         const Group &g = gs[i];
         KsgLaunch a;
         IDTX_TRY(prep_group(c, g, st, bp.sl[i], nullptr, nullptr, timeout_ns, a, launches[i]));
-        a.work = (unsigned long long *)c->buf[B_WORK] + (size_t)g.work_slot * kNumWork;
         cudaEvent_t l0 = nullptr, l1 = nullptr;
         if (c->profiling) {
             IDTX_TRY(take_event(c, &l0));
@@ -1633,7 +1685,8 @@ int batch_enqueue(idtx_ctx *c, const std::vector<Group> &gs, const BatchPlan &bp
         const Group &g = gs[i];
         const int n_jobs = (int)g.jobs.size();
         note_group(c, g, launches[i], g.use_list);
-        k_finalize<<<(n_jobs + 127) / 128, 128, 0, st>>>(bp.sl[i].partial, n_jobs, g.n_qt,
+        k_finalize<<<(n_jobs + kFinalWarps - 1) / kFinalWarps, kFinalWarps * 32, 0, st>>>(
+        bp.sl[i].partial, n_jobs, g.n_qt,
                                                           c->psi, g.k, g.n, cmi + g.off_cmi);
         IDTX_CUDA(cudaGetLastError());
     }
@@ -1687,10 +1740,16 @@ struct HostCopy {
     size_t off;  // float offset in B_IN
 };
 
-// Reset the per-call work counters for n_slots fused launches.
+// Reset the error word and the per-call work counters for n_slots fused
+// launches (in the status area, one operation, where they fit).
 int begin_call(idtx_ctx *c, int n_slots, cudaStream_t st)
 {
     c->call_shapes.clear();
+    if (n_slots <= kStatusSlots) {
+        c->work = status_work(c);
+        IDTX_CUDA(cudaMemsetAsync(c->d_err, 0, kStatusHead + n_slots * kNumWork * sizeof(unsigned long long), st));
+        return IDTX_OK;
+    }
     const size_t bytes = (size_t)std::max(n_slots, 1) * kNumWork * sizeof(unsigned long long);
     IDTX_TRY(ensure(c, B_WORK, bytes));
     if (c->h_work_cap < bytes) {
@@ -1700,19 +1759,21 @@ int begin_call(idtx_ctx *c, int n_slots, cudaStream_t st)
         IDTX_CUDA(cudaMallocHost(&c->h_work, bytes));
         c->h_work_cap = bytes;
     }
+    c->work = (unsigned long long *)c->buf[B_WORK];
     IDTX_CUDA(cudaMemsetAsync(c->buf[B_WORK], 0, bytes, st));
-    IDTX_CUDA(cudaMemsetAsync(c->d_err, 0, sizeof(int), st));
+    IDTX_CUDA(cudaMemsetAsync(c->d_err, 0, kStatusHead, st));
     return IDTX_OK;
 }
 
 int finish_call(idtx_ctx *c, cudaStream_t st)
 {
-    IDTX_CUDA(cudaMemcpyAsync(c->h_err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     const size_t n_shapes = c->call_shapes.size();
-    if (n_shapes)
-        IDTX_CUDA(cudaMemcpyAsync(c->h_work, c->buf[B_WORK],
-                                  n_shapes * kNumWork * sizeof(unsigned long long),
-                                  cudaMemcpyDeviceToHost, st));
+    const size_t work_bytes = n_shapes * kNumWork * sizeof(unsigned long long);
+    const bool in_status = c->work == status_work(c);
+    IDTX_CUDA(cudaMemcpyAsync(c->h_status, c->d_err, kStatusHead + (in_status ? work_bytes : 0),
+                              cudaMemcpyDeviceToHost, st));
+    if (n_shapes && !in_status)
+        IDTX_CUDA(cudaMemcpyAsync(c->h_work, c->work, work_bytes, cudaMemcpyDeviceToHost, st));
     IDTX_CUDA(cudaStreamSynchronize(st));
     for (size_t w = 0; w < n_shapes; ++w) {
         // Algorithmic lane operations of the work the fused kernel did:
@@ -1721,7 +1782,8 @@ int finish_call(idtx_ctx *c, cudaStream_t st)
         //  count pass: per scanned pair 2dz'+1; per passing pair 2dy (Y
         //    distance) and per job 2dx+7 (X distance, three compares, three adds).
         const WorkShape &ws = c->call_shapes[w];
-        const unsigned long long *k = c->h_work + w * kNumWork;
+        const unsigned long long *k =
+            (in_status ? (const unsigned long long *)(c->h_status + kStatusHead) : c->h_work) + w * kNumWork;
         const double jobs = ws.gb * ws.job_frac;
         c->stats.exhaustive_pairs += ws.exhaustive_pairs;
         if (ws.list) {
@@ -1775,7 +1837,7 @@ int finish_call(idtx_ctx *c, cudaStream_t st)
         c->event_pool.push_back(pe.second);
     }
     c->pending.clear();
-    const int e = *c->h_err;
+    const int e = *(const int *)c->h_status;
     if (e & kErrNonFinite) return fail(IDTX_EINVAL, "input contains NaN or Inf");
     if (e & kErrTimeout) return fail(IDTX_ETIMEOUT, "a bounded device wait ran out");
     if (e) return fail(IDTX_EINTERNAL, "device error word 0x%x", e);
@@ -1828,10 +1890,9 @@ int idtx_ctx_create(idtx_ctx **out, int device)
     n += ksg_variants_d22(tmp + n);
     n += ksg_variants_generic(tmp + n);
     c->variants.assign(tmp, tmp + n);
-    // the error word, then the list kernel's two counters (zero between launches)
-    cudaError_t e = cudaMalloc(&c->d_err, 64 * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, 64 * sizeof(int));
-    if (e == cudaSuccess) e = cudaMallocHost(&c->h_err, sizeof(int));
+    cudaError_t e = cudaMalloc(&c->d_err, kStatusBytes);
+    if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, kStatusBytes);
+    if (e == cudaSuccess) e = cudaMallocHost(&c->h_status, kStatusBytes);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         idtx_ctx_destroy(c);
@@ -1921,7 +1982,7 @@ int idtx_ctx_destroy(idtx_ctx *c)
     }
     if (c->psi) cudaFree(c->psi);
     if (c->d_err) cudaFree(c->d_err);
-    if (c->h_err) cudaFreeHost(c->h_err);
+    if (c->h_status) cudaFreeHost(c->h_status);
     if (c->h_work) cudaFreeHost(c->h_work);
     delete c;
     return IDTX_OK;
@@ -2022,10 +2083,11 @@ static int cmi_ksg_impl(idtx_ctx *c, const float *x, int dx, const float *y, int
                               st));
     float *eps_d = eps_out ? (eps_dev ? eps_out : (float *)c->buf[B_EPS]) : nullptr;
     int32_t *cnt_d = counts_out ? (cnt_dev ? counts_out : (int32_t *)c->buf[B_CNT]) : nullptr;
-    double *cmi_d = (double *)c->buf[B_CMI];
+    double *cmi_d = cmi_dev ? cmi_out : (double *)c->buf[B_CMI];
     IDTX_TRY(enqueue_group(c, g, st, cmi_d, eps_d, cnt_d, timeout_of(c, s)));
-    IDTX_CUDA(cudaMemcpyAsync(cmi_out, cmi_d, (size_t)n_jobs * sizeof(double),
-                              cmi_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
+    if (!cmi_dev)
+        IDTX_CUDA(cudaMemcpyAsync(cmi_out, cmi_d, (size_t)n_jobs * sizeof(double),
+                                  cudaMemcpyDeviceToHost, st));
     if (eps_out && !eps_dev)
         IDTX_CUDA(cudaMemcpyAsync(eps_out, eps_d, (size_t)n_jobs * n * sizeof(float),
                                   cudaMemcpyDeviceToHost, st));
@@ -2178,6 +2240,8 @@ int idtx_cmi_batch(idtx_ctx *c, const idtx_problem *probs, int n_probs, int k, d
         rc = ensure(c, B_DESC, arena.size());
         if (rc == IDTX_OK) rc = ensure(c, B_CMI, total_jobs * sizeof(double));
         if (rc == IDTX_OK) rc = ensure(c, B_WORK, (size_t)n_probs * kNumWork * 8);
+        unsigned long long *const call_work = c->work;
+        c->work = (unsigned long long *)c->buf[B_WORK];  // the graph's own
         if (rc == IDTX_OK) rc = batch_plan(c, gs, st, tmo, bp);
         if (rc == IDTX_OK && cudaMemcpyAsync(c->buf[B_DESC], arena.data(), arena.size(),
                                              cudaMemcpyHostToDevice, st) != cudaSuccess)
@@ -2225,6 +2289,7 @@ int idtx_cmi_batch(idtx_ctx *c, const idtx_problem *probs, int n_probs, int k, d
         }
         if (graph) cudaGraphDestroy(graph);
         swap_buffer_sets(c);
+        c->work = call_work;
         c->call_shapes.clear();  // the graph's work counters are not read back
         if (rc != IDTX_OK) {
             drop_graph(c);
@@ -2414,7 +2479,7 @@ int mte_step_impl(idtx_ctx *c, const float *series, int n_proc, int64_t T, int t
         mlp_work_carve((float *)c->buf[B_MLP], nc, &w);
         IDTX_CUDA(mlp_round(params, w, st));
         IDTX_CUDA(mlp_forward(params, w, feats, nullptr, 0, nc, mean, scale, st));
-        k_screen_keep<<<1, 1, 0, st>>>(cmi_a, nc, s0, w.y, c->screen.delta, keep_d, nkeep_d);
+        k_screen_keep<<<1, kGateThreads, 0, st>>>(cmi_a, nc, s0, w.y, c->screen.delta, keep_d, nkeep_d);
         IDTX_CUDA(cudaGetLastError());
         c->stats.kernel_launches += 7;
         keep.resize(nc + 1);
@@ -2431,7 +2496,7 @@ int mte_step_impl(idtx_ctx *c, const float *series, int n_proc, int64_t T, int t
     };
     std::vector<Chunk> chunks;
     if (!screened) {
-        k_gate<<<1, 256, 0, st>>>(cmi_a, n_alive, s0, cmi_b, n_keep, s->n_surr, ids_d, s->alpha,
+        k_gate<<<1, kGateThreads, 0, st>>>(cmi_a, n_alive, s0, cmi_b, n_keep, s->n_surr, ids_d, s->alpha,
                                   step_d);
         IDTX_CUDA(cudaGetLastError());
         c->stats.kernel_launches += 1;
@@ -2439,7 +2504,7 @@ int mte_step_impl(idtx_ctx *c, const float *series, int n_proc, int64_t T, int t
         // Count over the cheap surrogates, then chunk after chunk of the rest
         // until the count decides "not significant" or all indices are done.
         int *count_d = (int *)((unsigned char *)ids_d + align_up((size_t)n_cand_total * 4, 16));
-        k_gate_begin<<<1, 256, 0, st>>>(cmi_a, n_alive, s0, ids_d, step_d, count_d);
+        k_gate_begin<<<1, kGateThreads, 0, st>>>(cmi_a, n_alive, s0, ids_d, step_d, count_d);
         IDTX_CUDA(cudaGetLastError());
         c->stats.kernel_launches += 1;
         int decide = 0;  // smallest count c with c / n_surr >= alpha
@@ -2484,19 +2549,24 @@ int mte_step_impl(idtx_ctx *c, const float *series, int n_proc, int64_t T, int t
     if (est_out) {
         // Rows of est_out are [1 + n_surr] per candidate id; columns the kernel
         // did not compute (screened mode, skipped candidates) are left untouched.
+        // Candidates of consecutive ids go in one copy.
         const bool dev = device_accessible(est_out);
         const cudaMemcpyKind kind = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
         const size_t row = (size_t)(1 + s->n_surr) * sizeof(double);
-        for (int a = 0; a < n_alive; ++a)
-            IDTX_CUDA(cudaMemcpyAsync((unsigned char *)est_out + (size_t)ids[a] * row,
-                                      cmi_a + (size_t)a * (1 + s0), (size_t)(1 + s0) * 8, kind,
-                                      st));
+        auto copy_rows = [&](const std::vector<int32_t> &rows, size_t col, const double *src,
+                             size_t cols) -> int {
+            for (size_t a = 0, b; a < rows.size(); a = b) {
+                for (b = a + 1; b < rows.size() && rows[b] == rows[b - 1] + 1;) ++b;
+                IDTX_CUDA(cudaMemcpy2DAsync((unsigned char *)est_out + (size_t)rows[a] * row + col * 8, row,
+                                            src + a * cols, cols * 8, cols * 8, b - a, kind, st));
+            }
+            return IDTX_OK;
+        };
+        IDTX_TRY(copy_rows(ids, 0, cmi_a, 1 + (size_t)s0));
+        std::vector<int32_t> kept;
+        for (int t = 0; t < n_keep; ++t) kept.push_back(ids[keep[t]]);
         for (const Chunk &ch : chunks)
-            for (int t = 0; t < n_keep; ++t)
-                IDTX_CUDA(cudaMemcpyAsync((unsigned char *)est_out + (size_t)ids[keep[t]] * row +
-                                              (size_t)(1 + ch.lo) * 8,
-                                          cmi_b + ch.off + (size_t)t * ch.cnt, (size_t)ch.cnt * 8,
-                                          kind, st));
+            IDTX_TRY(copy_rows(kept, 1 + (size_t)ch.lo, cmi_b + ch.off, (size_t)ch.cnt));
     }
     return finish_call(c, st);
 }
@@ -3216,9 +3286,11 @@ int idtx_bivariate_te(idtx_ctx *c, const float *series, int n_proc, int64_t T, i
         // rows of the source variables only (the target's own rows are left untouched)
         const cudaMemcpyKind ek = device_accessible(est_out) ? cudaMemcpyDeviceToDevice
                                                              : cudaMemcpyDeviceToHost;
-        for (size_t a = 0; a < ids.size(); ++a)
-            IDTX_CUDA(cudaMemcpyAsync(est_out + (size_t)ids[a] * row, est + a * row, row * 8, ek,
-                                      st));
+        for (size_t a = 0, b; a < ids.size(); a = b) {  // consecutive ids in one copy
+            for (b = a + 1; b < ids.size() && ids[b] == ids[b - 1] + 1;) ++b;
+            IDTX_CUDA(cudaMemcpyAsync(est_out + (size_t)ids[a] * row, est + a * row,
+                                      (b - a) * row * 8, ek, st));
+        }
     }
     return finish_call(c, st);
 }
@@ -3407,11 +3479,9 @@ extern "C" int idtx_cmi_ksg_noalloc(const float *x, int dx, const float *y, int 
         IDTX_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
         k_psi_table<<<grid_for(psi_n + 1, 256), 256, 0, st>>>(psi, psi_n);
         IDTX_CUDA(cudaGetLastError());
-        k_pack_shared<<<grid_for(n_pad * v->dsp, 256), 256, 0, st>>>(
+        k_pack_tiles<<<(unsigned)(n_pad / kTJ), kTJ, 0, st>>>(
             (const Col *)(base + o_z), dz, v->dz, (const Col *)(base + o_y), dy, v->dy, v->dsp, n,
-            n_pad, nullptr, sh, err);
-        IDTX_CUDA(cudaGetLastError());
-        k_tile_boxes<<<(unsigned)(n_pad / kTJ), kTJ, 0, st>>>(sh, v->dsp, n);
+            nullptr, sh, err);
         IDTX_CUDA(cudaGetLastError());
         int unused_launches = 0;
         bool composed = false;
@@ -3439,7 +3509,8 @@ extern "C" int idtx_cmi_ksg_noalloc(const float *x, int dx, const float *y, int 
         a.k = s->k;
         a.timeout_ns = timeout_of(s);
         IDTX_CUDA(v->fn(a, n_groups, st));
-        k_finalize<<<(n_jobs + 127) / 128, 128, 0, st>>>(partial, n_jobs, n_qt, psi, s->k, n,
+        k_finalize<<<(n_jobs + kFinalWarps - 1) / kFinalWarps, kFinalWarps * 32, 0, st>>>(
+        partial, n_jobs, n_qt, psi, s->k, n,
                                                           cmi_out);
         IDTX_CUDA(cudaGetLastError());
         IDTX_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, st));

@@ -101,3 +101,17 @@ def test_at_most_one_z_column(idtx, dims, n, k):
         assert np.array_equal(cnt[0], np.stack([a, b, c]))
         ref = oracle.cmi_surrogates(x, y, z if dims[2] else None, k, 1, 11)
         assert np.max(np.abs(cmi[:2] - ref)) < 1e-10
+
+
+def test_long_runs_of_equal_distances(idtx):
+    """Distances in a few far-apart values, each many hundred times: bins that
+    the second binning cannot split, cut lists that end inside one."""
+    rng = np.random.default_rng(2)
+    n = 2600
+    z = rng.choice(np.array([0.0, 1.0, 1.0 + 1e-6, 1000.0], np.float32), (2, n))
+    x, y = (rng.standard_normal((1, n)).astype(np.float32) * 1e-3 for _ in range(2))
+    for caps in ((64, 96), (0, 0)):
+        _, eps, cnt = _both(idtx, x, y, z, caps)
+        e, a, b, c = oracle.ksg_counts(x, y, z, 4)
+        assert np.array_equal(eps[0], e)
+        assert np.array_equal(cnt[0], np.stack([a, b, c]))
