@@ -22,7 +22,6 @@
 #include <cstdint>
 #include <mutex>
 
-#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 namespace idtx {
@@ -171,23 +170,29 @@ cudaError_t sort_pairs_u32(void *tmp, size_t &tmp_bytes, const uint32_t *keys_in
 cudaError_t sort_floats(void *tmp, size_t &tmp_bytes, const float *in, float *out, int n,
                         cudaStream_t stream);
 
-// Learned-screen network kernels (screen.cu).  A work area holds the batch
-// activations (B rows), the gradient and the bf16 copy of the parameters.
+// Learned-screen network kernels (screen.cu).  A work area holds a batch's
+// activations and their gradients (B rows), and a gradient of the parameters.
+// base is 16-byte aligned.
 struct MlpWork {
-    float *xn, *z1, *a1, *z2, *a2, *d2, *d1, *y, *dy, *grad;
-    __nv_bfloat16 *wbf;
+    float *a1, *a2, *d2, *d1, *xn, *y, *dy, *grad;
 };
 size_t mlp_work_floats(int B);
 void mlp_work_carve(float *base, int B, MlpWork *w);
-cudaError_t mlp_round(const float *params, MlpWork &w, cudaStream_t st);
-cudaError_t mlp_forward(const float *params, MlpWork &w, const float *feats,
-                        const int32_t *order, int64_t start, int B, const float *mean,
-                        const float *scale, cudaStream_t st);
-cudaError_t mlp_loss(MlpWork &w, const float *targets, const int32_t *order, int64_t start, int B,
-                     float dy_scale, float quantile, bool want_dy, double *loss_acc,
-                     cudaStream_t st);
-cudaError_t mlp_backward(MlpWork &w, int B, bool accumulate, cudaStream_t st);
-cudaError_t mlp_adam(float *params, const float *grad, float *m, float *v, int step, float lr,
+// Outputs y of rows start .. start + B - 1.
+cudaError_t mlp_forward(const float *params, const MlpWork &w, const float *feats, int64_t start,
+                        int B, const float *mean, const float *scale, cudaStream_t st);
+// The same for rows order[start ..] (or start ..), and the loss's gradients at
+// the layers, for mlp_grad or mlp_adam.  early: the launch before it in the
+// stream is mlp_adam's (order, feats and targets are older), whose end it need
+// not wait for to start.  mlp_adam follows mlp_rows directly.
+cudaError_t mlp_rows(const float *params, const MlpWork &w, const float *feats,
+                     const float *targets, const int32_t *order, int64_t start, int B,
+                     const float *mean, const float *scale, float dy_scale, float quantile,
+                     bool early, cudaStream_t st);
+cudaError_t mlp_loss(const MlpWork &w, const float *targets, int64_t start, int B, float quantile,
+                     double *loss_acc, cudaStream_t st);
+cudaError_t mlp_grad(const MlpWork &w, int B, cudaStream_t st);  // into w.grad
+cudaError_t mlp_adam(const MlpWork &w, int B, float *params, float *m, float *v, int step, float lr,
                      cudaStream_t st);
 
 // One-time set-up per device (kernel attributes, occupancy, SM count).

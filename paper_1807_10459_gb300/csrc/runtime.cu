@@ -2477,11 +2477,10 @@ int mte_step_impl(idtx_ctx *c, const float *series, int n_proc, int64_t T, int t
         IDTX_CUDA(cudaGetLastError());
         MlpWork w;
         mlp_work_carve((float *)c->buf[B_MLP], nc, &w);
-        IDTX_CUDA(mlp_round(params, w, st));
-        IDTX_CUDA(mlp_forward(params, w, feats, nullptr, 0, nc, mean, scale, st));
+        IDTX_CUDA(mlp_forward(params, w, feats, 0, nc, mean, scale, st));
         k_screen_keep<<<1, kGateThreads, 0, st>>>(cmi_a, nc, s0, w.y, c->screen.delta, keep_d, nkeep_d);
         IDTX_CUDA(cudaGetLastError());
-        c->stats.kernel_launches += 7;
+        c->stats.kernel_launches += 3;
         keep.resize(nc + 1);
         IDTX_CUDA(cudaMemcpyAsync(keep.data(), keep_d, (size_t)(nc + 1) * sizeof(int32_t),
                                   cudaMemcpyDeviceToHost, st));
@@ -2724,9 +2723,8 @@ extern "C" int idtx_screen_predict(idtx_ctx *c, const idtx_screen *sc, const flo
     IDTX_TRY(device_floats(feats, (size_t)n * kScreenF, rest, st, &fd));
     MlpWork w;
     mlp_work_carve((float *)c->buf[B_MLP], n, &w);
-    IDTX_CUDA(mlp_round(params, w, st));
-    IDTX_CUDA(mlp_forward(params, w, fd, nullptr, 0, n, mean, scale, st));
-    c->stats.kernel_launches += 5;
+    IDTX_CUDA(mlp_forward(params, w, fd, 0, n, mean, scale, st));
+    c->stats.kernel_launches += 1;
     IDTX_CUDA(cudaMemcpyAsync(out, w.y, (size_t)n * sizeof(float),
                               device_accessible(out) ? cudaMemcpyDeviceToDevice
                                                      : cudaMemcpyDeviceToHost,
@@ -2758,12 +2756,11 @@ extern "C" int idtx_screen_loss_grad(idtx_ctx *c, const idtx_screen *sc, const f
     IDTX_CUDA(cudaMemsetAsync(loss_d, 0, sizeof(double), st));
     MlpWork w;
     mlp_work_carve((float *)c->buf[B_MLP], n, &w);
-    IDTX_CUDA(mlp_round(params, w, st));
-    IDTX_CUDA(mlp_forward(params, w, fd, nullptr, 0, n, mean, scale, st));
-    IDTX_CUDA(mlp_loss(w, td, nullptr, 0, n, (quantile > 0.0f ? 1.0f : 2.0f) / (float)n, quantile,
-                       true, loss_d, st));
-    IDTX_CUDA(mlp_backward(w, n, false, st));
-    c->stats.kernel_launches += 11;
+    IDTX_CUDA(mlp_rows(params, w, fd, td, nullptr, 0, n, mean, scale,
+                       (quantile > 0.0f ? 1.0f : 2.0f) / (float)n, quantile, false, st));
+    IDTX_CUDA(mlp_loss(w, td, 0, n, quantile, loss_d, st));
+    IDTX_CUDA(mlp_grad(w, n, st));
+    c->stats.kernel_launches += 3;
     double lsum = 0.0;
     IDTX_CUDA(cudaMemcpyAsync(&lsum, loss_d, sizeof(double), cudaMemcpyDeviceToHost, st));
     IDTX_CUDA(cudaMemcpyAsync(grad, w.grad, (size_t)kScreenP * sizeof(float),
@@ -2788,51 +2785,68 @@ extern "C" int idtx_screen_train(idtx_ctx *c, idtx_screen *sc, const float *feat
     batch = std::min(batch, n);
     float *params, *mean, *scale, *rest;
     IDTX_TRY(upload_screen(c, sc, 0, st, &params, &mean, &scale, &rest));
-    // training area: features, targets, order, Adam moments, loss accumulator
-    const size_t tr_floats = (size_t)n * (kScreenF + 1) + (size_t)n + 2 * (size_t)kScreenP + 16;
+    // training area: features, targets, the orders of up to kOrders epochs
+    // (drawn together: a warp each), Adam moments, loss accumulator
+    constexpr int kOrders = 64;
+    constexpr int64_t kOrderRows = (int64_t)1 << 22;
+    const int n_orders =
+        (int)std::max<int64_t>(1, std::min<int64_t>({epochs, kOrders, kOrderRows / n}));
+    const size_t tr_floats = (size_t)n * (kScreenF + 1) + (size_t)n * n_orders +
+                             2 * (size_t)kScreenP + 16;
     IDTX_TRY(ensure(c, B_TRAIN, tr_floats * sizeof(float)));
     const int wb = std::max(batch, std::min(n, 4096));
     IDTX_TRY(ensure(c, B_MLP, mlp_work_floats(wb) * sizeof(float)));
     float *tr = (float *)c->buf[B_TRAIN];
     float *fbuf = tr, *tbuf = fbuf + (size_t)n * kScreenF;
-    int32_t *order = (int32_t *)(tbuf + n);
-    float *m = (float *)(order + n), *v = m + kScreenP;
+    int32_t *orders = (int32_t *)(tbuf + n);
+    float *m = (float *)(orders + (size_t)n * n_orders), *v = m + kScreenP;
     double *loss_d = (double *)(((uintptr_t)(v + kScreenP) + 7) & ~(uintptr_t)7);
     const float *fd, *td;
     IDTX_TRY(device_floats(feats, (size_t)n * kScreenF, fbuf, st, &fd));
     IDTX_TRY(device_floats(targets, (size_t)n, tbuf, st, &td));
     IDTX_CUDA(cudaMemsetAsync(m, 0, 2 * (size_t)kScreenP * sizeof(float), st));
-    IDTX_TRY(ensure(c, B_DESC, 64));
-    uint64_t *rng = (uint64_t *)c->buf[B_DESC];  // [0] stream, [1] seed of the shuffle
+    // the shuffles' streams (the epochs), then their seeds
+    std::vector<uint64_t> rng((size_t)epochs + n_orders, seed);
+    for (int ep = 0; ep < epochs; ++ep) rng[ep] = (uint64_t)ep;
+    IDTX_TRY(ensure(c, B_DESC, rng.size() * sizeof(uint64_t)));
+    uint64_t *rng_d = (uint64_t *)c->buf[B_DESC];
+    IDTX_CUDA(cudaMemcpyAsync(rng_d, rng.data(), rng.size() * sizeof(uint64_t),
+                              cudaMemcpyHostToDevice, st));
     MlpWork w;
     mlp_work_carve((float *)c->buf[B_MLP], wb, &w);
-    int step = 0;
+    int step = 0, launches = 0;
     for (int ep = 0; ep < epochs; ++ep) {
-        const uint64_t rs[2] = {(uint64_t)ep, seed};
-        IDTX_CUDA(cudaMemcpyAsync(rng, rs, sizeof(rs), cudaMemcpyHostToDevice, st));
-        k_fisher_yates<<<1, 32, 0, st>>>(order, rng, rng + 1, n);
-        IDTX_CUDA(cudaGetLastError());
+        if (ep % n_orders == 0) {
+            bool composed;
+            const int rc = enqueue_permutations(orders, rng_d + ep, rng_d + epochs,
+                                                std::min(n_orders, epochs - ep), n, nullptr, st,
+                                                launches, &composed);
+            if (rc != IDTX_OK) {
+                cudaStreamSynchronize(st);  // the copy of rng may be running
+                return rc;
+            }
+        }
+        const int32_t *order = orders + (size_t)n * (ep % n_orders);
         for (int start = 0; start < n; start += batch) {
             const int bsz = std::min(batch, n - start);
-            IDTX_CUDA(mlp_round(params, w, st));
-            IDTX_CUDA(mlp_forward(params, w, fd, order, start, bsz, mean, scale, st));
-            IDTX_CUDA(mlp_loss(w, td, order, start, bsz,
-                               (quantile > 0.0f ? 1.0f : 2.0f) / (float)bsz, quantile, true,
-                               loss_d, st));
-            IDTX_CUDA(mlp_backward(w, bsz, false, st));
-            IDTX_CUDA(mlp_adam(params, w.grad, m, v, ++step, lr, st));
-            c->stats.kernel_launches += 12;
+            IDTX_CUDA(mlp_rows(params, w, fd, td, order, start, bsz, mean, scale,
+                               (quantile > 0.0f ? 1.0f : 2.0f) / (float)bsz, quantile,
+                               start > 0 || ep % n_orders != 0, st));
+            IDTX_CUDA(mlp_adam(w, bsz, params, m, v, ++step, lr, st));
+            launches += 2;
         }
-        IDTX_CUDA(cudaStreamSynchronize(st));  // keep the host copy of rs alive
+        // a long training reports an error within some epochs
+        if (ep % kOrders == kOrders - 1) IDTX_CUDA(cudaStreamSynchronize(st));
     }
     // full-data loss of the trained parameters
     IDTX_CUDA(cudaMemsetAsync(loss_d, 0, sizeof(double), st));
-    IDTX_CUDA(mlp_round(params, w, st));
     for (int start = 0; start < n; start += wb) {
         const int bsz = std::min(wb, n - start);
-        IDTX_CUDA(mlp_forward(params, w, fd, nullptr, start, bsz, mean, scale, st));
-        IDTX_CUDA(mlp_loss(w, td, nullptr, start, bsz, 0.0f, quantile, false, loss_d, st));
+        IDTX_CUDA(mlp_forward(params, w, fd, start, bsz, mean, scale, st));
+        IDTX_CUDA(mlp_loss(w, td, start, bsz, quantile, loss_d, st));
+        launches += 2;
     }
+    c->stats.kernel_launches += launches;
     double lsum = 0.0;
     IDTX_CUDA(cudaMemcpyAsync(&lsum, loss_d, sizeof(double), cudaMemcpyDeviceToHost, st));
     IDTX_CUDA(cudaMemcpyAsync(sc->params, params, sizeof(sc->params), cudaMemcpyDeviceToHost, st));
