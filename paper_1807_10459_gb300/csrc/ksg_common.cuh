@@ -20,6 +20,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <initializer_list>
 #include <mutex>
 
 #include <cuda_runtime.h>
@@ -225,6 +226,20 @@ int ksg_variants_d11(KsgVariant *out);
 int ksg_variants_d12(KsgVariant *out);
 int ksg_variants_d21(KsgVariant *out);
 int ksg_variants_d22(KsgVariant *out);
+int ksg_variants_k7_d1(KsgVariant *out);
+int ksg_variants_k7_d2(KsgVariant *out);
 int ksg_variants_generic(KsgVariant *out);
+
+// All of them: those of one k, then those of a runtime k by what they cover,
+// the narrowest first.
+constexpr int kMaxVariants = 96;
+inline int ksg_variants(KsgVariant *out)
+{
+    int n = 0;
+    for (auto f : {ksg_variants_d11, ksg_variants_d12, ksg_variants_d21, ksg_variants_d22,
+                   ksg_variants_k7_d1, ksg_variants_k7_d2, ksg_variants_generic})
+        n += f(out + n);
+    return n;
+}
 
 }  // namespace idtx

@@ -174,7 +174,7 @@ struct ListShape {
     static constexpr int QC = S::QC;
     // 32 warps (64 registers a thread) for the small specialisations; 16
     // warps give the wide runtime-k one 128 registers.
-    static constexpr int NW = (DX > 2 || K1 > 8) ? 16 : 32;
+        static constexpr int NW = (DX > 2 || K1 > 8) ? 16 : 32;
     static constexpr int THREADS = NW * 32;
     static constexpr int RING = kListRing;
     static_assert(QC <= 64, "the term ring holds tiles of up to 64 queries");
@@ -247,7 +247,8 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
     constexpr int KH = K1 - 1;  // smallest distances kept (EXACT: exactly k)
     constexpr int kShStage = kTileRows * DSP;
     constexpr unsigned kFull = 0xffffffffu;
-    constexpr bool LOW = SPLIT && (DZ == 1 || !EXACT);  // may serve calls of at most one z column
+    // may serve calls of at most one z column: the generic one covers any dz
+    constexpr bool LOW = SPLIT && (DZ == 1 || K1 > 8);
     constexpr int TAIL_A = IDTX_LIST_TAIL_A;  // jobs left after the shared neighbour walk
     const float kInf = CUDART_INF_F;
 

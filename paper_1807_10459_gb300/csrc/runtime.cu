@@ -865,7 +865,9 @@ bool device_accessible(const void *p)
 
 const int kZBuckets[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16};
 
-const KsgVariant *pick_variant(const idtx_ctx *c, int dx, int dy, int dz, int k)
+// The specialisation for a call's dimensions and k: its own (k = 4), else the
+// first that covers them (ksg_variants has the narrow ones first).
+const KsgVariant *choose_variant(const KsgVariant *vars, int n_vars, int dx, int dy, int dz, int k)
 {
     const int dze = std::max(dz, 1);
     if (k == 4 && dx <= 2 && dy <= 2) {
@@ -875,12 +877,21 @@ const KsgVariant *pick_variant(const idtx_ctx *c, int dx, int dy, int dz, int k)
                 zb = b;
                 break;
             }
-        for (const KsgVariant &v : c->variants)
+        for (int i = 0; i < n_vars; ++i) {
+            const KsgVariant &v = vars[i];
             if (v.exact && v.k1 == 5 && v.dx == dx && v.dy == dy && v.dz == zb) return &v;
+        }
     }
-    for (const KsgVariant &v : c->variants)
+    for (int i = 0; i < n_vars; ++i) {
+        const KsgVariant &v = vars[i];
         if (!v.exact && v.dx >= dx && v.dy >= dy && v.dz >= dze && v.k1 > k) return &v;
+    }
     return nullptr;
+}
+
+const KsgVariant *pick_variant(const idtx_ctx *c, int dx, int dy, int dz, int k)
+{
+    return choose_variant(c->variants.data(), (int)c->variants.size(), dx, dy, dz, k);
 }
 
 // Host-side description of one group of jobs sharing Y and Z.
@@ -1540,11 +1551,37 @@ struct BatchPlan {
     int *next_d = nullptr;
 };
 
+// The problems of a runtime k that the tile kernel serves share the narrowest
+// specialisation that covers them all: one persistent launch, in which the
+// problems fill the device together (apart, the last tasks of each launch
+// leave it idle), for some work on padding.
+void share_variant(const idtx_ctx *c, std::vector<Group> &gs)
+{
+    auto shares = [](const Group &g) { return !g.use_list && !g.v->exact; };
+    int dx = 0, dy = 0, dz = 0, k = 0;
+    for (const Group &g : gs)
+        if (shares(g)) {
+            dx = std::max(dx, g.dx);
+            dy = std::max(dy, g.dy);
+            dz = std::max(dz, g.dz);
+            k = std::max(k, g.k);
+        }
+    if (dx == 0) return;
+    const KsgVariant *v = pick_variant(c, dx, dy, dz, k);
+    if (!v || v->exact) return;
+    for (Group &g : gs)
+        if (shares(g)) {
+            g.v = v;
+            g.n_qt = (int)(g.n_pad / v->qc);
+        }
+}
+
 // Host part of a batch: scratch, launch descriptions and task offsets, the
 // latter uploaded to the device (B_TABLE) on st.
-int batch_plan(idtx_ctx *c, const std::vector<Group> &gs, cudaStream_t st, long long timeout_ns,
+int batch_plan(idtx_ctx *c, std::vector<Group> &gs, cudaStream_t st, long long timeout_ns,
                BatchPlan &bp)
 {
+    share_variant(c, gs);
     const size_t n = gs.size();
     std::vector<CallBuffers> off(n);
     CallBuffers tot;
@@ -1882,13 +1919,8 @@ int idtx_ctx_create(idtx_ctx **out, int device)
     DeviceGuard guard(device);
     idtx_ctx *c = new idtx_ctx();
     c->device = device;
-    KsgVariant tmp[64];
-    int n = 0;
-    n += ksg_variants_d11(tmp + n);
-    n += ksg_variants_d12(tmp + n);
-    n += ksg_variants_d21(tmp + n);
-    n += ksg_variants_d22(tmp + n);
-    n += ksg_variants_generic(tmp + n);
+    KsgVariant tmp[kMaxVariants];
+    const int n = ksg_variants(tmp);
     c->variants.assign(tmp, tmp + n);
     cudaError_t e = cudaMalloc(&c->d_err, kStatusBytes);
     if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, kStatusBytes);
@@ -3351,36 +3383,11 @@ int noalloc_scratch(int device, unsigned char **out)
 
 const KsgVariant *noalloc_variant(int dx, int dy, int dz, int k)
 {
-    static KsgVariant table[64];
+    static KsgVariant table[kMaxVariants];
     static int n_table = 0;
     static std::once_flag once;
-    std::call_once(once, [] {
-        int n = 0;
-        n += ksg_variants_d11(table + n);
-        n += ksg_variants_d12(table + n);
-        n += ksg_variants_d21(table + n);
-        n += ksg_variants_d22(table + n);
-        n += ksg_variants_generic(table + n);
-        n_table = n;
-    });
-    const int dze = std::max(dz, 1);
-    if (k == 4 && dx <= 2 && dy <= 2) {
-        int zb = 0;
-        for (int b : kZBuckets)
-            if (b >= dze) {
-                zb = b;
-                break;
-            }
-        for (int i = 0; i < n_table; ++i) {
-            const KsgVariant &v = table[i];
-            if (v.exact && v.k1 == 5 && v.dx == dx && v.dy == dy && v.dz == zb) return &v;
-        }
-    }
-    for (int i = 0; i < n_table; ++i) {
-        const KsgVariant &v = table[i];
-        if (!v.exact && v.dx >= dx && v.dy >= dy && v.dz >= dze && v.k1 > k) return &v;
-    }
-    return nullptr;
+    std::call_once(once, [] { n_table = ksg_variants(table); });
+    return choose_variant(table, n_table, dx, dy, dz, k);
 }
 
 }  // namespace
