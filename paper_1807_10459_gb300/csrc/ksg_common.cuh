@@ -14,7 +14,8 @@
 //   xi   [n_groups][n_pad][GB*DX]
 //                            per-job X values, GB jobs interleaved per sample:
 //                            element (j, g, d) = X_job[d][pi_job(j)], +inf for j >= n.
-//   psi  [n_max+1] fp64      digamma at the integers 1..n_max (index 0 unused).
+//   psi  [n_max+1] int64     digamma at the integers 1..n_max (index 0 unused) in
+//                            units of 2^-kPsiBits.
 //   partial [n_jobs][n_qt] fp64  per query tile sums of the digamma terms.
 #pragma once
 
@@ -40,6 +41,19 @@ enum : int {
     kErrInternal = 4,   // an internal check failed
 };
 
+// Digamma values and their sums over a query tile are 64-bit fixed-point
+// numbers: sums without rounding, in any order, and not on the fp64 unit, which
+// does two operations a clock and SM.  A term psi(n_z + 1) - psi(n_xz + 1) -
+// psi(n_yz + 1) lies within +-15.7 for up to 2 million samples, a tile's sum
+// (64 terms) within +-1005 < 2^10, so 53 fraction bits fit; they hold the fp64
+// values exactly (those below 1/2 in magnitude, psi(2) alone, too: it is
+// psi(1) + 1).  So a tile's sum is that of the fp64 values, rounded once.
+constexpr int kPsiBits = 53;
+__host__ __device__ __forceinline__ double digamma_sum(long long s)
+{
+    return (double)s * (1.0 / (double)(1ll << kPsiBits));
+}
+
 constexpr int kTileRows = kTJ + 2;  // samples + bounding box rows
 
 // Work counters written by the fused kernel (per launch, summed over CTAs):
@@ -63,18 +77,18 @@ constexpr int kMaxListB = 4096;  // by d_Z
 
 // The list kernel's ring of per-query digamma terms (ksg_list.cuh), in global
 // scratch after the lists: per CTA, kListRing query tiles of up to 64
-// queries x 32 jobs (fp64).  The kernel runs at most kListRingCtas CTAs.
+// queries x 32 jobs (64 bits each).  The kernel runs at most kListRingCtas CTAs.
 #ifndef IDTX_LIST_RING
 #define IDTX_LIST_RING 8
 #endif
 constexpr int kListRing = IDTX_LIST_RING;
 constexpr int kListRingCtas = 192;
-constexpr size_t kListRingBytes = (size_t)kListRingCtas * kListRing * 64 * 32 * sizeof(double);
+constexpr size_t kListRingBytes = (size_t)kListRingCtas * kListRing * 64 * 32 * sizeof(long long);
 
 struct KsgLaunch {
     const float *sh;
     const float *xi;
-    const double *psi;
+    const long long *psi;
     double *partial;
     float *eps_out;      // nullable, [n_jobs][n] in original sample order
     int32_t *cnt_out;    // nullable, [n_jobs][3][n]: n_xz, n_yz, n_z, original order
@@ -90,7 +104,7 @@ struct KsgLaunch {
     const int2 *list_a;
     const int2 *list_b;
     const int4 *lmeta;
-    double *ring;  // kListRingBytes of scratch for the list kernel's term ring
+    long long *ring;  // kListRingBytes of scratch for the list kernel's term ring
     void *lscratch;  // list_scratch_bytes of scratch for build_lists
     // list kernel, n_pad <= 65536 (else null): the counts n_yz, n_z, n_xz of
     // every (group, query, job), [n_groups][n_pad][32], for sum_terms
@@ -111,15 +125,15 @@ struct KsgLaunch {
 };
 
 // The digamma terms of the list kernel's counts, summed into partial: query
-// tiles of qc queries, nws interleaved sums each (sums.cu).
-cudaError_t sum_terms(const KsgLaunch &a, int qc, int nws, int n_groups, cudaStream_t st);
+// tiles of qc queries (sums.cu).
+cudaError_t sum_terms(const KsgLaunch &a, int qc, int n_groups, cudaStream_t st);
 
 typedef cudaError_t (*KsgLaunchFn)(const KsgLaunch &, int n_groups, cudaStream_t);
 
 // One estimate of one job by the plain schedule (ksg_plain.cuh): sh the
 // group's tiles, xj the job's X values [n_pad][dx bucket], partial the job's
 // n_pad / 8 partial sums.
-typedef cudaError_t (*KsgPlainFn)(const float *sh, const float *xj, const double *psi, int64_t n,
+typedef cudaError_t (*KsgPlainFn)(const float *sh, const float *xj, const long long *psi, int64_t n,
                                   int64_t n_pad, int k, double *partial, float *eps,
                                   int32_t *cnt, cudaStream_t);
 constexpr int kPlainQueriesPerPartial = 8;

@@ -289,7 +289,7 @@ __device__ __forceinline__ bool ksg_cta(const KsgLaunch &a, const int qt, const 
     __shared__ int s_fin[ST];    // units finished of the stage's current item
     __shared__ int s_abort;
     __shared__ int s_last[ST];   // item last issued into the stage
-    __shared__ double s_red[NW][GB];
+    __shared__ long long s_red[NW][GB];
     volatile int *abort_flag = &s_abort;
 
     const int tid = threadIdx.x;
@@ -672,8 +672,8 @@ __device__ __forceinline__ bool ksg_cta(const KsgLaunch &a, const int qt, const 
     if (tid == 0)
         for (int st = 0; st < ST; ++st) mbar_inval(&s_bar[st]);
 
-    // ---------------- epilogue: self pair, outputs, digamma terms (fixed order)
-    double tsum = 0.0;
+    // ---------------- epilogue: self pair, outputs, digamma terms
+    long long tsum = 0;
     for (int m = warp; m < QC; m += NW) {
         const int64_t qi = q0 + m;
         if (qi >= a.n || !job_ok) continue;
@@ -702,10 +702,10 @@ __device__ __forceinline__ bool ksg_cta(const KsgLaunch &a, const int qt, const 
     }
     __syncthreads();
     if (tid < GB && job_ok) {
-        double s = 0.0;
+        long long s = 0;
 #pragma unroll
         for (int w = 0; w < NW; ++w) s += s_red[w][tid];
-        a.partial[static_cast<int64_t>(job) * a.n_qt + qt] = s;
+        a.partial[static_cast<int64_t>(job) * a.n_qt + qt] = digamma_sum(s);
     }
     __syncthreads();  // shared state may be reused by the CTA's next task
     return true;

@@ -242,7 +242,6 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
     using S = KsgShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>;
     using LS = ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>;
     constexpr int DS = S::DS, DSP = S::DSP, XW = S::XW, GB = S::GB, QC = S::QC;
-    constexpr int NWS = S::NW;  // interleaved sums of the tile kernel
     constexpr int NW = LS::NW, RING = LS::RING;
     constexpr int KH = K1 - 1;  // smallest distances kept (EXACT: exactly k)
     constexpr int kShStage = kTileRows * DSP;
@@ -387,7 +386,7 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
         }
         const int job = grp * GB + lane;
         const bool job_ok = job < a.n_jobs;
-        double term = 0.0;
+        long long term = 0;
 
         if (qi < a.n) {
             const float *xg = a.xi + static_cast<int64_t>(grp) * a.n_pad * XW + lane * DX;
@@ -861,11 +860,10 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
         }
 
         // ---------------- the term goes to the tile's slot; the warp that
-        // finishes the tile's last query sums it in ksg_fused_kernel's order
-        // (NWS sums over the queries m = w, w + NWS, ..., then their sum in
-        // order of w), writes the partial and frees the slot.
+        // finishes the tile's last query sums them, writes the partial and
+        // frees the slot.
         if constexpr (SPLIT) continue;
-        double *ring = a.ring + (static_cast<int64_t>(blockIdx.x) * RING + slot) * QC * 32;
+        long long *ring = a.ring + (static_cast<int64_t>(blockIdx.x) * RING + slot) * QC * 32;
         __stcg(ring + m * 32 + lane, term);
         __threadfence_block();
         __syncwarp();
@@ -875,17 +873,12 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
         if (prev == QC - 1) {
             __threadfence_block();
             const int64_t q0 = static_cast<int64_t>(qt) * QC;
-            double s = 0.0;
-#pragma unroll 1
-            for (int w = 0; w < NWS; ++w) {
-                double tsum = 0.0;
-                for (int mm = w; mm < QC; mm += NWS) {
-                    if (q0 + mm >= a.n) continue;
-                    tsum += __ldcg(ring + mm * 32 + lane);
-                }
-                s += tsum;
-            }
-            if (job_ok && qt < a.n_qt) a.partial[static_cast<int64_t>(job) * a.n_qt + qt] = s;
+            long long s = 0;
+#pragma unroll 8
+            for (int mm = 0; mm < QC; ++mm)
+                if (q0 + mm < a.n) s += __ldcg(ring + mm * 32 + lane);
+            if (job_ok && qt < a.n_qt)
+                a.partial[static_cast<int64_t>(job) * a.n_qt + qt] = digamma_sum(s);
             __syncwarp();
             if (lane == 0) {
                 sm.done[slot] = 0;
@@ -1167,7 +1160,7 @@ cudaError_t launch_ksg_list(const KsgLaunch &a, int n_groups, cudaStream_t strea
         e = launch_list_form<DX, DY, DZ, K1, EXACT, QC, NWARPS, false>(a, n_groups, stream);
     if (e == cudaSuccess && (setup || a.cz))
         e = launch_list_form<DX, DY, DZ, K1, EXACT, QC, NWARPS, true>(a, n_groups, stream);
-    if (e == cudaSuccess && !setup && a.cz) e = sum_terms(a, QC, NWARPS, n_groups, stream);
+    if (e == cudaSuccess && !setup && a.cz) e = sum_terms(a, QC, n_groups, stream);
     return e;
 }
 

@@ -28,17 +28,17 @@ constexpr int kPlainWarps = kPlainQueriesPerPartial;  // queries per CTA of the 
 // eps_i; cnt (nullable): this job's [3][n] n_xz, n_yz, n_z.
 template <int DX, int DY, int DZ, int K1, bool EXACT, int DSP>
 __global__ void __launch_bounds__(kPlainWarps * 32)
-    k_ksg_plain(const float *sh, const float *xj, int64_t n, int k, const double *psi,
+    k_ksg_plain(const float *sh, const float *xj, int64_t n, int k, const long long *psi,
                 double *partial, float *eps, int32_t *cnt)
 {
     constexpr int DS = DZ + DY;
     constexpr int KH = K1;  // the k+1 smallest including the query (EXACT: exactly)
     constexpr unsigned kFull = 0xffffffffu;
-    __shared__ double s_t[kPlainWarps];
+    __shared__ long long s_t[kPlainWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t i = blockIdx.x * static_cast<int64_t>(kPlainWarps) + warp;
     auto row = [&](int64_t j) { return sh + ((j / kTJ) * kTileRows + (j % kTJ)) * DSP; };
-    double term = 0.0;
+    long long term = 0;
     if (i < n) {
         float q[DS], xq[DX];
         const float *qr = row(i);
@@ -111,17 +111,17 @@ __global__ void __launch_bounds__(kPlainWarps * 32)
     if (lane == 0) s_t[warp] = term;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double s = 0.0;
+        long long s = 0;
 #pragma unroll
         for (int w = 0; w < kPlainWarps; ++w) s += s_t[w];
-        partial[blockIdx.x] = s;
+        partial[blockIdx.x] = digamma_sum(s);
     }
 }
 
 // One CTA per kPlainWarps queries of the n_pad (a multiple of kTJ) padded
 // ones, so that every partial of the job is written (0 past n).
 template <int DX, int DY, int DZ, int K1, bool EXACT, int QC, int NWARPS>
-cudaError_t launch_ksg_plain(const float *sh, const float *xj, const double *psi, int64_t n,
+cudaError_t launch_ksg_plain(const float *sh, const float *xj, const long long *psi, int64_t n,
                              int64_t n_pad, int k, double *partial, float *eps, int32_t *cnt,
                              cudaStream_t stream)
 {

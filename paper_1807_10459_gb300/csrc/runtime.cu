@@ -70,28 +70,32 @@ struct Job {  // one estimate: X source and permutation slot (-1: identity)
     int32_t slot;
 };
 
-// psi(n) for n in [0, n_max]: psi(0) is NaN; n < 16 by the finite harmonic sum
-// psi(n) = -gamma + sum_{m<n} 1/m; n >= 16 by the asymptotic expansion
+// -gamma + sum_{m<n} 1/m = psi(n).
+__host__ __device__ inline double psi_harmonic(int64_t n)
+{
+    double v = -0.57721566490153286060651209008240243;  // Euler's constant
+    for (int64_t m = 1; m < n; ++m) v += 1.0 / (double)m;
+    return v;
+}
+
+// psi(n) for n in [1, n_max] in units of 2^-kPsiBits (0 at n = 0): n < 16 by the
+// finite harmonic sum; n >= 16 by the asymptotic expansion
 // ln n - 1/(2n) - sum_j B_2j / (2j n^2j) (Abramowitz & Stegun 6.3.18) through
 // j = 5, whose first omitted term is below 1e-16 there.
-__global__ void k_psi_table(double *psi, int64_t n_max)
+__global__ void k_psi_table(long long *psi, int64_t n_max)
 {
-    const double kEulerGamma = 0.57721566490153286060651209008240243;
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n <= n_max;
          n += (int64_t)gridDim.x * blockDim.x) {
         double v;
-        if (n == 0) {
-            v = nan("");
-        } else if (n < 16) {
-            v = -kEulerGamma;
-            for (int64_t m = 1; m < n; ++m) v += 1.0 / (double)m;
+        if (n < 16) {
+            v = n ? psi_harmonic(n) : 0.0;
         } else {
             const double x = (double)n, r = 1.0 / x, r2 = r * r;
             v = log(x) - 0.5 * r -
                 r2 * (1.0 / 12.0 -
                       r2 * (1.0 / 120.0 - r2 * (1.0 / 252.0 - r2 * (1.0 / 240.0 - r2 / 132.0))));
         }
-        psi[n] = v;
+        psi[n] = __double2ll_rn(v * (double)(1ll << kPsiBits));
     }
 }
 
@@ -331,7 +335,7 @@ static int64_t gather_blocks(int64_t n_groups, int64_t n_pad, int gb, int dxb)
 // (A thread per job read its row alone: 47 us for 101 jobs of 782 tiles, 124
 // for 201 of 1561.)
 constexpr int kFinalWarps = 4;
-__global__ void k_finalize(const double *partial, int n_jobs, int n_qt, const double *psi, int k,
+__global__ void k_finalize(const double *partial, int n_jobs, int n_qt, double psi_k,
                            int64_t n, double *cmi)
 {
     const int job = blockIdx.x * kFinalWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -339,7 +343,7 @@ __global__ void k_finalize(const double *partial, int n_jobs, int n_qt, const do
     double s = 0.0;
     for (int t = lane; t < n_qt; t += 32) s += partial[(int64_t)job * n_qt + t];
     for (int off = 16; off >= 1; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-    if (lane == 0) cmi[job] = psi[k] + s / (double)n;
+    if (lane == 0) cmi[job] = psi_k + s / (double)n;
 }
 
 // Threads of the gate kernels (one block), and the threads that share a
@@ -728,7 +732,7 @@ struct idtx_ctx {
     int device = 0;
     void *buf[kNumBufs] = {};
     size_t cap[kNumBufs] = {};
-    double *psi = nullptr;
+    long long *psi = nullptr;
     int64_t psi_n = 0;
     int *d_err = nullptr;
     unsigned char *h_status = nullptr;  // pinned copy of the status area
@@ -844,7 +848,7 @@ int ensure_psi(idtx_ctx *c, int64_t n_max, cudaStream_t st)
     if (c->psi) cudaFree(c->psi);
     c->psi = nullptr;
     c->psi_n = 0;
-    IDTX_CUDA(cudaMalloc(&c->psi, sizeof(double) * (size_t)(want + 1)));
+    IDTX_CUDA(cudaMalloc(&c->psi, sizeof(long long) * (size_t)(want + 1)));
     k_psi_table<<<grid_for(want + 1, 256), 256, 0, st>>>(c->psi, want);
     IDTX_CUDA(cudaGetLastError());
     c->stats.kernel_launches += 1;
@@ -1259,7 +1263,7 @@ void fill_launch(const idtx_ctx *c, const Group &g, const Slices &sl, float *eps
         a.list_a = (const int2 *)sl.lists;
         a.list_b = (const int2 *)(sl.lists + oa);
         a.lmeta = (const int4 *)(sl.lists + oa + ob);
-        a.ring = (double *)(sl.lists + oa + ob + om);
+        a.ring = (long long *)(sl.lists + oa + ob + om);
         unsigned char *sp = sl.lists + list_bytes(g.n, g.cap_a, g.cap_b);
         a.lscratch = sp + count_bytes(g) + xsort_bytes(g);
         if (g.b_form == 2) a.xsort = (const float *)(sp + count_bytes(g));
@@ -1530,8 +1534,7 @@ int enqueue_group(idtx_ctx *c, const Group &g, cudaStream_t st, double *cmi, flo
     }
     note_group(c, g, launches, use_list && !g.plain);
     k_finalize<<<(n_jobs + kFinalWarps - 1) / kFinalWarps, kFinalWarps * 32, 0, st>>>(
-        partial, n_jobs, g.n_qt, c->psi, g.k, g.n,
-                                                      cmi);
+        partial, n_jobs, g.n_qt, psi_harmonic(g.k), g.n, cmi);
     IDTX_CUDA(cudaGetLastError());
     return IDTX_OK;
 }
@@ -1723,8 +1726,7 @@ int batch_enqueue(idtx_ctx *c, const std::vector<Group> &gs, const BatchPlan &bp
         const int n_jobs = (int)g.jobs.size();
         note_group(c, g, launches[i], g.use_list);
         k_finalize<<<(n_jobs + kFinalWarps - 1) / kFinalWarps, kFinalWarps * 32, 0, st>>>(
-        bp.sl[i].partial, n_jobs, g.n_qt,
-                                                          c->psi, g.k, g.n, cmi + g.off_cmi);
+            bp.sl[i].partial, n_jobs, g.n_qt, psi_harmonic(g.k), g.n, cmi + g.off_cmi);
         IDTX_CUDA(cudaGetLastError());
     }
     // One fused launch per variant instead of one per tile-kernel group.
@@ -3482,7 +3484,7 @@ extern "C" int idtx_cmi_ksg_noalloc(const float *x, int dx, const float *y, int 
     }
     if (doff > kNoAllocDescBytes) return fail(IDTX_EINTERNAL, "descriptor block overflow");
     int *err = (int *)(base + at_err);
-    double *psi = (double *)(base + at_psi);
+    long long *psi = (long long *)(base + at_psi);
     float *sh = (float *)(base + at_sh);
     float *xi = (float *)(base + at_xi);
     int32_t *perm = (int32_t *)(base + at_perm);
@@ -3531,8 +3533,7 @@ extern "C" int idtx_cmi_ksg_noalloc(const float *x, int dx, const float *y, int 
         a.timeout_ns = timeout_of(s);
         IDTX_CUDA(v->fn(a, n_groups, st));
         k_finalize<<<(n_jobs + kFinalWarps - 1) / kFinalWarps, kFinalWarps * 32, 0, st>>>(
-        partial, n_jobs, n_qt, psi, s->k, n,
-                                                          cmi_out);
+            partial, n_jobs, n_qt, psi_harmonic(s->k), n, cmi_out);
         IDTX_CUDA(cudaGetLastError());
         IDTX_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, st));
         return IDTX_OK;
