@@ -109,8 +109,10 @@ struct KsgLaunch {
     // list kernel, n_pad <= 65536 (else null): the counts n_yz, n_z, n_xz of
     // every (group, query, job), [n_groups][n_pad][32], for sum_terms
     uint16_t *cyz, *cz, *cxz;
-    // with them: (group, query, jobs) left to ksg_scan_kernel, and counters, 0
-    // between launches: the next chunk, the CTAs done, the entries of scans
+    // with them: (group, query, jobs, those without eps) left to
+    // ksg_scan_kernel, n_groups * n_pad entries filled from both ends, and
+    // counters, 0 between launches: the next chunk, the CTAs done, the entries
+    // at the front and at the back, the next one at the front
     int4 *scans;
     int *next;
     // list kernel, calls of at most one z column (else 0): iv_a: no z and one

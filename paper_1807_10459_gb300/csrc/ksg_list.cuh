@@ -194,6 +194,10 @@ struct ListShape {
     static constexpr size_t SMEM = sizeof(Smem);
 };
 
+// (query, group)s with full scans for at most this many jobs, and for more,
+// are queued apart, from the two ends of KsgLaunch::scans (ksg_scan_kernel).
+constexpr int kFewJobs = 8;
+
 // Merge four distances into the ascending h[0..4): sort them, take the four
 // smallest of both (the element-wise minimum of one and the other reversed),
 // and order that bitonic sequence.  22 minima and maxima without a branch,
@@ -774,8 +778,19 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
             uint32_t bmask = __ballot_sync(kFull, fb);
             nfb = __popc(bmask);
             if (SPLIT && bmask) {
-                if (lane == 0)
-                    a.scans[atomicAdd(a.next + 2, 1)] = make_int4(grp, qi, static_cast<int>(bmask), 0);
+                // the jobs, and those of them whose eps is not known yet
+                const uint32_t amask = __ballot_sync(kFull, fa);
+                if (lane == 0) {
+                    const bool few = __popc(bmask) <= kFewJobs;
+                    const int64_t i = atomicAdd(a.next + (few ? 2 : 3), 1);
+                    a.scans[few ? i : static_cast<int64_t>(n_groups) * a.n_pad - 1 - i] =
+                        make_int4(grp, qi, static_cast<int>(bmask), static_cast<int>(amask));
+                }
+                // eps, or a bound of it, in the place of the counts to come
+                if (fb) {
+                    nz = __float_as_int(eps) & 0xffff;
+                    nyz = static_cast<int>(__float_as_uint(eps) >> 16);
+                }
                 bmask = 0;
             }
             while (bmask) {
@@ -906,18 +921,30 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
 }
 
 // Full scans, for the (query, group)s that the split form's lists did not
-// serve (a query far from the others has long neighbourhoods for all of its
-// jobs): eps and the counts of the marked jobs over every sample.  A CTA takes
-// one (query, group) at a time, each of its warps 32 samples of every eighth tile; in a warp
-// a lane per sample finds the samples within reach, 32 at a time, and a lane
-// per job uses them, their X rows loaded sixteen at a time.  The warps share
-// each job's smallest k-th distance so far (any warp's is at least the job's
-// own) and their heaps and counts meet in shared memory.
-// A single warp of the list kernel took up to 1 ms for one such query at N =
-// 9995 with 32 jobs, and the whole GPU often waited for it; here it takes 70
-// us, bound by the latency of its loads.
+// serve: the counts of the marked jobs over every sample, and first eps where
+// it is not known yet (item.w).  A query far from the others has long
+// neighbourhoods for all of its jobs; far more often one or two jobs of a query
+// have an outlying x, so that their neighbourhoods reach past the lists: of
+// 1611 items at N = 9995, three z, lists of 512 and 1024, 96 surrogates, 1311
+// had one job and 56 more than eight.  So there are two ways:
+//   * More than kFewJobs jobs: a CTA takes one item at a time, each of its warps
+//     32 samples of every eighth tile; in a warp a lane per sample finds the
+//     samples within reach, 32 at a time, and a lane per job uses them, their X
+//     rows loaded sixteen at a time.  (A single warp of the list kernel took up
+//     to 1 ms for one such query at N = 9995 with 32 jobs; 70 us here.)
+//   * Fewer: the CTA's four quarters take one item each, a lane per sample; the
+//     jobs' x values are loaded where the subspace distance is within reach, of
+//     four segments of 32 samples at once, and the counts are votes.
+// The warps share each job's smallest k-th distance so far (any warp's is at
+// least the job's own) and their heaps and counts meet in shared memory.
+// Both are bound by the latency of their loads.  Measured, N = 9995, 101
+// estimates, against the first way for every item with eps sought afresh: two
+// z columns, lists of 512 and 1024 (10117 scanned jobs), 978 -> 147 us; three
+// z, 556 -> 98 us; 2001 estimates (99543), 9.4 -> 1.4 ms.  Scans are then so
+// much cheaper that shorter lists win: the first call 1.43 -> 0.98 ms.
 constexpr int kScanWarps = 32;
-static_assert(kScanWarps % (kTJ / 32) == 0, "whole tiles per step");
+constexpr int kScanQuarter = kScanWarps / 4;
+static_assert(kScanQuarter % (kTJ / 32) == 0, "whole tiles per step");
 
 template <int DX, int DY, int DZ, int K1, bool EXACT, int QCTA, int NWARPS>
 __global__ void __launch_bounds__(kScanWarps * 32, 1)
@@ -933,12 +960,19 @@ __global__ void __launch_bounds__(kScanWarps * 32, 1)
     __shared__ int s_cnt[3][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n = static_cast<int>(a.n), n_tiles = (n + kTJ - 1) / kTJ;
-    const int n_items = a.next[2], kk = a.k;
+    const int n_few = a.next[2], n_many = a.next[3], kk = a.k;
+    const int4 *many = a.scans + static_cast<int64_t>((a.n_jobs + GB - 1) / GB) * a.n_pad - 1;
     auto kth = [&](const float(&h)[KH]) { return EXACT ? h[KH - 1] : select_kth<KH>(h, kk - 1); };
-    for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
-        const int4 item = a.scans[it];
+    // eps of a job, or a bound of it, as the list kernel left it
+    auto left = [&](int64_t at) {
+        return static_cast<unsigned>(a.cz[at]) | static_cast<unsigned>(a.cyz[at]) << 16;
+    };
+    for (int it = blockIdx.x; it < n_many; it += gridDim.x) {
+        const int4 item = many[-it];
         const int grp = item.x, qi = item.y;
         const bool mine = (static_cast<unsigned>(item.z) >> lane) & 1u;  // this lane's job is wanted
+        const bool seek = (static_cast<unsigned>(item.w) >> lane) & 1u;  // and its eps
+        const int64_t at = (static_cast<int64_t>(grp) * a.n_pad + qi) * GB + lane;
         const float *xg = a.xi + static_cast<int64_t>(grp) * a.n_pad * XW + lane * DX;
         float xq[DX], q[DS];
 #pragma unroll
@@ -1001,7 +1035,7 @@ __global__ void __launch_bounds__(kScanWarps * 32, 1)
             }
         };
         if (warp == 0) {
-            s_th[lane] = __float_as_uint(mine ? CUDART_INF_F : 0.0f);
+            s_th[lane] = mine ? left(at) : 0u;
             s_cnt[0][lane] = s_cnt[1][lane] = s_cnt[2][lane] = 0;
         }
         __syncthreads();
@@ -1009,12 +1043,12 @@ __global__ void __launch_bounds__(kScanWarps * 32, 1)
         float h[KH];
 #pragma unroll
         for (int t = 0; t < KH; ++t) h[t] = CUDART_INF_F;
-        float th = mine ? CUDART_INF_F : 0.0f;  // other jobs do not raise the limit
+        float th = seek ? CUDART_INF_F : 0.0f;  // other jobs do not raise the limit
         // A distance equal to the shared bound may be the k-th itself, so the
         // limit is the next float above it.
-        scan(std::false_type{},
+        if (item.w) scan(std::false_type{},
              [&] {
-                 if (mine && th < __uint_as_float(th_all[lane])) atomicMin(&s_th[lane], __float_as_uint(th));
+                 if (seek && th < __uint_as_float(th_all[lane])) atomicMin(&s_th[lane], __float_as_uint(th));
                  const unsigned m = __reduce_max_sync(kFull, min(th_all[lane], __float_as_uint(th)));
                  return m < 0x7f800000u ? __uint_as_float(m + 1) : CUDART_INF_F;
              },
@@ -1031,21 +1065,23 @@ __global__ void __launch_bounds__(kScanWarps * 32, 1)
                          if (d < kth(h)) sorted_insert<KH>(h, d);
                      }
                  }
-                 if (mine) th = kth(h);
+                 if (seek) th = kth(h);
              });
+        if (item.w) {
 #pragma unroll
-        for (int t = 0; t < KH; ++t) s_heap[warp][t][lane] = h[t];
-        __syncthreads();
-        if (warp == 0) {  // the k smallest of all warps
-            for (int w = 1; w < kScanWarps; ++w)
-                for (int t = 0; t < KH; ++t) {
-                    const float d = s_heap[w][t][lane];
-                    if (!__any_sync(kFull, mine && d < kth(h))) break;
-                    if (d < kth(h)) sorted_insert<KH>(h, d);
-                }
-            s_th[lane] = __float_as_uint(mine ? kth(h) : 0.0f);
+            for (int t = 0; t < KH; ++t) s_heap[warp][t][lane] = h[t];
+            __syncthreads();
+            if (warp == 0) {  // the k smallest of all warps
+                for (int w = 1; w < kScanWarps; ++w)
+                    for (int t = 0; t < KH; ++t) {
+                        const float d = s_heap[w][t][lane];
+                        if (!__any_sync(kFull, seek && d < kth(h))) break;
+                        if (d < kth(h)) sorted_insert<KH>(h, d);
+                    }
+                if (seek) s_th[lane] = __float_as_uint(kth(h));
+            }
+            __syncthreads();
         }
-        __syncthreads();
         const float eps = __uint_as_float(s_th[lane]);
         const float lim = warp_max_nn(eps);
         int cz = 0, cyz = 0, cxz = 0;
@@ -1065,7 +1101,6 @@ __global__ void __launch_bounds__(kScanWarps * 32, 1)
         }
         __syncthreads();
         if (warp == 0 && mine) {
-            const int64_t at = (static_cast<int64_t>(grp) * a.n_pad + qi) * GB + lane;
             a.cz[at] = static_cast<uint16_t>(s_cnt[0][lane]);
             a.cyz[at] = static_cast<uint16_t>(s_cnt[1][lane]);
             a.cxz[at] = static_cast<uint16_t>(s_cnt[2][lane]);
@@ -1076,13 +1111,201 @@ __global__ void __launch_bounds__(kScanWarps * 32, 1)
         }
         __syncthreads();  // shared state is set up afresh by the next item
     }
+
+    // ---------------- items of few jobs, by quarters of the CTA
+    constexpr int V = DSP <= 4 ? 4 : (DSP <= 12 ? 2 : 1);  // segments of 32 samples at once
+    __shared__ unsigned s_bound[4][kFewJobs];  // bits of each job's bound, then of its eps
+    __shared__ int s_few[4][3][kFewJobs], s_item[4];
+    const int part = warp / kScanQuarter, pw = warp % kScanQuarter;
+    auto part_sync = [&] {
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + part), "n"(kScanQuarter * 32) : "memory");
+    };
+    while (true) {
+        if (pw == 0 && lane == 0) s_item[part] = atomicAdd(a.next + 4, 1);
+        part_sync();
+        const int it = s_item[part];
+        if (it >= n_few) break;
+        const int4 item = a.scans[it];
+        const int grp = item.x, qi = item.y, m = __popc(item.z);
+        // lane l < m serves the l-th marked job
+        uint32_t rest = static_cast<uint32_t>(item.z);
+        for (int t = 0; t < lane && t + 1 < m; ++t) rest &= rest - 1;
+        const int job = __ffs(rest) - 1;
+        const bool mine = lane < m, seek = mine && ((static_cast<uint32_t>(item.w) >> job) & 1u);
+        const uint32_t seeks = __ballot_sync(kFull, seek);
+        const int64_t at = (static_cast<int64_t>(grp) * a.n_pad + qi) * GB + job;
+        const float *xg = a.xi + static_cast<int64_t>(grp) * a.n_pad * XW;
+        float xq[DX], q[DS];
+#pragma unroll
+        for (int d = 0; d < DX; ++d) xq[d] = xg[static_cast<int64_t>(qi) * XW + job * DX + d];
+        const float *qr = a.sh + (static_cast<int64_t>(qi / kTJ) * kTileRows + qi % kTJ) * DSP;
+#pragma unroll
+        for (int d = 0; d < DS; ++d) q[d] = qr[d];
+        if (pw == 0 && mine) {
+            s_bound[part][lane] = left(at);
+            s_few[part][0][lane] = s_few[part][1][lane] = s_few[part][2][lane] = 0;
+        }
+        part_sync();
+        volatile unsigned *bound = s_bound[part];
+        // use(samples, d_Z, d_YZ) of V samples a lane (+inf: none), for the tiles
+        // whose d_YZ (ZONLY: d_Z) may be below limit()
+        auto sweep = [&](auto zonly, auto limit, auto use) {
+            constexpr bool ZONLY = decltype(zonly)::value;
+            constexpr int SEGS = kTJ / 32, STEP = kScanQuarter / SEGS;
+            const int b = pw % SEGS * 32;
+            float lim = limit();
+            for (int i0 = 0; i0 * STEP < n_tiles; i0 += 32) {
+                const int u = (i0 + lane) * STEP + pw / SEGS;
+                const int my_tile = u < n_tiles ? spiral_tile(qi / kTJ, n_tiles, u) : 0;
+                const float my_gap =
+                    u < n_tiles ? point_gap<ZONLY ? DZ : DS, DSP>(
+                                      a.sh + static_cast<int64_t>(my_tile) * kTileRows * DSP, q)
+                                : CUDART_INF_F;
+                uint32_t todo = __ballot_sync(kFull, my_gap < lim);
+                while (todo) {
+                    int j[V];
+                    float dz[V], dyz[V];
+#pragma unroll
+                    for (int v = 0; v < V; ++v) {
+                        const int t = todo ? __shfl_sync(kFull, my_tile, (__ffs(todo) - 1) & 31) : -1;
+                        todo &= todo - 1;
+                        j[v] = t * kTJ + b + lane;
+                        const bool some = t >= 0 && j[v] < n && j[v] != qi;
+                        if (!some) j[v] = qi;
+                        const float4 *row = reinterpret_cast<const float4 *>(
+                            t >= 0 ? a.sh + (static_cast<int64_t>(t) * kTileRows + b + lane) * DSP : qr);
+                        float r[DSP];
+#pragma unroll
+                        for (int c = 0; c < DSP / 4; ++c) {
+                            const float4 f = row[c];
+                            r[4 * c] = f.x;
+                            r[4 * c + 1] = f.y;
+                            r[4 * c + 2] = f.z;
+                            r[4 * c + 3] = f.w;
+                        }
+                        dz[v] = some ? fabsf(q[0] - r[0]) : CUDART_INF_F;
+#pragma unroll
+                        for (int d = 1; d < DZ; ++d) dz[v] = fmaxf(dz[v], fabsf(q[d] - r[d]));
+                        dyz[v] = dz[v];
+#pragma unroll
+                        for (int d = DZ; d < DS; ++d) dyz[v] = fmaxf(dyz[v], fabsf(q[d] - r[d]));
+                    }
+                    use(j, dz, dyz);
+                    lim = limit();
+                    todo &= __ballot_sync(kFull, my_gap < lim);
+                }
+            }
+        };
+        // d_X of the l-th job to V samples, +inf where `near` is false
+        auto x_dists = [&](int l, const int(&j)[V], const bool(&near)[V], float(&dx)[V]) {
+            const float *xj = xg + __shfl_sync(kFull, job, l) * DX;
+            float xl[DX];
+#pragma unroll
+            for (int d = 0; d < DX; ++d) xl[d] = __shfl_sync(kFull, xq[d], l);
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const float *xr = xj + static_cast<int64_t>(j[v]) * XW;
+                dx[v] = near[v] ? fabsf(xl[0] - xr[0]) : CUDART_INF_F;
+#pragma unroll
+                for (int d = 1; d < DX; ++d) dx[v] = near[v] ? fmaxf(dx[v], fabsf(xl[d] - xr[d])) : dx[v];
+            }
+        };
+        // the next float above a bound: a distance equal to it may be the k-th
+        auto above = [](unsigned bits) {
+            return __uint_as_float(bits < 0x7f800000u ? bits + 1 : 0x7f800000u);
+        };
+        if (seeks) {
+            float h[KH];  // lane l: the l-th job's smallest distances
+#pragma unroll
+            for (int t = 0; t < KH; ++t) h[t] = CUDART_INF_F;
+            sweep(std::false_type{},
+                  [&] { return above(__reduce_max_sync(kFull, seek ? bound[lane] : 0u)); },
+                  [&](const int(&j)[V], const float(&)[V], const float(&dyz)[V]) {
+                      for (uint32_t left_l = seeks; left_l; left_l &= left_l - 1) {
+                          const int l = __ffs(left_l) - 1;
+                          const unsigned was = __shfl_sync(kFull, bound[l], 0);
+                          const float lim = above(was);
+                          bool near[V];
+#pragma unroll
+                          for (int v = 0; v < V; ++v) near[v] = dyz[v] < lim;
+                          float dx[V];
+                          x_dists(l, j, near, dx);
+#pragma unroll
+                          for (int v = 0; v < V; ++v) {
+                              const float d = fmaxf(dx[v], dyz[v]);
+                              uint32_t hits = __ballot_sync(kFull, d < lim);
+                              while (hits) {
+                                  const float dh = __shfl_sync(kFull, d, __ffs(hits) - 1);
+                                  hits &= hits - 1;
+                                  if (lane == l && dh < kth(h)) sorted_insert<KH>(h, dh);
+                              }
+                          }
+                          if (lane == l && __float_as_uint(kth(h)) < was)
+                              atomicMin(&s_bound[part][l], __float_as_uint(kth(h)));
+                      }
+                  });
+#pragma unroll
+            for (int t = 0; t < KH; ++t) s_heap[warp][t][lane] = h[t];
+            part_sync();
+            if (pw == 0 && seek) {  // the k smallest of the quarter's warps
+                for (int w = 1; w < kScanQuarter; ++w)
+                    for (int t = 0; t < KH; ++t) {
+                        const float d = s_heap[warp + w][t][lane];
+                        if (!(d < kth(h))) break;
+                        sorted_insert<KH>(h, d);
+                    }
+                s_bound[part][lane] = __float_as_uint(kth(h));
+            }
+            part_sync();
+        }
+        const float eps = mine ? __uint_as_float(bound[lane]) : 0.0f;
+        const float lim = warp_max_nn(eps);
+        int cz = 0, cyz = 0, cxz = 0;
+        sweep(std::true_type{}, [&] { return lim; },
+              [&](const int(&j)[V], const float(&dz)[V], const float(&dyz)[V]) {
+                  for (int l = 0; l < m; ++l) {
+                      const float el = __shfl_sync(kFull, eps, l);
+                      bool near[V];
+#pragma unroll
+                      for (int v = 0; v < V; ++v) near[v] = dz[v] < el;
+                      float dx[V];
+                      x_dists(l, j, near, dx);
+                      int c0 = 0, c1 = 0, c2 = 0;
+#pragma unroll
+                      for (int v = 0; v < V; ++v) {
+                          c0 += __popc(__ballot_sync(kFull, near[v]));
+                          c1 += __popc(__ballot_sync(kFull, dyz[v] < el));
+                          c2 += __popc(__ballot_sync(kFull, dx[v] < el));
+                      }
+                      if (lane == l) {
+                          cz += c0;
+                          cyz += c1;
+                          cxz += c2;
+                      }
+                  }
+              });
+        if (mine) {
+            atomicAdd(&s_few[part][0][lane], cz);
+            atomicAdd(&s_few[part][1][lane], cyz);
+            atomicAdd(&s_few[part][2][lane], cxz);
+        }
+        part_sync();
+        if (pw == 0 && mine) {
+            a.cz[at] = static_cast<uint16_t>(s_few[part][0][lane]);
+            a.cyz[at] = static_cast<uint16_t>(s_few[part][1][lane]);
+            a.cxz[at] = static_cast<uint16_t>(s_few[part][2][lane]);
+            if (a.eps_out) {
+                const int64_t orig = a.order ? static_cast<int64_t>(a.order[qi]) : static_cast<int64_t>(qi);
+                a.eps_out[static_cast<int64_t>(grp * GB + job) * a.n + orig] = eps;
+            }
+        }
+    }
     // the last CTA to come here empties the queue for the next launch
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(a.next + 1, 1) == static_cast<int>(gridDim.x) - 1) {
-            a.next[1] = 0;
-            a.next[2] = 0;
+            for (int t = 1; t < 5; ++t) a.next[t] = 0;
         }
     }
 }
