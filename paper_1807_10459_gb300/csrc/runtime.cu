@@ -1439,8 +1439,11 @@ int tune_group(idtx_ctx *c, const Group &g, KsgLaunch &a, cudaStream_t st, bool 
 {
     idtx_ctx::Trial trial{g.n, g.n_groups, {{false, 0, 0, 0.0f, 0.0f}, {true, g.cap_a, g.cap_b, 0.0f, 0.0f}}};
     std::vector<idtx_ctx::Timed> &way = trial.way;
-    if (c->cap_a == 0 && c->cap_b == 0 && !g.iv_a)  // capacities not fixed by the caller
-        for (int sh = 1; sh <= 2; ++sh) {
+    // Capacities not fixed by the caller: also lists of a half, a quarter and an
+    // eighth.  Which wins depends on how many jobs reach past them: of eleven calls,
+    // steps and batches an eighth (256, 512) took up to 13 % off some.
+    if (c->cap_a == 0 && c->cap_b == 0 && !g.iv_a)
+        for (int sh = 1; sh <= 3; ++sh) {
             const int ca = (g.cap_a >> sh) / 32 * 32, cb = (g.cap_b >> sh) / 32 * 32;
             if (ca >= 256 && (cb >= 256 || g.b_form)) way.push_back({true, ca, cb, 0.0f, 0.0f});
         }
