@@ -75,16 +75,6 @@ constexpr int kNumWork = 10;
 constexpr int kMaxListA = 2048;  // by d_YZ
 constexpr int kMaxListB = 4096;  // by d_Z
 
-// The list kernel's ring of per-query digamma terms (ksg_list.cuh), in global
-// scratch after the lists: per CTA, kListRing query tiles of up to 64
-// queries x 32 jobs (64 bits each).  The kernel runs at most kListRingCtas CTAs.
-#ifndef IDTX_LIST_RING
-#define IDTX_LIST_RING 8
-#endif
-constexpr int kListRing = IDTX_LIST_RING;
-constexpr int kListRingCtas = 192;
-constexpr size_t kListRingBytes = (size_t)kListRingCtas * kListRing * 64 * 32 * sizeof(long long);
-
 struct KsgLaunch {
     const float *sh;
     const float *xi;
@@ -104,13 +94,14 @@ struct KsgLaunch {
     const int2 *list_a;
     const int2 *list_b;
     const int4 *lmeta;
-    long long *ring;  // kListRingBytes of scratch for the list kernel's term ring
     void *lscratch;  // list_scratch_bytes of scratch for build_lists
-    // list kernel, n_pad <= 65536 (else null): the counts n_yz, n_z, n_xz of
-    // every (group, query, job), [n_groups][n_pad][32], for sum_terms
-    uint16_t *cyz, *cz, *cxz;
+    // list kernel: the counts n_yz, n_z, n_xz of every (group, query, job) of
+    // count_groups groups, [count_groups][n_pad][32], 16 bits each (wide: 32, for
+    // n_pad > 65536), for sum_terms
+    void *cyz, *cz, *cxz;
+    int wide, count_groups;
     // with them: (group, query, jobs, those without eps) left to
-    // ksg_scan_kernel, n_groups * n_pad entries filled from both ends, and
+    // ksg_scan_kernel, count_groups * n_pad entries filled from both ends, and
     // counters, 0 between launches: the next chunk, the CTAs done, the entries
     // at the front and at the back, the next one at the front
     int4 *scans;
@@ -125,6 +116,18 @@ struct KsgLaunch {
     const int2 *jobs;
     int cap_a, cap_b;
 };
+
+__device__ __forceinline__ void put_count(void *c, int64_t at, int v, int wide)
+{
+    if (wide)
+        static_cast<uint32_t *>(c)[at] = (uint32_t)v;
+    else
+        static_cast<uint16_t *>(c)[at] = (uint16_t)v;
+}
+__device__ __forceinline__ int get_count(const void *c, int64_t at, int wide)
+{
+    return wide ? (int)static_cast<const uint32_t *>(c)[at] : (int)static_cast<const uint16_t *>(c)[at];
+}
 
 // The digamma terms of the list kernel's counts, summed into partial: query
 // tiles of qc queries (sums.cu).

@@ -45,18 +45,13 @@
 //     neighbour walk most finish lane-split (the 32 lanes splitting the
 //     entries), the last of the count walk with the lanes shared out among
 //     them.
-//   * Split form (n_pad <= 65536): the counts go out as 16-bit numbers and
-//     sum_terms (sums.cu) forms and sums the terms.  No order of the queries
-//     matters then, so the CTAs take chunks as they come free; (query, group)s
-//     that need full scans are queued for ksg_scan_kernel.
-//   * Otherwise the terms go through a ring of tile slots in global memory, so
-//     that they can be summed in the fixed order once a tile's queries are
-//     done, the CTAs' chunks are fixed, and full scans run in place.  A warp
-//     that takes a query of tile t waits until tile t - RING has been summed
-//     (that tile's queries were all taken earlier, so the wait always ends).
-//     Every wait is bounded by %globaltimer; on expiry the CTA records
-//     kErrTimeout and stops.
-//   * Calls of at most one z column (split form) walk an order instead of a
+//   * The counts go out (16 bits each, 32 above 65536 samples) and sum_terms
+//     (sums.cu) forms and sums the terms.  No order of the queries matters, so
+//     the CTAs take chunks as they come free; (query, group)s that need full
+//     scans are queued for ksg_scan_kernel.  Waits (for a chunk being fetched)
+//     are bounded by %globaltimer; on expiry the CTA records kErrTimeout and
+//     stops.
+//   * Calls of at most one z column (n_pad <= 65536) walk an order instead of a
 //     list where the subspace has one dimension: with one z column the samples
 //     are ordered by it, and the samples after and before the query, whose d_Z
 //     ascends, are list B (up to thousands of entries there, beyond any list's
@@ -66,9 +61,10 @@
 //     kernel, 0.35; N = 20000: 30.1 and 1.7; one z, N = 3001: 0.95 (lists) and
 //     0.57; N = 50000, 101 estimates: 33.1 (tile) and 22.6.
 // Measured on GB300, greedy step of N = 9995 with 9447 estimates (one network;
-// lists of 2048 and 4096): 19.1 -> 13.2 ms with sum_terms; of N = 4997, six
-// conditions, 28341 estimates: 10.8 -> 9.7 ms; N = 1000, 101 estimates: 163 ->
-// 70 us.  Bound by issue (58 % of the slots) and the latency behind it: fewer,
+// lists of 2048 and 4096), against summing the terms in the kernel and scanning
+// in place: 19.1 -> 12.7 ms; of N = 4997, six conditions, 28341 estimates: 10.8
+// -> 8.5 ms; N = 1000, 101 estimates: 163 -> 24 us (each with sum_terms' 0.30,
+// 0.51 ms and 4 us to add).  Bound by issue (58 % of the slots) and the latency behind it: fewer,
 // fatter warps (24 of 80 registers) were 8 % slower.
 #pragma once
 
@@ -103,13 +99,7 @@
 #ifndef IDTX_LIST_GSB
 #define IDTX_LIST_GSB 16
 #endif
-// The form with the ring: most consecutive query tiles a CTA takes at a time
-// (fewer when the call has too few tiles to give every SM two chunks; the
-// ring's depth, kListRing, is in ksg_common.cuh).  The split form: queries
-// (256 to 1024 are alike).
-#ifndef IDTX_LIST_CHUNK
-#define IDTX_LIST_CHUNK 8
-#endif
+// Most consecutive queries a CTA takes at a time (256 to 1024 are alike).
 #ifndef IDTX_LIST_CHUNKQ
 #define IDTX_LIST_CHUNKQ 256
 #endif
@@ -165,9 +155,9 @@ __device__ __forceinline__ float warp_max_nn(float v)
     return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
 }
 
-// Launch shape of the list kernel for one specialisation.  QC, NWS: the tile
-// kernel's queries per CTA and interleaved sums, which fix the partial-sum
-// layout (one partial per QC queries) and the order of the sums.
+// Launch shape of the list kernel for one specialisation.  QC: the tile
+// kernel's queries per CTA, which fix the partial-sum layout (one partial per QC
+// queries).
 template <int DX, int DY, int DZ, int K1, bool EXACT, int QCTA, int NWARPS>
 struct ListShape {
     using S = KsgShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>;
@@ -176,17 +166,13 @@ struct ListShape {
     // warps give the wide runtime-k one 128 registers.
         static constexpr int NW = (DX > 2 || K1 > 8) ? 16 : 32;
     static constexpr int THREADS = NW * 32;
-    static constexpr int RING = kListRing;
-    static_assert(QC <= 64, "the term ring holds tiles of up to 64 queries");
+    static_assert(QC <= 64, "sum_terms takes tiles of up to 64 queries");
     struct Smem {
         int2 ent[NW][64];  // per warp: two chunks of staged list entries
         unsigned long long work[NW][kNumWork];
-        int owner[RING];  // the CTA-local tile number a slot currently serves
-        int done[RING];   // queries of that tile finished
-        int next;         // next CTA-local query position
-        // split form: the CTA's chunks in their order (number, chunk; a ring),
-        // the next query (number << 16 | query within the chunk), and the
-        // chunk to follow (-1: being fetched)
+        // the CTA's chunks in their order (number, chunk; a ring), the next query
+        // (number << 16 | query within the chunk), and the chunk to follow (-1:
+        // being fetched)
         int2 chunk[8];
         unsigned cur;
         int ahead;
@@ -226,32 +212,19 @@ __device__ __forceinline__ void merge4(float (&h)[4], float s0, float s1, float 
     cmp_swap(h[2], h[3]);
 }
 
-// Wait until *owner == want (tile slot free), bounded by timeout_ns.
-__device__ __forceinline__ bool wait_slot(const int *owner, int want, long long timeout_ns)
-{
-    const volatile int *o = owner;
-    if (*o == want) return true;
-    const long long t0 = global_ns();
-    while (*o != want) {
-        if (global_ns() - t0 > timeout_ns) return false;
-        __nanosleep(32);
-    }
-    return true;
-}
-
-template <int DX, int DY, int DZ, int K1, bool EXACT, int QCTA, int NWARPS, bool SPLIT>
+template <int DX, int DY, int DZ, int K1, bool EXACT, int QCTA, int NWARPS>
 __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>::THREADS, 1)
     ksg_list_kernel(const KsgLaunch a, const int n_groups, const int n_chunks, const int chunk_q)
 {
     using S = KsgShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>;
     using LS = ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>;
-    constexpr int DS = S::DS, DSP = S::DSP, XW = S::XW, GB = S::GB, QC = S::QC;
-    constexpr int NW = LS::NW, RING = LS::RING;
+    constexpr int DSP = S::DSP, XW = S::XW, GB = S::GB;
+    constexpr int NW = LS::NW;
     constexpr int KH = K1 - 1;  // smallest distances kept (EXACT: exactly k)
     constexpr int kShStage = kTileRows * DSP;
     constexpr unsigned kFull = 0xffffffffu;
     // may serve calls of at most one z column: the generic one covers any dz
-    constexpr bool LOW = SPLIT && (DZ == 1 || K1 > 8);
+    constexpr bool LOW = DZ == 1 || K1 > 8;
     constexpr int TAIL_A = IDTX_LIST_TAIL_A;  // jobs left after the shared neighbour walk
     const float kInf = CUDART_INF_F;
 
@@ -260,17 +233,10 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
-    if (tid < RING) {
-        sm.owner[tid] = tid;
-        sm.done[tid] = 0;
-    }
     if (tid == 0) {
-        sm.next = 0;
-        if (SPLIT) {
-            sm.cur = 0;
-            sm.chunk[0] = make_int2(0, atomicAdd(a.next, 1));
-            sm.ahead = atomicAdd(a.next, 1);
-        }
+        sm.cur = 0;
+        sm.chunk[0] = make_int2(0, atomicAdd(a.next, 1));
+        sm.ahead = atomicAdd(a.next, 1);
     }
     __syncthreads();
 
@@ -281,7 +247,7 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
     auto sh_row = [&](int64_t j) { return a.sh + (j / kTJ) * kShStage + (j % kTJ) * DSP; };
     const long long t_begin = clock64();
     unsigned long long my_work = 0;   // work counter `lane` of this warp (5: cycles)
-    int grp = 0, qt = 0, num_of = -1, q_of = 0;  // the last query's group, tile or chunk
+    int grp = 0, num_of = -1, q_of = 0;  // the last query's group and chunk
 
     while (true) {
         // ---------------- take the CTA's next query.  Chunks of consecutive
@@ -289,95 +255,57 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
         // by query block within a super-block, so the CTAs in flight share a
         // few groups' X rows and a range of queries' lists in L2, while each
         // CTA's warps serve consecutive queries of one group.
-        int slot = 0, lt = 0, m = 0;
-        int qi;  // the query (sorted position)
-        if constexpr (SPLIT) {
-            // Chunks of `chunk_q` queries, taken by the CTAs as they come free
-            // (the queries' work differs).  The warp that takes the first
-            // query past a chunk brings in the one fetched ahead; others that
-            // come before it has try again.
-            unsigned v = 0;
-            if (lane == 0) v = atomicAdd(&sm.cur, 1u);
-            v = __shfl_sync(kFull, v, 0);
-            const int num = static_cast<int>(v >> 16), at = static_cast<int>(v & 0xffffu);
-            if (at >= chunk_q) {
-                int ok = 1;
-                if (lane == 0) {
-                    const long long t0 = global_ns();
-                    if (at == chunk_q) {
-                        volatile int *ahead = &sm.ahead;
-                        while (ok && *ahead < 0) {
-                            __nanosleep(32);
-                            ok = global_ns() - t0 <= a.timeout_ns;
-                        }
-                        if (ok) {
-                            const int next = *ahead;
-                            *ahead = -1;
-                            sm.chunk[(num + 1) & 7] = make_int2((num + 1) & 0xffff, next);
-                            __threadfence_block();
-                            atomicExch(&sm.cur, static_cast<unsigned>(num + 1) << 16);
-                            *ahead = next < n_chunks ? atomicAdd(a.next, 1) : next;
-                        }
-                    } else {
-                        const volatile unsigned *cur = &sm.cur;
-                        while (ok && (*cur >> 16) == (v >> 16)) {
-                            __nanosleep(32);
-                            ok = global_ns() - t0 <= a.timeout_ns;
-                        }
+        // Chunks of `chunk_q` queries, taken by the CTAs as they come free
+        // (the queries' work differs).  The warp that takes the first
+        // query past a chunk brings in the one fetched ahead; others that
+        // come before it has try again.
+        unsigned v = 0;
+        if (lane == 0) v = atomicAdd(&sm.cur, 1u);
+        v = __shfl_sync(kFull, v, 0);
+        const int num = static_cast<int>(v >> 16), at = static_cast<int>(v & 0xffffu);
+        if (at >= chunk_q) {
+            int ok = 1;
+            if (lane == 0) {
+                const long long t0 = global_ns();
+                if (at == chunk_q) {
+                    volatile int *ahead = &sm.ahead;
+                    while (ok && *ahead < 0) {
+                        __nanosleep(32);
+                        ok = global_ns() - t0 <= a.timeout_ns;
+                    }
+                    if (ok) {
+                        const int next = *ahead;
+                        *ahead = -1;
+                        sm.chunk[(num + 1) & 7] = make_int2((num + 1) & 0xffff, next);
+                        __threadfence_block();
+                        atomicExch(&sm.cur, static_cast<unsigned>(num + 1) << 16);
+                        *ahead = next < n_chunks ? atomicAdd(a.next, 1) : next;
+                    }
+                } else {
+                    const volatile unsigned *cur = &sm.cur;
+                    while (ok && (*cur >> 16) == (v >> 16)) {
+                        __nanosleep(32);
+                        ok = global_ns() - t0 <= a.timeout_ns;
                     }
                 }
-                if (!__shfl_sync(kFull, ok, 0)) {
-                    if (lane == 0) atomicOr(a.err, kErrTimeout);
-                    break;
-                }
-                continue;
             }
-            if (num != num_of) {
-                num_of = num;
-                __threadfence_block();
-                const int2 mine = sm.chunk[num & 7];
-                if (mine.x != num) {  // overtaken by seven chunks: cannot be, and is not passed over
-                    if (lane == 0) atomicOr(a.err, kErrInternal);
-                    break;
-                }
-                const int chunk = mine.y;
-                if (chunk >= n_chunks) break;
-                const int n_qb = (static_cast<int>(a.n) + chunk_q - 1) / chunk_q;
-                const int per_sb = IDTX_LIST_GSB * n_qb;
-                const int sb = chunk / per_sb;
-                const int g0 = sb * IDTX_LIST_GSB;
-                const int gs = n_groups - g0 < IDTX_LIST_GSB ? n_groups - g0 : IDTX_LIST_GSB;
-                const int rc = chunk - sb * per_sb;
-                const int qblock = rc / gs;
-                grp = g0 + (rc - qblock * gs);
-                q_of = qblock * chunk_q;
-            }
-            qi = q_of + at;
-        } else {
-            // The ring sums the tiles in their order, so the CTA's stream is
-            // fixed: tile lt of it is tile lt mod 2^chunk_lg of chunk
-            // blockIdx.x + (lt >> chunk_lg) * gridDim.x; tiles past a group's
-            // last one (its last block may be short) are claimed as empty.
-            int p = 0;
-            if (lane == 0) p = atomicAdd(&sm.next, 1);
-            p = __shfl_sync(kFull, p, 0);
-            lt = p / QC;
-            m = p - lt * QC;
-            const int chunk_lg = chunk_q;
-            const int chunk =
-                static_cast<int>(blockIdx.x) + (lt >> chunk_lg) * static_cast<int>(gridDim.x);
-            if (chunk >= n_chunks) break;
-            slot = lt % RING;
-            int ok = 1;
-            if (lane == 0) ok = wait_slot(&sm.owner[slot], lt, a.timeout_ns) ? 1 : 0;
-            ok = __shfl_sync(kFull, ok, 0);
-            if (!ok) {
+            if (!__shfl_sync(kFull, ok, 0)) {
                 if (lane == 0) atomicOr(a.err, kErrTimeout);
                 break;
             }
+            continue;
+        }
+        if (num != num_of) {
+            num_of = num;
             __threadfence_block();
-            // (32-bit: n_chunks, the chunk count, fits an int; see the launcher)
-            const int n_qb = (a.n_qt + (1 << chunk_lg) - 1) >> chunk_lg;
+            const int2 mine = sm.chunk[num & 7];
+            if (mine.x != num) {  // overtaken by seven chunks: cannot be, and is not passed over
+                if (lane == 0) atomicOr(a.err, kErrInternal);
+                break;
+            }
+            const int chunk = mine.y;
+            if (chunk >= n_chunks) break;
+            const int n_qb = (static_cast<int>(a.n) + chunk_q - 1) / chunk_q;
             const int per_sb = IDTX_LIST_GSB * n_qb;
             const int sb = chunk / per_sb;
             const int g0 = sb * IDTX_LIST_GSB;
@@ -385,12 +313,11 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
             const int rc = chunk - sb * per_sb;
             const int qblock = rc / gs;
             grp = g0 + (rc - qblock * gs);
-            qt = (qblock << chunk_lg) + (lt & ((1 << chunk_lg) - 1));
-            qi = qt * QC + m;  // >= n_pad past the last tile
+            q_of = qblock * chunk_q;
         }
+        const int qi = q_of + at;  // the query (sorted position)
         const int job = grp * GB + lane;
         const bool job_ok = job < a.n_jobs;
-        long long term = 0;
 
         if (qi < a.n) {
             const float *xg = a.xi + static_cast<int64_t>(grp) * a.n_pad * XW + lane * DX;
@@ -427,20 +354,6 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
             } else {
                 la = Src{a.list_a + static_cast<int64_t>(qi) * a.cap_a, __ldg(&a.lmeta[qi].x), 0, 0};
             }
-
-            auto x_dist = [&](int j) {
-                const float *xr = xg + static_cast<int64_t>(j) * XW;
-                float dx = fabsf(xq[0] - xr[0]);
-#pragma unroll
-                for (int d = 1; d < DX; ++d) dx = fmaxf(dx, fabsf(xq[d] - xr[d]));
-                return dx;
-            };
-            // the query's shared coordinates (full-scan fallbacks only)
-            auto load_q = [&](float(&qc)[DS]) {
-                const float *qr = sh_row(qi);
-#pragma unroll
-                for (int d = 0; d < DS; ++d) qc[d] = qr[d];
-            };
 
             // ---------------- pass A: the k smallest joint distances
             float h[KH];
@@ -595,63 +508,17 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
                 walk_total += walked_a;
             }
             walked_a = walk_total;
-            // The list ran out before the job's k-th distance dropped to r_A:
-            // the job is recomputed over every sample, in the split form by
-            // ksg_scan_kernel, else here: the 32 lanes split the samples of
-            // one such job at a time, keep their own k smallest, and the warp
-            // merges them (repeatedly taking the smallest head).
+            // The list ran out before the job's k-th distance dropped to r_A: eps
+            // is sought over every sample (ksg_scan_kernel).
             const float r_a = iv_a ? kInf : __int_as_float(__ldg(&a.lmeta[qi].z));
             const bool fa = job_ok && th > r_a;
-            float eps_fix = 0.0f;
-            uint32_t fmask = __ballot_sync(kFull, fa);
-            nfa = __popc(fmask);
-            if (SPLIT) fmask = 0;
-            while (fmask) {
-                float qc[DS];
-                load_q(qc);
-                const int f = __ffs(fmask) - 1;
-                fmask &= fmask - 1;
-                float xf[DX];
-#pragma unroll
-                for (int d = 0; d < DX; ++d) xf[d] = __shfl_sync(kFull, xq[d], f);
-                const float *xgf = xg - lane * DX + f * DX;
-                float hl[KH];
-#pragma unroll
-                for (int t = 0; t < KH; ++t) hl[t] = kInf;
-                float thl = kInf;
-                for (int64_t j = lane; j < a.n; j += 32) {
-                    const float *row = sh_row(j);
-                    float dyz = fabsf(qc[0] - row[0]);
-#pragma unroll
-                    for (int d = 1; d < DS; ++d) dyz = fmaxf(dyz, fabsf(qc[d] - row[d]));
-                    const float *xr = xgf + j * XW;
-                    float dx = fabsf(xf[0] - xr[0]);
-#pragma unroll
-                    for (int d = 1; d < DX; ++d) dx = fmaxf(dx, fabsf(xf[d] - xr[d]));
-                    const float dd = fmaxf(dx, dyz);
-                    if (dd < thl && j != qi) {
-                        sorted_insert<KH>(hl, dd);
-                        thl = kth(hl);
-                    }
-                }
-                float kv = kInf;
-                for (int t = 0; t < kk; ++t) {
-                    kv = warp_min_nn(hl[0]);
-                    const uint32_t who = __ballot_sync(kFull, hl[0] == kv);
-                    if (lane == __ffs(who) - 1) {
-#pragma unroll
-                        for (int mm = 0; mm + 1 < KH; ++mm) hl[mm] = hl[mm + 1];
-                        hl[KH - 1] = kInf;
-                    }
-                }
-                if (lane == f) eps_fix = kv;
-            }
-            const float eps = job_ok ? (!SPLIT && fa ? eps_fix : kth(h)) : -1.0f;
+            nfa = __popc(__ballot_sync(kFull, fa));
+            const float eps = job_ok ? kth(h) : -1.0f;
 
             // ---------------- pass B: strict-radius counts
             const int b_form = LOW ? a.b_form : 0;
             const float r_b = b_form ? kInf : __int_as_float(__ldg(&a.lmeta[qi].w));
-            const bool fb = job_ok && (eps > r_a || eps > r_b || (SPLIT && fa));
+            const bool fb = fa || (job_ok && (eps > r_a || eps > r_b));
             int nz = 0, nyz = 0, nxz = 0;
             // Every list A entry below eps lies in the walked prefix (the walk
             // went on until each job's k-th value was at most the next entry).
@@ -772,12 +639,10 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
                     rem = still;
                 }
             }
-            // Jobs whose eps reaches past a list: counts by a full scan, in
-            // the split form by ksg_scan_kernel, else here, the 32 lanes
-            // splitting the samples of one such job at a time.
-            uint32_t bmask = __ballot_sync(kFull, fb);
+            // Jobs whose eps reaches past a list are left to ksg_scan_kernel.
+            const uint32_t bmask = __ballot_sync(kFull, fb);
             nfb = __popc(bmask);
-            if (SPLIT && bmask) {
+            if (bmask) {
                 // the jobs, and those of them whose eps is not known yet
                 const uint32_t amask = __ballot_sync(kFull, fa);
                 if (lane == 0) {
@@ -788,117 +653,30 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
                 }
                 // eps, or a bound of it, in the place of the counts to come
                 if (fb) {
-                    nz = __float_as_int(eps) & 0xffff;
+                    nz = __float_as_int(eps);
                     nyz = static_cast<int>(__float_as_uint(eps) >> 16);
                 }
-                bmask = 0;
             }
-            while (bmask) {
-                float qc[DS];
-                load_q(qc);
-                const int f = __ffs(bmask) - 1;
-                bmask &= bmask - 1;
-                float xf[DX];
-#pragma unroll
-                for (int d = 0; d < DX; ++d) xf[d] = __shfl_sync(kFull, xq[d], f);
-                const float ef = __shfl_sync(kFull, eps, f);
-                const float *xgf = xg - lane * DX + f * DX;
-                int cz = 0, cyz = 0, cxz = 0;
-                for (int64_t j = lane; j < a.n; j += 32) {
-                    const float *row = sh_row(j);
-                    float dz = fabsf(qc[0] - row[0]);
-#pragma unroll
-                    for (int d = 1; d < DZ; ++d) dz = fmaxf(dz, fabsf(qc[d] - row[d]));
-                    float dyz = dz;
-#pragma unroll
-                    for (int d = DZ; d < DS; ++d) dyz = fmaxf(dyz, fabsf(qc[d] - row[d]));
-                    const float *xr = xgf + j * XW;
-                    float dx = fabsf(xf[0] - xr[0]);
-#pragma unroll
-                    for (int d = 1; d < DX; ++d) dx = fmaxf(dx, fabsf(xf[d] - xr[d]));
-                    const bool self = j == qi;
-                    const bool pz = dz < ef && !self;
-                    cz += pz ? 1 : 0;
-                    cyz += (dyz < ef && !self) ? 1 : 0;
-                    cxz += (pz && dx < ef) ? 1 : 0;
-                }
-                cz = __reduce_add_sync(kFull, cz);
-                cyz = __reduce_add_sync(kFull, cyz);
-                cxz = __reduce_add_sync(kFull, cxz);
-                if (lane == f) {
-                    nz = cz;
-                    nyz = cyz;
-                    nxz = cxz;
-                }
-            }
-            if constexpr (SPLIT) {
-                const int64_t at = (static_cast<int64_t>(grp) * a.n_pad + qi) * GB + lane;
-                a.cyz[at] = static_cast<uint16_t>(nyz);
-                a.cz[at] = static_cast<uint16_t>(nz);
-                a.cxz[at] = static_cast<uint16_t>(nxz);
-            } else if (job_ok) {
-                term = a.psi[nz + 1] - a.psi[nxz + 1] - a.psi[nyz + 1];
-            }
-            if (job_ok) {
+            const int64_t at = (static_cast<int64_t>(grp) * a.n_pad + qi) * GB + lane;
+            put_count(a.cyz, at, nyz, a.wide);
+            put_count(a.cz, at, nz, a.wide);
+            put_count(a.cxz, at, nxz, a.wide);
+            if (a.eps_out && job_ok && !fb) {
                 const int64_t orig = a.order ? static_cast<int64_t>(a.order[qi]) : static_cast<int64_t>(qi);
-                if (a.eps_out && !(SPLIT && fb)) a.eps_out[static_cast<int64_t>(job) * a.n + orig] = eps;
-                if (!SPLIT && a.cnt_out) {
-                    int32_t *co = a.cnt_out + static_cast<int64_t>(job) * 3 * a.n;
-                    co[orig] = nxz;
-                    co[a.n + orig] = nyz;
-                    co[2 * a.n + orig] = nz;
-                }
+                a.eps_out[static_cast<int64_t>(job) * a.n + orig] = eps;
             }
             if (a.work) {
                 // lane k keeps counter k: no read-modify-write per query
-                unsigned snz = 0, snyz = 0;  // (the split form's are summed by sum_terms)
-                if (!SPLIT) {
-                    snz = __reduce_add_sync(kFull, static_cast<unsigned>(job_ok ? nz : 0));
-                    snyz = __reduce_add_sync(kFull, static_cast<unsigned>(job_ok ? nyz : 0));
-                }
+                // (sum_terms has the sums of n_z and n_yz)
                 unsigned v = static_cast<unsigned>(walked_a);
                 v = lane == 1 ? static_cast<unsigned>(walked_b) : v;
                 v = lane == 6 ? tb : v;
                 v = lane == 7 ? ta : v;
-                if (!SPLIT) {
-                    v = lane == 8 ? snz : v;
-                    v = lane == 9 ? snyz : v;
-                    my_work += lane < 2 || lane >= 6 ? v : 0u;
-                } else {
-                    my_work += lane < 2 || lane == 6 || lane == 7 ? v : 0u;
-                }
+                my_work += lane < 2 || lane == 6 || lane == 7 ? v : 0u;
                 if (nfa | nfb) {
                     const unsigned long long n1 = static_cast<unsigned long long>(a.n - 1);
                     my_work += lane == 2 ? nfa * n1 : (lane == 3 ? nfb * n1 : (lane == 4 ? nfa + nfb : 0ull));
                 }
-            }
-        }
-
-        // ---------------- the term goes to the tile's slot; the warp that
-        // finishes the tile's last query sums them, writes the partial and
-        // frees the slot.
-        if constexpr (SPLIT) continue;
-        long long *ring = a.ring + (static_cast<int64_t>(blockIdx.x) * RING + slot) * QC * 32;
-        __stcg(ring + m * 32 + lane, term);
-        __threadfence_block();
-        __syncwarp();
-        int prev = 0;
-        if (lane == 0) prev = atomicAdd(&sm.done[slot], 1);
-        prev = __shfl_sync(kFull, prev, 0);
-        if (prev == QC - 1) {
-            __threadfence_block();
-            const int64_t q0 = static_cast<int64_t>(qt) * QC;
-            long long s = 0;
-#pragma unroll 8
-            for (int mm = 0; mm < QC; ++mm)
-                if (q0 + mm < a.n) s += __ldcg(ring + mm * 32 + lane);
-            if (job_ok && qt < a.n_qt)
-                a.partial[static_cast<int64_t>(job) * a.n_qt + qt] = digamma_sum(s);
-            __syncwarp();
-            if (lane == 0) {
-                sm.done[slot] = 0;
-                __threadfence_block();
-                *reinterpret_cast<volatile int *>(&sm.owner[slot]) = lt + RING;
             }
         }
     }
@@ -906,7 +684,7 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
     if (lane == 5) my_work = static_cast<unsigned long long>(clock64() - t_begin);
     if (lane < kNumWork) sm.work[warp][lane] = my_work;
     __syncthreads();
-    if (SPLIT && tid == 0) {  // the last CTA to come here resets the counters for the next launch
+    if (tid == 0) {  // the last CTA to come here resets the counters for the next launch
         __threadfence();
         if (atomicAdd(a.next + 1, 1) == static_cast<int>(gridDim.x) - 1) {
             a.next[0] = 0;
@@ -920,9 +698,9 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
     }
 }
 
-// Full scans, for the (query, group)s that the split form's lists did not
-// serve: the counts of the marked jobs over every sample, and first eps where
-// it is not known yet (item.w).  A query far from the others has long
+// Full scans, for the (query, group)s that the lists did not serve: the counts
+// of the marked jobs over every sample, and first eps where it is not known yet
+// (item.w).  A query far from the others has long
 // neighbourhoods for all of its jobs; far more often one or two jobs of a query
 // have an outlying x, so that their neighbourhoods reach past the lists: of
 // 1611 items at N = 9995, three z, lists of 512 and 1024, 96 surrogates, 1311
@@ -965,7 +743,8 @@ __global__ void __launch_bounds__(kScanWarps * 32, 1)
     auto kth = [&](const float(&h)[KH]) { return EXACT ? h[KH - 1] : select_kth<KH>(h, kk - 1); };
     // eps of a job, or a bound of it, as the list kernel left it
     auto left = [&](int64_t at) {
-        return static_cast<unsigned>(a.cz[at]) | static_cast<unsigned>(a.cyz[at]) << 16;
+        const unsigned v = static_cast<unsigned>(get_count(a.cz, at, a.wide));
+        return a.wide ? v : v | static_cast<unsigned>(get_count(a.cyz, at, 0)) << 16;
     };
     for (int it = blockIdx.x; it < n_many; it += gridDim.x) {
         const int4 item = many[-it];
@@ -1101,9 +880,9 @@ __global__ void __launch_bounds__(kScanWarps * 32, 1)
         }
         __syncthreads();
         if (warp == 0 && mine) {
-            a.cz[at] = static_cast<uint16_t>(s_cnt[0][lane]);
-            a.cyz[at] = static_cast<uint16_t>(s_cnt[1][lane]);
-            a.cxz[at] = static_cast<uint16_t>(s_cnt[2][lane]);
+            put_count(a.cz, at, s_cnt[0][lane], a.wide);
+            put_count(a.cyz, at, s_cnt[1][lane], a.wide);
+            put_count(a.cxz, at, s_cnt[2][lane], a.wide);
             if (a.eps_out) {
                 const int64_t orig = a.order ? static_cast<int64_t>(a.order[qi]) : static_cast<int64_t>(qi);
                 a.eps_out[static_cast<int64_t>(grp * GB + lane) * a.n + orig] = eps;
@@ -1291,9 +1070,9 @@ __global__ void __launch_bounds__(kScanWarps * 32, 1)
         }
         part_sync();
         if (pw == 0 && mine) {
-            a.cz[at] = static_cast<uint16_t>(s_few[part][0][lane]);
-            a.cyz[at] = static_cast<uint16_t>(s_few[part][1][lane]);
-            a.cxz[at] = static_cast<uint16_t>(s_few[part][2][lane]);
+            put_count(a.cz, at, s_few[part][0][lane], a.wide);
+            put_count(a.cyz, at, s_few[part][1][lane], a.wide);
+            put_count(a.cxz, at, s_few[part][2][lane], a.wide);
             if (a.eps_out) {
                 const int64_t orig = a.order ? static_cast<int64_t>(a.order[qi]) : static_cast<int64_t>(qi);
                 a.eps_out[static_cast<int64_t>(grp * GB + job) * a.n + orig] = eps;
@@ -1310,11 +1089,17 @@ __global__ void __launch_bounds__(kScanWarps * 32, 1)
     }
 }
 
-template <int DX, int DY, int DZ, int K1, bool EXACT, int QC, int NWARPS, bool SPLIT>
-cudaError_t launch_list_form(const KsgLaunch &a, int n_groups, cudaStream_t stream)
+// The estimates of n_groups groups, as many at a time as the count buffers
+// hold: the list kernel, the scans it left, the sums.  n_qt * n_groups <= 0
+// only sets up.
+template <int DX, int DY, int DZ, int K1, bool EXACT, int QC, int NWARPS>
+cudaError_t launch_ksg_list(const KsgLaunch &all, int n_groups, cudaStream_t stream)
 {
     using LS = ListShape<DX, DY, DZ, K1, EXACT, QC, NWARPS>;
-    auto kern = ksg_list_kernel<DX, DY, DZ, K1, EXACT, QC, NWARPS, SPLIT>;
+    using S = typename LS::S;
+    auto kern = ksg_list_kernel<DX, DY, DZ, K1, EXACT, QC, NWARPS>;
+    auto scan = ksg_scan_kernel<DX, DY, DZ, K1, EXACT, QC, NWARPS>;
+    constexpr size_t kScanSmem = kScanWarps * (K1 - 1) * 32 * sizeof(float);
     // Per device: the dynamic shared memory, a carveout that leaves the rest
     // of the SM's memory to L1, and the SM count (one CTA per SM).
     static DeviceOnce setup;
@@ -1332,59 +1117,40 @@ cudaError_t launch_list_form(const KsgLaunch &a, int n_groups, cudaStream_t stre
             }
         }
         if (r == cudaSuccess) r = cudaDeviceGetAttribute(&n_sms[d], cudaDevAttrMultiProcessorCount, d);
-        if (SPLIT && r == cudaSuccess)
-            r = cudaFuncSetAttribute(ksg_scan_kernel<DX, DY, DZ, K1, EXACT, QC, NWARPS>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(kScanWarps * (K1 - 1) * 32 * sizeof(float)));
+        if (r == cudaSuccess)
+            r = cudaFuncSetAttribute(scan, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     static_cast<int>(kScanSmem));
         return r;
     });
-    if (e != cudaSuccess) return e;
-    const int64_t tiles = static_cast<int64_t>(a.n_qt) * n_groups;
-    if (tiles <= 0) return cudaSuccess;  // set-up only
+    if (e != cudaSuccess || static_cast<int64_t>(all.n_qt) * n_groups <= 0) return e;
     int dev = 0;
     e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    int chunk = 0;
-    int64_t chunks = 0;
-    if (SPLIT) {
+    if (all.count_groups < 1) return cudaErrorInvalidValue;
+    for (int g0 = 0; g0 < n_groups; g0 += all.count_groups) {
+        const int groups = n_groups - g0 < all.count_groups ? n_groups - g0 : all.count_groups;
+        const int64_t j0 = static_cast<int64_t>(g0) * S::GB;
+        KsgLaunch a = all;
+        a.n_jobs = static_cast<int>(all.n_jobs - j0 < groups * S::GB ? all.n_jobs - j0 : groups * S::GB);
+        a.xi += g0 * all.n_pad * S::XW;
+        a.partial += j0 * all.n_qt;
+        if (a.eps_out) a.eps_out += j0 * all.n;
+        if (a.cnt_out) a.cnt_out += j0 * 3 * all.n;
+        if (a.jobs) a.jobs += j0;
         // chunks of consecutive queries: eight per SM where that leaves 16 queries
-        const int64_t per = a.n * n_groups / (8 * n_sms[dev]);
-        chunk = per > IDTX_LIST_CHUNKQ ? IDTX_LIST_CHUNKQ : (per < 16 ? 16 : static_cast<int>(per));
-        chunks = static_cast<int64_t>(n_groups) * ((a.n + chunk - 1) / chunk);
-    } else {
-        // blocks of 2^chunk query tiles (a group's last one may be short): the
-        // largest (up to IDTX_LIST_CHUNK) giving every SM two
-        while ((2 << chunk) <= IDTX_LIST_CHUNK && (tiles >> (chunk + 1)) >= 2 * n_sms[dev]) ++chunk;
-        chunks = static_cast<int64_t>(n_groups) * ((a.n_qt + (1 << chunk) - 1) >> chunk);
-    }
-    if (chunks > 0x3fffffff) return cudaErrorInvalidValue;  // the kernel's chunk arithmetic is 32-bit
-    int64_t grid = chunks < n_sms[dev] ? chunks : n_sms[dev];
-    if (!SPLIT && grid > kListRingCtas) grid = kListRingCtas;
-    kern<<<static_cast<unsigned>(grid), LS::THREADS, LS::SMEM, stream>>>(
-        a, n_groups, static_cast<int>(chunks), chunk);
-    if (SPLIT) {
+        const int64_t per = a.n * groups / (8 * n_sms[dev]);
+        const int chunk = per > IDTX_LIST_CHUNKQ ? IDTX_LIST_CHUNKQ : (per < 16 ? 16 : static_cast<int>(per));
+        const int64_t chunks = groups * ((a.n + chunk - 1) / chunk);
+        if (chunks > 0x3fffffff) return cudaErrorInvalidValue;  // the kernel's chunk arithmetic is 32-bit
+        const int64_t grid = chunks < n_sms[dev] ? chunks : n_sms[dev];
+        kern<<<static_cast<unsigned>(grid), LS::THREADS, LS::SMEM, stream>>>(
+            a, groups, static_cast<int>(chunks), chunk);
+        scan<<<static_cast<unsigned>(n_sms[dev]), kScanWarps * 32, kScanSmem, stream>>>(a);
         e = cudaGetLastError();
+        if (e == cudaSuccess) e = sum_terms(a, QC, groups, stream);
         if (e != cudaSuccess) return e;
-        ksg_scan_kernel<DX, DY, DZ, K1, EXACT, QC, NWARPS>
-            <<<static_cast<unsigned>(n_sms[dev]), kScanWarps * 32, kScanWarps * (K1 - 1) * 32 * sizeof(float),
-               stream>>>(a);
     }
-    return cudaGetLastError();
-}
-
-// The split form (counts out, terms summed by sum_terms) where the counts fit
-// in 16 bits and the launch so has their buffer, else the one with the ring.
-template <int DX, int DY, int DZ, int K1, bool EXACT, int QC, int NWARPS>
-cudaError_t launch_ksg_list(const KsgLaunch &a, int n_groups, cudaStream_t stream)
-{
-    cudaError_t e = cudaSuccess;
-    const bool setup = static_cast<int64_t>(a.n_qt) * n_groups <= 0;  // of both forms
-    if (setup || !a.cz)
-        e = launch_list_form<DX, DY, DZ, K1, EXACT, QC, NWARPS, false>(a, n_groups, stream);
-    if (e == cudaSuccess && (setup || a.cz))
-        e = launch_list_form<DX, DY, DZ, K1, EXACT, QC, NWARPS, true>(a, n_groups, stream);
-    if (e == cudaSuccess && !setup && a.cz) e = sum_terms(a, QC, n_groups, stream);
-    return e;
+    return cudaSuccess;
 }
 
 // One compiled specialisation: the tile kernel (ksg_kernel.cuh), its

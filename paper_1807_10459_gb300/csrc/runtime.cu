@@ -1067,24 +1067,35 @@ struct CallBuffers {
     size_t sh = 0, xi = 0, perm = 0, partial = 0, order = 0, sort_tmp = 0, lists = 0;
 };
 
-// B_LIST layout for n queries: list_a [n][cap_a] | list_b [n][cap_b] | meta [n]
-// | the list kernel's term ring, all counted here | its counts
+// B_LIST layout for n queries: list_a [n][cap_a] | list_b [n][cap_b] | meta
+// [n], all counted here | the list kernel's counts and its queue
 // | the sorted columns of a call without z | build_lists' scratch.
 size_t list_bytes(int64_t n, int cap_a, int cap_b)
 {
     return align_up((size_t)n * cap_a * sizeof(int2), 256) +
            align_up((size_t)n * cap_b * sizeof(int2), 256) +
-           align_up((size_t)n * sizeof(int4), 256) + kListRingBytes;
+           align_up((size_t)n * sizeof(int4), 256);
 }
 
-// The list kernel's counts, part of B_LIST: three 16-bit ones per (group,
-// query, job) where they fit in 16 bits (else the kernel sums by its ring),
-// and its queue of (group, query)s to scan.
-size_t count_rows(const Group &g) { return g.n_pad <= 65536 ? (size_t)g.n_groups * g.n_pad * 32 : 0; }
-size_t count_bytes(const Group &g)
+// The list kernel's counts, part of B_LIST: three per (group, query, job), of
+// 16 bits where they fit, and its queue of (group, query)s to scan, of as many
+// groups as kCountBudget holds (the others take their turn).
+constexpr size_t kCountBudget = size_t(1) << 30;
+bool wide_counts(const Group &g) { return g.n_pad > 65536; }
+size_t count_rows(const Group &g)  // of one group
 {
-    return align_up(count_rows(g) * 3 * sizeof(uint16_t) + count_rows(g) / 32 * sizeof(int4), 256);
+    return (size_t)g.n_pad * 32;
 }
+size_t group_count_bytes(const Group &g)
+{
+    return count_rows(g) * 3 * (wide_counts(g) ? sizeof(uint32_t) : sizeof(uint16_t)) +
+           (size_t)g.n_pad * sizeof(int4);
+}
+int count_groups(const Group &g)
+{
+    return (int)std::min<size_t>(g.n_groups, std::max<size_t>(1, kCountBudget / group_count_bytes(g)));
+}
+size_t count_bytes(const Group &g) { return align_up(count_groups(g) * group_count_bytes(g), 256); }
 
 // The sorted source columns of a call without z, part of B_LIST.
 size_t xsort_bytes(const Group &g)
@@ -1247,9 +1258,9 @@ void fill_launch(const idtx_ctx *c, const Group &g, const Slices &sl, float *eps
     a.list_a = nullptr;
     a.list_b = nullptr;
     a.lmeta = nullptr;
-    a.ring = nullptr;
     a.lscratch = nullptr;
     a.cyz = a.cz = a.cxz = nullptr;
+    a.wide = a.count_groups = 0;
     a.scans = nullptr;
     a.iv_a = a.b_form = 0;
     a.xsort = nullptr;
@@ -1259,23 +1270,22 @@ void fill_launch(const idtx_ctx *c, const Group &g, const Slices &sl, float *eps
     if ((g.use_list || g.tune) && sl.lists) {
         const size_t oa = align_up((size_t)g.n * g.cap_a * sizeof(int2), 256);
         const size_t ob = align_up((size_t)g.n * g.cap_b * sizeof(int2), 256);
-        const size_t om = align_up((size_t)g.n * sizeof(int4), 256);
         a.list_a = (const int2 *)sl.lists;
         a.list_b = (const int2 *)(sl.lists + oa);
         a.lmeta = (const int4 *)(sl.lists + oa + ob);
-        a.ring = (long long *)(sl.lists + oa + ob + om);
         unsigned char *sp = sl.lists + list_bytes(g.n, g.cap_a, g.cap_b);
         a.lscratch = sp + count_bytes(g) + xsort_bytes(g);
         if (g.b_form == 2) a.xsort = (const float *)(sp + count_bytes(g));
         a.iv_a = g.iv_a;
         a.b_form = g.b_form;
         a.jobs = (const int2 *)((const unsigned char *)c->buf[B_DESC] + g.off_jobs);
-        if (const size_t rows = count_rows(g)) {
-            a.cyz = (uint16_t *)sp;
-            a.cz = a.cyz + rows;
-            a.cxz = a.cz + rows;
-            a.scans = (int4 *)(a.cxz + rows);  // rows is a multiple of 4096: 16-byte aligned
-        }
+        a.wide = wide_counts(g);
+        a.count_groups = count_groups(g);
+        const size_t bytes = count_rows(g) * a.count_groups * (a.wide ? sizeof(uint32_t) : sizeof(uint16_t));
+        a.cyz = sp;
+        a.cz = sp + bytes;
+        a.cxz = sp + 2 * bytes;
+        a.scans = (int4 *)(sp + 3 * bytes);  // bytes is a multiple of 256
     }
 }
 

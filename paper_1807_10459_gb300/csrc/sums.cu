@@ -14,6 +14,7 @@ namespace {
 // estimates: 0.58 -> 0.30 ms against terms and sums in fp64, of which an SM
 // does two operations a clock (see digamma_sum).
 constexpr int kRowsPerWarp = 8;
+template <typename Four>  // four counts: uint2 of 16 bits each, uint4 of 32
 __global__ void k_sum_terms(const KsgLaunch a, int qc)
 {
     __shared__ long long s_sum[32][32];  // [warp][job]
@@ -24,14 +25,14 @@ __global__ void k_sum_terms(const KsgLaunch a, int qc)
     unsigned sz = 0, syz = 0;  // for the work counters
     long long sum[4] = {0, 0, 0, 0};
     constexpr int kRows = kRowsPerWarp / 4;
-    uint2 z[kRows], xz[kRows], yz[kRows];
+    Four z[kRows], xz[kRows], yz[kRows];
 #pragma unroll
     for (int u = 0; u < kRows; ++u) {
         const int64_t qi = min(q0 + w * kRowsPerWarp + u * 4 + (lane >> 3), a.n_pad - 1);
         const int64_t at = (((int64_t)grp * a.n_pad + qi) * 32 + j0) / 4;
-        z[u] = __ldcs(reinterpret_cast<const uint2 *>(a.cz) + at);
-        xz[u] = __ldcs(reinterpret_cast<const uint2 *>(a.cxz) + at);
-        yz[u] = __ldcs(reinterpret_cast<const uint2 *>(a.cyz) + at);
+        z[u] = __ldcs(static_cast<const Four *>(a.cz) + at);
+        xz[u] = __ldcs(static_cast<const Four *>(a.cxz) + at);
+        yz[u] = __ldcs(static_cast<const Four *>(a.cyz) + at);
     }
 #pragma unroll
     for (int u = 0; u < kRows; ++u) {
@@ -42,8 +43,14 @@ __global__ void k_sum_terms(const KsgLaunch a, int qc)
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
             if (t >= n_job) break;
-            auto part = [&](const uint2 &v) {
-                return (int)((t < 2 ? v.x : v.y) >> (t & 1) * 16 & 0xffffu);
+            auto part = [&](const Four &v) {
+                if constexpr (sizeof(Four) == sizeof(uint4)) {
+                    // within psi's table also where the list kernel gave up
+                    const unsigned c = t == 0 ? v.x : (t == 1 ? v.y : (t == 2 ? v.z : v.w));
+                    return (int)min(c, (unsigned)a.n - 1u);
+                } else {  // (the table has at least 65536 entries)
+                    return (int)((t < 2 ? v.x : v.y) >> (t & 1) * 16 & 0xffffu);
+                }
             };
             const int nz = part(z[u]), nxz = part(xz[u]), nyz = part(yz[u]);
             sz += nz;
@@ -82,8 +89,12 @@ __global__ void k_sum_terms(const KsgLaunch a, int qc)
 cudaError_t sum_terms(const KsgLaunch &a, int qc, int n_groups, cudaStream_t st)
 {
     static_assert(64 % kRowsPerWarp == 0, "tiles of up to 64 queries, a multiple of 8");
-    k_sum_terms<<<dim3((unsigned)a.n_qt, (unsigned)n_groups),
-                  (unsigned)(qc / kRowsPerWarp * 32), 0, st>>>(a, qc);
+    const dim3 grid((unsigned)a.n_qt, (unsigned)n_groups);
+    const unsigned threads = (unsigned)(qc / kRowsPerWarp * 32);
+    if (a.wide)
+        k_sum_terms<uint4><<<grid, threads, 0, st>>>(a, qc);
+    else
+        k_sum_terms<uint2><<<grid, threads, 0, st>>>(a, qc);
     return cudaGetLastError();
 }
 

@@ -23,7 +23,7 @@ def idtx():
     return m
 
 
-def _both(idtx, x, y, z, caps, S=2, k=4):
+def _both(idtx, x, y, z, caps, S=2, k=4, full=True):
     out = []
     for kernel in (idtx.KERNEL_LIST, idtx.KERNEL_TILE):
         ctx = idtx.Context(0)
@@ -31,8 +31,8 @@ def _both(idtx, x, y, z, caps, S=2, k=4):
         ctx.set_list_caps(*caps)
         dev = [None if c is None else torch.from_numpy(np.ascontiguousarray(c)).cuda()
                for c in (x, y, z)]
-        r = idtx.cmi_ksg(*dev, k=k, n_surr=S, seed=11, want_eps=True, want_counts=True, ctx=ctx)
-        out.append([t.cpu().numpy() for t in r])
+        r = idtx.cmi_ksg(*dev, k=k, n_surr=S, seed=11, want_eps=full, want_counts=full, ctx=ctx)
+        out.append([t.cpu().numpy() for t in (r if full else (r,))])
     for a, b in zip(*out):
         assert np.array_equal(a, b)
     return out[0]
@@ -70,10 +70,17 @@ def test_lists_of_uneven_density_and_equal_distances(idtx):
 
 @pytest.mark.parametrize("n", [65536, 65537])
 def test_both_forms_of_the_list_kernel_at_their_boundary(idtx, n):
-    """Up to 65536 samples the counts leave the list kernel as 16-bit numbers
-    and the terms are summed apart; above, the kernel sums them itself."""
+    """Up to 65536 samples the counts leave the list kernel as 16-bit numbers,
+    above as 32-bit ones."""
     g = synth.gaussian_problem(n, 1, 1, 2, seed=9)
     _both(idtx, g.x, g.y, g.z, (256, 512), S=1)
+
+
+def test_more_groups_than_the_count_buffers_hold(idtx):
+    """1301 estimates of 65537 samples: the counts of 40 groups fit, so 41 take
+    two turns, the second one with 21 jobs."""
+    g = synth.gaussian_problem(65537, 1, 1, 3, seed=4)
+    _both(idtx, g.x, g.y, g.z, (64, 128), S=1300, full=False)
 
 
 @pytest.mark.parametrize("n,S,caps", [(129, 0, (32, 32)), (1000, 33, (32, 64)), (3000, 95, (96, 96))])
