@@ -238,7 +238,7 @@ int idtx_ctx_set_kernel(idtx_ctx *ctx, int kernel);
 int idtx_ctx_set_list_caps(idtx_ctx *ctx, int cap_a, int cap_b);
 
 /* Bound every device wait of this context's calls (the tile kernel's staged-
- * tile and lock waits, the list kernel's tile-ring waits) by ns nanoseconds
+ * tile and lock waits, the list kernel's waits for work) by ns nanoseconds
  * instead of settings->timeout_ms; 0 restores the settings' bound.  No
  * counterpart in the paper: with a bound shorter than a tile copy the waits
  * run out, the call returns IDTX_ETIMEOUT, and the context stays usable, so

@@ -8,8 +8,8 @@
 //
 // Every job of a group shares Y and Z (a surrogate only permutes X; the
 // candidates of one greedy step differ only in X), so the neighbourhoods in
-// the (Y,Z) and Z subspaces are the same for all of them.  k_build_lists
-// (lists.cu) sorts them once per query i, for all jobs together:
+// the (Y,Z) and Z subspaces are the same for all of them.  build_lists
+// (lists.cu) lists them once per query i, for all jobs together:
 //   list A: every j != i with d_YZ(i,j) < r_A(i), ascending by d_YZ,
 //   list B: every j != i with d_Z(i,j)  < r_B(i), ascending by d_Z,
 // at most cap_a / cap_b entries, r_A and r_B chosen so.  Per (query, job):
@@ -25,9 +25,9 @@
 //     are exact when eps <= r_A and eps <= r_B (every sample closer than eps
 //     is listed); otherwise the job's counts come from a full scan.
 // Every distance is formed from the same fp32 differences and maxima as in
-// the definition, so eps and the counts are exact, and the digamma terms are
-// summed in the same order as ksg_fused_kernel's: both kernels give
-// bit-identical estimates and either may serve a call.
+// the definition, so eps and the counts are exact, and a query tile's digamma
+// terms are summed without rounding (digamma_sum), as by ksg_fused_kernel: both
+// kernels give bit-identical estimates and either may serve a call.
 //
 // Design (GB300).  The kernel is persistent: one CTA of 32 warps per SM, one
 // job per lane.  A CTA takes chunks of consecutive queries of one job group

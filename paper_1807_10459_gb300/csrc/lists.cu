@@ -12,14 +12,14 @@
 //
 // Two kernels per chunk of queries, with the unsorted entries in scratch
 // between them:
-//   k_collect     a warp per QW consecutive queries: a radius for each list
+//   k_collect     a warp per one or two queries: a radius for each list
 //                 from a sample of the distances, then one pass over the
 //                 tiles whose box is within a radius, appending the entries.
 //   k_sort_lists  a block per (query, list): counting sort on the distance.
 // Measured on GB300 against one block per query with two histogram passes over
 // all rows and block radix sorts, both kernels together: N = 9995, three z and
-// one y column, lists of 2048 and 4096: 1.68 -> 0.84 ms; N = 4997, six z,
-// 1024 and 2048: 0.51 -> 0.30 ms; N = 99850, ten z, 512 and 1024: 44.3 ->
+// one y column, lists of 2048 and 4096: 1.68 -> 0.77 ms; N = 4997, six z,
+// 1024 and 2048: 0.51 -> 0.29 ms; N = 99850, ten z, 512 and 1024: 44.3 ->
 // 8.8 ms (that kernel read every visited row once per query, and visited 60 to
 // 95 % of the tiles for its histogram).
 #include <cuda_runtime.h>
@@ -160,7 +160,7 @@ __device__ __noinline__ Shrunk shrink_list(int2 *buf, int cnt, int cap, int *his
     return Shrunk{kept, radius};
 }
 
-// One warp per two consecutive queries.
+// One warp per QW (one or two) consecutive queries.
 //
 // Radii.  The distances to n_sample rows spread evenly over the samples (in
 // Morton order, so over space) go into a histogram per list; the radius is
@@ -175,7 +175,7 @@ __device__ __noinline__ Shrunk shrink_list(int2 *buf, int cnt, int cap, int *his
 // gap reaches both radii of both queries are skipped, 32 tiles being tested
 // at a time, one per lane.
 //
-// A visited tile's rows are loaded once for the two queries, whose
+// A visited tile's rows are loaded once for the warp's queries, whose
 // coordinates stay in registers, and the entries below a radius are appended
 // to the query's buffers (the counts are the warp's own: no atomics).  With
 // more than six dimensions the first four are tested first: a group of 32
@@ -183,12 +183,12 @@ __device__ __noinline__ Shrunk shrink_list(int2 *buf, int cnt, int cap, int *his
 // Bound by issue (the differences and maxima) at few dimensions and by L1 at
 // many; two queries per warp at 80 registers ran N = 99850, ten z in 7.1 ms,
 // four queries at 167 registers (half the warps) in 15.4.
-template <int DZ, int DY>
-__global__ void __launch_bounds__(kCollectThreads, DZ + DY <= 12 ? 3 : 2)
+template <int DZ, int DY, int QW>
+__global__ void __launch_bounds__(kCollectThreads, QW == 1 ? 4 : (DZ + DY <= 12 ? 3 : 2))
     k_collect(const CollectArgs a)
 {
     constexpr int DS = DZ + DY, NC = (DS + 3) / 4, DSP = NC * 4;
-    constexpr int QW = 2, kSegs = kTJ / 32;
+    constexpr int kSegs = kTJ / 32;
     constexpr int U = NC == 1 ? 4 : 2;  // rows a lane has in flight
     constexpr bool EARLY = DZ > 6;
     static_assert(kTJ % QW == 0 && kSegs % U == 0, "query groups and row steps tile a tile");
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kCollectThreads, DZ + DY <= 12 ? 3 : 2)
     };
     // The second query past the chunk's end (odd counts) repeats the first
     // and lists nothing.
-    const bool two = g0 + 1 < a.n_q;
+    const bool two = QW > 1 && g0 + 1 < a.n_q;
     const int q0 = (int)a.q0 + g0;
     float q[QW][DSP], ra[QW], rb[QW];
     int ca[QW], cb[QW];
@@ -261,8 +261,11 @@ __global__ void __launch_bounds__(kCollectThreads, DZ + DY <= 12 ? 3 : 2)
         }
         __syncwarp();
     }
-    if (a.cap_b == 0) rb[0] = rb[1] = -1.0f;  // list A only
-    if (!two) ra[1] = rb[1] = -1.0f;
+#pragma unroll
+    for (int u = 0; u < QW; ++u) {
+        if (a.cap_b == 0) rb[u] = -1.0f;  // list A only
+        if (u > 0 && !two) ra[u] = rb[u] = -1.0f;
+    }
     int2 *const oa = a.raw_a + (int64_t)g0 * a.buf_a, *const ob = a.raw_b + (int64_t)g0 * a.buf_b;
     const int n_tiles = (n + kTJ - 1) / kTJ;
     const int home = q0 / kTJ;  // the tile of both queries
@@ -345,7 +348,9 @@ __global__ void __launch_bounds__(kCollectThreads, DZ + DY <= 12 ? 3 : 2)
     }
     if (lane == 0) {
         a.raw_meta[g0] = make_int4(ca[0], cb[0], __float_as_int(ra[0]), __float_as_int(rb[0]));
-        if (two) a.raw_meta[g0 + 1] = make_int4(ca[1], cb[1], __float_as_int(ra[1]), __float_as_int(rb[1]));
+        if (two)
+            a.raw_meta[g0 + 1] =
+                make_int4(ca[QW - 1], cb[QW - 1], __float_as_int(ra[QW - 1]), __float_as_int(rb[QW - 1]));
     }
 }
 
@@ -602,11 +607,23 @@ __global__ void __launch_bounds__(T, E > 8 ? 1536 / T : 2048 / T)
     }
 }
 
+// Two queries a warp share a visited tile's rows, one leaves more registers for
+// warps (four blocks an SM instead of three) and twice the warps: better as long
+// as the rows stay in L1 and are short, and for few queries.  One against two,
+// us: N = 1000, two z, 11 and 17; 2500, eight, 39 and 49; 4997, six, 86 and
+// 100; 9995, three, 205 and 269; 30000, three, 513 and 610; 50000, two, 736 and
+// 706; 4000, eight, 88 (at three blocks) and 73; 30000, eight, 1705 and 1469.
+template <int DZ, int DY>
+constexpr int kCollectSingle = DZ + DY <= 8 ? 32768 : 2560;
 template <int DZ, int DY>
 cudaError_t launch_collect(const CollectArgs &a, cudaStream_t st)
 {
-    const int per = kCollectWarps * 2;  // queries per block
-    k_collect<DZ, DY><<<(unsigned)((a.n_q + per - 1) / per), kCollectThreads, 0, st>>>(a);
+    if (a.n <= kCollectSingle<DZ, DY>)
+        k_collect<DZ, DY, 1><<<(unsigned)((a.n_q + kCollectWarps - 1) / kCollectWarps), kCollectThreads,
+                               0, st>>>(a);
+    else
+        k_collect<DZ, DY, 2><<<(unsigned)((a.n_q + 2 * kCollectWarps - 1) / (2 * kCollectWarps)),
+                               kCollectThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -6,10 +6,12 @@
 // the original estimate and its surrogates (idtx_cmi_ksg), one batch problem
 // (idtx_cmi_batch), or every candidate of a greedy step with its surrogates
 // (idtx_mte_step).  A group runs as
-//   pack_shared  : Y/Z columns -> sh [n_pad][dsp] (row per sample, +inf pads)
+//   pack_tiles   : Y/Z columns -> sh, tiles of 128 samples and their boxes
 //   shuffle      : surrogate permutations, one warp per permutation
-//   gather_x     : X values of every job, permuted, -> xi [groups][n_pad][GB*DX]
-//   ksg_fused    : kNN + counts + digamma partial sums (ksg_kernel.cuh)
+//   gather       : X values of every job, permuted, -> xi [groups][n_pad][GB*DX]
+//   build_lists  : per query, its neighbours in (Y,Z) and Z (lists.cu)
+//   estimator    : kNN + counts + digamma partial sums, over the lists
+//                  (ksg_list.cuh) or all pairs (ksg_kernel.cuh)
 //   finalize     : psi(k) + sum / N per job, fixed order
 // and the greedy step adds the max-statistic gate kernel.
 #include <algorithm>
