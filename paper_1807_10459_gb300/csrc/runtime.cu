@@ -3521,7 +3521,14 @@ const KsgVariant *noalloc_variant(int dx, int dy, int dz, int k)
     static KsgVariant table[kMaxVariants];
     static int n_table = 0;
     static std::once_flag once;
-    std::call_once(once, [] { n_table = ksg_variants(table); });
+    // Without the runtime k <= 7 ones: a problem's scratch, and so whether it is
+    // taken, is that of the generic specialisation.
+    std::call_once(once, [] {
+        KsgVariant all[kMaxVariants];
+        const int n = ksg_variants(all);
+        for (int i = 0; i < n; ++i)
+            if (all[i].exact || all[i].k1 > 8) table[n_table++] = all[i];
+    });
     return choose_variant(table, n_table, dx, dy, dz, k);
 }
 
