@@ -73,8 +73,8 @@
 #include "ksg_kernel.cuh"
 #include "ksg_plain.cuh"
 
-// List entries whose X rows a walk has in flight (a multiple of 4, at most 16;
-// compile-time knobs, the defaults are the tuned values: 4 / 8 / 16 give the
+// List entries whose X rows a walk has in flight (4, 8 or 16: whole steps of the
+// 32 entries staged at a time; compile-time knobs, the defaults are the tuned values: 4 / 8 / 16 give the
 // greedy step 13.8 / 13.2 / 13.4 ms).
 #ifndef IDTX_LIST_SA
 #define IDTX_LIST_SA 8
@@ -367,6 +367,7 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
             // of the warp's buffer that was used up; past the list's end
             // sentinels), their distances and X values.
             constexpr int SW = IDTX_LIST_SA;
+            static_assert(SW % 4 == 0 && 32 % SW == 0, "steps stay within the staged entries");
             float row_d[SW], row_x[SW][DX];
             int2 nxt;
             auto fetch = [&](int e) {
