@@ -74,26 +74,28 @@
 #include "ksg_plain.cuh"
 
 // List entries whose X rows a walk has in flight (4, 8 or 16: whole steps of the
-// 32 entries staged at a time; compile-time knobs, the defaults are the tuned values: 4 / 8 / 16 give the
-// greedy step 13.8 / 13.2 / 13.4 ms).
+// 32 entries staged at a time; compile-time knobs, the defaults are the tuned
+// values).  N = 9995, three z, 2001 estimates, the kernel: 2.96 / 2.84 / 3.15 ms.
 #ifndef IDTX_LIST_SA
 #define IDTX_LIST_SA 8
 #endif
-// Jobs of a warp whose neighbour walk goes on past the others' and is
-// finished with the lanes splitting its entries.
+// Jobs of a warp whose neighbour walk goes on past the others' and is finished
+// with the lanes splitting its entries (1 / 2 / 3 / 4: 2.89 / 2.84 / 2.86 / 2.92).
 #ifndef IDTX_LIST_TAIL_A
 #define IDTX_LIST_TAIL_A 2
 #endif
 // The shared count walk hands over to the repacked phases once at most this
-// many jobs (a power of two <= 16) still need entries (4 / 8 / 16: within 1 %).
+// many jobs (a power of two <= 16) still need entries (4 / 8 / 16: 2.95 / 2.84 /
+// 2.87).
 #ifndef IDTX_LIST_REPACK
 #define IDTX_LIST_REPACK 8
 #endif
 // Entries a lane takes per step of a repacked count phase (their loads are in
-// flight together; entries past the lane's job are predicated off): 2 / 4
-// entries give the greedy step 13.5 / 13.2 ms.
+// flight together; entries past the lane's job are predicated off); four with
+// more than one x column.  N = 9995, three z, 2001 estimates, the kernel at 2 /
+// 4 / 5 / 6 / 8: 2.91 / 2.84 / 2.82 / 2.80 / 2.86 ms.
 #ifndef IDTX_LIST_PHASE_STEP
-#define IDTX_LIST_PHASE_STEP 4
+#define IDTX_LIST_PHASE_STEP 6
 #endif
 // Job groups per super-block of the chunk order (see the kernel).
 #ifndef IDTX_LIST_GSB
@@ -598,7 +600,7 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
                     int cz = 0, cx = 0;
                     uint32_t still;
                     do {
-                        constexpr int PS = IDTX_LIST_PHASE_STEP;
+                        constexpr int PS = DX == 1 ? IDTX_LIST_PHASE_STEP : 4;
                         int js[PS];
                         float xv[PS][DX];
 #pragma unroll
