@@ -57,15 +57,16 @@
 //     ascends, are list B (up to thousands of entries there, beyond any list's
 //     capacity); with none and one y column the order is by y and stands for
 //     list A.  Without z, n_z is all and n_xz with one x column is a range of
-//     the sorted column.  N = 3001, no z, 201 estimates: 2.0 ms by the tile
-//     kernel, 0.35; N = 20000: 30.1 and 1.7; one z, N = 3001: 0.95 (lists) and
-//     0.57; N = 50000, 101 estimates: 33.1 (tile) and 22.6.
+//     the sorted column.  The call, by the tile kernel and so: N = 3001, no z,
+//     201 estimates, 1.92 and 0.32 ms; N = 20000, 49.4 and 2.5; one z, N = 3001,
+//     0.73 and 0.52 (0.95 with a list B); N = 50000, 101 estimates, 29.6 and 14.6.
 // Measured on GB300, greedy step of N = 9995 with 9447 estimates (one network;
 // lists of 2048 and 4096), against summing the terms in the kernel and scanning
 // in place: 19.1 -> 12.7 ms; of N = 4997, six conditions, 28341 estimates: 10.8
-// -> 8.5 ms; N = 1000, 101 estimates: 163 -> 24 us (each with sum_terms' 0.30,
-// 0.51 ms and 4 us to add).  Bound by issue (58 % of the slots) and the latency behind it: fewer,
-// fatter warps (24 of 80 registers) were 8 % slower.
+// -> 8.5 ms; N = 1000, 101 estimates: 163 -> 24 us (each with sum_terms' 0.27,
+// 0.38 ms and 4 us to add).  Bound by issue (71 % of the slots in a capture of 752
+// estimates) and L1 (78 % of its rate): fewer, fatter warps (24 of 80 registers)
+// were 8 % slower.
 #pragma once
 
 #include <type_traits>
