@@ -208,7 +208,8 @@ int idtx_ctx_set_profiling(idtx_ctx *ctx, int enable);
 int idtx_ctx_set_graphs(idtx_ctx *ctx, int enable);
 
 /* Which kernel computes the estimates of a call (no counterpart in the paper,
- * whose GPU estimator is not described; both give bit-identical results):
+ * whose GPU estimator is not described; both give bit-identical results, as
+ * do a batch and separate calls, and the plain schedule):
  *   IDTX_KERNEL_TILE: the tile kernel scans reference tiles staged into
  *     shared memory, skipping tiles that are provably out of reach.
  *   IDTX_KERNEL_LIST: the list kernel first sorts, once per query and for
@@ -503,13 +504,11 @@ int idtx_screen_features(idtx_ctx *ctx, const double *est, int n_cand, int s0, i
  * CUDA device and takes all its scratch from one fixed array of
  * IDTX_NOALLOC_SCRATCH_BYTES bytes in device memory that the library
  * declares at file scope.  Every GPU that loads the library holds that array
- * until the process exits.  The per-sample eps and counts behind the
- * estimates are the same as idtx_cmi_ksg's; the estimates agree within
- * 1e-10 nats but not always bit for bit, because this entry point keeps the
- * samples in their given order (idtx_cmi_ksg sorts them along a Morton curve
- * for n > 256), so its fp64 partial sums are added in another order.  For
- * the same reason its tile kernel skips few reference tiles, and for large n
- * it is markedly slower than idtx_cmi_ksg.
+ * until the process exits.  The estimates, and the per-sample eps and counts
+ * behind them, are the same as idtx_cmi_ksg's, to the last bit.  This entry
+ * point keeps the samples in their given order (idtx_cmi_ksg sorts them for
+ * n > 256), so its tile kernel skips few reference tiles, and for large n it
+ * is markedly slower than idtx_cmi_ksg.
  *   - x, y, z and cmi_out must be device memory; cmi_out [1+n_surr] fp64.
  *   - 0 <= settings->n_surr <= IDTX_NOALLOC_MAX_SURR; a problem whose scratch
  *     does not fit in the array returns IDTX_EINVAL with the bytes it needs.

@@ -16,7 +16,8 @@
 //                            element (j, g, d) = X_job[d][pi_job(j)], +inf for j >= n.
 //   psi  [n_max+1] int64     digamma at the integers 1..n_max (index 0 unused) in
 //                            units of 2^-kPsiBits.
-//   partial [n_jobs][n_qt] fp64  per query tile sums of the digamma terms.
+//   partial [n_jobs][n_qt] int64  per query tile sums of the digamma terms, in
+//                            the same units.
 #pragma once
 
 #include <cstddef>
@@ -47,12 +48,10 @@ enum : int {
 // psi(n_yz + 1) lies within +-15.7 for up to 2 million samples, a tile's sum
 // (64 terms) within +-1005 < 2^10, so 53 fraction bits fit; they hold the fp64
 // values exactly (those below 1/2 in magnitude, psi(2) alone, too: it is
-// psi(1) + 1).  So a tile's sum is that of the fp64 values, rounded once.
+// psi(1) + 1).  k_finalize adds the tiles' sums exactly and rounds once, so an
+// estimate's bits depend neither on the tiles' size nor on the samples' order:
+// every kernel, specialisation and schedule gives the same.
 constexpr int kPsiBits = 53;
-__host__ __device__ __forceinline__ double digamma_sum(long long s)
-{
-    return (double)s * (1.0 / (double)(1ll << kPsiBits));
-}
 
 constexpr int kTileRows = kTJ + 2;  // samples + bounding box rows
 
@@ -79,7 +78,7 @@ struct KsgLaunch {
     const float *sh;
     const float *xi;
     const long long *psi;
-    double *partial;
+    long long *partial;
     float *eps_out;      // nullable, [n_jobs][n] in original sample order
     int32_t *cnt_out;    // nullable, [n_jobs][3][n]: n_xz, n_yz, n_z, original order
     const int32_t *order;  // nullable: original index of sorted position m
@@ -139,7 +138,7 @@ typedef cudaError_t (*KsgLaunchFn)(const KsgLaunch &, int n_groups, cudaStream_t
 // group's tiles, xj the job's X values [n_pad][dx bucket], partial the job's
 // n_pad / 8 partial sums.
 typedef cudaError_t (*KsgPlainFn)(const float *sh, const float *xj, const long long *psi, int64_t n,
-                                  int64_t n_pad, int k, double *partial, float *eps,
+                                  int64_t n_pad, int k, long long *partial, float *eps,
                                   int32_t *cnt, cudaStream_t);
 constexpr int kPlainQueriesPerPartial = 8;
 

@@ -307,7 +307,7 @@ __device__ __forceinline__ bool ksg_cta(const KsgLaunch &a, const int qt, const 
     if (qv <= 0) {
         // Only padding queries (n_pad is a multiple of the reference tile, not
         // of QC): zero partial sums, and no copy is ever issued.
-        if (tid < GB && job_ok) a.partial[static_cast<int64_t>(job) * a.n_qt + qt] = 0.0;
+        if (tid < GB && job_ok) a.partial[static_cast<int64_t>(job) * a.n_qt + qt] = 0;
         return true;
     }
 
@@ -705,7 +705,7 @@ __device__ __forceinline__ bool ksg_cta(const KsgLaunch &a, const int qt, const 
         long long s = 0;
 #pragma unroll
         for (int w = 0; w < NW; ++w) s += s_red[w][tid];
-        a.partial[static_cast<int64_t>(job) * a.n_qt + qt] = digamma_sum(s);
+        a.partial[static_cast<int64_t>(job) * a.n_qt + qt] = s;
     }
     __syncthreads();  // shared state may be reused by the CTA's next task
     return true;

@@ -26,7 +26,7 @@
 //     is listed); otherwise the job's counts come from a full scan.
 // Every distance is formed from the same fp32 differences and maxima as in
 // the definition, so eps and the counts are exact, and a query tile's digamma
-// terms are summed without rounding (digamma_sum), as by ksg_fused_kernel: both
+// terms are summed without rounding (kPsiBits), as by ksg_fused_kernel: both
 // kernels give bit-identical estimates and either may serve a call.
 //
 // Design (GB300).  The kernel is persistent: one CTA of 32 warps per SM, one
@@ -1158,9 +1158,8 @@ cudaError_t launch_ksg_list(const KsgLaunch &all, int n_groups, cudaStream_t str
 }
 
 // One compiled specialisation: the tile kernel (ksg_kernel.cuh), its
-// persistent form, and the list kernel, all with the same launch shape so
-// that their digamma partial sums agree bit for bit; and the plain schedule
-// (ksg_plain.cuh) of the same dimension bucket.
+// persistent form, the list kernel with the same query tiles, and the plain
+// schedule (ksg_plain.cuh) of the same dimension bucket.
 template <int DX, int DY, int DZ, int K1, bool EXACT, int QC, int NWARPS>
 KsgVariant make_variant()
 {

@@ -9,11 +9,10 @@
 // distance 0, included), and the warp merges them by repeated minima, so the
 // (k+1)-th smallest is eps_i.  A second sweep counts the strict-radius
 // neighbours in the subspaces, the self pair removed.  A CTA of 8 warps
-// serves 8 consecutive queries and writes their digamma terms' sum, in warp
-// order, as one partial; k_finalize sums the partials in order.  Distances
-// are the definition's fp32 |a - b| and maxima, so eps and the counts equal
-// the other kernels'; only the order of the fp64 sum differs (estimates
-// agree within rounding).
+// serves 8 consecutive queries and writes their digamma terms' sum as one
+// partial.  Distances are the definition's fp32 |a - b| and maxima, so eps and
+// the counts equal the other kernels', and with the exact sums (kPsiBits) the
+// estimates do, to the last bit.
 #pragma once
 
 #include "ksg_kernel.cuh"
@@ -29,7 +28,7 @@ constexpr int kPlainWarps = kPlainQueriesPerPartial;  // queries per CTA of the 
 template <int DX, int DY, int DZ, int K1, bool EXACT, int DSP>
 __global__ void __launch_bounds__(kPlainWarps * 32)
     k_ksg_plain(const float *sh, const float *xj, int64_t n, int k, const long long *psi,
-                double *partial, float *eps, int32_t *cnt)
+                long long *partial, float *eps, int32_t *cnt)
 {
     constexpr int DS = DZ + DY;
     constexpr int KH = K1;  // the k+1 smallest including the query (EXACT: exactly)
@@ -114,7 +113,7 @@ __global__ void __launch_bounds__(kPlainWarps * 32)
         long long s = 0;
 #pragma unroll
         for (int w = 0; w < kPlainWarps; ++w) s += s_t[w];
-        partial[blockIdx.x] = digamma_sum(s);
+        partial[blockIdx.x] = s;
     }
 }
 
@@ -122,7 +121,7 @@ __global__ void __launch_bounds__(kPlainWarps * 32)
 // ones, so that every partial of the job is written (0 past n).
 template <int DX, int DY, int DZ, int K1, bool EXACT, int QC, int NWARPS>
 cudaError_t launch_ksg_plain(const float *sh, const float *xj, const long long *psi, int64_t n,
-                             int64_t n_pad, int k, double *partial, float *eps, int32_t *cnt,
+                             int64_t n_pad, int k, long long *partial, float *eps, int32_t *cnt,
                              cudaStream_t stream)
 {
     using S = KsgShape<DX, DY, DZ, K1, EXACT, QC, NWARPS>;

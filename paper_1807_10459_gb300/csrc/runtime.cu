@@ -408,19 +408,30 @@ static int64_t gather_blocks(int64_t n_groups, int64_t n_pad, int gb, int dxb)
     return b > 0x7fffffff ? 0 : b;
 }
 
-// cmi[job] = psi(k) + (sum over query tiles) / n, a warp per job: lane l adds
-// the tiles l, l + 32, ... in order, then the lanes' sums are added pairwise.
-// (A thread per job read its row alone: 47 us for 101 jobs of 782 tiles, 124
-// for 201 of 1561.)
+// cmi[job] = psi(k) + (sum over query tiles) / n, a warp per job.  The sum is
+// exact, of the partial sums' high and low 32 bits apart (up to 2^18 tiles of
+// 2^31 and 2^32), and rounded once, when the two halves, exact in fp64, are
+// added.  (A thread per job read its row alone: 47 us for 101 jobs of 782
+// tiles, 124 for 201 of 1561.)
 constexpr int kFinalWarps = 4;
-__global__ void k_finalize(const double *partial, int n_jobs, int n_qt, double psi_k,
+__global__ void k_finalize(const long long *partial, int n_jobs, int n_qt, double psi_k,
                            int64_t n, double *cmi)
 {
     const int job = blockIdx.x * kFinalWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (job >= n_jobs) return;
-    double s = 0.0;
-    for (int t = lane; t < n_qt; t += 32) s += partial[(int64_t)job * n_qt + t];
-    for (int off = 16; off >= 1; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+    long long hi = 0, lo = 0;
+    for (int t = lane; t < n_qt; t += 32) {
+        const long long v = partial[(int64_t)job * n_qt + t];
+        hi += v >> 32;
+        lo += v & 0xffffffffll;
+    }
+    for (int off = 16; off >= 1; off >>= 1) {
+        hi += __shfl_down_sync(0xffffffffu, hi, off);
+        lo += __shfl_down_sync(0xffffffffu, lo, off);
+    }
+    hi += lo >> 32;
+    lo &= 0xffffffffll;
+    const double s = ((double)hi * 4294967296.0 + (double)lo) * (1.0 / (double)(1ll << kPsiBits));
     if (lane == 0) cmi[job] = psi_k + s / (double)n;
 }
 
@@ -1069,7 +1080,8 @@ int plan(idtx_ctx *c, Group &g)
     g.n_groups = (int)((g.jobs.size() + g.v->gb - 1) / g.v->gb);
     if (g.n_groups > 65535) return fail(IDTX_EINVAL, "too many estimates in one group");
     g.sort = !g.plain && g.n > 2 * kTJ;
-    // The order fixes that of the sums, so it is the same for both kernels.
+    // The same order for both kernels, so that a trial runs both on one
+    // preparation.
     g.col_order = 0;
     if (g.sort && g.n_pad <= 65536)
         g.col_order = g.dz == 1 ? 1 : (g.dz == 0 && g.dy == 1 ? 2 : 0);
@@ -1202,7 +1214,7 @@ CallBuffers bytes_of(const Group &g)
     }
     b.xi = align_up((size_t)g.n_groups * g.n_pad * g.v->gb * g.v->dx * sizeof(float), 256);
     b.perm = align_up(g.slot_stream.size() * (size_t)(g.n + g.n_reps) * sizeof(int32_t), 256);
-    b.partial = align_up(g.jobs.size() * (size_t)g.n_qt * sizeof(double), 256);
+    b.partial = align_up(g.jobs.size() * (size_t)g.n_qt * sizeof(long long), 256);
     if (g.use_list || g.tune)
         b.lists = list_bytes(g.n, g.cap_a, g.cap_b) + count_bytes(g) + xsort_bytes(g) +
                   list_scratch_bytes(g.n, g.cap_a, g.cap_b);
@@ -1227,7 +1239,7 @@ struct Slices {
     float *sh;
     float *xi;
     int32_t *perm;
-    double *partial;
+    long long *partial;
     unsigned char *order;
     void *sort_tmp;
     size_t sort_cap;
@@ -1413,7 +1425,7 @@ int prep_group(idtx_ctx *c, const Group &g, cudaStream_t st, const Slices &sl, f
     float *sh = sl.sh;
     float *xi = sl.xi;
     int32_t *perm = sl.perm;
-    double *partial = sl.partial;
+    long long *partial = sl.partial;
     const KsgVariant &v = *g.v;
     const int n_jobs = (int)g.jobs.size();
     const int n_slots = (int)g.slot_stream.size();
@@ -1628,7 +1640,7 @@ int enqueue_group(idtx_ctx *c, const Group &g, cudaStream_t st, double *cmi, flo
                   int32_t *cnt_out, long long timeout_ns)
 {
     const Slices sl{(float *)c->buf[B_SH],       (float *)c->buf[B_XI],
-                    (int32_t *)c->buf[B_PERM],   (double *)c->buf[B_PARTIAL],
+                    (int32_t *)c->buf[B_PERM],   (long long *)c->buf[B_PARTIAL],
                     (unsigned char *)c->buf[B_ORDER], c->buf[B_SORT], c->cap[B_SORT],
                     (unsigned char *)c->buf[B_LIST]};
     KsgLaunch a;
@@ -1639,7 +1651,7 @@ int enqueue_group(idtx_ctx *c, const Group &g, cudaStream_t st, double *cmi, flo
     if (g.tune) IDTX_TRY(tune_group(c, g, a, st, use_list));
     const int n_jobs = (int)g.jobs.size();
     float *xi = sl.xi;
-    double *partial = sl.partial;
+    long long *partial = sl.partial;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     if (c->profiling) {
         IDTX_TRY(take_event(c, &ev0));
@@ -1744,7 +1756,7 @@ int batch_plan(idtx_ctx *c, std::vector<Group> &gs, cudaStream_t st, long long t
         bp.sl[i] = Slices{(float *)((unsigned char *)c->buf[B_SH] + off[i].sh),
                           (float *)((unsigned char *)c->buf[B_XI] + off[i].xi),
                           (int32_t *)((unsigned char *)c->buf[B_PERM] + off[i].perm),
-                          (double *)((unsigned char *)c->buf[B_PARTIAL] + off[i].partial),
+                          (long long *)((unsigned char *)c->buf[B_PARTIAL] + off[i].partial),
                           (unsigned char *)c->buf[B_ORDER] + off[i].order,
                           (unsigned char *)c->buf[B_SORT] + off[i].sort_tmp,
                           bytes_of(gs[i]).sort_tmp, (unsigned char *)c->buf[B_LIST]};
@@ -1886,7 +1898,7 @@ int resolve_tuning(idtx_ctx *c, std::vector<Group> &gs, cudaStream_t st, long lo
             IDTX_TRY(ensure(c, B_SORT, b.sort_tmp));
             IDTX_TRY(ensure(c, B_LIST, b.lists));
             const Slices sl{(float *)c->buf[B_SH],       (float *)c->buf[B_XI],
-                            (int32_t *)c->buf[B_PERM],   (double *)c->buf[B_PARTIAL],
+                            (int32_t *)c->buf[B_PERM],   (long long *)c->buf[B_PARTIAL],
                             (unsigned char *)c->buf[B_ORDER], c->buf[B_SORT], c->cap[B_SORT],
                             (unsigned char *)c->buf[B_LIST]};
             KsgLaunch a;
@@ -3573,7 +3585,7 @@ extern "C" int idtx_cmi_ksg_noalloc(const float *x, int dx, const float *y, int 
     const size_t at_sh = take((size_t)(n_pad / kTJ) * kTileRows * v->dsp * sizeof(float));
     const size_t at_xi = take((size_t)n_groups * n_pad * v->gb * v->dx * sizeof(float));
     const size_t at_perm = take((size_t)n_slots * n * sizeof(int32_t));
-    const size_t at_partial = take((size_t)n_jobs * n_qt * sizeof(double));
+    const size_t at_partial = take((size_t)n_jobs * n_qt * sizeof(long long));
     if (off > kNoAllocBytes)
         return fail(IDTX_EINVAL,
                     "problem needs %zu bytes of scratch; the allocation-free entry point has "
@@ -3628,7 +3640,7 @@ extern "C" int idtx_cmi_ksg_noalloc(const float *x, int dx, const float *y, int 
     float *sh = (float *)(base + at_sh);
     float *xi = (float *)(base + at_xi);
     int32_t *perm = (int32_t *)(base + at_perm);
-    double *partial = (double *)(base + at_partial);
+    long long *partial = (long long *)(base + at_partial);
     const int64_t psi_n = std::max<int64_t>(n, s->k) + 1;
     int h_err = 0;
     // Everything from the first enqueue on: on an error the stream is

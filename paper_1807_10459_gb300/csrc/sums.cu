@@ -15,7 +15,7 @@ namespace {
 // memory, which nearly all counts are below (a gather there costs its bank
 // conflicts, three to four, and in L1 a cycle for every line).
 // N = 9995, 9447 estimates: 0.58 -> 0.30 ms against terms and sums in fp64, of
-// which an SM does two operations a clock (see digamma_sum), 0.27 with the
+// which an SM does two operations a clock (see kPsiBits), 0.27 with the
 // table in shared memory; N = 4997, 28 thousand: 0.89 -> 0.51 -> 0.38.
 constexpr int kRowsPerWarp = 8, kTable = 2048;
 template <typename Four, bool TABLE>  // four counts: uint2 of 16 bits each, uint4 of 32
@@ -88,7 +88,7 @@ __global__ void k_sum_terms(const KsgLaunch a, int qc, int64_t n_tasks)
         if (w == 0 && job < a.n_jobs) {
             long long s = 0;
             for (int v = 0; v < nw; ++v) s += s_sum[v][lane];
-            a.partial[(int64_t)job * a.n_qt + qt] = digamma_sum(s);
+            a.partial[(int64_t)job * a.n_qt + qt] = s;
         }
         __syncthreads();
     }
