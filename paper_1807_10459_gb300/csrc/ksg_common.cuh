@@ -171,12 +171,12 @@ struct KsgVariant {
 };
 
 // Per-query sorted neighbour lists of a group prepared into sh (lists.cu):
-// rows of dzb z columns, then dyb y columns.  scratch: list_scratch_bytes(n,
+// rows of dzb z columns, then dyb y columns (dz and dy of them used).  scratch: list_scratch_bytes(n,
 // cap_a, cap_b), which also covers smaller capacities.  *launches (nullable)
 // receives the kernels launched.  n <= 0 only sets kernel attributes.
 size_t list_scratch_bytes(int64_t n, int cap_a, int cap_b);
-cudaError_t build_lists(const float *sh, int dzb, int dyb, int64_t n, int cap_a, int cap_b,
-                        int2 *list_a, int2 *list_b, int4 *meta, void *scratch, cudaStream_t st,
+cudaError_t build_lists(const float *sh, int dzb, int dyb, int dz, int dy, int64_t n, int cap_a,
+                        int cap_b, int2 *list_a, int2 *list_b, int4 *meta, void *scratch, cudaStream_t st,
                         int *launches);
 
 // Radix sort of (key, index) pairs on the low end_bit key bits (sort.cu).

@@ -1532,7 +1532,7 @@ int prep_group(idtx_ctx *c, const Group &g, cudaStream_t st, const Slices &sl, f
     if (fork) IDTX_CUDA(cudaEventRecord(join, xs));
     if (a.list_a && !g.iv_a) {
         int built = 0;
-        IDTX_CUDA(build_lists(sh, v.dz, v.dy, g.n, g.cap_a, g.cap_b,
+        IDTX_CUDA(build_lists(sh, v.dz, v.dy, g.dz, g.dy, g.n, g.cap_a, g.cap_b,
                               const_cast<int2 *>(a.list_a), const_cast<int2 *>(a.list_b),
                               const_cast<int4 *>(a.lmeta), a.lscratch, st, &built));
         launches += built;
@@ -1594,7 +1594,7 @@ int tune_group(idtx_ctx *c, const Group &g, KsgLaunch &a, cudaStream_t st, bool 
     auto build = [&](int ca, int cb) -> int {
         int built = 0;
         if (g.iv_a) return IDTX_OK;
-        IDTX_CUDA(build_lists(a.sh, v.dz, v.dy, g.n, ca, cb, const_cast<int2 *>(a.list_a),
+        IDTX_CUDA(build_lists(a.sh, v.dz, v.dy, g.dz, g.dy, g.n, ca, cb, const_cast<int2 *>(a.list_a),
                               const_cast<int2 *>(a.list_b), const_cast<int4 *>(a.lmeta),
                               a.lscratch, st, &built));
         c->stats.kernel_launches += built;
@@ -2435,7 +2435,7 @@ int idtx_cmi_batch(idtx_ctx *c, const idtx_problem *probs, int n_probs, int k, d
             else
                 c->event_pool.push_back(ev);
         }
-        if (rc == IDTX_OK && build_lists(nullptr, 1, 1, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, st,
+        if (rc == IDTX_OK && build_lists(nullptr, 1, 1, 1, 1, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, st,
                                          nullptr) != cudaSuccess)
             rc = fail(IDTX_ECUDA, "list kernel attribute setup failed");
         for (const KsgVariant *v : bp.vars)
