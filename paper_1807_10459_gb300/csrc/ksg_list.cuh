@@ -247,6 +247,11 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
     constexpr unsigned kFull = 0xffffffffu;
     // may serve calls of at most one z column: the generic one covers any dz
     constexpr bool LOW = DZ == 1 || K1 > 8;
+    // One z column: n_z is in the thousands, and is found by bisection after the
+    // walk for n_xz, not counted in it (which also spilled 32 bytes, now 8).  N =
+    // 9995, 9045 estimates, 59.1 -> 56.2 ms; N = 1000, 1001 estimates, 177 -> 182
+    // us, and for a runtime k 135 -> 142, with nothing gained at N = 10000.
+    constexpr bool SEARCH_Z = DZ == 1 && EXACT;
     constexpr int TAIL_A = IDTX_LIST_TAIL_A;  // jobs left after the shared neighbour walk
     const float kInf = CUDART_INF_F;
 
@@ -587,7 +592,7 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
 #pragma unroll
                     for (int t = 0; t < SW; ++t) {
                         const bool pz = dz[t] < ev;
-                        nz += pz ? 1 : 0;
+                        if (!SEARCH_Z) nz += pz ? 1 : 0;
                         nxz += (pz && dx[t] < ev) ? 1 : 0;
                     }
                 }
@@ -640,7 +645,7 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
                             float dxv = fabsf(xs[0] - xv[t][0]);
 #pragma unroll
                             for (int d = 1; d < DX; ++d) dxv = fmaxf(dxv, fabsf(xs[d] - xv[t][d]));
-                            cz += js[t] >= 0 ? 1 : 0;
+                            if (!SEARCH_Z) cz += js[t] >= 0 ? 1 : 0;
                             cx += dxv < es ? 1 : 0;
                         }
                         still = __ballot_sync(kFull, ((rem >> lane) & 1u) && ev > dn);
@@ -648,16 +653,23 @@ __global__ void __launch_bounds__(ListShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>
                     tb += static_cast<unsigned>(c * (pos - from));
                     // each slot's totals over its lanes, then to the job's lane
                     for (int off = M; off < 32; off <<= 1) {
-                        cz += __shfl_xor_sync(kFull, cz, off);
+                        if (!SEARCH_Z) cz += __shfl_xor_sync(kFull, cz, off);
                         cx += __shfl_xor_sync(kFull, cx, off);
                     }
-                    const int vz = __shfl_sync(kFull, cz, rank & 31);
+                    const int vz = SEARCH_Z ? 0 : __shfl_sync(kFull, cz, rank & 31);
                     const int vx = __shfl_sync(kFull, cx, rank & 31);
                     if ((rem >> lane) & 1u) {
                         nz += vz;
                         nxz += vx;
                     }
                     rem = still;
+                }
+                if (SEARCH_Z) {  // n_z, of the entries that the walk reached
+                    const int hi = pos < lb.len ? pos : lb.len;
+                    int lo = 0;
+                    for (int b = 1 << (31 - __clz(hi | 1)); b; b >>= 1)
+                        if (lo + b <= hi && entry_d(lb, lo + b - 1) < ev) lo += b;
+                    nz += lo;
                 }
             }
             // Jobs whose eps reaches past a list are left to ksg_scan_kernel.
