@@ -1137,6 +1137,27 @@ const idtx_ctx::Timed &best_way(const idtx_ctx::Trial &t, const Group &g)
     return t.way[best];
 }
 
+// What a trial for g times.  Not the tile kernel where the list kernel is always
+// the faster: with up to 1023 samples (tile over list time, 65 to 1000 samples,
+// 13 shapes, 0 to 300 surrogates: 1.1 to 3.7), and without z (257 to 10000
+// samples, also of few values: 1.4 to 14).  Unless the capacities are fixed by
+// the caller, from 512 samples on also lists of a half, a quarter and an eighth:
+// which wins depends on how many jobs reach past them (of eleven calls, steps
+// and batches an eighth, 256 and 512, took up to 13 % off some).
+constexpr int kAlwaysLists = 1023, kNeverLists = 64, kShorterLists = 512;
+std::vector<idtx_ctx::Timed> ways_of(const idtx_ctx *c, const Group &g)
+{
+    std::vector<idtx_ctx::Timed> way;
+    const bool fixed = c->cap_a != 0 || c->cap_b != 0;
+    if ((g.n > kAlwaysLists || fixed) && g.b_form != 2) way.push_back({false, 0, 0, 0.0f, 0.0f});
+    way.push_back({true, g.cap_a, g.cap_b, 0.0f, 0.0f});
+    for (int sh = 1; sh <= 3 && !fixed && !g.iv_a && g.n >= kShorterLists; ++sh) {
+        const int ca = (g.cap_a >> sh) / 32 * 32, cb = (g.cap_b >> sh) / 32 * 32;
+        if (ca >= 256 && (cb >= 256 || g.b_form)) way.push_back({true, ca, cb, 0.0f, 0.0f});
+    }
+    return way;
+}
+
 void take_way(Group &g, const idtx_ctx::Timed &w)
 {
     g.use_list = w.list;
@@ -1182,9 +1203,13 @@ int plan(idtx_ctx *c, Group &g)
         if (g.b_form) g.cap_b = 0;
         if (g.iv_a) g.cap_a = 32;  // unused
         if (g.cap_a > 0) {
+            // (few samples: the tile kernel's one launch is shorter than the list
+            // kernel's chain; no trial where there is one way only)
             if (c->kernel_pref == IDTX_KERNEL_LIST) {
                 g.use_list = true;
-            } else {
+            } else if (g.n > kNeverLists && ways_of(c, g).size() == 1) {
+                g.use_list = true;
+            } else if (g.n > kNeverLists) {
                 auto it = c->tuned.find(tune_key(g));
                 if (it == c->tuned.end()) {
                     g.tune = true;
@@ -1667,28 +1692,19 @@ void note_group(idtx_ctx *c, const Group &g, int launches, bool list)
 }
 
 // Time the candidate ways of running a prepared group -- the tile kernel, and
-// the list kernel with the group's list capacities and with two smaller ones
+// the list kernel with the group's list capacities and smaller ones (ways_of)
 // -- and remember the times for this (variant, log2 N).  Every candidate
 // writes the same partial sums.  On return the lists in the buffer, and a's
 // capacities, are those of the choice.
 int tune_group(idtx_ctx *c, const Group &g, KsgLaunch &a, cudaStream_t st, bool &use_list)
 {
-    idtx_ctx::Trial trial{g.n, g.n_groups, {{false, 0, 0, 0.0f, 0.0f}, {true, g.cap_a, g.cap_b, 0.0f, 0.0f}}};
+    idtx_ctx::Trial trial{g.n, g.n_groups, ways_of(c, g)};
     std::vector<idtx_ctx::Timed> &way = trial.way;
-    // Capacities not fixed by the caller: also lists of a half, a quarter and an
-    // eighth.  Which wins depends on how many jobs reach past them: of eleven calls,
-    // steps and batches an eighth (256, 512) took up to 13 % off some.
-    if (c->cap_a == 0 && c->cap_b == 0 && !g.iv_a)
-        for (int sh = 1; sh <= 3; ++sh) {
-            const int ca = (g.cap_a >> sh) / 32 * 32, cb = (g.cap_b >> sh) / 32 * 32;
-            if (ca >= 256 && (cb >= 256 || g.b_form)) way.push_back({true, ca, cb, 0.0f, 0.0f});
-        }
     const KsgVariant &v = *g.v;
     KsgLaunch t = a;
     t.work = nullptr;
     auto build = [&](int ca, int cb) -> int {
         int built = 0;
-        if (g.iv_a) return IDTX_OK;
         IDTX_CUDA(build_lists(a.sh, v.dz, v.dy, g.dz, g.dy, g.n, ca, cb, const_cast<int2 *>(a.list_a),
                               const_cast<int2 *>(a.list_b), const_cast<int4 *>(a.lmeta),
                               a.lscratch, st, &built));
@@ -1712,7 +1728,7 @@ int tune_group(idtx_ctx *c, const Group &g, KsgLaunch &a, cudaStream_t st, bool 
         IDTX_CUDA(cudaEventElapsedTime(&way[i].build_ms, ev[2 * i], ev[2 * i + 1]));
         IDTX_CUDA(cudaEventElapsedTime(&way[i].est_ms, ev[2 * i + 1], ev[2 * i + 2]));
     }
-    way[0].build_ms = 0.0f;
+    if (!way[0].list) way[0].build_ms = 0.0f;
     for (auto &e : ev) c->event_pool.push_back(e);
     const idtx_ctx::Timed b = best_way(trial, g);
     use_list = b.list;
