@@ -896,6 +896,7 @@ struct WorkShape {
 
 struct idtx_ctx {
     int device = 0;
+    int n_sms = 0;
     void *buf[kNumBufs] = {};
     size_t cap[kNumBufs] = {};
     long long *psi = nullptr;
@@ -1120,15 +1121,22 @@ std::pair<const KsgVariant *, int> tune_key(const Group &g)
 // Building lists and the tile kernel grow as n^2, the walks as n; the
 // estimators with the job groups, while the lists are built once for all of
 // them: a call of few groups may want the tile kernel or shorter lists where
-// one of many groups does not.
-const idtx_ctx::Timed &best_way(const idtx_ctx::Trial &t, const Group &g)
+// one of many groups does not.  A call that leaves SMs idle takes no less than
+// one that fills them: a query and job group is a warp's work in the list kernel
+// (32 a SM), an eighth of one in the tile kernel (64 a SM at least).
+const idtx_ctx::Timed &best_way(const idtx_ctx *c, const idtx_ctx::Trial &t, const Group &g)
 {
-    const float rn = (float)g.n / (float)t.n, rg = (float)g.n_groups / (float)t.groups;
+    const float rn = (float)g.n / (float)t.n;
+    auto grown = [&](bool list) {  // the estimator's work against the trial's
+        const float full = (float)c->n_sms * (list ? 32.0f : 64.0f);
+        return std::max((float)g.n * g.n_groups, full) / std::max((float)t.n * t.groups, full) *
+               (list ? 1.0f : rn);
+    };
     size_t best = 0;
     float best_ms = 0.0f;
     for (size_t i = 0; i < t.way.size(); ++i) {
         const idtx_ctx::Timed &w = t.way[i];
-        const float ms = w.build_ms * rn * rn + w.est_ms * rg * (w.list ? rn : rn * rn);
+        const float ms = w.build_ms * rn * rn + w.est_ms * grown(w.list);
         if (i == 0 || ms < best_ms) {
             best = i;
             best_ms = ms;
@@ -1214,7 +1222,7 @@ int plan(idtx_ctx *c, Group &g)
                 if (it == c->tuned.end()) {
                     g.tune = true;
                 } else {
-                    take_way(g, best_way(it->second, g));
+                    take_way(g, best_way(c, it->second, g));
                 }
             }
         }
@@ -1639,7 +1647,7 @@ int prep_group(idtx_ctx *c, const Group &g, cudaStream_t st, const Slices &sl, f
         IDTX_TRY(init_gather_cols());
         // rows per CTA: enough to be worth the columns, and CTAs to fill the SMs
         const int64_t tiles = g.n_pad / kGatherRows;
-        const int64_t chunks = std::max<int64_t>(1, std::min<int64_t>(tiles / 16, 152 * 8 / g.n_groups));
+        const int64_t chunks = std::max<int64_t>(1, std::min<int64_t>(tiles / 16, c->n_sms * 8 / g.n_groups));
         const int chunk_rows = (int)((tiles + chunks - 1) / chunks) * kGatherRows;
         k_gather_cols<<<dim3((unsigned)((g.n_pad + chunk_rows - 1) / chunk_rows), (unsigned)g.n_groups),
                         kColsThreads, gather_cols_smem(g.n), xs>>>(
@@ -1730,7 +1738,7 @@ int tune_group(idtx_ctx *c, const Group &g, KsgLaunch &a, cudaStream_t st, bool 
     }
     if (!way[0].list) way[0].build_ms = 0.0f;
     for (auto &e : ev) c->event_pool.push_back(e);
-    const idtx_ctx::Timed b = best_way(trial, g);
+    const idtx_ctx::Timed b = best_way(c, trial, g);
     use_list = b.list;
     if (b.list) {
         // the lists in the buffer are the last candidate's
@@ -2019,7 +2027,7 @@ int resolve_tuning(idtx_ctx *c, std::vector<Group> &gs, cudaStream_t st, long lo
             IDTX_TRY(tune_group(c, g, a, st, unused));
             c->stats.kernel_launches += launches - 2;
         }
-        take_way(g, best_way(c->tuned[tune_key(g)], g));
+        take_way(g, best_way(c, c->tuned[tune_key(g)], g));
         g.tune = false;
     }
     return IDTX_OK;
@@ -2179,7 +2187,8 @@ int idtx_ctx_create(idtx_ctx **out, int device)
     KsgVariant tmp[kMaxVariants];
     const int n = ksg_variants(tmp);
     c->variants.assign(tmp, tmp + n);
-    cudaError_t e = cudaMalloc(&c->d_err, kStatusBytes);
+    cudaError_t e = cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, device);
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_err, kStatusBytes);
     if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, kStatusBytes);
     if (e == cudaSuccess) e = cudaMallocHost(&c->h_status, kStatusBytes);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking);

@@ -31,3 +31,20 @@ def test_trials(n, dims, k, trials):
     assert ctx.stats()["tune_trials"] == trials
     ref = oracle.cmi_surrogates(g.x, g.y, z, k, 5, 2)
     assert np.max(np.abs(got.cpu().numpy() - ref)) < 1e-10
+
+
+def test_a_call_of_one_estimate_after_a_trial_of_many():
+    """A trial's times of 32 job groups do not fall to a 32nd for one group, which
+    leaves most SMs idle: the lists, half as long as the tile kernel there, are
+    still taken."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1807_10459_gb300 as idtx
+    g = synth.gaussian_problem(2000, 1, 1, 2, seed=3)
+    dev = [_dev(v) for v in (g.x, g.y, g.z)]
+    ctx = idtx.Context(0)
+    idtx.cmi_ksg(*dev, k=4, n_surr=1000, seed=2, ctx=ctx)
+    ctx.reset_stats()
+    idtx.cmi_ksg(*dev, k=4, n_surr=0, seed=2, ctx=ctx)
+    st = ctx.stats()
+    assert st["tune_trials"] == 0 and st["list_launches"] == 1
