@@ -130,7 +130,7 @@ __device__ __forceinline__ int get_count(const void *c, int64_t at, int wide)
 
 // The digamma terms of the list kernel's counts, summed into partial: query
 // tiles of qc queries (sums.cu).
-cudaError_t sum_terms(const KsgLaunch &a, int qc, int n_groups, cudaStream_t st);
+cudaError_t sum_terms(const KsgLaunch &a, int qc, int n_groups, int n_sms, cudaStream_t st);
 
 typedef cudaError_t (*KsgLaunchFn)(const KsgLaunch &, int n_groups, cudaStream_t);
 

@@ -1189,7 +1189,7 @@ cudaError_t launch_ksg_list(const KsgLaunch &all, int n_groups, cudaStream_t str
             a, groups, static_cast<int>(chunks), chunk);
         scan<<<static_cast<unsigned>(n_sms[dev]), kScanWarps * 32, kScanSmem, stream>>>(a);
         e = cudaGetLastError();
-        if (e == cudaSuccess) e = sum_terms(a, QC, groups, stream);
+        if (e == cudaSuccess) e = sum_terms(a, QC, groups, n_sms[dev], stream);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

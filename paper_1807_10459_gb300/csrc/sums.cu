@@ -102,14 +102,14 @@ __global__ void k_sum_terms(const KsgLaunch a, int qc, int64_t n_tasks)
 }
 
 template <typename Four>
-cudaError_t launch_sum(const KsgLaunch &a, int qc, int64_t n_tasks, cudaStream_t st)
+cudaError_t launch_sum(const KsgLaunch &a, int qc, int64_t n_tasks, int n_sms, cudaStream_t st)
 {
-    // With the table: as many blocks as an SM holds on 152 of them, when each
-    // then has at least four tiles to take.
-    constexpr int64_t kBlocks = 152 * 8;
+    // With the table: as many blocks as the SMs hold, when each then has at
+    // least four tiles to take.
+    const int64_t blocks = n_sms * 8;
     const unsigned threads = (unsigned)(qc / kRowsPerWarp * 32);
-    if (n_tasks >= 4 * kBlocks)
-        k_sum_terms<Four, true><<<(unsigned)kBlocks, threads, kTable * sizeof(long long), st>>>(a, qc, n_tasks);
+    if (n_tasks >= 4 * blocks)
+        k_sum_terms<Four, true><<<(unsigned)blocks, threads, kTable * sizeof(long long), st>>>(a, qc, n_tasks);
     else
         k_sum_terms<Four, false><<<(unsigned)n_tasks, threads, 0, st>>>(a, qc, n_tasks);
     return cudaGetLastError();
@@ -117,11 +117,11 @@ cudaError_t launch_sum(const KsgLaunch &a, int qc, int64_t n_tasks, cudaStream_t
 
 }  // namespace
 
-cudaError_t sum_terms(const KsgLaunch &a, int qc, int n_groups, cudaStream_t st)
+cudaError_t sum_terms(const KsgLaunch &a, int qc, int n_groups, int n_sms, cudaStream_t st)
 {
     static_assert(64 % kRowsPerWarp == 0, "tiles of up to 64 queries, a multiple of 8");
     const int64_t tasks = (int64_t)a.n_qt * n_groups;
-    return a.wide ? launch_sum<uint4>(a, qc, tasks, st) : launch_sum<uint2>(a, qc, tasks, st);
+    return a.wide ? launch_sum<uint4>(a, qc, tasks, n_sms, st) : launch_sum<uint2>(a, qc, tasks, n_sms, st);
 }
 
 }  // namespace idtx
