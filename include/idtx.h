@@ -115,8 +115,8 @@ int idtx_version(void);
 
 /* Counters of a context, for measurement (no counterpart in the paper: they
  * report what the library did).  kernel_launches counts every kernel the
- * library enqueued; the fused_* fields cover the fused estimator kernel
- * only: its launches, its device time (CUDA events recorded on the caller's
+ * library enqueued (a sort of CUB's as one); the fused_* fields cover the fused
+ * estimator kernel only: its launches, its device time (CUDA events recorded on the caller's
  * stream around each launch, only while profiling is enabled), and its
  * algorithmic lane operations: for every (query, reference sample, group of
  * jobs sharing Y and Z) that the kernel scans, 2(dy+dz')+1 operations in the

@@ -1295,6 +1295,8 @@ int count_groups(const Group &g)
 {
     return (int)std::min<size_t>(g.n_groups, std::max<size_t>(1, kCountBudget / group_count_bytes(g)));
 }
+// Kernels of a list estimate: the walk, the scans and the sums, turn by turn.
+int list_launches(const Group &g) { return 3 * ((g.n_groups + count_groups(g) - 1) / count_groups(g)); }
 size_t count_bytes(const Group &g) { return align_up(count_groups(g) * group_count_bytes(g), 256); }
 
 // The sorted source columns of a call without z, part of B_LIST.
@@ -1695,7 +1697,7 @@ void note_group(idtx_ctx *c, const Group &g, int launches, bool list)
     if ((int)c->call_shapes.size() <= g.work_slot) c->call_shapes.resize(g.work_slot + 1);
     c->call_shapes[g.work_slot] = ws;
     c->stats.fused_launches += 1;
-    c->stats.kernel_launches += launches;
+    c->stats.kernel_launches += launches + (list ? list_launches(g) - 1 : 0);  // (one is counted as the estimator)
     if (list && g.dz > 0) c->stats.list_launches += 1;  // (without z there is no list B)
 }
 
@@ -1748,7 +1750,7 @@ int tune_group(idtx_ctx *c, const Group &g, KsgLaunch &a, cudaStream_t st, bool 
         a.cap_b = b.cap_b;
     }
     c->stats.tune_trials += 1;
-    c->stats.kernel_launches += (int64_t)way.size();  // the estimator launches
+    for (const idtx_ctx::Timed &w : way) c->stats.kernel_launches += w.list ? list_launches(g) : 1;
     c->tuned[tune_key(g)] = std::move(trial);
     return IDTX_OK;
 }
