@@ -140,7 +140,8 @@ typedef struct {
     double exhaustive_pairs;
     double wait_cycles, warp_cycles;
     int64_t graph_launches;  /* calls served by replaying a captured graph */
-    /* List kernel (see idtx_ctx_set_kernel): launches, list entries walked in
+    /* List kernel (see idtx_ctx_set_kernel): launches that walk neighbour
+     * lists (all count in fused_launches), list entries walked in
      * the neighbour pass (list A) and the count pass (list B) per (query,
      * group of 32 jobs), samples scanned by full-scan fallbacks, fallbacks
      * taken (a (query, group) whose lists did not cover some job), and
@@ -218,10 +219,11 @@ int idtx_ctx_set_graphs(idtx_ctx *ctx, int enable);
  *     capacity; each estimate then walks only the prefix it needs, with a
  *     full scan for a (query, estimate) whose neighbourhood the lists do not
  *     cover.  With n in (256, 65536] and one z column the samples' order by
- *     it takes the place of the lists by Z distance; without z, counts in
- *     sorted columns take that of both counts' walks (dx = 1; these launches
- *     are not counted as list_launches).  Other dz = 0 calls use the tile
- *     kernel.
+ *     it takes the place of the lists by Z distance; without z and with dx = 1,
+ *     counts in sorted columns take that of both counts' walks, and with dy = 1
+ *     the samples' order by y that of the lists by (Y,Z) distance (such a call
+ *     has no lists, and does not count as one of list_launches).  Other dz = 0
+ *     calls use the tile kernel.
  *   IDTX_KERNEL_AUTO (default): the tile kernel up to 64 samples, the list
  *     kernel up to 511 and without z (where it is always the faster one); else
  *     on the first call of a shape (kernel variant, floor(log2 N)) both

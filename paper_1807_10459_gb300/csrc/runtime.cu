@@ -1698,7 +1698,7 @@ void note_group(idtx_ctx *c, const Group &g, int launches, bool list)
     c->call_shapes[g.work_slot] = ws;
     c->stats.fused_launches += 1;
     c->stats.kernel_launches += launches + (list ? list_launches(g) - 1 : 0);  // (one is counted as the estimator)
-    if (list && g.dz > 0) c->stats.list_launches += 1;  // (without z there is no list B)
+    if (list && !g.iv_a) c->stats.list_launches += 1;  // (those have no lists)
 }
 
 // Time the candidate ways of running a prepared group -- the tile kernel, and

@@ -1,4 +1,5 @@
-"""The launch counters: kernel_launches against the profiler's count of kernels."""
+"""The launch counters: kernel_launches against the profiler's count of kernels,
+list_launches where one of a call's two lists is missing."""
 import numpy as np
 import pytest
 
@@ -12,8 +13,9 @@ def _dev(a):
     return None if a is None else torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
-@pytest.mark.parametrize("dims", [(1, 1, 2), (2, 1, 1), (1, 1, 0), (1, 2, 0)])
-def test_launches_are_counted(dims):
+@pytest.mark.parametrize("dims,listed", [((1, 1, 2), 1), ((2, 1, 1), 1), ((1, 1, 0), 0),
+                                         ((1, 2, 0), 1)])
+def test_launches_are_counted(dims, listed):
     """At most 4096 samples, where a sort of CUB's is one kernel."""
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
@@ -42,3 +44,4 @@ def test_launches_are_counted(dims):
         kernels = [n for n in names if not n.startswith("Mem")]
         assert st["kernel_launches"] == len(kernels), kernels
         assert st["fused_launches"] == 1
+        assert st["list_launches"] == (listed if kernel == idtx.KERNEL_LIST else 0)
