@@ -171,10 +171,10 @@ struct KsgVariant {
 };
 
 // Per-query sorted neighbour lists of a group prepared into sh (lists.cu):
-// rows of dzb z columns, then dyb y columns (dz and dy of them used).  scratch: list_scratch_bytes(n,
-// cap_a, cap_b), which also covers smaller capacities.  *launches (nullable)
-// receives the kernels launched.  n <= 0 only sets kernel attributes.
-size_t list_scratch_bytes(int64_t n, int cap_a, int cap_b);
+// rows of dzb z columns, then dyb y columns (dz and dy of them used).
+// scratch: list_scratch_bytes(n, cap_a, cap_b) (list_scratch.cuh), which also
+// covers smaller capacities.  *launches (nullable) receives the kernels
+// launched.  n <= 0 only sets kernel attributes.
 cudaError_t build_lists(const float *sh, int dzb, int dyb, int dz, int dy, int64_t n, int cap_a,
                         int cap_b, int2 *list_a, int2 *list_b, int4 *meta, void *scratch, cudaStream_t st,
                         int *launches);

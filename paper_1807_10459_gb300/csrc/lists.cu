@@ -29,6 +29,7 @@
 #include <type_traits>
 
 #include "ksg_common.cuh"
+#include "list_scratch.cuh"
 
 namespace idtx {
 
@@ -701,38 +702,10 @@ cudaError_t sort_lists(const SortPair &p, int n_q, int lists, int buf, cudaStrea
     return launch_sort<512, 12, 4096>(p, n_q, lists, buf, st);
 }
 
-// Scratch entries per query of a list (see the sampling above), or every sample.
-int buf_of(int cap, int64_t n)
-{
-    const int64_t all = (n + 31) / 32 * 32;
-    return (int)std::max<int64_t>(64, std::min<int64_t>(cap >= 2048 ? cap + cap / 2 : 2 * cap, all));
-}
 static_assert(kMaxListB + kMaxListB / 2 <= 512 * 12, "the largest buffer");
-
-size_t query_scratch(int64_t n, int cap_a, int cap_b)
-{
-    return ((size_t)buf_of(cap_a, n) + buf_of(cap_b, n)) * sizeof(int2) + sizeof(int4);
-}
-
-// Scratch of one chunk of queries: enough of them to fill the GPU several
-// times over, without another list-sized buffer for large n.
-constexpr size_t kScratchBudget = size_t(5) << 28;
-constexpr int64_t kMinChunk = 4096;
-
-int64_t chunk_of(int64_t n, int cap_a, int cap_b)
-{
-    const int64_t fit = (int64_t)(kScratchBudget / query_scratch(n, cap_a, cap_b));
-    return std::min(n, std::max(kMinChunk, fit / kTJ * kTJ));  // whole tiles: warps share their home tile
-}
+static_assert(kScratchTile == kTJ && kListEntry == sizeof(int2) && kListMeta == sizeof(int4), "list_scratch.cuh");
 
 }  // namespace
-
-// Enough for these capacities and for any smaller ones.
-size_t list_scratch_bytes(int64_t n, int cap_a, int cap_b)
-{
-    const size_t per = query_scratch(n, cap_a, cap_b);
-    return std::min((size_t)n * per, std::max(kScratchBudget, (size_t)kMinChunk * per)) + 512;
-}
 
 cudaError_t build_lists(const float *sh, int dzb, int dyb, int dz, int dy, int64_t n, int cap_a, int cap_b,
                         int2 *list_a, int2 *list_b, int4 *meta, void *scratch, cudaStream_t st,

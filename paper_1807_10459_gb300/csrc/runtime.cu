@@ -29,6 +29,7 @@
 
 #include "idtx.h"
 #include "ksg_common.cuh"
+#include "list_scratch.cuh"
 #include "shuffle.cuh"
 
 namespace idtx {
