@@ -1035,6 +1035,20 @@ bool device_accessible(const void *p)
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// Whether k_finalize may store its results at p: aligned memory of this device
+// (another one's is out of a kernel's reach without peer access, but not out of
+// a copy's).
+bool storable(const double *p, int device)
+{
+    cudaPointerAttributes at;
+    if (!p || (uintptr_t)p % alignof(double) != 0) return false;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == device;
+}
+
 const int kZBuckets[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16};
 
 // The specialisation for a call's dimensions and k: its own (k = 4), else the
@@ -2366,7 +2380,7 @@ static int cmi_ksg_impl(idtx_ctx *c, const float *x, int dx, const float *y, int
     sizes_of(g, b);
     const bool eps_dev = eps_out && device_accessible(eps_out);
     const bool cnt_dev = counts_out && device_accessible(counts_out);
-    const bool cmi_dev = device_accessible(cmi_out);
+    const bool cmi_stored = storable(cmi_out, c->device);
     IDTX_TRY(ensure(c, B_DESC, arena.size()));
     IDTX_TRY(ensure(c, B_SH, b.sh));
     IDTX_TRY(ensure(c, B_XI, b.xi));
@@ -2384,11 +2398,12 @@ static int cmi_ksg_impl(idtx_ctx *c, const float *x, int dx, const float *y, int
                               st));
     float *eps_d = eps_out ? (eps_dev ? eps_out : (float *)c->buf[B_EPS]) : nullptr;
     int32_t *cnt_d = counts_out ? (cnt_dev ? counts_out : (int32_t *)c->buf[B_CNT]) : nullptr;
-    double *cmi_d = cmi_dev ? cmi_out : (double *)c->buf[B_CMI];
+    double *cmi_d = cmi_stored ? cmi_out : (double *)c->buf[B_CMI];
     IDTX_TRY(enqueue_group(c, g, st, cmi_d, eps_d, cnt_d, timeout_of(c, s)));
-    if (!cmi_dev)
+    if (!cmi_stored)
         IDTX_CUDA(cudaMemcpyAsync(cmi_out, cmi_d, (size_t)n_jobs * sizeof(double),
-                                  cudaMemcpyDeviceToHost, st));
+                                  device_accessible(cmi_out) ? cudaMemcpyDeviceToDevice
+                                                             : cudaMemcpyDeviceToHost, st));
     if (eps_out && !eps_dev)
         IDTX_CUDA(cudaMemcpyAsync(eps_out, eps_d, (size_t)n_jobs * n * sizeof(float),
                                   cudaMemcpyDeviceToHost, st));
