@@ -1243,6 +1243,20 @@ int plan(idtx_ctx *c, Group &g)
         }
         if (!g.use_list && !g.tune) g.iv_a = g.b_form = 0;
     }
+    // Few CTAs of the tile kernel: the generic specialisation has 16 queries a
+    // CTA, those of k <= 7 have 64, so where its CTAs just fill the SMs it is the
+    // faster for all its padding, if there is little else to gain: without z
+    // every pair is visited, and the widest z bucket is its own.  k = 3, dx = 2, no
+    // z, one group, N = 500, 1000, 2000: 293, 430, 730 us by 64 and 289, 407, 626
+    // by 16; N = 300 and 3000: 249 and 1078 against 279 and 1429.
+    if (!g.use_list && !g.tune && !g.plain && !g.v->exact && (g.dz == 0 || g.v->dz == IDTX_MAX_DZ) &&
+        g.n > 384) {
+        const KsgVariant *w = &c->variants.back();
+        if ((g.n_pad / w->qc) * g.n_groups <= c->n_sms) {
+            g.v = w;
+            g.n_qt = (int)(g.n_pad / w->qc);
+        }
+    }
     return IDTX_OK;
 }
 

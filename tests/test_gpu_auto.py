@@ -16,7 +16,8 @@ def _dev(a):
 @pytest.mark.parametrize("n,dims,k,trials", [(64, (1, 1, 2), 4, 0), (65, (1, 1, 2), 4, 0),
                                              (511, (2, 1, 1), 3, 0), (512, (1, 1, 2), 4, 1),
                                              (2000, (1, 1, 0), 4, 0), (2000, (1, 2, 0), 4, 1),
-                                             (2000, (2, 1, 0), 4, 0)])
+                                             (2000, (2, 1, 0), 4, 0), (385, (2, 1, 0), 3, 0),
+                                             (2430, (2, 2, 0), 7, 0), (2433, (2, 2, 0), 7, 0)])
 def test_trials(n, dims, k, trials):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
