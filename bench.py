@@ -33,11 +33,11 @@ METRIC = "KSG CMI estimates/s incl. surrogates (N=1e4,k=4); batched/screened vs 
 # Tile kernel: profiles/ksg_fused_kernel_greedy_step_small.md (15-surrogate case,
 # 31.68 MB, scaled by job groups 296/24).  List kernel: captured directly on the
 # full-size launch (profiles/ksg_list_kernel_greedy_step_small.md).
-TRAFFIC_BYTES = {"tile": 390.7e6, "list": 3180.0e6 + 564.7e6}
+TRAFFIC_BYTES = {"tile": 390.7e6, "list": 3240.0e6 + 564.8e6}
 # Pipe utilisation of the list kernel from its committed full ncu capture
 # (small case of the same step; profiles/ksg_list_kernel_greedy_step_small.md).
-PIPES_FROM_PROFILE = {"alu_pct": 46.7, "fma_pct": 30.2, "lsu_pct": 34.4, "issue_active_pct": 71.1,
-                      "l1_hit_pct": 67.9, "unit": "% of each pipe's peak, sustained active",
+PIPES_FROM_PROFILE = {"alu_pct": 47.7, "fma_pct": 30.1, "lsu_pct": 34.9, "issue_active_pct": 71.4,
+                      "l1_hit_pct": 67.5, "unit": "% of each pipe's peak, sustained active",
                       "source": "profiles/ksg_list_kernel_greedy_step_small.md"}
 
 WORKLOAD = dict(n_proc=10, order=5, T=10000, n_past=3, min_lag=1, max_lag=5, k=4, n_surr=200,

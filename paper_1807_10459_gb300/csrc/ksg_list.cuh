@@ -58,14 +58,17 @@
 //     capacity); with none and one y column the order is by y and stands for
 //     list A.  Without z, n_z is all and n_xz with one x column is a range of
 //     the sorted column.  The call, by the tile kernel and so: N = 3001, no z,
-//     201 estimates, 1.92 and 0.32 ms; N = 20000, 49.4 and 2.5; one z, N = 3001,
-//     0.73 and 0.52 (0.95 with a list B); N = 50000, 101 estimates, 29.6 and 14.6.
+//     201 estimates, 1.93 and 0.32 ms; N = 20000, 48.5 and 2.2; one z, N = 3001,
+//     0.65 and 0.50 (0.95 with a list B); N = 50000, 101 estimates, 23.1 and 11.5
+//     (on data of few values the tile kernel is up to a tenth slower in this
+//     order than along a Morton curve, on continuous data faster by up to two
+//     thirds).
 // Measured on GB300, greedy step of N = 9995 with 9447 estimates (one network;
 // lists of 2048 and 4096), against summing the terms in the kernel and scanning
 // in place: 19.1 -> 12.7 ms; of N = 4997, six conditions, 28341 estimates: 10.8
 // -> 8.5 ms; N = 1000, 101 estimates: 163 -> 24 us (each with sum_terms' 0.27,
 // 0.38 ms and 4 us to add).  Bound by issue (71 % of the slots in a capture of 752
-// estimates) and L1 (78 % of its rate): fewer, fatter warps (24 of 80 registers)
+// estimates) and L1 (80 % of its rate): fewer, fatter warps (24 of 80 registers)
 // were 8 % slower.
 #pragma once
 
@@ -178,15 +181,14 @@ __device__ __forceinline__ float warp_max_nn(float v)
 }
 
 // Launch shape of the list kernel for one specialisation.  QC: the tile
-// kernel's queries per CTA, which fix the partial-sum layout (one partial per QC
-// queries).
+// kernel's queries per CTA: sum_terms writes one partial sum per QC queries.
 template <int DX, int DY, int DZ, int K1, bool EXACT, int QCTA, int NWARPS>
 struct ListShape {
     using S = KsgShape<DX, DY, DZ, K1, EXACT, QCTA, NWARPS>;
     static constexpr int QC = S::QC;
     // 32 warps (64 registers a thread) for the small specialisations; 16
     // warps give the wide runtime-k one 128 registers.
-        static constexpr int NW = (DX > 2 || K1 > 8) ? 16 : 32;
+    static constexpr int NW = (DX > 2 || K1 > 8) ? 16 : 32;
     static constexpr int THREADS = NW * 32;
     static_assert(QC <= 64, "sum_terms takes tiles of up to 64 queries");
     struct Smem {

@@ -358,7 +358,8 @@ __global__ void __launch_bounds__(kCollectThreads, QW == 1 ? 4 : (DZ + DY <= 12 
 constexpr int kBigBin = 16;  // bins above this are sorted by the whole block
 // Bins to sort in place that a block lists (more are found again by a walk over
 // all bins).  Short: three blocks of the largest lists take 195.6 of the 196 KB
-// that leave the other 60 to L1 (with room for all bins it sorted 6 % slower).
+// that leave the other 60 to L1 (with room for all bins it sorted 6 % slower, as it
+// is 3 than without a list).
 constexpr int kUnequal = 64;
 
 struct SortArgs {

@@ -1,7 +1,7 @@
 // sort.cu -- the library's one use of a vendor primitive: CUB's device radix
 // sort, of (32-bit key, int32 index) pairs to order the samples before the
-// estimator runs, and of a single short column's values for counts in it.  Kept in its own
-// translation unit so the template instantiations compile in parallel.
+// estimator runs, and of a single short column's values for counts in it.  Kept
+// in its own translation unit so the template instantiations compile in parallel.
 #include <cub/device/device_radix_sort.cuh>
 
 #include "ksg_common.cuh"
