@@ -224,13 +224,13 @@ int idtx_ctx_set_graphs(idtx_ctx *ctx, int enable);
  *     the samples' order by y that of the lists by (Y,Z) distance (such a call
  *     has no lists, and does not count as one of list_launches).  Other dz = 0
  *     calls use the tile kernel.
- *   IDTX_KERNEL_AUTO (default): the tile kernel up to 64 samples, the list
- *     kernel up to 511 and without z (where it is always the faster one); else
- *     on the first call of a shape (kernel variant, floor(log2 N)) both
- *     kernels run (from 1024 samples on), or the list kernel with several
- *     capacities, timed, and from then on in this context the way serves a
- *     call of that shape that is the fastest by these times, scaled to the
- *     call's N and number of estimates.
+ *   IDTX_KERNEL_AUTO (default): the list kernel for 65 to 511 samples and
+ *     without z (where it is always the faster one); else on the first call of
+ *     a shape (kernel variant, floor(log2 N)) both kernels run, or, from 512
+ *     to 1023 samples, the list kernel with several capacities, timed, and
+ *     from then on in this context the way serves a call of that shape that is
+ *     the fastest by these times, scaled to the call's N and number of
+ *     estimates.
  * Returns IDTX_EINVAL for a NULL ctx or an unknown value. */
 #define IDTX_KERNEL_AUTO 0
 #define IDTX_KERNEL_TILE 1

@@ -1161,18 +1161,18 @@ const idtx_ctx::Timed &best_way(const idtx_ctx *c, const idtx_ctx::Trial &t, con
 }
 
 // What a trial for g times.  Not the tile kernel where the list kernel is always
-// the faster: with up to 1023 samples (tile over list time, 65 to 1000 samples,
-// 13 shapes, 0 to 300 surrogates: 1.1 to 3.7), and without z (257 to 10000
+// the faster: with 65 to 1023 samples (tile over list time, 129 to 1000 samples,
+// 13 shapes, 0 to 300 surrogates: 1.1 to 3.7; 40 samples: 0.84 to 1.27), and without z (257 to 10000
 // samples, also of few values: 1.4 to 14).  Unless the capacities are fixed by
 // the caller, from 512 samples on also lists of a half, a quarter and an eighth:
 // which wins depends on how many jobs reach past them (of eleven calls, steps
 // and batches an eighth, 256 and 512, took up to 13 % off some).
-constexpr int kAlwaysLists = 1023, kNeverLists = 64, kShorterLists = 512;
+constexpr int kListsFrom = 65, kListsTo = 1023, kShorterLists = 512;
 std::vector<idtx_ctx::Timed> ways_of(const idtx_ctx *c, const Group &g)
 {
     std::vector<idtx_ctx::Timed> way;
     const bool fixed = c->cap_a != 0 || c->cap_b != 0;
-    if ((g.n > kAlwaysLists || fixed) && g.b_form != 2) way.push_back({false, 0, 0, 0.0f, 0.0f});
+    if ((g.n < kListsFrom || g.n > kListsTo || fixed) && g.b_form != 2) way.push_back({false, 0, 0, 0.0f, 0.0f});
     way.push_back({true, g.cap_a, g.cap_b, 0.0f, 0.0f});
     for (int sh = 1; sh <= 3 && !fixed && !g.iv_a && g.n >= kShorterLists; ++sh) {
         const int ca = (g.cap_a >> sh) / 32 * 32, cb = (g.cap_b >> sh) / 32 * 32;
@@ -1226,13 +1226,10 @@ int plan(idtx_ctx *c, Group &g)
         if (g.b_form) g.cap_b = 0;
         if (g.iv_a) g.cap_a = 32;  // unused
         if (g.cap_a > 0) {
-            // (few samples: the tile kernel's one launch is shorter than the list
-            // kernel's chain; no trial where there is one way only)
-            if (c->kernel_pref == IDTX_KERNEL_LIST) {
+            // (no trial where there is one way only)
+            if (c->kernel_pref == IDTX_KERNEL_LIST || ways_of(c, g).size() == 1) {
                 g.use_list = true;
-            } else if (g.n > kNeverLists && ways_of(c, g).size() == 1) {
-                g.use_list = true;
-            } else if (g.n > kNeverLists) {
+            } else {
                 auto it = c->tuned.find(tune_key(g));
                 if (it == c->tuned.end()) {
                     g.tune = true;
