@@ -1161,8 +1161,9 @@ const idtx_ctx::Timed &best_way(const idtx_ctx *c, const idtx_ctx::Trial &t, con
 }
 
 // What a trial for g times.  Not the tile kernel where the list kernel is always
-// the faster: with 65 to 1023 samples (tile over list time, 129 to 1000 samples,
-// 13 shapes, 0 to 300 surrogates: 1.1 to 3.7; 40 samples: 0.84 to 1.27), and without z (257 to 10000
+// the faster: with 65 to 1023 samples (tile over list time, 13 shapes, 0 to 300
+// surrogates: 40 samples 0.84 to 1.27, 65 0.94 to 1.38, 80 0.98 to 1.43, 100 to
+// 1000 1.03 to 3.7), and without z (257 to 10000
 // samples, also of few values: 1.4 to 14).  Unless the capacities are fixed by
 // the caller, from 512 samples on also lists of a half, a quarter and an eighth:
 // which wins depends on how many jobs reach past them (of eleven calls, steps
