@@ -1174,16 +1174,17 @@ cudaError_t launch_ksg_list(const KsgLaunch &all, int n_groups, cudaStream_t str
         if (a.eps_out) a.eps_out += j0 * all.n;
         if (a.cnt_out) a.cnt_out += j0 * 3 * all.n;
         if (a.jobs) a.jobs += j0;
-        // chunks of consecutive queries: eight per SM where that leaves 16 queries,
-        // else 16, or, if these would leave SMs without any, one per SM (the
-        // queries of a small call are one wave of warps: 21 estimates, one z
-        // column, dx = 3, N = 1000, 192 us in chunks of 16, 93 in 143 of 7; k = 4,
-        // two z columns, 23.8 and 20.9)
+        // Chunks of consecutive queries: eight per SM where that leaves 16 queries,
+        // else 16, or, if these would leave SMs without any, one per SM of at
+        // least four (the queries of a small call are one wave of warps: 21
+        // estimates, one z column, dx = 3, N = 1000, 192 us in chunks of 16, 93 in 143
+        // of 7; k = 4, two z columns, 23.8 and 20.9; one estimate, N = 129, 8.2 in
+        // chunks of 16, 7.4 of four, 12.9 of one, most of a CTA's warps in each
+        // other's way to it).
         const int64_t per = a.n * groups / (8 * n_sms[dev]);
         const int64_t one = (a.n * groups + n_sms[dev] - 1) / n_sms[dev];
-        const int chunk = static_cast<int>(per > IDTX_LIST_CHUNKQ ? IDTX_LIST_CHUNKQ
-                                           : per >= 16            ? per
-                                                                  : (one < 16 ? one : 16));
+        const int64_t few = one < 4 ? 4 : (one < 16 ? one : 16);
+        const int chunk = static_cast<int>(per > IDTX_LIST_CHUNKQ ? IDTX_LIST_CHUNKQ : (per >= 16 ? per : few));
         const int64_t chunks = groups * ((a.n + chunk - 1) / chunk);
         if (chunks > 0x3fffffff) return cudaErrorInvalidValue;  // the kernel's chunk arithmetic is 32-bit
         const int64_t grid = chunks < n_sms[dev] ? chunks : n_sms[dev];
